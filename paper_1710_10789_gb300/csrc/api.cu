@@ -124,7 +124,6 @@ static tetra_status_t plan_geometry(Plan &P, const int box[3], int ctas_per_sm) 
         P.tile_copies = (int)std::min<size_t>(8, 1 + room / copy);
         P.smem_bytes += (size_t)(P.tile_copies - 1) * copy;
     }
-    P.threads = pairs ? 384 : 512;
     const int ctas = std::max(1, ctas_per_sm) * P.sm_count;
     P.grid_x = std::max(1, std::min(P.n_boxes, (ctas + P.n_chunks - 1) / P.n_chunks));
     // Fixed-point fraction bits. A DOS value is a sum of N contributions of

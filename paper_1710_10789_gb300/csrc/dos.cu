@@ -23,8 +23,7 @@
 //    heavily, so one walk over the union of the two windows adds both
 //    tetrahedra's contributions at each energy before touching the shared
 //    tile: about half the shared-memory traffic of one tetrahedron each.
-//    (Integrated mode: each tetrahedron adds its weights below its own E4
-//    and puts its own saturation step.)
+//    (Integrated mode: beyond the union the pair puts one saturation step.)
 //  * Items of a box are ranked by window length (counting sort), so the 32
 //    lanes of a warp walk windows of nearly equal length.
 //  * Each visited energy adds sum_l b_{l,s} dw_l to the CTA's tile for every
@@ -48,6 +47,7 @@
 //    CTA's int64 partial in global memory before it could overflow.
 //  * tetra_dos_reduce sums the per-CTA int64 partials (exact) and scales by u;
 //    for a batch, each model's accumulator is scaled.
+#include <algorithm>
 #include <atomic>
 #include <memory>
 #include <new>
@@ -61,20 +61,21 @@ namespace {
 constexpr float kMagic = 12582912.0f;   // 1.5 * 2^23: float + kMagic rounds to an integer
 constexpr int kMagicBits = 0x4B400000;  // bit pattern of kMagic
 constexpr uint32_t kSmemAlign = 1024;
-// Work unit, threads per CTA and registers per thread. Point mode with up to
-// 8 orbitals walks face-sharing tetrahedron pairs, holding two tetrahedra's
-// weights and constants in registers; 16 orbitals would not fit, so there, as
-// in bin mode, a unit is one tetrahedron. Each of the SM's four
-// sub-partitions has 16K registers for its warps: 12 warps (3 per
-// sub-partition) can use 168 registers per thread, 16 warps 128.
-template <int MODE, int NORB>
+// Work unit, threads per CTA and registers per thread. With up to 8 orbitals
+// a unit is a face-sharing tetrahedron pair, holding two tetrahedra's weights
+// and constants in registers; 16 orbitals would not fit, so there a unit is
+// one tetrahedron. Each of the SM's four sub-partitions has 16K registers for
+// its warps: 16 warps can use 128 registers per thread. (A pair with 8
+// orbitals fits them since its corner derivatives need ten constants per
+// tetrahedron; 64^3 points, 8 bands, 2000 energies: 1742 us with 12 warps of
+// 168 registers, 1670 us with 16; 256^3 and 4000 energies 45.8 and 43.8 ms.)
+constexpr int kThreads = 512;
+constexpr int kMaxRegs = 128;
+template <int NORB>
 struct Cfg {
     static constexpr bool pairs = NORB <= 8;
-    static constexpr int threads = pairs ? 384 : 512;
-    static constexpr int max_regs = pairs ? 168 : 128;
     static constexpr int units_per_cube = pairs ? 3 : 6;
 };
-constexpr int kMaxThreads = 512;
 constexpr int kKBins = 256;     // window-length histogram bins (K >= 255 share one)
 
 // Table I, corner labels minus one; label c sits at offset (c&1, (c>>1)&1, (c>>2)&1).
@@ -194,160 +195,69 @@ __device__ __forceinline__ int fdivq(int a, int d) {
 
 __device__ __forceinline__ float safe_rcp(float x) { return x > 0.f ? __fdividef(1.0f, x) : 0.f; }
 
-// Per-item constants of the weight formulas, in fixed-point units.
+// The corner weights of one tetrahedron, without cases. With sorted corner
+// energies and the crossing fractions of the edges clamped to [0, 1],
+//   f_jl = sat((E - E_l) / (E_j - E_l)),  f_lj = 1 - f_jl  (j > l),
+// every case of Sec. II.C is one sum over simplices that have zero size
+// where the case does not hold:
+//  * the surface D = E is the triangle with vertices 13, 14 and "12 or 23"
+//    (size f21 f23 f31) plus the triangle 14, 24 and "23 or 34" (size
+//    f32 f34 f24), "ab" being the point of edge (a, b) at energy E:
+//      dw_l/dE = 4 f / E41 * sum over both of size * sum_vertices lambda_l
+//    (lambda the barycentric coordinates; E <= E2 has no second triangle,
+//    E >= E3 no first one, outside (E1, E4) there is neither);
+//  * the volume D < E is {1, 12|2, 13|3, 14|4} (f21 f31 f41), {2, 13, 14, 23}
+//    (f41 f32 f13), {2, 14, 23|3, 24} (f42 f32 f14) and {3, 14, 24, 34}
+//    (f43 f24 f14): w_l = f * sum of size * sum_vertices lambda_l / 4 * 4.
+// The clamps are the multiplies' own .sat, so no energy costs a compare, a
+// select or a branch that the lanes of a warp do not share, the set-up is six
+// reciprocals (the cubic coefficients of the middle case took about 90
+// operations and 16 registers per tetrahedron), and every term is positive. Equal
+// corner energies give infinite reciprocals: inf * 0 = NaN saturates to 0
+// and inf * positive to 1, which is the half-open step wanted there.
 struct Tet {
-    float e1, e2, e3, e4;
+    float e1, e2, e3;
     float r21, r31, r41, r32, r42, r43;
-    float P1, S1, P3, S3, k1, k2, k3, fq;
+    float scale;   // point: 4 f / E41 (0 for a flat tetrahedron); bin, integrated: f
 };
 
+template <int MODE>
 __device__ __forceinline__ void tet_setup(Tet &T, float e1, float e2, float e3, float e4, float fq) {
-    T.e1 = e1; T.e2 = e2; T.e3 = e3; T.e4 = e4;
-    T.r21 = safe_rcp(e2 - e1); T.r31 = safe_rcp(e3 - e1); T.r41 = safe_rcp(e4 - e1);
-    T.r32 = safe_rcp(e3 - e2); T.r42 = safe_rcp(e4 - e2); T.r43 = safe_rcp(e4 - e3);
-    T.P1 = 4.f * fq * T.r21 * T.r31 * T.r41;
-    T.S1 = T.r21 + T.r31 + T.r41;
-    T.P3 = 4.f * fq * T.r41 * T.r42 * T.r43;
-    T.S3 = T.r41 + T.r42 + T.r43;
-    T.k1 = fq * T.r31 * T.r41;
-    T.k2 = fq * T.r31 * T.r32 * T.r41;
-    T.k3 = fq * T.r32 * T.r41 * T.r42;
-    T.fq = fq;
+    T.e1 = e1; T.e2 = e2; T.e3 = e3;
+    T.r21 = __fdividef(1.f, e2 - e1); T.r31 = __fdividef(1.f, e3 - e1); T.r41 = __fdividef(1.f, e4 - e1);
+    T.r32 = __fdividef(1.f, e3 - e2); T.r42 = __fdividef(1.f, e4 - e2); T.r43 = __fdividef(1.f, e4 - e3);
+    T.scale = (MODE == TETRA_POINT) ? (e4 > e1 ? 4.f * fq * T.r41 : 0.f) : fq;
 }
 
-// Point-mode constants of one item, for a branch-free evaluation of the four
-// corner derivatives dw_l/dE at any E strictly inside (E1, E4):
-//  * cases E1 < E <= E2 and E3 < E < E4 share one mirrored form: with
-//    v = E - E1 (or E4 - E), g = P v^2, the apex corner (1, or 4) gets
-//    g (3 - v S) and the other three g v / E_j1 (or g v / E_4j);
-//  * in E2 < E <= E3 every dw_l is a cubic in t = E - E2, evaluated by
-//    Horner from coefficients expanded from the printed C1, C2, C3 forms.
-// e2c is the upper end of the first case: E2, or the float just below E4 when
-// E2 = E4 (then no energy below E4 may take the first case's form).
-struct TetP {
-    float e1, e2, e3, e4, e2c;
-    float P1, S1, r21, r31, r41;
-    float P3, S3, r42, r43;
-    float c[4][4];   // c[l][m]: coefficient of t^m in dw_l (case E2 < E <= E3)
-};
-
-__device__ __forceinline__ void tetp_setup(TetP &T, float e1, float e2, float e3, float e4, float fq) {
-    T.e1 = e1; T.e2 = e2; T.e3 = e3; T.e4 = e4;
-    T.e2c = (e2 < e4) ? e2 : nextafterf(e4, -INFINITY);
-    const float A = e2 - e1, B = e3 - e2, C = e4 - e2;
-    T.r21 = safe_rcp(A); T.r31 = safe_rcp(e3 - e1); T.r41 = safe_rcp(e4 - e1);
-    const float r32 = safe_rcp(B);
-    T.r42 = safe_rcp(C); T.r43 = safe_rcp(e4 - e3);
-    T.P1 = 4.f * fq * T.r21 * T.r31 * T.r41;
-    T.S1 = T.r21 + T.r31 + T.r41;
-    T.P3 = 4.f * fq * T.r41 * T.r42 * T.r43;
-    T.S3 = T.r41 + T.r42 + T.r43;
-    const float r31 = T.r31, r41 = T.r41, r42 = T.r42;
-    const float k1 = fq * r31 * r41, k2 = fq * r31 * r32 * r41, k3 = fq * r32 * r41 * r42;
-    const float k1r31 = k1 * r31, k1r41 = k1 * r41, k2r31 = k2 * r31, k2r41 = k2 * r41;
-    const float k2r32 = k2 * r32, k3r41 = k3 * r41, k3r32 = k3 * r32, k3r42 = k3 * r42;
-    T.c[0][0] = -A * (A * (k1r31 + k1r41) - B * B * k2r31 - B * C * k2r41 - 2.f * B * k1r31 -
-                      2.f * C * k1r41 - 2.f * k1);
-    T.c[0][1] = -2.f * (2.f * A * B * k2r31 + A * B * k2r41 + A * C * k2r41 + 2.f * A * k1r31 +
-                        2.f * A * k1r41 - B * B * k2r31 - B * C * k2r41 - B * k1r31 -
-                        C * C * k3r41 - C * k1r41 - k1);
-    T.c[0][2] = -3.f * (-A * k2r31 - A * k2r41 + 2.f * B * k2r31 + B * k2r41 + C * k2r41 +
-                        2.f * C * k3r41 + k1r31 + k1r41);
-    T.c[0][3] = 4.f * (k2r31 + k2r41 + k3r41);
-    T.c[1][0] = A * (B * B * k2r32 + B * k2 + 2.f * k1);
-    T.c[1][1] = -2.f * (2.f * A * B * k2r32 + A * k2 - B * B * k2r32 - B * C * k3r32 - B * k2 -
-                        C * C * k3r42 - C * k3 - k1);
-    T.c[1][2] = 3.f * (A * k2r32 - 2.f * B * k2r32 - B * k3r32 - C * k3r32 - 2.f * C * k3r42 - k2 - k3);
-    T.c[1][3] = 4.f * (k2r32 + k3r32 + k3r42);
-    T.c[2][0] = A * A * r31 * (B * k2 + 3.f * k1);
-    T.c[2][1] = 2.f * A * (-A * k2r31 + 2.f * B * k2r31 + B * k2r32 + 3.f * k1r31);
-    T.c[2][2] = 3.f * (-2.f * A * k2r31 - A * k2r32 + B * k2r31 + B * k2r32 + C * k3r32 + k1r31);
-    T.c[2][3] = -4.f * (k2r31 + k2r32 + k3r32);
-    T.c[3][0] = A * A * r41 * (B * k2 + 3.f * k1);
-    T.c[3][1] = 2.f * A * r41 * (-A * k2 + 2.f * B * k2 + C * k3 + 3.f * k1);
-    T.c[3][2] = 3.f * (-2.f * A * k2r41 - A * k3r41 + B * k2r41 + C * k3r41 + C * k3r42 + k1r41);
-    T.c[3][3] = -4.f * (k2r41 + k3r41 + k3r42);
+// Point mode: dw_l/dE at any E, sorted corners (30 operations).
+__device__ __forceinline__ void tet_dw(const Tet &T, float E, float (&d)[4]) {
+    const float x = E - T.e1, t = E - T.e2, y = E - T.e3;
+    const float f21 = __saturatef(x * T.r21), f31 = __saturatef(x * T.r31), f41 = __saturatef(x * T.r41);
+    const float f32 = __saturatef(t * T.r32), f42 = __saturatef(t * T.r42), f43 = __saturatef(y * T.r43);
+    const float p = fmaf(-f21, f32, f21);   // f21 f23
+    const float q = fmaf(-f32, f43, f32);   // f32 f34
+    const float qs = q * T.scale;
+    const float a = (p * T.scale) * f31, b = fmaf(-qs, f42, qs), s = a + b;
+    d[0] = fmaf((1.f - f21) + (1.f - f31), a, fmaf(-f41, s, s));
+    d[1] = fmaf((1.f - f32) + (1.f - f42), b, p * a);
+    d[2] = fmaf(f31 + f32, a, q * b);
+    d[3] = fmaf(f42 + f43, b, f41 * s);
 }
 
-// Valid at any E: outside (E1, E4) the clamped distance v = 0 makes every
-// derivative exactly zero (E >= E4 always takes the E4 - E form). At E = E3
-// the third case's form is used (equal to the second's by continuity). The
-// two mirrored forms give, in sorted corner order, (apex, u r21, u r31, u r41)
-// for the first case and (u r41, u r42, u r43, apex) for the third, so the
-// first and last outputs swap apex and u r41 and the middle two pick their
-// reciprocal: fewer selects than choosing every parameter first.
-// LEAN (the single-model kernel): the first case tested against the stored
-// e2c, and the mirrored forms' outputs picked as above. Otherwise (the
-// batched kernel, which has no register to spare for the leaner form: it
-// spilled there) the same values from the five selected parameters of the
-// case and one test E <= E2 and E < E4 (the same set as E <= e2c).
-template <bool LEAN = true>
-__device__ __forceinline__ void tetp_dw(const TetP &T, float E, float d[4]) {
-    const bool in1 = LEAN ? E <= T.e2c : (E <= T.e2 && E < T.e4);
-    const bool in3 = !in1 && E >= T.e3;
-    const float v = fmaxf(in1 ? E - T.e1 : T.e4 - E, 0.f);
-    const float P = in1 ? T.P1 : T.P3;
-    const float S = in1 ? T.S1 : T.S3;
-    const float g = P * v * v;
-    const float apex = g * fmaf(-v, S, 3.f);
-    const float u = g * v;
-    float m0, m1, m2, m3;
-    if constexpr (LEAN) {
-        const float u41 = u * T.r41;
-        m0 = in1 ? apex : u41;
-        m1 = u * (in1 ? T.r21 : T.r42);
-        m2 = u * (in1 ? T.r31 : T.r43);
-        m3 = in1 ? u41 : apex;
-    } else {
-        const float ra = in1 ? T.r21 : T.r41, rb = in1 ? T.r31 : T.r42, rc = in1 ? T.r41 : T.r43;
-        const float o1 = u * ra, o2 = u * rb, o3 = u * rc;
-        m0 = in1 ? apex : o1;
-        m1 = in1 ? o1 : o2;
-        m2 = in1 ? o2 : o3;
-        m3 = in1 ? o3 : apex;
-    }
-    const float t = E - T.e2;
-    float h[4];
-#pragma unroll
-    for (int l = 0; l < 4; ++l) h[l] = fmaf(fmaf(fmaf(T.c[l][3], t, T.c[l][2]), t, T.c[l][1]), t, T.c[l][0]);
-    const bool in2 = !in1 && !in3;
-    d[0] = in2 ? h[0] : m0;
-    d[1] = in2 ? h[1] : m1;
-    d[2] = in2 ? h[2] : m2;
-    d[3] = in2 ? h[3] : m3;
-}
-
-// w_l(E) for any E (Sec. II.C, all five cases), sorted corners.
-template <bool OPEN = false>
-__device__ __forceinline__ void tet_weights(const Tet &T, float E, float w[4]) {
-    if (E <= T.e1) {
-        w[0] = w[1] = w[2] = w[3] = 0.f;
-    } else if (E >= T.e4) {
-        // saturated; OPEN: zero, the saturated part being added elsewhere
-        w[0] = w[1] = w[2] = w[3] = OPEN ? 0.f : T.fq;
-    } else if (E <= T.e2) {
-        const float x = E - T.e1;
-        const float C = 0.25f * T.P1 * x * x * x;
-        w[0] = C * fmaf(-x, T.S1, 4.f);
-        const float cx = C * x;
-        w[1] = cx * T.r21; w[2] = cx * T.r31; w[3] = cx * T.r41;
-    } else if (E <= T.e3) {
-        const float a = E - T.e1, bq = E - T.e2, c = T.e3 - E, dd = T.e4 - E;
-        const float C1 = T.k1 * a * a;
-        const float C2 = T.k2 * a * bq * c;
-        const float C3 = T.k3 * bq * bq * dd;
-        const float S12 = C1 + C2, S23 = C2 + C3, S123 = S12 + C3;
-        w[0] = C1 + S12 * c * T.r31 + S123 * dd * T.r41;
-        w[1] = S123 + S23 * c * T.r32 + C3 * dd * T.r42;
-        w[2] = S12 * a * T.r31 + S23 * bq * T.r32;
-        w[3] = S123 * a * T.r41 + C3 * bq * T.r42;
-    } else {
-        const float y = T.e4 - E;
-        const float C = 0.25f * T.P3 * y * y * y;
-        const float cy = C * y;
-        w[0] = T.fq - cy * T.r41; w[1] = T.fq - cy * T.r42; w[2] = T.fq - cy * T.r43;
-        w[3] = T.fq - C * fmaf(-y, T.S3, 4.f);
-    }
+// w_l(E) at any E (0 below E1, f above E4), sorted corners (49 operations).
+__device__ __forceinline__ void tet_w(const Tet &T, float E, float (&w)[4]) {
+    const float x = E - T.e1, t = E - T.e2, y = E - T.e3;
+    const float f21 = __saturatef(x * T.r21), f31 = __saturatef(x * T.r31), f41 = __saturatef(x * T.r41);
+    const float f32 = __saturatef(t * T.r32), f42 = __saturatef(t * T.r42), f43 = __saturatef(y * T.r43);
+    const float f13 = 1.f - f31, f14 = 1.f - f41, f24 = 1.f - f42, g23 = 2.f - f32;   // 1 + f23
+    const float fa = T.scale * f41, fb = T.scale * f14;
+    const float v1 = (f21 * f31) * fa, v2 = (f32 * f13) * fa;
+    const float v3 = (f32 * f42) * fb, v4 = (f43 * f24) * fb;
+    const float c13 = f13 + f14, s42 = f41 + f42;
+    w[0] = fmaf(v3 + v4, f14, fmaf(v2, c13, fmaf(v1, c13 + (1.f - f21), v1)));
+    w[1] = fmaf(v4, f24, fmaf(v3, g23 + f24, fmaf(v2, g23, v1 * f21)));
+    w[2] = fmaf(v4, 2.f - f43, fmaf(v3, f32, fmaf(v2, f31 + f32, v1 * f31)));
+    w[3] = fmaf(v4, s42 + f43, fmaf(v3, s42, (v1 + v2) * f41));
 }
 
 // Adds one energy's contribution of an item directly to the CTA's int64
@@ -426,7 +336,7 @@ struct Batch {
 };
 
 template <int NORB, typename WT, int MODE, int MAXM>
-__global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
+__global__ void __maxnreg__(kMaxRegs)
     tetra_dos_fwd_kernel(const __grid_constant__ Batch<MAXM> B, const FwdArgs A) {
     // tile row: NORB orbitals + the row's add count (differences); the odd
     // row length also spreads consecutive rows over the shared-memory banks
@@ -448,10 +358,10 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
     int *tile = reinterpret_cast<int *>(wstage + A.w_stage);   // [copies][chunk_w + 1][TS]
     // (copies only for single-model bin-mode pairs; elsewhere one, known at
     // compile time: the batched kernel measured faster without them)
-    constexpr bool kCopies = MODE == TETRA_BIN && Cfg<MODE, NORB>::pairs && MAXM == 1;
+    constexpr bool kCopies = MODE == TETRA_BIN && Cfg<NORB>::pairs && MAXM == 1;
     const int n_copies = kCopies ? A.tile_copies : 1, copy_ints = TS * (A.chunk_w + 1);
     // integrated mode: per-orbital sums of the saturated weights of the items
-    // whose E4 lies between energy j-1 and j, [chunk_w][NORB] (plain integers)
+    // whose (larger) E4 lies between energy j-1 and j, [chunk_w][NORB] (plain integers)
     int *stile = tile + copy_ints * n_copies;
     float *om = reinterpret_cast<float *>(stile + (MODE == TETRA_INTEGRATED ? NORB * A.chunk_w : 0));
     float *iw = om + A.chunk_w + 1;                                   // 1/bin width (bin mode)
@@ -466,8 +376,8 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
     int *kcursor = khist + kKBins;           // rank cursors per window length
     uint64_t *mbar = reinterpret_cast<uint64_t *>(
         (reinterpret_cast<uintptr_t>(kcursor + kKBins) + 15) & ~uintptr_t(15));
-    __shared__ float red_f[kMaxThreads / 32];
-    __shared__ int s_wsum[kMaxThreads / 32];
+    __shared__ float red_f[kThreads / 32];
+    __shared__ int s_wsum[kThreads / 32];
     __shared__ int s_abort, s_active, s_slot;
     __shared__ int s_cdelta[8];   // staged-box point offset of cube corner c
     __shared__ int n_issued[3];   // TMA loads issued per mbarrier (thread 0 keeps them)
@@ -726,8 +636,8 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
                     // grid get lo = w0 + wc, which makes them inactive
                     int K = 0, lo = (MODE == TETRA_INTEGRATED) ? w0 + wc : 0;
                     if (it < A.items_per_box) {
-                        constexpr bool PAIRS = Cfg<MODE, NORB>::pairs;
-                        constexpr int UPC = Cfg<MODE, NORB>::units_per_cube;
+                        constexpr bool PAIRS = Cfg<NORB>::pairs;
+                        constexpr int UPC = Cfg<NORB>::units_per_cube;
                         const int cube = it & (ncube - 1);
                         const int rest = it >> lcube;
                         const int t = rest % UPC, n = rest / UPC;
@@ -736,10 +646,12 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
                             // a pair's window is the union of its two tetrahedra's:
                             // the window of the min / max over its five corners
                             float e1 = 3.0e38f, e4 = -3.0e38f;
+                            bool flat_face = false;
                             const uint32_t code = PAIRS ? pair_code(t) : tet_code(t);
                             const int p0 = cx + PX * (cy + PY * cz);
 #pragma unroll
                             for (int q = 0; q < (PAIRS ? 5 : 4); ++q) {
+                                if (q == 3) flat_face = e1 == e4;   // of a pair: corners 0..2
                                 const int p = p0 + s_cdelta[(code >> (3 * q)) & 7];
                                 const float ev = Es[p * A.eps_stride + n];
                                 e1 = fminf(e1, ev);
@@ -747,6 +659,10 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
                             }
                             int hi;
                             item_window<MODE>(e1, e4, om, w0, wc, om0, inv_de, M.n_omega, lo, hi);
+                            // a flat tetrahedron at a pair's upper end is empty at an
+                            // energy equal to it: there the walk, not the pair's step
+                            if (MODE == TETRA_INTEGRATED && PAIRS && flat_face)
+                                while (hi < w0 + wc - 1 && om[hi + 1 - w0] <= e4) ++hi;
                             K = max(0, hi - lo + 1);
                         }
                     }
@@ -762,7 +678,7 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
                         s_K[it] = (unsigned short)K;
                     }
                     const bool act = it < A.items_per_box && (K > 0 || (MODE == TETRA_INTEGRATED && lo + K < w0 + wc));
-                    if constexpr (MODE == TETRA_INTEGRATED && Cfg<MODE, NORB>::pairs) {
+                    if constexpr (MODE == TETRA_INTEGRATED && Cfg<NORB>::pairs) {
                         // items with an empty window (only a step: every tetrahedron
                         // below the chunk) all count in bin 0, one add per warp
                         const unsigned zm = __ballot_sync(0xffffffffu, act && K == 0);
@@ -801,7 +717,7 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
             const int K = it < A.items_per_box ? (int)s_K[it] : 0;
             const bool act = it < A.items_per_box &&
                              (K > 0 || (MODE == TETRA_INTEGRATED && s_lo[it] + K < wc));
-            if constexpr (MODE == TETRA_INTEGRATED && Cfg<MODE, NORB>::pairs) {
+            if constexpr (MODE == TETRA_INTEGRATED && Cfg<NORB>::pairs) {
                 // empty windows: consecutive ranks from one cursor add per warp
                 const unsigned zm = __ballot_sync(0xffffffffu, act && K == 0);
                 if (act && K > 0) s_list[atomicAdd(&kcursor[min(K, kKBins - 1)], 1)] = (unsigned short)it;
@@ -870,7 +786,7 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
             const int hi = valid ? lo + s_K[it] - 1 : w0 - 1;
             const uint32_t gcube = (uint32_t)(gx0 + cx) +
                                    (uint32_t)M.n1 * ((uint32_t)(gy0 + cy) + (uint32_t)M.n2 * (uint32_t)(gz0 + cz));
-            if constexpr (Cfg<MODE, NORB>::pairs) {
+            if constexpr (Cfg<NORB>::pairs) {
                 // integrated mode: the lanes that hold an item, for the warp sums of
                 // the steps on the chunk's first energy
                 const unsigned vmask = (MODE == TETRA_INTEGRATED) ? __ballot_sync(0xffffffffu, valid) : 0u;
@@ -899,24 +815,21 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
                 }
                 const float dith = item_dither((gcube * 3u + (uint32_t)pr) * (uint32_t)A.nb + (uint32_t)n);
                 if constexpr (MODE == TETRA_INTEGRATED) {
-                    // Occupation: the walk over the union window adds each
-                    // tetrahedron's weights below its own E4 (zero at and above
-                    // it); from its step, the first energy at or above its E4,
-                    // the saturated weights fq sum_l b_l enter the step tile.
+                    // Occupation: the walk over the union window adds both
+                    // tetrahedra's weights (saturated above a tetrahedron's own
+                    // E4); from the first energy beyond it on, the pair's step
+                    // fq sum_l b_l of both enters through the step tile.
                     // Every corner weight is at most V_T/(4 V_G): the pair adds
                     // at most 8 fq Bmax to any entry.
                     const float qmax = bmax * 8.f * fq * 1.01f;
                     const bool fast = qmax < (float)A.fast_cap;
-                    int loa, hia, lob, hib;
-                    item_window<MODE>(ea[0], ea[3], om, w0, wc, om0, inv_de, M.n_omega, loa, hia);
-                    item_window<MODE>(eb[0], eb[3], om, w0, wc, om0, inv_de, M.n_omega, lob, hib);
-                    // the first energy with saturated weights: at or above E4 and
-                    // above E1 (a flat tetrahedron, E1 = E4, is empty at E = E1)
-                    const int hsa = max(hia + 1, loa), hsb = max(hib + 1, lob);
-                    const bool stepa = hsa < w0 + wc, stepb = hsb < w0 + wc;
+                    // the first energy beyond the window (a flat pair, E1 = E4, is
+                    // empty at E = E1: lo is above E1)
+                    const int hs = hi + 1;
+                    const bool step = hs < w0 + wc;
                     // steps on the chunk's first energy (there go the steps of all
                     // tetrahedra below the chunk) are summed over the warp first
-                    const bool firsta = fast && stepa && hsa == w0, firstb = fast && stepb && hsb == w0;
+                    const bool first = fast && step && hs == w0;
                     const unsigned qbnd = fast ? (unsigned)qmax + 2u : 0u;
                     if (fast) {
                         if (hi >= lo) {
@@ -924,29 +837,24 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
                             atomicAdd(&tile[(lo - w0) * TS + CNT], 1);
                             atomicAdd(&tile[(hi + 1 - w0) * TS + CNT], -1);
                         }
-                        if (stepa && !firsta) atomicAdd(&blk_bound[(hsa - w0) >> 6], qbnd);
-                        if (stepb && !firstb) atomicAdd(&blk_bound[(hsb - w0) >> 6], qbnd);
+                        if (step && !first) atomicAdd(&blk_bound[(hs - w0) >> 6], qbnd);
                     }
                     Tet TA, TB;
-                    tet_setup(TA, ea[0], ea[1], ea[2], ea[3], fq);
-                    tet_setup(TB, eb[0], eb[1], eb[2], eb[3], fq);
-                    float sa[NORB], sb[NORB];   // saturated contributions fq sum_l b_{l,s}
-#pragma unroll
-                    for (int s = 0; s < NORB; ++s) {
-                        sa[s] = fq * ((ba[0][s] + ba[1][s]) + (ba[2][s] + ba[3][s]));
-                        sb[s] = fq * ((bb[0][s] + bb[1][s]) + (bb[2][s] + bb[3][s]));
-                    }
-                    if (__any_sync(vmask, firsta || firstb)) {
-                        // the warp's first-energy steps (a tetrahedron whose step is
-                        // there adds nothing in the window): integer sums, one add per orbital
+                    tet_setup<MODE>(TA, ea[0], ea[1], ea[2], ea[3], fq);
+                    tet_setup<MODE>(TB, eb[0], eb[1], eb[2], eb[3], fq);
+                    // the pair's saturated contribution of orbital s
+                    auto full = [&](int s) {
+                        return fq * (((ba[0][s] + ba[1][s]) + (ba[2][s] + ba[3][s])) +
+                                     ((bb[0][s] + bb[1][s]) + (bb[2][s] + bb[3][s]))) + dith;
+                    };
+                    if (__any_sync(vmask, first)) {
+                        // the warp's first-energy steps: integer sums, one add per orbital
                         const bool lead = lane == __ffs(vmask) - 1;
-                        const unsigned bsum = __reduce_add_sync(vmask, (firsta ? qbnd : 0u) + (firstb ? qbnd : 0u));
+                        const unsigned bsum = __reduce_add_sync(vmask, first ? qbnd : 0u);
                         if (lead && bsum) atomicAdd(&blk_bound[0], bsum);
 #pragma unroll
                         for (int s = 0; s < NORB; ++s) {
-                            const int v = (firsta ? __float_as_int(sa[s] + dith + kMagic) - kMagicBits : 0) +
-                                          (firstb ? __float_as_int(sb[s] + dith + kMagic) - kMagicBits : 0);
-                            const int tot = __reduce_add_sync(vmask, v);
+                            const int tot = __reduce_add_sync(vmask, first ? __float_as_int(full(s) + kMagic) - kMagicBits : 0);
                             if (lead && tot) atomicAdd(&stile[s], tot);
                         }
                     }
@@ -955,8 +863,8 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
                         int i = lo + ((lane * max(K, 1)) >> 5);
                         for (int j = 0; j < K; ++j) {
                             float wa[4], wb[4];
-                            tet_weights<true>(TA, om[i - w0], wa);
-                            tet_weights<true>(TB, om[i - w0], wb);
+                            tet_w(TA, om[i - w0], wa);
+                            tet_w(TB, om[i - w0], wb);
                             int *col = tile + (i - w0) * TS;
 #pragma unroll
                             for (int s = 0; s < NORB; ++s) {
@@ -972,18 +880,16 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
                             }
                             i = (i == hi) ? lo : i + 1;
                         }
+                        if (step && !first) {
 #pragma unroll
-                        for (int s = 0; s < NORB; ++s) {
-                            if (stepa && !firsta)
-                                atomicAdd(&stile[(hsa - w0) * NORB + s], __float_as_int(sa[s] + dith + kMagic) - kMagicBits);
-                            if (stepb && !firstb)
-                                atomicAdd(&stile[(hsb - w0) * NORB + s], __float_as_int(sb[s] + dith + kMagic) - kMagicBits);
+                            for (int s = 0; s < NORB; ++s)
+                                atomicAdd(&stile[(hs - w0) * NORB + s], __float_as_int(full(s) + kMagic) - kMagicBits);
                         }
                     } else {
                         for (int i = lo; i <= hi; ++i) {
                             float wa[4], wb[4];
-                            tet_weights<true>(TA, om[i - w0], wa);
-                            tet_weights<true>(TB, om[i - w0], wb);
+                            tet_w(TA, om[i - w0], wa);
+                            tet_w(TB, om[i - w0], wb);
 #pragma unroll
                             for (int s = 0; s < NORB; ++s) {
                                 if (s >= A.n_orb) continue;
@@ -1001,8 +907,7 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
 #pragma unroll
                         for (int s = 0; s < NORB; ++s) {
                             if (s >= A.n_orb) continue;
-                            if (stepa) deposit_one(sa[s] + dith, Gsc + (long)s * A.chunk_w + (hsa - w0), A.status);
-                            if (stepb) deposit_one(sb[s] + dith, Gsc + (long)s * A.chunk_w + (hsb - w0), A.status);
+                            if (step) deposit_one(full(s), Gsc + (long)s * A.chunk_w + (hs - w0), A.status);
                         }
                     }
                     continue;
@@ -1027,16 +932,16 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
                         atomicAdd(&tl[(hi + 1 - w0) * TS + CNT], -1);
                     }
                     Tet TA, TB;
-                    tet_setup(TA, ea[0], ea[1], ea[2], ea[3], fq);
-                    tet_setup(TB, eb[0], eb[1], eb[2], eb[3], fq);
+                    tet_setup<MODE>(TA, ea[0], ea[1], ea[2], ea[3], fq);
+                    tet_setup<MODE>(TB, eb[0], eb[1], eb[2], eb[3], fq);
                     float wpa[4], wpb[4];
-                    tet_weights(TA, om[lo - w0], wpa);
-                    tet_weights(TB, om[lo - w0], wpb);
+                    tet_w(TA, om[lo - w0], wpa);
+                    tet_w(TB, om[lo - w0], wpb);
                     int *col = tl + (lo - w0) * TS;
                     for (int i = lo; i <= hi; ++i, col += TS) {
                         float wna[4], wnb[4], da[4], db[4];
-                        tet_weights(TA, om[i + 1 - w0], wna);
-                        tet_weights(TB, om[i + 1 - w0], wnb);
+                        tet_w(TA, om[i + 1 - w0], wna);
+                        tet_w(TB, om[i + 1 - w0], wnb);
                         const float sc = iw[i - w0];
 #pragma unroll
                         for (int r4 = 0; r4 < 4; ++r4) {
@@ -1077,22 +982,17 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
                     atomicAdd(&tile[(lo - w0) * TS + CNT], 1);
                     atomicAdd(&tile[(hi + 1 - w0) * TS + CNT], -1);
                 }
-                TetP TA, TB;
-                tetp_setup(TA, ea[0], ea[1], ea[2], ea[3], fq);
-                tetp_setup(TB, eb[0], eb[1], eb[2], eb[3], fq);
-                // both tetrahedra's corner derivatives at E (zero outside a
-                // tetrahedron's own window (E1, E4), see tetp_dw)
-                auto both = [&](float E, float (&da)[4], float (&db)[4]) {
-                    tetp_dw<MAXM == 1>(TA, E, da);
-                    tetp_dw<MAXM == 1>(TB, E, db);
-                };
+                Tet TA, TB;
+                tet_setup<MODE>(TA, ea[0], ea[1], ea[2], ea[3], fq);
+                tet_setup<MODE>(TB, eb[0], eb[1], eb[2], eb[3], fq);
                 if (fast) {
                     // lane-dependent start, wrapping walk (see below)
                     const int K = hi - lo + 1;
                     int i = lo + ((lane * K) >> 5);
                     for (int j = 0; j < K; ++j) {
-                        float da[4], db[4];
-                        both(om[i - w0], da, db);
+                        float da[4], db[4];   // zero outside a tetrahedron's own window
+                        tet_dw(TA, om[i - w0], da);
+                        tet_dw(TB, om[i - w0], db);
                         int *col = tile + (i - w0) * TS;
 #pragma unroll
                         for (int s = 0; s < NORB; ++s) {
@@ -1110,8 +1010,9 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
                     }
                 } else {
                     for (int i = lo; i <= hi; ++i) {
-                        float da[4], db[4];
-                        both(om[i - w0], da, db);
+                        float da[4], db[4];   // zero outside a tetrahedron's own window
+                        tet_dw(TA, om[i - w0], da);
+                        tet_dw(TB, om[i - w0], db);
 #pragma unroll
                         for (int s = 0; s < NORB; ++s) {
                             if (s >= A.n_orb) continue;
@@ -1172,7 +1073,7 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
             }
             if constexpr (MODE == TETRA_INTEGRATED) {
                 Tet T;
-                tet_setup(T, e[0], e[1], e[2], e[3], fq);
+                tet_setup<MODE>(T, e[0], e[1], e[2], e[3], fq);
                 float bsum[NORB];   // saturated contribution: fq sum_l b_{l,s}
 #pragma unroll
                 for (int s = 0; s < NORB; ++s) bsum[s] = fq * ((b[0][s] + b[1][s]) + (b[2][s] + b[3][s]));
@@ -1181,7 +1082,7 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
                     int i = lo + ((lane * max(K, 1)) >> 5);
                     for (int j = 0; j < K; ++j) {
                         float wl[4];
-                        tet_weights(T, om[i - w0], wl);
+                        tet_w(T, om[i - w0], wl);
                         int *col = tile + (i - w0) * TS;
 #pragma unroll
                         for (int s = 0; s < NORB; ++s) {
@@ -1201,7 +1102,7 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
                 } else {
                     for (int i = lo; i <= hi; ++i) {
                         float wl[4];
-                        tet_weights(T, om[i - w0], wl);
+                        tet_w(T, om[i - w0], wl);
                         deposit_slow<NORB>(b, wl, A.n_orb, dith, Gc + (i - w0), A.chunk_w, A.status);
                     }
                     if (step) {
@@ -1213,8 +1114,8 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
                 continue;
             }
             if constexpr (MODE == TETRA_POINT) {
-                TetP TP;
-                tetp_setup(TP, e[0], e[1], e[2], e[3], fq);
+                Tet TP;
+                tet_setup<MODE>(TP, e[0], e[1], e[2], e[3], fq);
                 if (fast) {
                     // The walk over the window starts at a lane-dependent offset
                     // and wraps: lanes whose windows coincide then add to
@@ -1224,7 +1125,7 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
                     int i = lo + ((lane * K) >> 5);
                     for (int j = 0; j < K; ++j) {
                         float d[4];
-                        tetp_dw<MAXM == 1>(TP, om[i - w0], d);
+                        tet_dw(TP, om[i - w0], d);
                         int *col = tile + (i - w0) * TS;
 #pragma unroll
                         for (int s = 0; s < NORB; ++s) {
@@ -1239,19 +1140,19 @@ __global__ void __maxnreg__((Cfg<MODE, NORB>::max_regs))
                 } else {
                     for (int i = lo; i <= hi; ++i) {
                         float d[4];
-                        tetp_dw<MAXM == 1>(TP, om[i - w0], d);
+                        tet_dw(TP, om[i - w0], d);
                         deposit_slow<NORB>(b, d, A.n_orb, dith, Gc + (i - w0), A.chunk_w, A.status);
                     }
                 }
             } else {
                 Tet T;
-                tet_setup(T, e[0], e[1], e[2], e[3], fq);
+                tet_setup<MODE>(T, e[0], e[1], e[2], e[3], fq);
                 float wp[4];
-                tet_weights(T, om[lo - w0], wp);
+                tet_w(T, om[lo - w0], wp);
                 int *col = tile + (lo - w0) * TS;
                 for (int i = lo; i <= hi; ++i, col += TS) {
                     float wn[4], d[4];
-                    tet_weights(T, om[i + 1 - w0], wn);
+                    tet_w(T, om[i + 1 - w0], wn);
                     const float sc = iw[i - w0];
 #pragma unroll
                     for (int r4 = 0; r4 < 4; ++r4) { d[r4] = (wn[r4] - wp[r4]) * sc; wp[r4] = wn[r4]; }
@@ -1465,7 +1366,9 @@ cudaError_t launch_t(size_t smem, dim3 grid, const Batch<MAXM> &Bt, const FwdArg
             }
         }
     }
-    k<<<grid, Cfg<MODE, NORB>::threads, smem, stream>>>(Bt, A);
+    // no more warps than a box has items for (idle ones only slow its barriers)
+    const int threads = std::min(kThreads, std::max(128, (A.items_per_box + 31) & ~31));
+    k<<<grid, threads, smem, stream>>>(Bt, A);
     return cudaGetLastError();
 }
 

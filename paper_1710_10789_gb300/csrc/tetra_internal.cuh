@@ -23,7 +23,6 @@ struct tetra_plan_s {
     int nbx, nby, nbz, n_boxes;
     int chunk_w, n_chunks;      // energy chunking of the shared-memory tile
     int grid_x;                 // persistent CTAs per energy chunk
-    int threads;
     int fixed_bits;             // fixed-point fraction bits (see dos.cu)
     int flush_bits;             // a tile block is flushed once its bound reaches 2^flush_bits
     int items_per_box;          // work units per box: (pair, band) in point mode, (tetrahedron, band) in bin mode
