@@ -223,7 +223,9 @@ struct Tet {
 
 template <int MODE>
 __device__ __forceinline__ void tet_setup(Tet &T, float e1, float e2, float e3, float e4, float fq) {
-    T.e1 = e1; T.e2 = e2; T.e3 = e3;
+    T.e1 = e1; T.e3 = e3;
+    // E2 = E3 = E4: the section jumps to zero at E4, where f32 has to be 1
+    T.e2 = (MODE == TETRA_POINT && !(e2 < e4)) ? nextafterf(e4, -INFINITY) : e2;
     T.r21 = __fdividef(1.f, e2 - e1); T.r31 = __fdividef(1.f, e3 - e1); T.r41 = __fdividef(1.f, e4 - e1);
     T.r32 = __fdividef(1.f, e3 - e2); T.r42 = __fdividef(1.f, e4 - e2); T.r43 = __fdividef(1.f, e4 - e3);
     T.scale = (MODE == TETRA_POINT) ? (e4 > e1 ? 4.f * fq * T.r41 : 0.f) : fq;
