@@ -662,8 +662,10 @@ __global__ void __maxnreg__(kMaxRegs)
                             int hi;
                             item_window<MODE>(e1, e4, om, w0, wc, om0, inv_de, M.n_omega, lo, hi);
                             // a flat tetrahedron at a pair's upper end is empty at an
-                            // energy equal to it: there the walk, not the pair's step
-                            if (MODE == TETRA_INTEGRATED && PAIRS && flat_face)
+                            // energy (bin edge) equal to it: in integrated mode there
+                            // the walk, not the pair's step; in bin mode the bin above
+                            // takes its whole step
+                            if (MODE != TETRA_POINT && PAIRS && flat_face)
                                 while (hi < w0 + wc - 1 && om[hi + 1 - w0] <= e4) ++hi;
                             K = max(0, hi - lo + 1);
                         }
