@@ -133,9 +133,8 @@ tetra_status_t tetra_dos(tetra_plan_t plan, const float *eps, const void *w,
  * convenience.
  *   Scratch: a static device array of 32 MiB inside libtetra (held on every
  *   GPU that loads the library until the process exits). The call allocates
- *   nothing. If the plan's per-CTA partial sums do not fit, fewer persistent
- *   CTAs are used (same result, bit for bit); if they do not fit even with one
- *   CTA, returns TETRA_ENOMEM. With one CTA the scratch holds
+ *   nothing. If the plan's accumulators do not fit, returns TETRA_ENOMEM; they
+ *   take
  *     256 + m * 8 * n_orb * n_chunks * ceil(n_omega / n_chunks)  bytes,
  *   m = 2 in TETRA_INTEGRATED mode and 1 otherwise, where n_chunks is the
  *   number of shared-memory energy tiles of the plan (1 up to about 4300

@@ -44,9 +44,10 @@
 //    is at most 3/E41 of V_T/V_G) decides between this fast path and a 64-bit
 //    global integer path for rare near-flat tetrahedra. The sum of q_max over
 //    processed items bounds every tile entry; the tile is flushed into the
-//    CTA's int64 partial in global memory before it could overflow.
-//  * tetra_dos_reduce sums the per-CTA int64 partials (exact) and scales by u;
-//    for a batch, each model's accumulator is scaled.
+//    int64 accumulator in global memory before it could overflow.
+//  * The CTAs flush into one int64 accumulator (integer atomics: exact, any
+//    order); the CTA that finishes last scales it by u. For a batch a second
+//    kernel scales each model's accumulator.
 #include <algorithm>
 #include <atomic>
 #include <memory>
@@ -120,10 +121,12 @@ struct FwdArgs {
     int items_per_box;   // items per box: (pair, band) in point mode, (tetrahedron, band) otherwise
     int fast_cap;
     unsigned flush_at;   // a 64-energy block is flushed once its bound reaches this
-    long long *G;        // int64 partials, [slot][n_orb][chunk_w]
-    long long *Gs;       // integrated mode: int64 partial step sums, [slot][n_orb][chunk_w]
+    long long *G;        // int64 accumulators, [slot][n_orb][chunk_w]; slot = chunk, or model of a batch
+    long long *Gs;       // integrated mode: int64 accumulators of the step sums, the same shape
     int *status;
     int *queue;          // batched: next unclaimed (model, box) work item
+    int *done;           // single model: CTAs that have flushed, [kDoneGroups] (chunk % kDoneGroups)
+    float *dos;          // single model: the result, written by the CTA that finishes a chunk
 };
 
 // Fixed-point unit, identical in every kernel that uses it. The DOS modes
@@ -570,9 +573,9 @@ __global__ void __maxnreg__(kMaxRegs)
             cur = mi;
             w0 = (MAXM == 1) ? chunk * A.chunk_w : 0;
             wc = min(A.chunk_w, M.n_omega - w0);
-            // partial slot: one per (energy chunk, CTA) for a single model, one
-            // per model for a batch (CTAs flush into it with integer atomics)
-            const long slot = (MAXM == 1) ? (long)chunk * gridDim.x + blockIdx.x : (long)mi;
+            // accumulator: one per energy chunk of a single model, one per model
+            // of a batch (CTAs flush into it with integer atomics)
+            const long slot = (MAXM == 1) ? (long)chunk : (long)mi;
             Gc = A.G + slot * (long)A.n_orb * A.chunk_w;
             if (MODE == TETRA_INTEGRATED) Gsc = A.Gs + slot * (long)A.n_orb * A.chunk_w;
             for (int i = tid; i < copy_ints * n_copies; i += blockDim.x) tile[i] = 0;
@@ -1254,83 +1257,73 @@ __global__ void __maxnreg__(kMaxRegs)
         }
     }
     __syncthreads();
-    if (s_abort) {
-        // a TMA wait timed out: wait (bounded) for copies still in flight, then leave
+    const bool aborted = s_abort != 0;
+    if (aborted) {
+        // a TMA wait timed out: wait (bounded) for copies still in flight
         if (tid == 0) {
             for (int b = 0; b < 3; ++b)
                 if (n_issued[b] > 0)
                     mbar_wait_bounded(&mbar[b], (uint32_t)(n_issued[b] - 1) & 1u, nullptr, 100000000ull);
         }
-        return;
+        if (MAXM > 1) return;
+    } else if (cur >= 0) {
+        flush_tile();
     }
-    if (cur >= 0) flush_tile();
-}
-
-// Single model: dos[s][w0+j] = u * sum over CTAs of the int64 partials (exact).
-__global__ void tetra_dos_reduce_kernel(const long long *G, int grid_x, int n_orb, int n_omega,
-                                        int chunk_w, int mode, const float *omega, double vtvg,
-                                        int bits, float *dos) {
-    const double u = fixed_unit(omega, n_omega, mode, vtvg, bits);
-    const long total = (long)n_orb * n_omega;
-    for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < total;
-         idx += (long)gridDim.x * blockDim.x) {
-        const int s = (int)(idx / n_omega), i = (int)(idx - (long)s * n_omega);
-        const int chunk = i / chunk_w, j = i - chunk * chunk_w;
-        const long long *g = G + ((long)chunk * grid_x * n_orb + s) * chunk_w + j;
-        long long acc = 0;
-        for (int c = 0; c < grid_x; ++c) acc += g[(long)c * n_orb * chunk_w];
-        dos[idx] = (float)((double)acc * u);
-    }
-}
-
-// Integrated mode: block (s, c) = orbital s, energy chunk c. A chunk's CTAs
-// put the steps of every tetrahedron below the chunk on its first energy, so
-// the running sum of the step partials starts afresh in each chunk:
-// dos[s][w0 + j] = u * (sum over CTAs of the window partials at j + the
-// running sum over j' <= j of the chunk's step partials), exact int64
-// arithmetic up to the scaling.
-__global__ void tetra_dos_reduce_integrated(const long long *G, const long long *Gs, int grid_x, int n_orb,
-                                            int n_omega, int chunk_w, const float *omega, double vtvg,
-                                            int bits, float *dos) {
-    __shared__ long long s_warp[32];
-    __shared__ long long s_carry;
-    const int s = blockIdx.x, chunk = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nw = (int)(blockDim.x >> 5);
-    const int w0 = chunk * chunk_w, wc = min(chunk_w, n_omega - w0);
-    const long cta_stride = (long)n_orb * chunk_w;
-    const long first = ((long)chunk * grid_x * n_orb + s) * chunk_w;
-    const double u = fixed_unit(omega, n_omega, TETRA_INTEGRATED, vtvg, bits);
-    if (tid == 0) s_carry = 0;
-    __syncthreads();
-    for (int base = 0; base < wc; base += blockDim.x) {
-        const int j = base + tid;
-        long long wsum = 0, ssum = 0;
-        if (j < wc) {
-            for (int c = 0; c < grid_x; ++c) {
-                const long off = first + c * cta_stride + j;
-                wsum += G[off];
-                ssum += Gs[off];
+    if constexpr (MAXM == 1) {
+        // The last CTA of a chunk scales the exact sums to the result. (One
+        // accumulator for all CTAs: a slot per CTA took a 39 MB memset, a
+        // separate launch and 26 us of serial reads at 256^3 and 4000
+        // energies; the flushes are integer atomics either way.)
+        __threadfence();
+        __syncthreads();
+        const int group = chunk % kDoneGroups;
+        const int chunks = ((int)gridDim.y - group + kDoneGroups - 1) / kDoneGroups;   // chunks that share the counter
+        if (tid == 0) s_active = atomicAdd(&A.done[group], 1) == chunks * (int)gridDim.x - 1;
+        __syncthreads();
+        if (!s_active) return;
+        __threadfence();
+        const ModelP &M = B.m[0];
+        u = fixed_unit(M.omega, M.n_omega, MODE, M.vtvg, M.fixed_bits);
+        for (int c = group; c < (int)gridDim.y; c += kDoneGroups) {
+            const int f0 = c * A.chunk_w, fn = min(A.chunk_w, M.n_omega - f0);
+            const long long *G = A.G + (long)c * A.n_orb * A.chunk_w;
+            if constexpr (MODE == TETRA_INTEGRATED) {
+                // running sum of the chunk's steps (a chunk's first energy holds the
+                // steps of every tetrahedron below the chunk): one warp per orbital,
+                // in the shared memory of the two tiles
+                const long long *Gs = A.Gs + (long)c * A.n_orb * A.chunk_w;
+                long long *buf = reinterpret_cast<long long *>(tile);
+                __syncthreads();
+                for (int i = tid; i < A.n_orb * fn; i += blockDim.x) {
+                    const int s = i / fn;
+                    buf[i] = __ldcg(Gs + (long)s * A.chunk_w + (i - s * fn));
+                }
+                __syncthreads();
+                const int lane = tid & 31;
+                for (int s = tid >> 5; s < A.n_orb; s += (int)(blockDim.x >> 5)) {
+                    long long carry = 0;
+                    for (int j0 = 0; j0 < fn; j0 += 32) {
+                        const int j = j0 + lane;
+                        long long x = j < fn ? buf[s * fn + j] : 0;
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const long long y = __shfl_up_sync(0xffffffffu, x, o);
+                            if (lane >= o) x += y;
+                        }
+                        x += carry;
+                        carry = __shfl_sync(0xffffffffu, x, 31);
+                        if (j < fn) buf[s * fn + j] = x;
+                    }
+                }
+                __syncthreads();
+            }
+            for (int i = tid; i < A.n_orb * fn; i += blockDim.x) {
+                const int s = i / fn, j = i - s * fn;
+                long long v = __ldcg(G + (long)s * A.chunk_w + j);
+                if (MODE == TETRA_INTEGRATED) v += reinterpret_cast<const long long *>(tile)[i];
+                A.dos[(long)s * M.n_omega + f0 + j] = (float)((double)v * u);
             }
         }
-        long long x = ssum;   // inclusive scan over the block
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const long long y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) s_warp[warp] = x;
-        __syncthreads();
-        long long off = s_carry;
-        for (int w2 = 0; w2 < warp; ++w2) off += s_warp[w2];
-        x += off;
-        if (j < wc) dos[(long)s * n_omega + w0 + j] = (float)((double)(wsum + x) * u);
-        __syncthreads();
-        if (tid == 0) {
-            long long tot = 0;
-            for (int w2 = 0; w2 < nw; ++w2) tot += s_warp[w2];
-            s_carry += tot;
-        }
-        __syncthreads();
     }
 }
 
@@ -1447,7 +1440,7 @@ int norb_template(int n_orb) {
 
 size_t dos_forward_workspace(const Plan &P) {
     // integrated mode: a second array of the same size for the step sums
-    const size_t parts = sizeof(long long) * (size_t)P.n_chunks * P.grid_x * P.d.n_orb * (size_t)P.chunk_w;
+    const size_t parts = sizeof(long long) * (size_t)P.n_chunks * P.d.n_orb * (size_t)P.chunk_w;
     return kStatusBytes + (P.d.mode == TETRA_INTEGRATED ? 2 : 1) * parts;
 }
 
@@ -1467,7 +1460,9 @@ tetra_status_t launch_dos_forward(const Plan &P, const float *eps, const void *w
     A.status = reinterpret_cast<int *>(ws);
     A.queue = nullptr;
     A.G = reinterpret_cast<long long *>(static_cast<unsigned char *>(ws) + kStatusBytes);
-    A.Gs = A.G + (size_t)P.n_chunks * P.grid_x * P.d.n_orb * (size_t)P.chunk_w;
+    A.Gs = A.G + (size_t)P.n_chunks * P.d.n_orb * (size_t)P.chunk_w;
+    A.done = reinterpret_cast<int *>(static_cast<unsigned char *>(ws) + kDoneOffset);
+    A.dos = dos;
     cudaError_t e = cudaMemsetAsync(ws, 0, need, stream);
     if (e != cudaSuccess) return TETRA_ECUDA;
     const dim3 grid(P.grid_x, P.n_chunks);
@@ -1476,23 +1471,7 @@ tetra_status_t launch_dos_forward(const Plan &P, const float *eps, const void *w
         : mode == TETRA_BIN ? launch_norb<TETRA_BIN, 1>(P.d.n_orb, P.d.weight_dtype, P.smem_bytes, grid, Bt, A, stream)
                             : launch_norb<TETRA_INTEGRATED, 1>(P.d.n_orb, P.d.weight_dtype, P.smem_bytes, grid, Bt,
                                                                A, stream);
-    if (e != cudaSuccess) return TETRA_ECUDA;
-    if (mode == TETRA_INTEGRATED) {
-        const dim3 rgrid(P.d.n_orb, P.n_chunks);
-        tetra_dos_reduce_integrated<<<rgrid, 256, 0, stream>>>(A.G, A.Gs, P.grid_x, P.d.n_orb, P.d.n_omega,
-                                                               P.chunk_w, omega, Bt.m[0].vtvg, P.fixed_bits,
-                                                               dos);
-        if (cudaGetLastError() != cudaSuccess) return TETRA_ECUDA;
-        return TETRA_OK;
-    }
-    const long total = (long)P.d.n_orb * P.d.n_omega;
-    const int rb = 256;
-    const int rg = (int)std::min<long>((total + rb - 1) / rb, 4L * P.sm_count);
-    tetra_dos_reduce_kernel<<<rg, rb, 0, stream>>>(A.G, P.grid_x, P.d.n_orb, P.d.n_omega,
-                                                   P.chunk_w, P.d.mode, omega, Bt.m[0].vtvg,
-                                                   P.fixed_bits, dos);
-    if (cudaGetLastError() != cudaSuccess) return TETRA_ECUDA;
-    return TETRA_OK;
+    return e == cudaSuccess ? TETRA_OK : TETRA_ECUDA;
 }
 
 size_t dos_batched_workspace(const BatchPlan &B) {
@@ -1526,6 +1505,8 @@ tetra_status_t launch_dos_batched(const BatchPlan &BP, const float *const *eps, 
     A.queue = reinterpret_cast<int *>(static_cast<unsigned char *>(ws) + kQueueOffset);
     A.G = reinterpret_cast<long long *>(static_cast<unsigned char *>(ws) + kStatusBytes);
     A.Gs = nullptr;
+    A.done = nullptr;
+    A.dos = nullptr;
     cudaError_t e = cudaMemsetAsync(ws, 0, need, stream);   // status, counter, accumulators
     if (e != cudaSuccess) return TETRA_ECUDA;
     const dim3 grid(BP.grid_x, 1);

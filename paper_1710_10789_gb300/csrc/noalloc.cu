@@ -19,7 +19,7 @@ namespace tetra {
 namespace {
 
 // Scratch of the allocation-free entry point: the status words and the int64
-// per-CTA partial DOS of tetra_dos. It is a static device array, so every GPU
+// accumulators of tetra_dos. It is a static device array, so every GPU
 // that loads libtetra holds these bytes until the process exits.
 constexpr size_t kNoAllocScratchBytes = size_t(32) << 20;   // 32 MiB
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocScratchBytes];
@@ -81,18 +81,13 @@ extern "C" tetra_status_t tetra_dos_noalloc(tetra_plan_t plan, const float *eps,
     if (!plan || !eps || !w || !omega || !dos) return TETRA_EINVAL;
     if ((reinterpret_cast<uintptr_t>(eps) & 15u) || (reinterpret_cast<uintptr_t>(w) & 15u))
         return TETRA_EINVAL;
-    // Same kernels as tetra_dos; only the number of persistent CTAs is lowered
-    // when their int64 partials would not fit the fixed scratch. The result does
-    // not depend on that number (exact integer accumulation).
-    tetra::Plan q = *plan;
-    while (q.grid_x > 1 && tetra::dos_forward_workspace(q) > tetra::kNoAllocScratchBytes) --q.grid_x;
-    if (tetra::dos_forward_workspace(q) > tetra::kNoAllocScratchBytes) return TETRA_ENOMEM;
+    if (tetra::dos_forward_workspace(*plan) > tetra::kNoAllocScratchBytes) return TETRA_ENOMEM;
     const tetra::DeviceGuard dg(plan->device);
     if (!dg.ok()) return TETRA_ECUDA;
     void *scratch = nullptr;
     const tetra_status_t st = tetra::scratch_address(plan->device, &scratch, true);
     if (st != TETRA_OK) return st;
-    return tetra::launch_dos_forward(q, eps, w, omega, dos, scratch, tetra::kNoAllocScratchBytes,
+    return tetra::launch_dos_forward(*plan, eps, w, omega, dos, scratch, tetra::kNoAllocScratchBytes,
                                      stream);
 }
 

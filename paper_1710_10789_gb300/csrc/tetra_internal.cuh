@@ -56,6 +56,9 @@ namespace tetra {
 enum : int { kFlagTimeout = 1, kFlagRange = 2, kFlagConfig = 4 };
 constexpr size_t kStatusBytes = 256;
 constexpr size_t kQueueOffset = 64;   // batched launches: work counter inside the status bytes
+constexpr size_t kDoneOffset = 128;   // single-model launches: counters of finished CTAs
+constexpr int kDoneGroups = 32;       // energy chunks c, c + 32, ... share a counter
+static_assert(kDoneOffset + kDoneGroups * sizeof(int) <= kStatusBytes, "status bytes");
 
 using Plan = ::tetra_plan_s;
 
