@@ -2,28 +2,33 @@
 // DOS_s[i] = sum_{T,n} sum_l b_{l,s} [w_l(e_{i+1}) - w_l(e_i)] / (e_{i+1} - e_i),
 // computes dL/db and dL/deps at every k-point.
 //
-// One thread owns one (cube, band). For each of the cube's six tetrahedra it
-// sorts the corners once and, for every bin the tetrahedron overlaps,
-// evaluates the corner weights of Sec. II.C together with their derivatives
-// along all four corner energies (forward mode with four tangents; the six
-// reciprocal energy differences and their tangents are formed once per
-// tetrahedron, so the paper's formulas run on multiplies only). Then
-//   dL/db_{l,s}  += g_si dW_l/dE_i                                (bin averages)
-//   dL/de_r      += sum_i (1/width_i) sum_l [sum_s g_si b_{l,s}] d(dW_l)/de_r
-// for the sorted corners l, r, added into the cube's eight corner
-// accumulators (thread-private shared memory). Cubes are processed in eight
-// launches, one per parity class of the cube origin (x, y, z mod 2): two
-// cubes of one class share no point of the padded layout (the layout holds
-// the periodic images x = n1 etc. as separate points), so each class adds its
-// corner sums to the gradient arrays without atomics. A last pass folds the
-// periodic images onto the interior points. Every sum runs in a fixed order,
-// so the result is deterministic.
+// With the edge values D_{e,s} = G_{e-1,s} - G_{e,s}, G_{i,s} = g_si / width_i
+// (G_{-1} = G_{n_bins} = 0), the sum over bins is a sum over bin edges,
+//   L = sum_{T,n} sum_l sum_s b_{l,s} sum_e D_{e,s} w_l(e),
+// where edges at or below a tetrahedron's E1 give nothing and those at or
+// above E4 telescope to f G_{j-1,s} (w_l = f = V_T/(4 V_G) there; e_j the first
+// of them). So only the edges inside (E1, E4) cost work, a few or none:
+//   dL/db_{l,s} = f G_{j-1,s} + sum_e w_l(e) D_{e,s},
+//   dL/de_r     = - sum_e sum_l M_rl(e) k_l(e),  k_l(e) = sum_s b_{l,s} D_{e,s},
+// with M_rl(E) = int lambda_r lambda_l delta(E - D) over the tetrahedron, since
+// dw_l/de_r = -M_lr. The section at E is two triangles (12|23, 13, 14) and
+// (14, 24, 23|34) with corners on edges (see the forward kernel: the same
+// clamped edge fractions, no energy cases), and over a triangle of weight a
+// the integral of lambda_r lambda_l is a/12 (sum_v lambda_r^v lambda_l^v +
+// (sum_v lambda_r^v)(sum_v lambda_l^v)), so M k needs the three corner values
+// lambda^v . k only. (The weights with four forward-mode tangents at every
+// bin edge before took 2.4 ms at 64^3 points, 8 bands, 200 bins.)
 //
-// The kernel is bound by the latency of its loads and branches, not by its
-// arithmetic: three blocks per SM (168 registers) hide more of it than two.
-// To fit that register count, the third weight case runs through the first
-// case's code on the mirrored tetrahedron, which also keeps a warp whose
-// lanes sit in both outer cases on one path.
+// One thread owns one (cube, band) and adds its six tetrahedra's corner sums
+// into the cube's eight corner accumulators (thread-private shared memory).
+// Cubes are processed in eight launches, one per parity class of the cube
+// origin (x, y, z mod 2): two cubes of one class share no point of the padded
+// layout (the layout holds the periodic images x = n1 etc. as separate
+// points), so each class adds its corner sums to the gradient arrays without
+// atomics. A last pass folds the periodic images onto the interior points.
+// Every sum runs in a fixed order, so the result is deterministic.
+#include <algorithm>
+
 #include "tetra_internal.cuh"
 
 namespace tetra {
@@ -31,95 +36,57 @@ namespace tetra {
 namespace {
 
 constexpr int kBwdThreads = 128;
+constexpr int kBwdBlocks = 3;   // per SM
 
-// A value and its derivatives along the four sorted corner energies.
-struct F4 {
-    float v, d[4];
+// Sorted corner energies, the reciprocals of their differences and
+// V_T/(4 V_G) (f) and f / E41. A difference of zero gives an infinite
+// reciprocal, which the clamped products below turn into a step.
+struct TetB {
+    float e1, e2, e3;
+    float r21, r31, r41, r32, r42, r43;
+    float f, fr;
 };
-__device__ __forceinline__ F4 operator+(const F4 &a, const F4 &b) {
-    return F4{a.v + b.v, {a.d[0] + b.d[0], a.d[1] + b.d[1], a.d[2] + b.d[2], a.d[3] + b.d[3]}};
-}
-__device__ __forceinline__ F4 operator-(const F4 &a, const F4 &b) {
-    return F4{a.v - b.v, {a.d[0] - b.d[0], a.d[1] - b.d[1], a.d[2] - b.d[2], a.d[3] - b.d[3]}};
-}
-__device__ __forceinline__ F4 operator*(const F4 &a, const F4 &b) {
-    F4 r;
-    r.v = a.v * b.v;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) r.d[i] = fmaf(a.d[i], b.v, a.v * b.d[i]);
-    return r;
-}
-__device__ __forceinline__ F4 operator*(float s, const F4 &a) {
-    return F4{s * a.v, {s * a.d[0], s * a.d[1], s * a.d[2], s * a.d[3]}};
-}
-__device__ __forceinline__ F4 operator-(float s, const F4 &a) {
-    return F4{s - a.v, {-a.d[0], -a.d[1], -a.d[2], -a.d[3]}};
-}
-__device__ __forceinline__ F4 konst(float v) { return F4{v, {0.f, 0.f, 0.f, 0.f}}; }
-
-// Per-tetrahedron constants: the sorted corner energies with their tangents
-// (unit vectors) and the reciprocal energy differences 1/E_ab with theirs
-// (d(1/x) = -dx/x^2). A difference that is not positive gets 0: no region
-// that reads it is ever entered then (the regions are half-open, so every
-// executed branch has positive denominators).
-struct TetD {
-    F4 e1, e2, e3, e4;
-    F4 r21, r31, r41, r32, r42, r43;
-};
-__device__ __forceinline__ F4 rcp_diff(const F4 &a, const F4 &b) {   // 1 / (a - b)
-    const float x = a.v - b.v;
-    const float r = x > 0.f ? __fdividef(1.0f, x) : 0.f;
-    const float r2 = r * r;
-    return F4{r, {-(a.d[0] - b.d[0]) * r2, -(a.d[1] - b.d[1]) * r2, -(a.d[2] - b.d[2]) * r2,
-                  -(a.d[3] - b.d[3]) * r2}};
-}
-__device__ __forceinline__ void tetd_setup(TetD &T, const float e[4]) {
-    T.e1 = F4{e[0], {1.f, 0.f, 0.f, 0.f}};
-    T.e2 = F4{e[1], {0.f, 1.f, 0.f, 0.f}};
-    T.e3 = F4{e[2], {0.f, 0.f, 1.f, 0.f}};
-    T.e4 = F4{e[3], {0.f, 0.f, 0.f, 1.f}};
-    T.r21 = rcp_diff(T.e2, T.e1); T.r31 = rcp_diff(T.e3, T.e1); T.r41 = rcp_diff(T.e4, T.e1);
-    T.r32 = rcp_diff(T.e3, T.e2); T.r42 = rcp_diff(T.e4, T.e2); T.r43 = rcp_diff(T.e4, T.e3);
+__device__ __forceinline__ void tetb_setup(TetB &T, const float e[4], float f) {
+    T.e1 = e[0]; T.e3 = e[2];
+    // E2 = E3 = E4: no edge below E4 may see f32 > 0, and at E4 it is 1
+    T.e2 = e[1] < e[3] ? e[1] : nextafterf(e[3], -INFINITY);
+    T.r21 = __fdividef(1.f, e[1] - e[0]); T.r31 = __fdividef(1.f, e[2] - e[0]);
+    T.r41 = __fdividef(1.f, e[3] - e[0]); T.r32 = __fdividef(1.f, e[2] - e[1]);
+    T.r42 = __fdividef(1.f, e[3] - e[1]); T.r43 = __fdividef(1.f, e[3] - e[2]);
+    T.f = f;
+    T.fr = f * T.r41;
 }
 
-// Corner weights w_l(E) (Sec. II.C, all five cases) with their derivatives
-// along the four corner energies; f = V_T/(4 V_G). Regions are taken
-// half-open as in the forward kernel.
-__device__ __forceinline__ void weights4(const TetD &T, float E, float f, F4 w[4]) {
-    if (E <= T.e1.v) {
-#pragma unroll
-        for (int l = 0; l < 4; ++l) w[l] = konst(0.f);
-    } else if (E >= T.e4.v) {
-#pragma unroll
-        for (int l = 0; l < 4; ++l) w[l] = konst(f);
-    } else if (E > T.e2.v && E <= T.e3.v) {
-        const F4 a = konst(E) - T.e1, bq = konst(E) - T.e2, c = T.e3 - konst(E), dd = T.e4 - konst(E);
-        const F4 r3141 = T.r31 * T.r41;
-        const F4 C1 = f * ((a * a) * r3141);
-        const F4 C2 = f * (((a * bq) * c) * (r3141 * T.r32));
-        const F4 C3 = f * (((bq * bq) * dd) * ((T.r32 * T.r41) * T.r42));
-        const F4 C12 = C1 + C2, C23 = C2 + C3, C123 = C12 + C3;
-        w[0] = C1 + (C12 * c) * T.r31 + (C123 * dd) * T.r41;
-        w[1] = C123 + (C23 * c) * T.r32 + (C3 * dd) * T.r42;
-        w[2] = (C12 * a) * T.r31 + (C23 * bq) * T.r32;
-        w[3] = (C123 * a) * T.r41 + (C3 * bq) * T.r42;
-    } else {
-        // E1 < E <= E2, or E3 < E < E4 as the first case of the mirrored
-        // tetrahedron (energies -E4 <= -E3 <= -E2 <= -E1 at -E: distance
-        // E4 - E, reciprocals 1/E43, 1/E42, 1/E41), whose weights are f minus
-        // the original's in reverse corner order
-        const bool mir = E > T.e2.v;
-        const F4 x = mir ? T.e4 - konst(E) : konst(E) - T.e1;
-        const F4 ra = mir ? T.r43 : T.r21, rb = mir ? T.r42 : T.r31;
-        const F4 C = f * (((x * x) * x) * ((ra * rb) * T.r41));
-        const F4 S = ra + rb + T.r41;
-        const F4 Cx = C * x;
-        const F4 u0 = C * (4.f - x * S), u1 = Cx * ra, u2 = Cx * rb, u3 = Cx * T.r41;
-        w[0] = mir ? f - u3 : u0;
-        w[1] = mir ? f - u2 : u1;
-        w[2] = mir ? f - u1 : u2;
-        w[3] = mir ? f - u0 : u3;
-    }
+// At an edge E inside (E1, E4): the corner weights w and m = M k (both for the
+// sorted corners).
+__device__ __forceinline__ void edge_terms(const TetB &T, float E, const float (&k)[4], float (&w)[4], float (&m)[4]) {
+    const float x = E - T.e1, t = E - T.e2, y = E - T.e3;
+    const float f21 = __saturatef(x * T.r21), f31 = __saturatef(x * T.r31), f41 = __saturatef(x * T.r41);
+    const float f32 = __saturatef(t * T.r32), f42 = __saturatef(t * T.r42), f43 = __saturatef(y * T.r43);
+    const float f12 = 1.f - f21, f13 = 1.f - f31, f14 = 1.f - f41, f23 = 1.f - f32, f24 = 1.f - f42;
+    // volume below E: four simplices (forward kernel, tet_w)
+    const float fa = T.f * f41, fb = T.f * f14;
+    const float v1 = (f21 * f31) * fa, v2 = (f32 * f13) * fa;
+    const float v3 = (f32 * f42) * fb, v4 = (f43 * f24) * fb;
+    const float c13 = f13 + f14, s42 = f41 + f42, g23 = 1.f + f23;
+    w[0] = fmaf(v3 + v4, f14, fmaf(v2, c13, fmaf(v1, c13 + f12, v1)));
+    w[1] = fmaf(v4, f24, fmaf(v3, g23 + f24, fmaf(v2, g23, v1 * f21)));
+    w[2] = fmaf(v4, 2.f - f43, fmaf(v3, f32, fmaf(v2, f31 + f32, v1 * f31)));
+    w[3] = fmaf(v4, s42 + f43, fmaf(v3, s42, (v1 + v2) * f41));
+    // section at E: triangles of weight 12 fr p f31 and 12 fr q f24
+    const float p = f21 * f23, q = fmaf(-f32, f43, f32);
+    const float a = (p * f31) * T.fr, b = (q * f24) * T.fr;
+    const float k13 = fmaf(f13, k[0], f31 * k[2]), k14 = fmaf(f14, k[0], f41 * k[3]);
+    const float k24 = fmaf(f24, k[1], f42 * k[3]);
+    const float kx = fmaf(f12, k[0], fmaf(p, k[1], f32 * k[2]));   // corner 12 | 23
+    const float ky = fmaf(f23, k[1], fmaf(q, k[2], f43 * k[3]));   // corner 23 | 34
+    const float sa = k13 + k14 + kx, sb = k14 + k24 + ky;
+    const float t13 = a * (k13 + sa), tx = a * (kx + sa), t24 = b * (k24 + sb), ty = b * (ky + sb);
+    const float t14 = fmaf(a, k14 + sa, b * (k14 + sb));
+    m[0] = fmaf(f13, t13, fmaf(f14, t14, f12 * tx));
+    m[1] = fmaf(p, tx, fmaf(f24, t24, f23 * ty));
+    m[2] = fmaf(f31, t13, fmaf(f32, tx, q * ty));
+    m[3] = fmaf(f41, t14, fmaf(f42, t24, f43 * ty));
 }
 
 // Table I corner labels minus one.
@@ -135,13 +102,15 @@ struct BwdArgs {
     const float *edges;      // n_bins + 1
     const float *grad_dos;   // [n_orb][n_bins]
     float *geps, *gw;
-    int staged;              // grad_dos, edges and 1/widths copied to shared memory
+    int vec;                 // gw is 16-byte aligned (the caller's array may not be)
+    int staged;              // edges, G and D staged in shared memory
 };
 
-// Shared-memory bytes of the staged bin data, or 0 when it does not fit the
-// 64 KB budget.
-inline size_t bwd_stage_bytes(int n_orb, int n_bins) {
-    const size_t b = sizeof(float) * ((size_t)n_orb * n_bins + 2 * (size_t)n_bins + 1);
+// Shared-memory bytes of the staged edges, G and D (n_bins + 1 rows each;
+// row e of the first holds G_{e-1}), or 0 when they do not fit the 64 KB
+// budget.
+inline size_t bwd_stage_bytes(int norb_t, int n_bins) {
+    const size_t b = sizeof(float) * (((size_t)n_bins + 1 + 3) / 4 * 4 + 2 * (size_t)norb_t * (n_bins + 1));
     return b <= 64 * 1024 ? b : 0;
 }
 
@@ -150,137 +119,172 @@ inline size_t bwd_stage_bytes(int n_orb, int n_bins) {
 inline size_t bwd_scratch_bytes(int n_orb) { return sizeof(float) * (1 + (size_t)n_orb) * 8 * kBwdThreads; }
 
 template <int NORB, typename WT>
-__global__ void __launch_bounds__(kBwdThreads, 3) tetra_dos_bwd_kernel(const BwdArgs A, int px, int py, int pz) {
-    extern __shared__ float s_mem[];
-    const int ng = A.n_orb * A.n_bins;
-    const size_t stage = A.staged ? (size_t)ng + 2 * (size_t)A.n_bins + 1 : 0;
-    float *scr = s_mem + ((stage + 3) & ~size_t(3));   // [(1 + n_orb) * 8][blockDim]
-    const float *gd = A.grad_dos, *ed = A.edges, *siw = nullptr;
+__global__ void __launch_bounds__(kBwdThreads, kBwdBlocks) tetra_dos_bwd_kernel(const BwdArgs A, int px, int py, int pz) {
+    extern __shared__ __align__(16) float s_mem[];
+    const int n_e = A.n_bins + 1;
+    const int ed_words = (n_e + 3) & ~3;
+    const size_t stage = A.staged ? (size_t)ed_words + 2 * (size_t)NORB * n_e : 0;
+    float *scr = s_mem + stage;   // [(1 + n_orb) * 8][blockDim]
+    // G_{e-1,s}, from the gradient (0 beyond either end)
+    auto g_below = [&](int e, int s) -> float {
+        return e > 0 ? A.grad_dos[(long)s * A.n_bins + e - 1] / (A.edges[e] - A.edges[e - 1]) : 0.f;
+    };
+    const float *ed = A.edges, *sG = nullptr, *sD = nullptr;
     if (A.staged) {
-        for (int i = threadIdx.x; i < ng; i += blockDim.x) s_mem[i] = A.grad_dos[i];
-        for (int i = threadIdx.x; i <= A.n_bins; i += blockDim.x) s_mem[ng + i] = A.edges[i];
-        for (int i = threadIdx.x; i < A.n_bins; i += blockDim.x)
-            s_mem[ng + A.n_bins + 1 + i] = 1.0f / (A.edges[i + 1] - A.edges[i]);
+        for (int i = threadIdx.x; i < n_e; i += blockDim.x) s_mem[i] = A.edges[i];
+        float *G = s_mem + ed_words, *D = G + (size_t)NORB * n_e;
+        for (int i = threadIdx.x; i < NORB * n_e; i += blockDim.x) {
+            const int s = i / n_e, e = i - s * n_e;
+            const float lo = s < A.n_orb ? g_below(e, s) : 0.f;
+            const float hi = s < A.n_orb && e < A.n_bins ? g_below(e + 1, s) : 0.f;
+            G[e * NORB + s] = lo;
+            D[e * NORB + s] = lo - hi;
+        }
         __syncthreads();
-        gd = s_mem;
-        ed = s_mem + ng;
-        siw = s_mem + ng + A.n_bins + 1;
+        ed = s_mem;
+        sG = G;
+        sD = D;
     }
+    // row e of G_{e-1} or D_e
+    auto row = [&](bool diff, int e, float (&r)[NORB]) {
+        if (A.staged) {
+            load_weights<NORB, float>((diff ? sD : sG) + (size_t)e * NORB, NORB, r);
+        } else {
+#pragma unroll
+            for (int s = 0; s < NORB; ++s) {
+                r[s] = s < A.n_orb ? g_below(e, s) : 0.f;
+                if (diff && s < A.n_orb && e < A.n_bins) r[s] -= g_below(e + 1, s);
+            }
+        }
+    };
     // cubes of this parity class: x = px, px + 2, ... < n1 (same for y, z)
     const int cxn = (A.n1 - px + 1) >> 1, cyn = (A.n2 - py + 1) >> 1, czn = (A.n3 - pz + 1) >> 1;
-    const long gid = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (gid >= (long)cxn * cyn * czn * A.nb) return;
-    const int n = (int)(gid % A.nb);
-    const long cube = gid / A.nb;
-    const int x = px + 2 * (int)(cube % cxn), y = py + 2 * (int)((cube / cxn) % cyn),
-              z = pz + 2 * (int)(cube / ((long)cxn * cyn));
+    const long total = (long)cxn * cyn * czn * A.nb;
     const WT *W = static_cast<const WT *>(A.w);
     const int nv = 1 + A.n_orb;
     const int tid = threadIdx.x, nt = blockDim.x;
-    for (int v = 0; v < nv * 8; ++v) scr[v * nt + tid] = 0.f;
     const float om0 = ed[0];
     const float inv_de = (float)A.n_bins / (ed[A.n_bins] - om0);
-    for (int t = 0; t < 6; ++t) {
-        float e[4];
-        int pt[4], slot[4];
+    for (long gid = blockIdx.x * (long)blockDim.x + threadIdx.x; gid < total; gid += (long)gridDim.x * blockDim.x) {
+        const int n = (int)(gid % A.nb);
+        const long cube = gid / A.nb;
+        const int x = px + 2 * (int)(cube % cxn), y = py + 2 * (int)((cube / cxn) % cyn),
+                  z = pz + 2 * (int)(cube / ((long)cxn * cyn));
+        for (int v = 0; v < nv * 8; ++v) scr[v * nt + tid] = 0.f;
+        for (int t = 0; t < 6; ++t) {
+            float e[4];
+            int pt[4], slot[4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int cc = c_tab[t][q];
-            pt[q] = (x + (cc & 1)) + A.nx * ((y + ((cc >> 1) & 1)) + A.ny * (z + ((cc >> 2) & 1)));
-            e[q] = A.eps[(long)pt[q] * A.eps_stride + n];
-            slot[q] = q;
-        }
-        // sort corners by energy, carrying their Table-I slot (stable for ties)
+            for (int q = 0; q < 4; ++q) {
+                const int cc = c_tab[t][q];
+                pt[q] = (x + (cc & 1)) + A.nx * ((y + ((cc >> 1) & 1)) + A.ny * (z + ((cc >> 2) & 1)));
+                e[q] = A.eps[(long)pt[q] * A.eps_stride + n];
+                slot[q] = q;
+            }
+            // sort corners by energy, carrying their Table-I slot (stable for ties)
 #pragma unroll
-        for (int i = 1; i < 4; ++i)
+            for (int i = 1; i < 4; ++i)
 #pragma unroll
-            for (int j = i; j > 0; --j)
-                if (e[j] < e[j - 1]) {
-                    const float te = e[j]; e[j] = e[j - 1]; e[j - 1] = te;
-                    const int ts = slot[j]; slot[j] = slot[j - 1]; slot[j - 1] = ts;
-                }
-        // bins whose weight difference can be non-zero
-        int lo = (int)floorf(fminf(fmaxf((e[0] - om0) * inv_de, -2.f), (float)A.n_bins + 2.f));
-        int hi = (int)ceilf(fminf(fmaxf((e[3] - om0) * inv_de, -2.f), (float)A.n_bins + 2.f));
-        lo = min(max(lo, 0), A.n_bins);
-        hi = max(min(hi, A.n_bins - 1), -1);
-        while (lo > 0 && ed[lo] > e[0]) --lo;
-        while (lo < A.n_bins && ed[lo + 1] <= e[0]) ++lo;
-        while (hi < A.n_bins - 1 && (ed[hi + 1] < e[3] || ed[hi + 1] <= e[0])) ++hi;
-        while (hi >= 0 && !(ed[hi] < e[3] || ed[hi] <= e[0])) --hi;
-        if (lo > hi) continue;
-        // orbital weights of the four corners, in sorted order
-        float b[4][NORB];
+                for (int j = i; j > 0; --j)
+                    if (e[j] < e[j - 1]) {
+                        const float te = e[j]; e[j] = e[j - 1]; e[j - 1] = te;
+                        const int ts = slot[j]; slot[j] = slot[j - 1]; slot[j - 1] = ts;
+                    }
+            // edges inside (E1, E4): [lo, hi); hi is the first edge at or above E4
+            // and above E1 (a flat tetrahedron is empty at an edge equal to it)
+            int lo = (int)ceilf(fminf(fmaxf((e[0] - om0) * inv_de, -2.f), (float)A.n_bins + 2.f));
+            int hi = (int)ceilf(fminf(fmaxf((e[3] - om0) * inv_de, -2.f), (float)A.n_bins + 2.f));
+            lo = min(max(lo, 0), n_e);
+            hi = min(max(hi, 0), n_e);
+            while (lo > 0 && ed[lo - 1] > e[0]) --lo;
+            while (lo < n_e && ed[lo] <= e[0]) ++lo;
+            while (hi > 0 && ed[hi - 1] >= e[3]) --hi;
+            while (hi < n_e && ed[hi] < e[3]) ++hi;
+            hi = max(hi, lo);
+            // nothing below the first or above the last edge reaches a bin
+            if (hi == 0 || lo == n_e) continue;
+            float acc_e[4] = {0.f, 0.f, 0.f, 0.f};
+            float acc_w[4][NORB];
+            {
+                float g[NORB];   // f G_{hi-1}: the edges at or above E4
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
-            load_weights<NORB, WT>(W + (long)pt[slot[r]] * A.w_stride + (long)n * A.n_orb, A.n_orb, b[r]);
-        TetD TD;
-        tetd_setup(TD, e);
-        float acc_e[4] = {0.f, 0.f, 0.f, 0.f};
-        float acc_w[4][NORB];
+                for (int s = 0; s < NORB; ++s) g[s] = 0.f;
+                if (hi < n_e) row(false, hi, g);
 #pragma unroll
-        for (int r = 0; r < 4; ++r)
+                for (int s = 0; s < NORB; ++s)
 #pragma unroll
-            for (int s = 0; s < NORB; ++s) acc_w[r][s] = 0.f;
-        F4 wl[4], wu[4];
-        weights4(TD, ed[lo], A.f, wl);
-        for (int i = lo; i <= hi; ++i) {
-            weights4(TD, ed[i + 1], A.f, wu);
-            const float iw = siw ? siw[i] : 1.0f / (ed[i + 1] - ed[i]);
-            float dW[4], h[4] = {0.f, 0.f, 0.f, 0.f};
+                    for (int r = 0; r < 4; ++r) acc_w[r][s] = A.f * g[s];
+            }
+            if (lo < hi) {
+                float b[4][NORB];
 #pragma unroll
-            for (int l = 0; l < 4; ++l) dW[l] = (wu[l].v - wl[l].v) * iw;
+                for (int r = 0; r < 4; ++r)
+                    load_weights<NORB, WT>(W + (long)pt[slot[r]] * A.w_stride + (long)n * A.n_orb, A.n_orb, b[r]);
+                TetB T;
+                tetb_setup(T, e, A.f);
+                for (int i = lo; i < hi; ++i) {
+                    float g[NORB], k[4] = {0.f, 0.f, 0.f, 0.f}, w[4], m[4];
+                    row(true, i, g);
 #pragma unroll
-            for (int s = 0; s < NORB; ++s) {
-                if (s >= A.n_orb) continue;
-                const float g = gd[(long)s * A.n_bins + i];
+                    for (int s = 0; s < NORB; ++s)
 #pragma unroll
-                for (int l = 0; l < 4; ++l) {
-                    acc_w[l][s] = fmaf(g, dW[l], acc_w[l][s]);
-                    h[l] = fmaf(g, b[l][s], h[l]);
+                        for (int l = 0; l < 4; ++l) k[l] = fmaf(g[s], b[l][s], k[l]);
+                    edge_terms(T, ed[i], k, w, m);
+#pragma unroll
+                    for (int l = 0; l < 4; ++l) {
+                        acc_e[l] -= m[l];
+#pragma unroll
+                        for (int s = 0; s < NORB; ++s) acc_w[l][s] = fmaf(g[s], w[l], acc_w[l][s]);
+                    }
                 }
             }
-            // d(bin DOS contribution)/d(sorted corner energy r)
+            // add the sorted corners' sums to the cube-corner accumulators
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-                float de = 0.f;
+                const int c = c_tab[t][slot[r]];
+                scr[(0 * 8 + c) * nt + tid] += acc_e[r];
 #pragma unroll
-                for (int l = 0; l < 4; ++l) de = fmaf(h[l], wu[l].d[r] - wl[l].d[r], de);
-                acc_e[r] = fmaf(iw, de, acc_e[r]);
+                for (int s = 0; s < NORB; ++s)
+                    if (s < A.n_orb) scr[((1 + s) * 8 + c) * nt + tid] += acc_w[r][s];
             }
-#pragma unroll
-            for (int l = 0; l < 4; ++l) wl[l] = wu[l];
         }
-        // add the sorted corners' sums to the cube-corner accumulators
+        // this class's cubes share no point: plain read-modify-write
+        for (int c = 0; c < 8; ++c) {
+            const long p = (x + (c & 1)) + (long)A.nx * ((y + ((c >> 1) & 1)) + (long)A.ny * (z + (c >> 2)));
+            A.geps[p * A.eps_stride + n] += scr[(0 * 8 + c) * nt + tid];
+            float *gwp = A.gw + p * A.w_stride + (long)n * A.n_orb;
+            if (NORB % 4 == 0 && A.vec && A.n_orb == NORB) {
 #pragma unroll
-        for (int r = 0; r < 4; ++r) {
-            const int c = c_tab[t][slot[r]];
-            scr[(0 * 8 + c) * nt + tid] += acc_e[r];
-#pragma unroll
-            for (int s = 0; s < NORB; ++s)
-                if (s < A.n_orb) scr[((1 + s) * 8 + c) * nt + tid] += acc_w[r][s];
+                for (int v = 0; v < NORB / 4; ++v) {
+                    float4 *g4 = reinterpret_cast<float4 *>(gwp) + v;
+                    float4 g = *g4;
+                    g.x += scr[((1 + 4 * v) * 8 + c) * nt + tid];
+                    g.y += scr[((2 + 4 * v) * 8 + c) * nt + tid];
+                    g.z += scr[((3 + 4 * v) * 8 + c) * nt + tid];
+                    g.w += scr[((4 + 4 * v) * 8 + c) * nt + tid];
+                    *g4 = g;
+                }
+            } else {
+                for (int s = 0; s < A.n_orb; ++s) gwp[s] += scr[((1 + s) * 8 + c) * nt + tid];
+            }
         }
-    }
-    // this class's cubes share no point: plain read-modify-write
-    for (int c = 0; c < 8; ++c) {
-        const long p = (x + (c & 1)) + (long)A.nx * ((y + ((c >> 1) & 1)) + (long)A.ny * (z + (c >> 2)));
-        A.geps[p * A.eps_stride + n] += scr[(0 * 8 + c) * nt + tid];
-        float *gwp = A.gw + p * A.w_stride + (long)n * A.n_orb;
-        for (int s = 0; s < A.n_orb; ++s) gwp[s] += scr[((1 + s) * 8 + c) * nt + tid];
     }
 }
 
 // Folds the periodic images (x = n1, y = n2, z = n3 in the padded layout) onto
 // the interior point they copy and zeroes them: one thread per (interior
-// point on a face x = 0, y = 0 or z = 0, band), images added in a fixed order.
-// The face points are enumerated plane by plane: x = 0; y = 0 with x >= 1;
-// z = 0 with x, y >= 1.
+// point on a face x = 0, y = 0 or z = 0, value of its rows of both arrays),
+// images added in a fixed order. The face points are enumerated plane by
+// plane: x = 0; y = 0 with x >= 1; z = 0 with x, y >= 1. (One thread per
+// value: per (point, band) the orbitals' loads ran one after another, 81 us
+// at 64^3.)
 __global__ void tetra_dos_bwd_fold(const BwdArgs A) {
     const long fa = (long)A.n2 * A.n3, fb = (long)(A.n1 - 1) * A.n3, fc = (long)(A.n1 - 1) * (A.n2 - 1);
+    const int vals = A.nb * (1 + A.n_orb);
     const long gid = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (gid >= (fa + fb + fc) * A.nb) return;
-    const int n = (int)(gid % A.nb);
-    long k = gid / A.nb;
+    if (gid >= (fa + fb + fc) * vals) return;
+    const int v = (int)(gid % vals);
+    long k = gid / vals;
     int x, y, z;
     if (k < fa) {                      // plane x = 0
         x = 0; y = (int)(k % A.n2); z = (int)(k / A.n2);
@@ -290,37 +294,29 @@ __global__ void tetra_dos_bwd_fold(const BwdArgs A) {
         k -= fb;
         x = 1 + (int)(k % (A.n1 - 1)); y = 1 + (int)(k / (A.n1 - 1)); z = 0;
     }
-    const int mx = x == 0 ? 2 : 1, my = y == 0 ? 2 : 1, mz = z == 0 ? 2 : 1;
-    const long p0 = x + (long)A.nx * (y + (long)A.ny * z);
-    float se = A.geps[p0 * A.eps_stride + n];
-    for (int iz = 0; iz < mz; ++iz)
-        for (int iy = 0; iy < my; ++iy)
-            for (int ix = 0; ix < mx; ++ix) {
-                if (ix == 0 && iy == 0 && iz == 0) continue;
-                const long q = (x + ix * A.n1) + (long)A.nx * ((y + iy * A.n2) + (long)A.ny * (z + iz * A.n3));
-                se += A.geps[q * A.eps_stride + n];
-                A.geps[q * A.eps_stride + n] = 0.f;
-            }
-    A.geps[p0 * A.eps_stride + n] = se;
-    for (int s = 0; s < A.n_orb; ++s) {
-        float sw = A.gw[p0 * A.w_stride + (long)n * A.n_orb + s];
-        for (int iz = 0; iz < mz; ++iz)
-            for (int iy = 0; iy < my; ++iy)
-                for (int ix = 0; ix < mx; ++ix) {
-                    if (ix == 0 && iy == 0 && iz == 0) continue;
-                    const long q = (x + ix * A.n1) + (long)A.nx * ((y + iy * A.n2) + (long)A.ny * (z + iz * A.n3));
-                    float *gq = A.gw + q * A.w_stride + (long)n * A.n_orb + s;
-                    sw += *gq;
-                    *gq = 0.f;
-                }
-        A.gw[p0 * A.w_stride + (long)n * A.n_orb + s] = sw;
+    const bool is_e = v < A.nb;
+    float *base = is_e ? A.geps + v : A.gw + (v - A.nb);
+    const long stride = is_e ? A.eps_stride : A.w_stride;
+    float q[8], sum = 0.f;
+    float *at[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {   // the loads first: they overlap
+        const bool in = (x == 0 || !(i & 1)) && (y == 0 || !(i & 2)) && (z == 0 || !(i & 4));
+        const long p = (x + (i & 1) * A.n1) + (long)A.nx * ((y + ((i >> 1) & 1) * A.n2) + (long)A.ny * (z + (i >> 2) * A.n3));
+        at[i] = in ? base + p * stride : nullptr;
+        q[i] = in ? *at[i] : 0.f;
     }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) sum += q[i];
+    *at[0] = sum;
+#pragma unroll
+    for (int i = 1; i < 8; ++i)
+        if (at[i]) *at[i] = 0.f;
 }
 
 template <int NORB>
 cudaError_t launch_bwd_n(const Plan &P, const BwdArgs &A, cudaStream_t stream) {
-    const size_t stage = A.staged ? bwd_stage_bytes(A.n_orb, A.n_bins) : 0;
-    const size_t smem = ((stage + 15) & ~size_t(15)) + bwd_scratch_bytes(A.n_orb);
+    const size_t smem = (A.staged ? bwd_stage_bytes(NORB, A.n_bins) : 0) + bwd_scratch_bytes(A.n_orb);
     auto go = [&](auto kfn) {
         cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
@@ -329,12 +325,14 @@ cudaError_t launch_bwd_n(const Plan &P, const BwdArgs &A, cudaStream_t stream) {
             const long cubes = (long)((A.n1 - px + 1) >> 1) * ((A.n2 - py + 1) >> 1) * ((A.n3 - pz + 1) >> 1);
             const long total = cubes * A.nb;
             if (total == 0) continue;
-            const int grid = (int)((total + kBwdThreads - 1) / kBwdThreads);
+            // as many blocks as run at once: each stages the bin tables once
+            const int grid = (int)std::min<long>((total + kBwdThreads - 1) / kBwdThreads, (long)kBwdBlocks * P.sm_count);
             kfn<<<grid, kBwdThreads, smem, stream>>>(A, px, py, pz);
             e = cudaGetLastError();
             if (e != cudaSuccess) return e;
         }
-        const long face = ((long)A.n2 * A.n3 + (long)(A.n1 - 1) * A.n3 + (long)(A.n1 - 1) * (A.n2 - 1)) * A.nb;
+        const long face = ((long)A.n2 * A.n3 + (long)(A.n1 - 1) * A.n3 + (long)(A.n1 - 1) * (A.n2 - 1)) *
+                          A.nb * (1 + A.n_orb);
         tetra_dos_bwd_fold<<<(int)((face + 255) / 256), 256, 0, stream>>>(A);
         return cudaGetLastError();
     };
@@ -360,7 +358,8 @@ tetra_status_t launch_dos_backward(const Plan &P, const float *eps, const void *
     A.eps_stride = P.eps_stride; A.w_stride = P.w_stride;
     A.f = (float)(0.25 / (6.0 * (double)P.d.n1 * (double)P.d.n2 * (double)P.d.n3));
     A.eps = eps; A.w = w; A.edges = omega; A.grad_dos = grad_dos; A.geps = grad_eps; A.gw = grad_w;
-    A.staged = bwd_stage_bytes(A.n_orb, A.n_bins) > 0;
+    A.vec = (reinterpret_cast<uintptr_t>(grad_w) & 15u) == 0;
+    A.staged = bwd_stage_bytes(norb_template(A.n_orb), A.n_bins) > 0;
     if (cudaMemsetAsync(ws, 0, kStatusBytes, stream) != cudaSuccess) return TETRA_ECUDA;
     // the parity classes add into the arrays: start from zero (halo and
     // padding entries stay zero)
