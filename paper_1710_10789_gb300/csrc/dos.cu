@@ -722,6 +722,15 @@ __global__ void __maxnreg__(kMaxRegs)
                     load_weights<NORB, WT>(Ws + (long)pa[r4] * A.w_stride + n * A.n_orb, A.n_orb, ba[r4]);
                     load_weights<NORB, WT>(Ws + (long)pb[r4] * A.w_stride + n * A.n_orb, A.n_orb, bb[r4]);
                 }
+                if constexpr (NORB == 1) {
+                    // all weights zero: every contribution rounds to zero (the dither
+                    // is at most 1/2). Two thirds of a susceptibility's transition
+                    // bands have both ends occupied or both empty.
+                    float any = 0.f;
+#pragma unroll
+                    for (int r4 = 0; r4 < 4; ++r4) any = fmaxf(any, fmaxf(fabsf(ba[r4][0]), fabsf(bb[r4][0])));
+                    if (MODE != TETRA_INTEGRATED && any == 0.f) continue;
+                }
                 const float dith = item_dither((gcube * 3u + (uint32_t)pr) * (uint32_t)A.nb + (uint32_t)n);
                 if constexpr (MODE == TETRA_INTEGRATED) {
                     // Occupation: the walk over the union window adds both

@@ -15,44 +15,66 @@ __device__ __forceinline__ float occupation(float e, float mu, float inv_kT) {
     return 0.5f * (1.0f - tanhf(0.5f * (e - mu) * inv_kT));
 }
 
-// One thread per padded point of the pair plan's layout (halo included).
+// A block takes kPairPoints padded points of the pair plan's layout (halo
+// included): one thread per (point, band) evaluates both points' energies and
+// occupations into shared memory, then the block writes the NB^2 values of
+// each point in order. Bound by the two output arrays (140 MB at 64^3 points
+// and 8 bands: 21 us at the copy bandwidth); one thread per point, writing
+// its own row 4 bytes at a time and 256 bytes from its neighbour's, took
+// 231 us.
+constexpr int kPairPoints = 64;
+constexpr int kPairThreads = 256;
 template <int NB>
-__global__ void pair_bands_kernel(const float *eps, int eps_stride, int n1, int n2, int n3, int nx, int ny,
-                                  int qx, int qy, int qz, float mu, float inv_kT, long n_pts,
-                                  float *eps_p, int eps_stride_p, float *w_p, int w_stride_p) {
-    const long p = blockIdx.x * (long)blockDim.x + threadIdx.x;
-    if (p >= n_pts) return;
-    const int px = (int)(p % nx), py = (int)((p / nx) % ny), pz = (int)(p / ((long)nx * ny));
-    const int x = px % n1, y = py % n2, z = pz % n3;
-    const long pk = x + (long)nx * (y + (long)ny * z);
-    const int xq = (x + qx) % n1, yq = (y + qy) % n2, zq = (z + qz) % n3;
-    const long pkq = xq + (long)nx * (yq + (long)ny * zq);
-    float ek[NB], ekq[NB], fk[NB], fkq[NB];
-#pragma unroll
-    for (int n = 0; n < NB; ++n) {
-        ek[n] = eps[pk * eps_stride + n];
-        ekq[n] = eps[pkq * eps_stride + n];
-        fk[n] = occupation(ek[n], mu, inv_kT);
-        fkq[n] = occupation(ekq[n], mu, inv_kT);
+__global__ void __launch_bounds__(kPairThreads)
+    pair_bands_kernel(const float *eps, int eps_stride, int n1, int n2, int n3, int nx, int ny, int qx, int qy, int qz,
+                      float mu, float inv_kT, long n_pts, float *eps_p, int eps_stride_p, float *w_p, int w_stride_p) {
+    __shared__ float ek[kPairPoints][NB], ekq[kPairPoints][NB], fk[kPairPoints][NB], fkq[kPairPoints][NB];
+    const long p0 = blockIdx.x * (long)kPairPoints;
+    const int np = (int)min((long)kPairPoints, n_pts - p0);
+    for (int i = threadIdx.x; i < np * NB; i += kPairThreads) {
+        const int l = i / NB, n = i - l * NB;
+        const long p = p0 + l;
+        const int px = (int)(p % nx), py = (int)((p / nx) % ny), pz = (int)(p / ((long)nx * ny));
+        const int x = px % n1, y = py % n2, z = pz % n3;
+        const int xq = (x + qx) % n1, yq = (y + qy) % n2, zq = (z + qz) % n3;
+        const float a = eps[(x + (long)nx * (y + (long)ny * z)) * eps_stride + n];
+        const float c = eps[(xq + (long)nx * (yq + (long)ny * zq)) * eps_stride + n];
+        ek[l][n] = a;
+        ekq[l][n] = c;
+        fk[l][n] = occupation(a, mu, inv_kT);
+        fkq[l][n] = occupation(c, mu, inv_kT);
     }
-    float *eo = eps_p + p * eps_stride_p;
-    float *wo = w_p + p * w_stride_p;
+    __syncthreads();
+    // whole 16-byte vectors where a row is a multiple of them (rows start on
+    // 16-byte boundaries in both layouts)
+    constexpr int V = NB % 2 == 0 ? 4 : 1;
+    constexpr int RV = NB * NB / V;
+    for (int i = threadIdx.x; i < np * RV; i += kPairThreads) {
+        const int l = i / RV, j0 = (i - l * RV) * V;
+        float e[V], w[V];
 #pragma unroll
-    for (int n = 0; n < NB; ++n)
-#pragma unroll
-        for (int m = 0; m < NB; ++m) {
-            eo[n * NB + m] = ekq[m] - ek[n];
-            wo[n * NB + m] = fk[n] - fkq[m];
+        for (int v = 0; v < V; ++v) {
+            const int n = (j0 + v) / NB, m = (j0 + v) - n * NB;
+            e[v] = ekq[l][m] - ek[l][n];
+            w[v] = fk[l][n] - fkq[l][m];
         }
+        float *eo = eps_p + (p0 + l) * eps_stride_p + j0, *wo = w_p + (p0 + l) * w_stride_p + j0;
+        if constexpr (V == 4) {
+            *reinterpret_cast<float4 *>(eo) = make_float4(e[0], e[1], e[2], e[3]);
+            *reinterpret_cast<float4 *>(wo) = make_float4(w[0], w[1], w[2], w[3]);
+        } else {
+            *eo = e[0];
+            *wo = w[0];
+        }
+    }
 }
 
 template <int NB>
 cudaError_t launch_nb(const Plan &P, const Plan &Q, const float *eps, const int q[3], float mu, float inv_kT,
                       float *eps_p, float *w_p, cudaStream_t stream) {
     const long n_pts = (long)Q.nx * Q.ny * Q.nz;
-    const int threads = 128;
-    const long blocks = (n_pts + threads - 1) / threads;
-    pair_bands_kernel<NB><<<(unsigned)blocks, threads, 0, stream>>>(
+    const long blocks = (n_pts + kPairPoints - 1) / kPairPoints;
+    pair_bands_kernel<NB><<<(unsigned)blocks, kPairThreads, 0, stream>>>(
         eps, P.eps_stride, P.d.n1, P.d.n2, P.d.n3, P.nx, P.ny, q[0], q[1], q[2], mu, inv_kT, n_pts, eps_p,
         Q.eps_stride, w_p, Q.w_stride);
     return cudaGetLastError();
