@@ -149,8 +149,42 @@ static tetra_status_t plan_geometry(Plan &P, const int box[3], int ctas_per_sm) 
     return TETRA_OK;
 }
 
+// Box of a single-model plan. CTAs take boxes in rounds of grid_x, so the time
+// goes with rounds x (cubes per box + overhead of a box): a small grid wants
+// boxes that fill a round (60x60x10 points, 4x4x4 boxes: 4.4 rounds and every
+// sixth cube plane off the grid; 8x4x2: 3.9), a large one wants large boxes
+// (256^3, 200 bins: 26.3 ms with 4x4x4, 23.8 ms with 8x4x4, from which the
+// overhead of about 8 cubes; less in point mode, more in bin mode). A shape
+// may hold up to twice the default's items where the shared memory has room
+// beside the same energy tile and tile copies. The result does not depend on
+// the shape.
+static void choose_box(const Plan &P0, int box[3]) {
+    if (std::getenv("TETRA_BOX_X") || std::getenv("TETRA_BOX_Y") || std::getenv("TETRA_BOX_Z")) return;
+    auto cost = [](const Plan &P) {
+        const long rounds = ((long)P.n_boxes + P.grid_x - 1) / P.grid_x;
+        return (double)rounds * (P.BX * P.BY * P.BZ + 8);
+    };
+    const int per_cube = P0.items_per_box / (P0.BX * P0.BY * P0.BZ);
+    const int most = std::max(P0.items_per_box, 2 * 1536);
+    double best = cost(P0) * 0.98;   // (the default unless another is clearly better)
+    for (int bx = 2; bx <= 8; bx *= 2)
+        for (int by = 2; by <= 8; by *= 2)
+            for (int bz = 1; bz <= 8; bz *= 2) {
+                if ((long)bx * by * bz * per_cube > most) continue;
+                Plan P = P0;
+                const int b[3] = {bx, by, bz};
+                if (plan_geometry(P, b, env_int("TETRA_CTAS_PER_SM", 1)) != TETRA_OK) continue;
+                if (P.n_chunks != P0.n_chunks || P.tile_copies < P0.tile_copies) continue;
+                const double c = cost(P);
+                if (c < best) {
+                    best = c;
+                    for (int i = 0; i < 3; ++i) box[i] = b[i];
+                }
+            }
+}
+
 // Validates a description and fills a plan for it (box shape given).
-tetra_status_t plan_init(Plan &P, const tetra_desc_t &d, int device, const int box[3], int ctas_per_sm) {
+tetra_status_t plan_init(Plan &P, const tetra_desc_t &d, int device, const int box[3], int ctas_per_sm, bool choose) {
     if (d.n1 < 1 || d.n2 < 1 || d.n3 < 1 || d.n1 > 4096 || d.n2 > 4096 || d.n3 > 4096)
         return TETRA_EINVAL;
     if (d.n_bands < 1 || d.n_bands > 64 || d.n_orb < 1 || d.n_orb > 16 || d.n_omega < 1)
@@ -182,7 +216,11 @@ tetra_status_t plan_init(Plan &P, const tetra_desc_t &d, int device, const int b
         return TETRA_ECUDA;
     P.sm_count = sms;
     P.smem_optin = (size_t)optin;
-    return plan_geometry(P, box, ctas_per_sm);
+    const tetra_status_t st = plan_geometry(P, box, ctas_per_sm);
+    if (st != TETRA_OK || !choose) return st;
+    int best[3] = {box[0], box[1], box[2]};
+    choose_box(P, best);
+    return plan_geometry(P, best, ctas_per_sm);
 }
 
 }  // namespace tetra
@@ -198,7 +236,7 @@ tetra_status_t tetra_plan(tetra_plan_t *plan, const tetra_desc_t *desc, int devi
     tetra::default_box(*desc, box);
     Plan *P = new (std::nothrow) Plan();
     if (!P) return TETRA_ENOMEM;
-    tetra_status_t st = tetra::plan_init(*P, *desc, device, box, tetra::env_int("TETRA_CTAS_PER_SM", 1));
+    tetra_status_t st = tetra::plan_init(*P, *desc, device, box, tetra::env_int("TETRA_CTAS_PER_SM", 1), true);
     if (st != TETRA_OK) {
         delete P;
         return st;
@@ -322,7 +360,7 @@ tetra_status_t tetra_plan_batched(tetra_batch_plan_t *plan, const tetra_desc_t *
     B->device = device;
     B->big = 0;
     for (int m = 0; m < n_models; ++m) {
-        tetra_status_t st = tetra::plan_init(B->models[m], descs[m], device, box, ctas_per_sm);
+        tetra_status_t st = tetra::plan_init(B->models[m], descs[m], device, box, ctas_per_sm, false);
         if (st != TETRA_OK) return fail(st);
         if (descs[m].n_omega > descs[B->big].n_omega) B->big = m;
     }

@@ -102,7 +102,8 @@ struct FwdArgs {
     uint32_t e_stage, w_stage;           // their shared-memory slots (128-byte multiples)
     int chunk_w;         // energies per shared tile (largest model of a batch)
     int tile_copies;     // copies of the tile; lane l of a bin-mode pair adds into copy l % tile_copies
-    int items_per_box;   // items per box: (pair, band) in point mode, (tetrahedron, band) otherwise
+    int items_per_box;   // items per box: (pair, band), with more than 8 orbitals (tetrahedron, band)
+    int split;           // log2 of the lanes that share a pair's walk (point and integrated mode)
     int fast_cap;
     unsigned flush_at;   // a 64-energy block is flushed once its bound reaches this
     long long *G;        // int64 accumulators, [slot][n_orb][chunk_w]; slot = chunk, or model of a batch
@@ -673,7 +674,9 @@ __global__ void __maxnreg__(kMaxRegs)
         bmax = 0.f;
         for (int i = 0; i < nwarp; ++i) bmax = fmaxf(bmax, red_f[i]);
         const int n_active = s_active;
-        const int n_slots = (n_active + 31) >> 5;
+        // (lanes per pair: bin mode walks in order, 16 orbitals have one tetrahedron)
+        const int ls = MODE != TETRA_BIN && Cfg<NORB>::pairs ? A.split : 0;
+        const int n_slots = ((n_active << ls) + 31) >> 5;
 
         // Pass B: slot q holds the 32 items of ranks 32q .. 32q+31 (nearly equal
         // window length, so a warp's lanes finish together). Warps claim slots
@@ -685,8 +688,9 @@ __global__ void __maxnreg__(kMaxRegs)
             claim = __shfl_sync(0xffffffffu, claim, 0);
             if (claim >= n_slots) break;
             const int pos = (n_slots - 1 - claim) * 32 + lane;
-            const bool valid = pos < n_active;
-            const int it = valid ? (int)s_list[pos] : 0;
+            const bool valid = pos < (n_active << ls);
+            const int it = valid ? (int)s_list[pos >> ls] : 0;
+            const int part = pos & ((1 << ls) - 1);   // this lane takes the window's energies part, part + 2^ls, ...
             const int cube = it & (ncube - 1);
             const int rest = it >> lcube;
             const int cx = cube & (A.BX - 1), cy = (cube >> A.lbx) & (A.BY - 1), cz = cube >> (A.lbx + A.lby);
@@ -744,13 +748,13 @@ __global__ void __maxnreg__(kMaxRegs)
                     // the first energy beyond the window (a flat pair, E1 = E4, is
                     // empty at E = E1: lo is above E1)
                     const int hs = hi + 1;
-                    const bool step = hs < w0 + wc;
+                    const bool step = part == 0 && hs < w0 + wc;
                     // steps on the chunk's first energy (there go the steps of all
                     // tetrahedra below the chunk) are summed over the warp first
                     const bool first = fast && step && hs == w0;
                     const unsigned qbnd = fast ? (unsigned)qmax + 2u : 0u;
                     if (fast) {
-                        if (hi >= lo) {
+                        if (hi >= lo && part == 0) {
                             for (int bk = (lo - w0) >> 6; bk <= ((hi - w0) >> 6); ++bk) atomicAdd(&blk_bound[bk], qbnd);
                             atomicAdd(&tile[(lo - w0) * TS + CNT], 1);
                             atomicAdd(&tile[(hi + 1 - w0) * TS + CNT], -1);
@@ -777,8 +781,8 @@ __global__ void __maxnreg__(kMaxRegs)
                         }
                     }
                     if (fast) {
-                        const int K = hi - lo + 1;
-                        int i = lo + ((lane * max(K, 1)) >> 5);
+                        const int K = (hi - lo - part + (1 << ls)) >> ls, i0 = lo + part, i1 = i0 + ((K - 1) << ls);
+                        int i = i0 + (((lane * max(K, 1)) >> 5) << ls);
                         for (int j = 0; j < K; ++j) {
                             float wa[4], wb[4];
                             tet_w(TA, om[i - w0], wa);
@@ -796,7 +800,7 @@ __global__ void __maxnreg__(kMaxRegs)
                                 acc = fmaf(bb[3][s], wb[3], acc);
                                 atomicAdd(col + s, __float_as_int(acc + kMagic));
                             }
-                            i = (i == hi) ? lo : i + 1;
+                            i = (i == i1) ? i0 : i + (1 << ls);
                         }
                         if (step && !first) {
 #pragma unroll
@@ -804,7 +808,7 @@ __global__ void __maxnreg__(kMaxRegs)
                                 atomicAdd(&stile[(hs - w0) * NORB + s], __float_as_int(full(s) + kMagic) - kMagicBits);
                         }
                     } else {
-                        for (int i = lo; i <= hi; ++i) {
+                        for (int i = lo + part; i <= hi; i += 1 << ls) {
                             float wa[4], wb[4];
                             tet_w(TA, om[i - w0], wa);
                             tet_w(TB, om[i - w0], wb);
@@ -894,7 +898,7 @@ __global__ void __maxnreg__(kMaxRegs)
                 const float qb = (eb[3] > eb[0]) ? bmax * 4.f * fq * 3.1f * safe_rcp(eb[3] - eb[0]) : 0.f;
                 const float qmax = qa + qb;
                 const bool fast = qmax < (float)A.fast_cap;
-                if (fast) {
+                if (fast && part == 0) {
                     const unsigned qbnd = (unsigned)qmax + 2u;
                     for (int bk = (lo - w0) >> 6; bk <= ((hi - w0) >> 6); ++bk) atomicAdd(&blk_bound[bk], qbnd);
                     atomicAdd(&tile[(lo - w0) * TS + CNT], 1);
@@ -905,8 +909,8 @@ __global__ void __maxnreg__(kMaxRegs)
                 tet_setup<MODE>(TB, eb[0], eb[1], eb[2], eb[3], fq);
                 if (fast) {
                     // lane-dependent start, wrapping walk (see below)
-                    const int K = hi - lo + 1;
-                    int i = lo + ((lane * K) >> 5);
+                    const int K = (hi - lo - part + (1 << ls)) >> ls, i0 = lo + part, i1 = i0 + ((K - 1) << ls);
+                    int i = i0 + (((lane * K) >> 5) << ls);
                     for (int j = 0; j < K; ++j) {
                         float da[4], db[4];   // zero outside a tetrahedron's own window
                         tet_dw(TA, om[i - w0], da);
@@ -924,10 +928,10 @@ __global__ void __maxnreg__(kMaxRegs)
                             acc = fmaf(bb[3][s], db[3], acc);
                             atomicAdd(col + s, __float_as_int(acc + kMagic));
                         }
-                        i = (i == hi) ? lo : i + 1;
+                        i = (i == i1) ? i0 : i + (1 << ls);
                     }
                 } else {
-                    for (int i = lo; i <= hi; ++i) {
+                    for (int i = lo + part; i <= hi; i += 1 << ls) {
                         float da[4], db[4];   // zero outside a tetrahedron's own window
                         tet_dw(TA, om[i - w0], da);
                         tet_dw(TB, om[i - w0], db);
@@ -1275,7 +1279,8 @@ cudaError_t launch_t(size_t smem, dim3 grid, const Batch<MAXM> &Bt, const FwdArg
         }
     }
     // no more warps than a box has items for (idle ones only slow its barriers)
-    const int threads = std::min(kThreads, std::max(128, (A.items_per_box + 31) & ~31));
+    const int items = A.items_per_box << (MODE != TETRA_BIN && Cfg<NORB>::pairs ? A.split : 0);
+    const int threads = std::min(kThreads, std::max(128, (items + 31) & ~31));
     k<<<grid, threads, smem, stream>>>(Bt, A);
     return cudaGetLastError();
 }
@@ -1315,6 +1320,10 @@ void fill_common(const Plan &P, FwdArgs &A) {
     A.chunk_w = P.chunk_w;
     A.tile_copies = P.tile_copies;
     A.items_per_box = P.items_per_box;
+    // few items per box (few bands): up to 8 lanes share a pair's walk, so that
+    // the box still has work for all warps and the walks are that much shorter
+    A.split = 0;
+    while (A.split < 3 && (P.items_per_box << (A.split + 1)) <= kThreads) ++A.split;
     A.flush_at = 1u << P.flush_bits;
     long cap = ((1L << 30) - (1L << 20)) / A.items_per_box;
     if (cap > (1L << 21)) cap = 1L << 21;

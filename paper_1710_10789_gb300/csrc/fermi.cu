@@ -271,14 +271,15 @@ __global__ void __launch_bounds__(kFermiThreads, 3) fermi_round_kernel(const Fer
     if (!(nhi - nlo < hi - lo) || nhi <= nextafterf(nlo, INFINITY)) S->done = 1;
 }
 
-// The integrated-mode plan of a plan (same grid, box and orbitals): a plan
-// without one has no Fermi level.
+// The integrated-mode plan of a plan (same grid and orbitals, default box): a
+// plan without one has no Fermi level.
 tetra_status_t integrated_plan(const Plan &P, Plan &Q) {
     tetra_desc_t d = P.d;
     d.mode = TETRA_INTEGRATED;
     d.n_omega = 64;
-    const int box[3] = {P.BX, P.BY, P.BZ};
-    return plan_init(Q, d, P.device, box, 1);
+    int box[3];
+    default_box(d, box);
+    return plan_init(Q, d, P.device, box, 1, false);
 }
 
 // Tile of at most 128 cubes with at most kTilePoints points whose values fit

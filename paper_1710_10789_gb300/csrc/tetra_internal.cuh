@@ -221,7 +221,7 @@ tetra_status_t launch_dos_batched(const BatchPlan &B, const float *const *eps, c
                                   const float *const *omega, float *const *dos, void *ws,
                                   size_t ws_bytes, cudaStream_t stream);
 size_t dos_batched_workspace(const BatchPlan &B);
-tetra_status_t plan_init(Plan &P, const tetra_desc_t &d, int device, const int box[3], int ctas_per_sm);
+tetra_status_t plan_init(Plan &P, const tetra_desc_t &d, int device, const int box[3], int ctas_per_sm, bool choose);
 void default_box(const tetra_desc_t &d, int box[3]);
 tetra_status_t launch_dos_backward(const Plan &P, const float *eps, const void *w,
                                    const float *omega, const float *grad_dos, float *grad_eps,
