@@ -76,6 +76,10 @@ template <int NORB>
 struct Cfg {
     static constexpr bool pairs = NORB <= 8;
     static constexpr int units_per_cube = pairs ? 3 : 6;
+    // a pair's corner values added per corner before the projection
+    // (merge_pair): 15 operations against 3 multiply-adds per orbital
+    static constexpr bool merge = NORB >= 8;
+    static constexpr int rows = merge ? 5 : 8;   // weight rows of a pair
 };
 constexpr int kKBins = 256;     // window-length histogram bins (K >= 255 share one)
 
@@ -218,6 +222,48 @@ __device__ __forceinline__ void item_window(float e1, float e4, const float *om,
         while (lo < w0 + wc && om[lo + 1 - w0] <= e1) ++lo;
         while (hi < w0 + wc - 1 && (om[hi + 1 - w0] < e4 || om[hi + 1 - w0] <= e1)) ++hi;
         while (hi >= w0 && !(om[hi - w0] < e4 || om[hi - w0] <= e1)) --hi;
+    }
+}
+
+// A tetrahedron of a pair: its own corner's energy x merged into the sorted
+// face (e, ascending), and where it lies (below face corner j).
+struct PairOrder {
+    float e[4];
+    bool below[3];
+    __device__ __forceinline__ PairOrder(const float (&f)[3], float x) {
+        e[0] = fminf(x, f[0]);
+        e[1] = fmaxf(f[0], fminf(x, f[1]));
+        e[2] = fmaxf(f[1], fminf(x, f[2]));
+        e[3] = fmaxf(f[2], x);
+#pragma unroll
+        for (int j = 0; j < 3; ++j) below[j] = x < f[j];
+    }
+    // the points of the sorted corners: p[0..2] the face's, x the own one
+    __device__ __forceinline__ void place(const int *p, int x, int (&o)[4]) const {
+        o[0] = below[0] ? x : p[0];
+        o[1] = below[0] ? p[0] : (below[1] ? x : p[1]);
+        o[2] = below[1] ? p[1] : (below[2] ? x : p[2]);
+        o[3] = below[2] ? p[2] : x;
+    }
+};
+
+// Corner values of a pair's two tetrahedra (each in its own sorted order)
+// added per corner: the face's three, then the two own corners. 15 selects
+// and adds that save 3 n_orb multiply-adds of the projection and 3 n_orb
+// registers. With few orbitals (8 rows) they stay apart.
+__device__ __forceinline__ void merge_pair(const PairOrder &A, const PairOrder &B, const float (&a)[4],
+                                           const float (&b)[4], float (&d)[5]) {
+#pragma unroll
+    for (int j = 0; j < 3; ++j) d[j] = (A.below[j] ? a[j + 1] : a[j]) + (B.below[j] ? b[j + 1] : b[j]);
+    d[3] = A.below[1] ? (A.below[0] ? a[0] : a[1]) : (A.below[2] ? a[2] : a[3]);
+    d[4] = B.below[1] ? (B.below[0] ? b[0] : b[1]) : (B.below[2] ? b[2] : b[3]);
+}
+__device__ __forceinline__ void merge_pair(const PairOrder &, const PairOrder &, const float (&a)[4],
+                                           const float (&b)[4], float (&d)[8]) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        d[j] = a[j];
+        d[4 + j] = b[j];
     }
 }
 
@@ -707,32 +753,51 @@ __global__ void __maxnreg__(kMaxRegs)
                 // ---- a pair of tetrahedra sharing a face, walked over the union window
                 const int pr = rest % 3, n = rest / 3;
                 const uint32_t code = pair_code(pr);
-                float ea[4], eb[4];
-                int pa[4], pb[4];
+                // the face's three corners sorted, the first and the second
+                // tetrahedron's own corner merged into that order
+                float es[3];
+                int ps[5];
 #pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    pa[q] = pb[q] = p0 + s_cdelta[(code >> (3 * q)) & 7];
-                    ea[q] = eb[q] = Es[pa[q] * A.eps_stride + n];
-                }
-                pa[3] = p0 + s_cdelta[(code >> 9) & 7];
-                pb[3] = p0 + s_cdelta[(code >> 12) & 7];
-                ea[3] = Es[pa[3] * A.eps_stride + n];
-                eb[3] = Es[pb[3] * A.eps_stride + n];
-                sort4(ea, pa);
-                sort4(eb, pb);
-                float ba[4][NORB], bb[4][NORB];
+                for (int q = 0; q < 5; ++q) ps[q] = p0 + s_cdelta[(code >> (3 * q)) & 7];
 #pragma unroll
-                for (int r4 = 0; r4 < 4; ++r4) {
-                    load_weights<NORB, WT>(Ws + (long)pa[r4] * A.w_stride + n * A.n_orb, A.n_orb, ba[r4]);
-                    load_weights<NORB, WT>(Ws + (long)pb[r4] * A.w_stride + n * A.n_orb, A.n_orb, bb[r4]);
+                for (int q = 0; q < 3; ++q) es[q] = Es[ps[q] * A.eps_stride + n];
+                cswap(es[0], es[1], ps[0], ps[1]);
+                cswap(es[1], es[2], ps[1], ps[2]);
+                cswap(es[0], es[1], ps[0], ps[1]);
+                const PairOrder oa(es, Es[ps[3] * A.eps_stride + n]), ob(es, Es[ps[4] * A.eps_stride + n]);
+                const float (&ea)[4] = oa.e, (&eb)[4] = ob.e;
+                // weights: of the face's corners and the two own ones, or of each
+                // tetrahedron's corners in its sorted order
+                constexpr int ROWS = Cfg<NORB>::rows;
+                float bw[ROWS][NORB];
+                if constexpr (Cfg<NORB>::merge) {
+#pragma unroll
+                    for (int q = 0; q < 5; ++q)
+                        load_weights<NORB, WT>(Ws + (long)ps[q] * A.w_stride + n * A.n_orb, A.n_orb, bw[q]);
+                } else {
+                    int pa[4], pb[4];
+                    oa.place(ps, ps[3], pa);
+                    ob.place(ps, ps[4], pb);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        load_weights<NORB, WT>(Ws + (long)pa[q] * A.w_stride + n * A.n_orb, A.n_orb, bw[q]);
+                        load_weights<NORB, WT>(Ws + (long)pb[q] * A.w_stride + n * A.n_orb, A.n_orb, bw[ROWS - 4 + q]);
+                    }
                 }
+                // both tetrahedra's corner values (rows of bw) of orbital s, dithered
+                auto project = [&](const float (&d)[ROWS], int s, float dith) {
+                    float acc = fmaf(bw[0][s], d[0], dith);
+#pragma unroll
+                    for (int q = 1; q < ROWS; ++q) acc = fmaf(bw[q][s], d[q], acc);
+                    return acc;
+                };
                 if constexpr (NORB == 1) {
                     // all weights zero: every contribution rounds to zero (the dither
                     // is at most 1/2). Two thirds of a susceptibility's transition
                     // bands have both ends occupied or both empty.
                     float any = 0.f;
 #pragma unroll
-                    for (int r4 = 0; r4 < 4; ++r4) any = fmaxf(any, fmaxf(fabsf(ba[r4][0]), fabsf(bb[r4][0])));
+                    for (int q = 0; q < ROWS; ++q) any = fmaxf(any, fabsf(bw[q][0]));
                     if (MODE != TETRA_INTEGRATED && any == 0.f) continue;
                 }
                 const float dith = item_dither((gcube * 3u + (uint32_t)pr) * (uint32_t)A.nb + (uint32_t)n);
@@ -766,8 +831,11 @@ __global__ void __maxnreg__(kMaxRegs)
                     tet_setup<MODE>(TB, eb[0], eb[1], eb[2], eb[3], fq);
                     // the pair's saturated contribution of orbital s
                     auto full = [&](int s) {
-                        return fq * (((ba[0][s] + ba[1][s]) + (ba[2][s] + ba[3][s])) +
-                                     ((bb[0][s] + bb[1][s]) + (bb[2][s] + bb[3][s]))) + dith;
+                        if constexpr (Cfg<NORB>::merge)
+                            return fq * (2.f * ((bw[0][s] + bw[1][s]) + bw[2][s]) + (bw[3][s] + bw[4][s])) + dith;
+                        else
+                            return fq * (((bw[0][s] + bw[1][s]) + (bw[2][s] + bw[3][s])) +
+                                         ((bw[ROWS - 4][s] + bw[ROWS - 3][s]) + (bw[ROWS - 2][s] + bw[ROWS - 1][s]))) + dith;
                     };
                     if (__any_sync(vmask, first)) {
                         // the warp's first-energy steps: integer sums, one add per orbital
@@ -784,20 +852,14 @@ __global__ void __maxnreg__(kMaxRegs)
                         const int K = (hi - lo - part + (1 << ls)) >> ls, i0 = lo + part, i1 = i0 + ((K - 1) << ls);
                         int i = i0 + (((lane * max(K, 1)) >> 5) << ls);
                         for (int j = 0; j < K; ++j) {
-                            float wa[4], wb[4];
+                            float wa[4], wb[4], d5[ROWS];
                             tet_w(TA, om[i - w0], wa);
                             tet_w(TB, om[i - w0], wb);
+                            merge_pair(oa, ob, wa, wb, d5);
                             int *col = tile + (i - w0) * TS;
 #pragma unroll
                             for (int s = 0; s < NORB; ++s) {
-                                float acc = fmaf(ba[0][s], wa[0], dith);
-                                acc = fmaf(ba[1][s], wa[1], acc);
-                                acc = fmaf(ba[2][s], wa[2], acc);
-                                acc = fmaf(ba[3][s], wa[3], acc);
-                                acc = fmaf(bb[0][s], wb[0], acc);
-                                acc = fmaf(bb[1][s], wb[1], acc);
-                                acc = fmaf(bb[2][s], wb[2], acc);
-                                acc = fmaf(bb[3][s], wb[3], acc);
+                                const float acc = project(d5, s, dith);
                                 atomicAdd(col + s, __float_as_int(acc + kMagic));
                             }
                             i = (i == i1) ? i0 : i + (1 << ls);
@@ -809,20 +871,14 @@ __global__ void __maxnreg__(kMaxRegs)
                         }
                     } else {
                         for (int i = lo + part; i <= hi; i += 1 << ls) {
-                            float wa[4], wb[4];
+                            float wa[4], wb[4], d5[ROWS];
                             tet_w(TA, om[i - w0], wa);
                             tet_w(TB, om[i - w0], wb);
+                            merge_pair(oa, ob, wa, wb, d5);
 #pragma unroll
                             for (int s = 0; s < NORB; ++s) {
                                 if (s >= A.n_orb) continue;
-                                float acc = fmaf(ba[0][s], wa[0], dith);
-                                acc = fmaf(ba[1][s], wa[1], acc);
-                                acc = fmaf(ba[2][s], wa[2], acc);
-                                acc = fmaf(ba[3][s], wa[3], acc);
-                                acc = fmaf(bb[0][s], wb[0], acc);
-                                acc = fmaf(bb[1][s], wb[1], acc);
-                                acc = fmaf(bb[2][s], wb[2], acc);
-                                acc = fmaf(bb[3][s], wb[3], acc);
+                                const float acc = project(d5, s, dith);
                                 deposit_one(acc, Gc + (long)s * A.chunk_w + (i - w0), A.status);
                             }
                         }
@@ -856,33 +912,29 @@ __global__ void __maxnreg__(kMaxRegs)
                     Tet TA, TB;
                     tet_setup<MODE>(TA, ea[0], ea[1], ea[2], ea[3], fq);
                     tet_setup<MODE>(TB, eb[0], eb[1], eb[2], eb[3], fq);
-                    float wpa[4], wpb[4];
-                    tet_w(TA, om[lo - w0], wpa);
-                    tet_w(TB, om[lo - w0], wpb);
+                    // (weights of both by corner, then differences)
+                    auto both = [&](float E, float (&w5)[ROWS]) {
+                        float wa[4], wb[4];
+                        tet_w(TA, E, wa);
+                        tet_w(TB, E, wb);
+                        merge_pair(oa, ob, wa, wb, w5);
+                    };
+                    float wp[ROWS];
+                    both(om[lo - w0], wp);
                     int *col = tl + (lo - w0) * TS;
                     for (int i = lo; i <= hi; ++i, col += TS) {
-                        float wna[4], wnb[4], da[4], db[4];
-                        tet_w(TA, om[i + 1 - w0], wna);
-                        tet_w(TB, om[i + 1 - w0], wnb);
+                        float wn[ROWS], d5[ROWS];
+                        both(om[i + 1 - w0], wn);
                         const float sc = iw[i - w0];
 #pragma unroll
-                        for (int r4 = 0; r4 < 4; ++r4) {
-                            da[r4] = (wna[r4] - wpa[r4]) * sc;
-                            wpa[r4] = wna[r4];
-                            db[r4] = (wnb[r4] - wpb[r4]) * sc;
-                            wpb[r4] = wnb[r4];
+                        for (int q = 0; q < ROWS; ++q) {
+                            d5[q] = (wn[q] - wp[q]) * sc;
+                            wp[q] = wn[q];
                         }
 #pragma unroll
                         for (int s = 0; s < NORB; ++s) {
                             if (!fast && s >= A.n_orb) continue;
-                            float acc = fmaf(ba[0][s], da[0], dith);
-                            acc = fmaf(ba[1][s], da[1], acc);
-                            acc = fmaf(ba[2][s], da[2], acc);
-                            acc = fmaf(ba[3][s], da[3], acc);
-                            acc = fmaf(bb[0][s], db[0], acc);
-                            acc = fmaf(bb[1][s], db[1], acc);
-                            acc = fmaf(bb[2][s], db[2], acc);
-                            acc = fmaf(bb[3][s], db[3], acc);
+                            const float acc = project(d5, s, dith);
                             if (fast)
                                 atomicAdd(col + s, __float_as_int(acc + kMagic));
                             else
@@ -912,40 +964,28 @@ __global__ void __maxnreg__(kMaxRegs)
                     const int K = (hi - lo - part + (1 << ls)) >> ls, i0 = lo + part, i1 = i0 + ((K - 1) << ls);
                     int i = i0 + (((lane * K) >> 5) << ls);
                     for (int j = 0; j < K; ++j) {
-                        float da[4], db[4];   // zero outside a tetrahedron's own window
+                        float da[4], db[4], d5[ROWS];   // zero outside a tetrahedron's own window
                         tet_dw(TA, om[i - w0], da);
                         tet_dw(TB, om[i - w0], db);
+                        merge_pair(oa, ob, da, db, d5);
                         int *col = tile + (i - w0) * TS;
 #pragma unroll
                         for (int s = 0; s < NORB; ++s) {
-                            float acc = fmaf(ba[0][s], da[0], dith);
-                            acc = fmaf(ba[1][s], da[1], acc);
-                            acc = fmaf(ba[2][s], da[2], acc);
-                            acc = fmaf(ba[3][s], da[3], acc);
-                            acc = fmaf(bb[0][s], db[0], acc);
-                            acc = fmaf(bb[1][s], db[1], acc);
-                            acc = fmaf(bb[2][s], db[2], acc);
-                            acc = fmaf(bb[3][s], db[3], acc);
+                            const float acc = project(d5, s, dith);
                             atomicAdd(col + s, __float_as_int(acc + kMagic));
                         }
                         i = (i == i1) ? i0 : i + (1 << ls);
                     }
                 } else {
                     for (int i = lo + part; i <= hi; i += 1 << ls) {
-                        float da[4], db[4];   // zero outside a tetrahedron's own window
+                        float da[4], db[4], d5[ROWS];   // zero outside a tetrahedron's own window
                         tet_dw(TA, om[i - w0], da);
                         tet_dw(TB, om[i - w0], db);
+                        merge_pair(oa, ob, da, db, d5);
 #pragma unroll
                         for (int s = 0; s < NORB; ++s) {
                             if (s >= A.n_orb) continue;
-                            float acc = fmaf(ba[0][s], da[0], dith);
-                            acc = fmaf(ba[1][s], da[1], acc);
-                            acc = fmaf(ba[2][s], da[2], acc);
-                            acc = fmaf(ba[3][s], da[3], acc);
-                            acc = fmaf(bb[0][s], db[0], acc);
-                            acc = fmaf(bb[1][s], db[1], acc);
-                            acc = fmaf(bb[2][s], db[2], acc);
-                            acc = fmaf(bb[3][s], db[3], acc);
+                            const float acc = project(d5, s, dith);
                             deposit_one(acc, Gc + (long)s * A.chunk_w + (i - w0), A.status);
                         }
                     }
