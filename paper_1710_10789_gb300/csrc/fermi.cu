@@ -9,13 +9,15 @@
 // block narrows the bracket and keeps N(lo), exact integers, so the rounds
 // run back to back without the host.
 //
-// One block takes tiles of cubes: it stages the band energies of the tile's
-// points in shared memory and the summed weights of the bands that reach the
-// bracket; a warp takes 32 cubes of
-// one band (their windows nearly coincide, so an energy that no lane's cube
-// contains is skipped by a vote: below a cube nothing, above it the full
-// weight). The corner weights need no energy cases (tet_common.cuh).
-// Each cube's N(E) - N(lo) is rounded once to an integer of 2^-26 of a full
+// One block takes tiles of cubes. It stages the band energies of the tile's
+// points in shared memory, lists the (cube, band) items that reach the bracket
+// (a few percent from the second round on), stages the summed weights of their
+// bands, and hands the items out 32 at a time, kPer energies to a task, so
+// that warps are full and all of them have work (a warp per row of 32 cubes,
+// active or not, took 4.8 ms at the size below). An energy that no lane's
+// cube contains is skipped by a vote: below a cube nothing, above it the full
+// weight. The corner weights need no energy cases (tet_common.cuh). Each
+// cube's N(E) - N(lo) is rounded once to an integer of 2^-26 of a full
 // tetrahedron, summed over the warp by two 32-bit reductions, over the
 // block's warps and over the grid by integer adds: exact in any order.
 //
@@ -33,11 +35,12 @@ namespace tetra {
 namespace {
 
 constexpr int kPts = 16;           // energies per round: bracket / 16
+constexpr int kPer = 4;            // energies per task
 constexpr int kRounds = 64;        // at most; FP32 resolution takes about six
 constexpr int kRoundsPerSync = 7;
 constexpr int kFermiThreads = 256;
+constexpr int kFermiBlocks = 3;    // per SM
 constexpr int kUnitBits = 26;
-constexpr int kTilePoints = 297;   // (32 + 1) (2 + 1) (2 + 1), the largest tile below
 
 // Order-preserving map of a float to an unsigned int (for atomic min / max).
 __device__ __forceinline__ unsigned ordered(float f) {
@@ -89,7 +92,7 @@ __global__ void band_range_kernel(const float4 *eps, long n_vec, int row_vec, in
 
 struct FermiArgs {
     int n1, n2, n3, nx, ny, nb, n_orb, eps_stride, w_stride;
-    int tx, ty, tz;          // tile of cubes (tx ty tz = 128 at most)
+    int tx, lty, ltz;        // tile of cubes: tx (at most 31: a row of its points is a warp), 2^lty, 2^ltz
     int ntx, nty, n_tiles;
     double n_electrons, vtvg;
     const float *eps;
@@ -102,14 +105,35 @@ __device__ __forceinline__ float grid_energy(float lo, float hi, int j) {
     return j == kPts - 1 ? hi : lo + (hi - lo) * ((float)(j + 1) * (1.0f / kPts));
 }
 
+// Sum of n_orb weights, 16 bytes at a time where they fill whole vectors (the
+// rows of the layout start on 16-byte boundaries).
 template <typename WT>
-__global__ void __launch_bounds__(kFermiThreads, 3) fermi_round_kernel(const FermiArgs A) {
-    extern __shared__ float s_pt[];   // energies, then summed weights, [tile point][nb]
+__device__ __forceinline__ float sum_weights(const WT *b, int n_orb, bool vec) {
+    float t = 0.f;
+    if (vec) {
+        constexpr int V = 16 / sizeof(WT);
+        for (int s = 0; s < n_orb; s += V) {
+            const uint4 q = *reinterpret_cast<const uint4 *>(b + s);
+            const WT *e = reinterpret_cast<const WT *>(&q);
+#pragma unroll
+            for (int v = 0; v < V; ++v) t += to_f32<WT>(e[v]);
+        }
+    } else {
+        for (int s = 0; s < n_orb; ++s) t += to_f32<WT>(b[s]);
+    }
+    return t;
+}
+
+template <typename WT>
+__global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kernel(const FermiArgs A) {
+    extern __shared__ float s_pt[];   // energies, then summed weights, [band][ps]; items
     __shared__ unsigned long long s_sum[kPts];
     __shared__ float s_om[kPts];
-    __shared__ unsigned s_reach[2][2][2];   // of two tiles in turn
+    __shared__ unsigned s_band[2][2];   // bands with an item, of two tiles in turn
+    __shared__ int s_count[2];          // items, of two tiles in turn
     __shared__ int s_last;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nwarp = kFermiThreads / 32;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    constexpr int nwarp = kFermiThreads / 32;
     FermiState *S = A.S;
     const bool first = S->round == 0;
     if (S->done) return;   // (set by an earlier launch only)
@@ -126,111 +150,157 @@ __global__ void __launch_bounds__(kFermiThreads, 3) fermi_round_kernel(const Fer
         s_sum[tid] = 0ull;
         s_om[tid] = grid_energy(lo, hi, tid);
     }
-    const int px = A.tx + 1, py = A.ty + 1, npt = px * py * (A.tz + 1), nv = npt * A.nb;
-    float *se = s_pt, *sw = s_pt + nv;
-    const int ncube = A.tx * A.ty * A.tz, groups = (ncube + 31) >> 5;
+    // tile points (x, row) at 32 row + x, band by band: a warp reads and
+    // writes consecutive words
+    const int ty = 1 << A.lty, tz = 1 << A.ltz, py = ty + 1, rows = py * (tz + 1), ps = rows * 32 + 1;
+    const int lcol = A.lty + A.ltz;   // log2 of the (y, z) columns
+    float *se = s_pt, *sw = s_pt + A.nb * ps;
+    unsigned short *item = reinterpret_cast<unsigned short *>(sw + A.nb * ps);   // (band, column, x)
     const float fq = (float)(1 << kUnitBits) * 0.25f;
     const WT *W = static_cast<const WT *>(A.w);
+    const bool vec = (A.n_orb * sizeof(WT)) % 16 == 0;
+    // an item's first corner in the tile
+    auto point_of = [&](int it) {
+        const int col = (it >> 5) & ((1 << lcol) - 1), cy = col & (ty - 1), cz = col >> A.lty;
+        return (it >> (5 + lcol)) * ps + (it & 31) + 32 * (cy + py * cz);
+    };
+    const int dy = 32, dz = 32 * py;
     long long acc = 0;   // lane j: this warp's sum at energy j
-    int tile_par = 0;
-    for (int tile = blockIdx.x; tile < A.n_tiles; tile += gridDim.x) {
+    int par = 0;
+    for (int tile = blockIdx.x; tile < A.n_tiles; tile += gridDim.x, par ^= 1) {
         const int bx = tile % A.ntx, by = (tile / A.ntx) % A.nty, bz = tile / (A.ntx * A.nty);
-        const int x0 = bx * A.tx, y0 = by * A.ty, z0 = bz * A.tz;
-        if (tid < 4) s_reach[tile_par][tid >> 1][tid & 1] = 0u;
+        const int x0 = bx * A.tx, y0 = by << A.lty, z0 = bz << A.ltz;
+        const bool in_x = lane <= A.tx && x0 + lane <= A.n1;
+        if (tid < 2) s_band[par][tid] = 0u;
+        if (tid == 2) s_count[par] = 0;
         __syncthreads();   // the previous tile is read
-        // bands with some energy at or above lo / at or below hi
-        unsigned long long up = 0ull, down = 0ull;
-        for (int i = tid; i < nv; i += kFermiThreads) {
-            const int p = i / A.nb, n = i - p * A.nb;
-            const int x = min(x0 + p % px, A.n1), y = min(y0 + (p / px) % py, A.n2), z = min(z0 + p / (px * py), A.n3);
-            const float e = A.eps[(x + (long)A.nx * (y + (long)A.ny * z)) * A.eps_stride + n];
-            se[i] = e;
-            up |= (unsigned long long)(e >= lo) << n;
-            down |= (unsigned long long)(e <= hi) << n;
+        for (int r = warp; r < rows; r += nwarp) {
+            const int y = min(y0 + r % py, A.n2), z = min(z0 + r / py, A.n3);
+            const float4 *src = reinterpret_cast<const float4 *>(
+                A.eps + (x0 + lane + (long)A.nx * (y + (long)A.ny * z)) * A.eps_stride);
+#pragma unroll 2
+            for (int v = 0; v < A.eps_stride / 4; ++v) {
+                const float4 q = in_x ? src[v] : make_float4(0.f, 0.f, 0.f, 0.f);
+                float *o = se + 4 * v * ps + r * 32 + lane;
+                o[0] = q.x;
+                if (4 * v + 1 < A.nb) o[ps] = q.y;
+                if (4 * v + 2 < A.nb) o[2 * ps] = q.z;
+                if (4 * v + 3 < A.nb) o[3 * ps] = q.w;
+            }
         }
-        // (nb <= 64: two 32-bit votes each; s_reach was cleared before the first barrier)
+        __syncthreads();
+        for (int q = warp; q < A.nb << lcol; q += nwarp) {
+            const int n = q >> lcol, it = q * 32 + lane, col = q & ((1 << lcol) - 1);
+            const int p = point_of(it);
+            bool act = false;
+            if (lane < A.tx && x0 + lane < A.n1 && y0 + (col & (ty - 1)) < A.n2 && z0 + (col >> A.lty) < A.n3) {
+                float emin = INFINITY, emax = -INFINITY;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const unsigned u = __reduce_or_sync(0xffffffffu, (unsigned)(up >> (32 * h)));
-            const unsigned d = __reduce_or_sync(0xffffffffu, (unsigned)(down >> (32 * h)));
-            if (lane == 0 && u) atomicOr(&s_reach[tile_par][0][h], u);
-            if (lane == 0 && d) atomicOr(&s_reach[tile_par][1][h], d);
+                for (int k = 0; k < 8; ++k) {
+                    const float e = se[p + (k & 1) + ((k >> 1) & 1) * dy + (k >> 2) * dz];
+                    emin = fminf(emin, e);
+                    emax = fmaxf(emax, e);
+                }
+                act = emax >= lo && emin <= hi;
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, act);
+            if (!m) continue;
+            int base = 0;
+            if (lane == 0) {
+                base = atomicAdd(&s_count[par], __popc(m));
+                atomicOr(&s_band[par][n >> 5], 1u << (n & 31));
+            }
+            base = __shfl_sync(0xffffffffu, base, 0);
+            if (act) item[base + __popc(m & ((1u << lane) - 1u))] = (unsigned short)it;
         }
         __syncthreads();
-        const unsigned long long reach =
-            ((unsigned long long)(s_reach[tile_par][0][1] & s_reach[tile_par][1][1]) << 32) |
-            (s_reach[tile_par][0][0] & s_reach[tile_par][1][0]);
-        tile_par ^= 1;
-        if (!reach) continue;
-        for (int i = tid; i < nv; i += kFermiThreads) {
-            const int p = i / A.nb, n = i - p * A.nb;
-            if (!((reach >> n) & 1ull)) continue;
-            const int x = min(x0 + p % px, A.n1), y = min(y0 + (p / px) % py, A.n2), z = min(z0 + p / (px * py), A.n3);
-            const WT *b = W + (x + (long)A.nx * (y + (long)A.ny * z)) * A.w_stride + (long)n * A.n_orb;
-            float t = 0.f;
-            for (int s = 0; s < A.n_orb; ++s) t += to_f32<WT>(b[s]);
-            sw[i] = t;
+        const int count = s_count[par];
+        if (count == 0) continue;
+        unsigned long long bands = ((unsigned long long)s_band[par][1] << 32) | s_band[par][0];
+        while (bands) {
+            const int n = __ffsll((long long)bands) - 1;
+            bands &= bands - 1;
+#pragma unroll 2
+            for (int r = warp; r < rows; r += nwarp) {
+                const int y = min(y0 + r % py, A.n2), z = min(z0 + r / py, A.n3);
+                if (in_x)
+                    sw[n * ps + r * 32 + lane] = sum_weights<WT>(
+                        W + (x0 + lane + (long)A.nx * (y + (long)A.ny * z)) * A.w_stride + n * A.n_orb, A.n_orb, vec);
+            }
         }
         __syncthreads();
-        for (int item = warp; item < A.nb * groups; item += nwarp) {
-            const int n = item / groups, cube = (item - n * groups) * 32 + lane;
-            if (!((reach >> n) & 1ull)) continue;
-            const int cx = cube % A.tx, cy = (cube / A.tx) % A.ty, cz = cube / (A.tx * A.ty);
-            const bool in = cube < ncube && x0 + cx < A.n1 && y0 + cy < A.n2 && z0 + cz < A.n3;
+        const int groups = (count + 31) >> 5;
+        for (int task = warp; task < groups * (kPts / kPer); task += nwarp) {
+            const int g = task % groups, j0 = (task / groups) * kPer;
+            const bool act = g * 32 + lane < count;
+            const int p = point_of(item[act ? g * 32 + lane : 0]);
             float e[8], b[8];
             float emin = INFINITY, emax = -INFINITY;
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const int p = (in ? cx + px * (cy + py * cz) : 0) + (q & 1) + px * (((q >> 1) & 1) + py * (q >> 2));
-                e[q] = se[p * A.nb + n];
-                b[q] = sw[p * A.nb + n];
-                emin = fminf(emin, e[q]);
-                emax = fmaxf(emax, e[q]);
+            for (int k = 0; k < 8; ++k) {
+                const int o = p + (k & 1) + ((k >> 1) & 1) * dy + (k >> 2) * dz;
+                e[k] = se[o];
+                b[k] = sw[o];
+                emin = fminf(emin, e[k]);
+                emax = fmaxf(emax, e[k]);
             }
-            const bool act = in && emax >= lo && emin <= hi;
-            if (!__any_sync(0xffffffffu, act)) continue;
-            Tet T[6];
-            float bs[6][4], at_lo = 0.f, full = 0.f;
+            // which of the task's energies some lane's cube contains, and whether
+            // some lane's cube holds lo: without either no tetrahedron is set up
+            float E[kPer];
+            bool in[kPer], any[kPer], some = __any_sync(0xffffffffu, act && lo > emin);
 #pragma unroll
-            for (int t = 0; t < 6; ++t) {
-                float es[4], w[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int c = (tet_code(t) >> (3 * q)) & 7;
-                    es[q] = e[c];
-                    bs[t][q] = b[c];
-                }
-                sort4(es, bs[t]);
-                tet_setup<TETRA_INTEGRATED>(T[t], es[0], es[1], es[2], es[3], fq);
-                tet_w(T[t], lo, w);
-                full = fmaf(fq, (bs[t][0] + bs[t][1]) + (bs[t][2] + bs[t][3]), full);
-#pragma unroll
-                for (int q = 0; q < 4; ++q) at_lo = fmaf(bs[t][q], w[q], at_lo);
+            for (int j = 0; j < kPer; ++j) {
+                E[j] = s_om[j0 + j];
+                in[j] = act && E[j] >= emin && E[j] <= emax;
+                any[j] = __any_sync(0xffffffffu, in[j]);
+                some = some || any[j];
             }
-            // one rounding per energy; the same integers whatever the bracket
-            const long long q_lo = __float2ll_rn(at_lo), q_full = __float2ll_rn(full);
-#pragma unroll 1
-            for (int j = 0; j < kPts; ++j) {
-                const float E = s_om[j];
-                long long q = 0;
-                // a flat tetrahedron at E is empty there: only above emax all is full
-                if (act) q = (E > emax ? q_full : 0) - q_lo;
-                const bool in_cube = act && E >= emin && E <= emax;
-                if (__any_sync(0xffffffffu, in_cube)) {
-                    float v = 0.f;
+            float at_lo = 0.f, v[kPer];
 #pragma unroll
-                    for (int t = 0; t < 6; ++t) {
-                        float w[4];
-                        tet_w(T[t], E, w);
+            for (int j = 0; j < kPer; ++j) v[j] = 0.f;
+            if (some) {
+                // one tetrahedron after another; the sums run in the same order for
+                // every energy, so a cube's value at an energy does not depend on the
+                // bracket it is asked in
 #pragma unroll
-                        for (int r = 0; r < 4; ++r) v = fmaf(bs[t][r], w[r], v);
+                for (int t = 0; t < 6; ++t) {
+                    float es[4], bs[4], w[4];
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int c = (tet_code(t) >> (3 * k)) & 7;
+                        es[k] = e[c];
+                        bs[k] = b[c];
                     }
-                    if (in_cube) q = __float2ll_rn(v) - q_lo;
+                    sort4(es, bs);
+                    Tet T;
+                    tet_setup<TETRA_INTEGRATED>(T, es[0], es[1], es[2], es[3], fq);
+                    tet_w(T, lo, w);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) at_lo = fmaf(bs[k], w[k], at_lo);
+#pragma unroll
+                    for (int j = 0; j < kPer; ++j) {
+                        if (!any[j]) continue;
+                        tet_w(T, E[j], w);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) v[j] = fmaf(bs[k], w[k], v[j]);
+                    }
                 }
+            }
+            // all six full: a corner counts once for each tetrahedron that has it
+            float full = 0.f;
+#pragma unroll
+            for (int t = 0; t < 6; ++t)
+#pragma unroll
+                for (int k = 0; k < 4; ++k) full += fq * b[(tet_code(t) >> (3 * k)) & 7];
+            const long long q_lo = __float2ll_rn(at_lo), q_full = __float2ll_rn(full);
+#pragma unroll
+            for (int j = 0; j < kPer; ++j) {
+                // (a flat tetrahedron at E is empty there: only above emax all is full)
+                const long long q = act ? (in[j] ? __float2ll_rn(v[j]) : (E[j] > emax ? q_full : 0)) - q_lo : 0;
                 // q = high 2^24 + low, low in [0, 2^24): sums of 32 fit 32 bits
                 const long long sum = ((long long)__reduce_add_sync(0xffffffffu, (int)(q >> 24)) << 24) +
                                       (long long)__reduce_add_sync(0xffffffffu, (unsigned)(q & 0xFFFFFF));
-                if (lane == j) acc += sum;
+                if (lane == j0 + j) acc += sum;
             }
         }
     }
@@ -282,14 +352,22 @@ tetra_status_t integrated_plan(const Plan &P, Plan &Q) {
     return plan_init(Q, d, P.device, box, 1, false);
 }
 
-// Tile of at most 128 cubes with at most kTilePoints points whose values fit
-// the shared memory: long rows in x, for the warps' 32 cubes.
+// Shared memory of a tile: energies and summed weights of its points, items.
+size_t tile_bytes(const FermiArgs &A) {
+    const int ty = 1 << A.lty, tz = 1 << A.ltz;
+    return A.nb * (2 * sizeof(float) * ((size_t)(ty + 1) * (tz + 1) * 32 + 1) + sizeof(unsigned short) * 32 * ty * tz);
+}
+
+// Rows of nearly equal length in x, up to 4 x 4 columns as long as three
+// blocks share an SM's shared memory (at most 70 KB: 64 bands, one column).
 void choose_tile(const Plan &P, FermiArgs &A) {
-    A.tx = std::min(32, P.d.n1);
-    A.ty = std::min(2, P.d.n2);
-    A.tz = std::min(2, P.d.n3);
-    while (A.tx * A.ty * A.tz < 128 && A.ty < P.d.n2 && (A.tx + 1) * (A.ty + 2) * (A.tz + 1) <= kTilePoints) ++A.ty;
-    while (A.tx * A.ty * A.tz < 128 && A.tz < P.d.n3 && (A.tx + 1) * (A.ty + 1) * (A.tz + 2) <= kTilePoints) ++A.tz;
+    A.ntx = (P.d.n1 + 30) / 31;
+    A.tx = (P.d.n1 + A.ntx - 1) / A.ntx;
+    A.lty = P.d.n2 >= 4 ? 2 : P.d.n2 >= 2 ? 1 : 0;
+    A.ltz = P.d.n3 >= 4 ? 2 : P.d.n3 >= 2 ? 1 : 0;
+    while (tile_bytes(A) > 70 * 1024 && A.lty + A.ltz > 0) --(A.lty > A.ltz ? A.lty : A.ltz);
+    A.nty = (P.d.n2 + (1 << A.lty) - 1) >> A.lty;
+    A.n_tiles = A.ntx * A.nty * ((P.d.n3 + (1 << A.ltz) - 1) >> A.ltz);
 }
 
 template <typename WT>
@@ -323,12 +401,8 @@ tetra_status_t fermi_level(const Plan &P, const float *eps, const void *w, doubl
     A.eps = eps; A.w = w;
     A.S = reinterpret_cast<FermiState *>(static_cast<unsigned char *>(ws) + kStatusBytes);
     choose_tile(P, A);
-    A.ntx = (A.n1 + A.tx - 1) / A.tx;
-    A.nty = (A.n2 + A.ty - 1) / A.ty;
-    A.n_tiles = A.ntx * A.nty * ((A.n3 + A.tz - 1) / A.tz);
-    const size_t smem = 2 * sizeof(float) * (size_t)(A.tx + 1) * (A.ty + 1) * (A.tz + 1) * A.nb;
-    if (smem > P.smem_optin - 1024) return TETRA_EUNSUPPORTED;
-    const int grid = std::min(A.n_tiles, 3 * P.sm_count);
+    const size_t smem = tile_bytes(A);
+    const int grid = std::min(A.n_tiles, kFermiBlocks * P.sm_count);
     if (cudaMemsetAsync(ws, 0, kStatusBytes + sizeof(FermiState), stream) != cudaSuccess) return TETRA_ECUDA;
     const long n_vec = (long)P.nx * P.ny * P.nz * (P.eps_stride / 4);
     band_range_kernel<<<(int)std::min<long>((n_vec + 255) / 256, 8L * P.sm_count), 256, 0, stream>>>(
