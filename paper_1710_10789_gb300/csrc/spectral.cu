@@ -39,7 +39,9 @@
 // 1/(w - D), below), so the sub-tetrahedra are kept in per-lane segments and
 // the whole warp evaluates them, lane by lane in a fixed order, at all
 // energies (each lane owning every 32nd energy).
+#include <algorithm>
 #include <atomic>
+#include <cmath>
 
 #include "tetra_internal.cuh"
 
@@ -50,9 +52,12 @@ namespace {
 constexpr int kSpecThreads = 128;
 constexpr int kSpecWarps = kSpecThreads / 32;
 constexpr int kSpecBlocksPerSM = 4;
-constexpr int kSpecBits = 26;   // fixed-point fraction bits of the unit below
+constexpr int kReBits = 26;     // fixed-point fraction bits of the real part's unit (S: spec_bits)
 constexpr int kQueueCap = 256;  // sub-tetrahedra per warp queue
 constexpr int kDrainAt = 64;    // a queue this full is drained before the next band pair
+constexpr int kWide = 20;       // a sub-tetrahedron with this many energies is taken by the whole warp
+constexpr float kEntryCap = 4.1e6f;         // below 2^22: larger contributions go to the 64-bit accumulator
+constexpr unsigned kTileLimit = 1u << 30;   // the int32 tile is flushed before its sums could pass this
 // the real part of chi0 (kKindRe) next to the spectral function (kKindS)
 constexpr int kKindS = 0, kKindRe = 1;
 constexpr int kReBlocksPerSM = 3;
@@ -119,50 +124,53 @@ struct __align__(16) ReStage {
 // Constants of a launch that the sub-tetrahedron accumulation needs.
 struct SpecArgs {
     const float *om;        // shared: energies (point) or bin edges (bin)
-    long long *tile;        // shared: int64 accumulators per energy / bin
+    long long *tile;        // shared, real part: int64 accumulators per energy
+    int *tile32;            // shared, S: int32 accumulators per energy / bin
+    unsigned *bound;        // shared, S: bound on what any entry of tile32 holds
+    long long *sums;        // global: int64 accumulators per energy / bin
     int n_om;               // energies or bins
     int mode;               // TETRA_POINT or TETRA_BIN
     float scale;            // V_T/V_G over the fixed-point unit
+    float max_iw;           // bin mode: 1 / narrowest bin
     int *status;
     float om0, om_last;     // first and last grid energy (edge)
     float inv_de;           // 1 / mean spacing, for the index estimates
     SubTet *q;              // shared: this warp's queue [kQueueCap]
-    int *qn;                // shared: its fill count (real part: this lane's)
+    int *qn;                // shared: its fill count (real part: each lane's)
+    struct SpecTet *st;     // shared, S: this warp's set-ups [32]
     float *racc;            // shared, real part: this warp's FP32 sums per energy
-    ReSeg *rq;              // shared, real part: this lane's segment [kSubPerPair]
+    ReSeg *rq;              // shared, real part: the lanes' segments [32][kSubPerPair]
     ReStage *stage;         // shared, real part: this warp's set-ups [32]
 };
 
-// Normalised density g and cumulative G of a linear function with sorted
-// corner values d0 <= d1 <= d2 <= d3 at w (reciprocals precomputed).
-struct Lin {
-    float d0, d1, d2, d3;
-    float k1, k2a, k2b, k3;   // g = k1 x^2 | k2a (d21 + 2x - k2b x^2) | k3 y^2
-    float g2c;                     // G case 2: (d21^2 + 3 d21 x + 3 x^2 - k2b x^3) * g2c
+// One sub-tetrahedron set up for its energies [i0, i1): the density of D, and
+// its cumulative, with the clamped edge fractions of the DOS kernel (no cases;
+// equal corner energies give infinite reciprocals, whose products saturate).
+struct __align__(16) SpecTet {
+    float e1, e2, e3, r21, r31, r41, r32, r42, r43;
+    float amp;    // point: amplitude * 3 / E41; bin: amplitude
+    float dith;
+    int i0, i1, pad[3];
 };
 
-// (All three pieces are evaluated and one is selected: the lanes of a warp
-// walk different sub-tetrahedra, so a branch per piece would diverge.)
-__device__ __forceinline__ float lin_g(const Lin &L, float w) {
-    const float x1 = w - L.d0, x2 = w - L.d1, y = L.d3 - w;
-    const float g1 = L.k1 * x1 * x1;
-    const float g2 = L.k2a * fmaf(-L.k2b * x2, x2, fmaf(2.f, x2, L.d1 - L.d0));
-    const float g3 = L.k3 * y * y;
-    const float g = (w <= L.d1) ? g1 : ((w <= L.d2) ? g2 : g3);
-    return (w > L.d0 && w < L.d3) ? g : 0.f;
+__device__ __forceinline__ float spec_density(const SpecTet &T, float E) {   // over amp
+    const float x = E - T.e1, t = E - T.e2, y = E - T.e3;
+    const float f21 = __saturatef(x * T.r21), f31 = __saturatef(x * T.r31), f32 = __saturatef(t * T.r32);
+    const float f42 = __saturatef(t * T.r42), f43 = __saturatef(y * T.r43);
+    const float p = fmaf(-f21, f32, f21), q = fmaf(-f32, f43, f32);   // f21 f23, f32 f34
+    return fmaf(p, f31, fmaf(-q, f42, q));
 }
 
-__device__ __forceinline__ float lin_G(const Lin &L, float w) {
-    const float x1 = w - L.d0, x2 = w - L.d1, y = L.d3 - w, d21 = L.d1 - L.d0;
-    const float G1 = L.k1 * (1.f / 3.f) * x1 * x1 * x1;
-    const float G2 = L.g2c * (d21 * d21 + x2 * (3.f * d21 + x2 * (3.f - L.k2b * x2)));
-    const float G3 = 1.f - L.k3 * (1.f / 3.f) * y * y * y;
-    const float G = (w <= L.d1) ? G1 : ((w <= L.d2) ? G2 : G3);
-    return !(w > L.d0) ? 0.f : (!(w < L.d3) ? 1.f : G);
+__device__ __forceinline__ float spec_below(const SpecTet &T, float E) {
+    const float x = E - T.e1, t = E - T.e2, y = E - T.e3;
+    const float f21 = __saturatef(x * T.r21), f31 = __saturatef(x * T.r31), f41 = __saturatef(x * T.r41);
+    const float f32 = __saturatef(t * T.r32), f42 = __saturatef(t * T.r42), f43 = __saturatef(y * T.r43);
+    const float f14 = 1.f - f41;
+    return fmaf(f41, fmaf(f32, 1.f - f31, f21 * f31), f14 * fmaf(f32, f42, f43 * (1.f - f42)));
 }
 
 // Mean spacing of the energy grid (or bin width), the scale of the
-// fixed-point unit = (V_T/V_G) / de * 2^-26.
+// fixed-point unit = (V_T/V_G) / de * 2^-bits.
 __device__ __forceinline__ double mean_spacing(const float *om, int n_om, int mode) {
     const int spacings = mode == TETRA_BIN ? n_om : n_om - 1;
     double de = spacings > 0 ? ((double)om[spacings] - (double)om[0]) / spacings : 1.0;
@@ -199,51 +207,53 @@ __device__ __forceinline__ int lower_index(const float *om, int n, float x, floa
     return i;
 }
 
-// Adds one sub-tetrahedron's distribution of D to the tile.
-__device__ void deposit(const SubTet &T, const SpecArgs &S) {
-    Lin L;
-    L.d0 = T.d0; L.d1 = T.d1; L.d2 = T.d2; L.d3 = T.d3;
-    const float d21 = T.d1 - T.d0, d31 = T.d2 - T.d0, d41 = T.d3 - T.d0;
-    const float d32 = T.d2 - T.d1, d42 = T.d3 - T.d1, d43 = T.d3 - T.d2;
-    L.k1 = d21 > 0.f ? 3.f / (d21 * d31 * d41) : 0.f;
-    L.k2a = (d31 > 0.f) ? 3.f / (d31 * d41) : 0.f;
-    L.k2b = (d32 > 0.f && d42 > 0.f) ? (d31 + d42) / (d32 * d42) : 0.f;
-    L.k3 = d43 > 0.f ? 3.f / (d41 * d42 * d43) : 0.f;
-    L.g2c = (d31 > 0.f) ? 1.f / (d31 * d41) : 0.f;
-    int i0, i1;   // indices [i0, i1)
+// Sets one queued sub-tetrahedron up.
+__device__ __forceinline__ void spec_setup(const SubTet &Q, const SpecArgs &S, SpecTet &T) {
+    T.e1 = Q.d0; T.e3 = Q.d2;
+    // E2 = E3 = E4: the density jumps to zero at E4, which is not below it
+    T.e2 = (Q.d1 < Q.d3) ? Q.d1 : nextafterf(Q.d3, -INFINITY);
+    T.r21 = __frcp_rn(Q.d1 - Q.d0); T.r31 = __frcp_rn(Q.d2 - Q.d0); T.r41 = __frcp_rn(Q.d3 - Q.d0);
+    T.r32 = __frcp_rn(Q.d2 - Q.d1); T.r42 = __frcp_rn(Q.d3 - Q.d1); T.r43 = __frcp_rn(Q.d3 - Q.d2);
+    T.dith = hash_dither(Q.key);
     if (S.mode == TETRA_BIN) {
-        i0 = max(0, upper_index(S.om, S.n_om + 1, T.d0, S.om0, S.inv_de) - 1);   // bins with upper edge > d0
-        i1 = min(S.n_om, upper_index(S.om, S.n_om + 1, T.d3, S.om0, S.inv_de));   // and lower edge <= d3
+        T.e2 = Q.d1;
+        T.amp = Q.amp;
+        T.i0 = max(0, upper_index(S.om, S.n_om + 1, Q.d0, S.om0, S.inv_de) - 1);   // bins with upper edge > d0
+        T.i1 = min(S.n_om, upper_index(S.om, S.n_om + 1, Q.d3, S.om0, S.inv_de));   // and lower edge <= d3
     } else {
-        i0 = upper_index(S.om, S.n_om, T.d0, S.om0, S.inv_de);
-        i1 = lower_index(S.om, S.n_om, T.d3, S.om0, S.inv_de);
+        T.amp = Q.amp * 3.f * T.r41;
+        T.i0 = upper_index(S.om, S.n_om, Q.d0, S.om0, S.inv_de);
+        T.i1 = lower_index(S.om, S.n_om, Q.d3, S.om0, S.inv_de);
     }
-    const float dith = hash_dither(T.key);
-    float Gp = (S.mode == TETRA_BIN && i0 < i1) ? lin_G(L, S.om[i0]) : 0.f;
-    for (int i = i0; i < i1; ++i) {
-        float v;
-        if (S.mode == TETRA_BIN) {
-            const float Gn = lin_G(L, S.om[i + 1]);
-            v = (Gn - Gp) / (S.om[i + 1] - S.om[i]);
-            Gp = Gn;
-        } else {
-            v = lin_g(L, S.om[i]);
-        }
-        const float x = fmaf(T.amp, v, dith);
-        long long qv;
-        if (fabsf(x) < 4194304.f) {
-            // round to nearest even by adding 1.5 * 2^23 (exact below 2^22):
-            // the same integer as the 64-bit conversion, without the FP64
-            // pipe that conversion runs on
-            qv = __float_as_int(x + 12582912.f) - 0x4B400000;
-        } else if (fabsf(x) < 4.0e18f) {
-            qv = __float2ll_rn(x);
+}
+
+// Its contribution to energy (bin) i, before rounding.
+__device__ __forceinline__ float spec_value(const SpecTet &T, const float *om, bool bin, int i) {
+    if (bin) return fmaf(T.amp, __fdividef(spec_below(T, om[i + 1]) - spec_below(T, om[i]), om[i + 1] - om[i]), T.dith);
+    return fmaf(T.amp, spec_density(T, om[i]), T.dith);
+}
+
+// Adds a sub-tetrahedron to the 64-bit accumulator in global memory: the path
+// of contributions too large for the int32 tile and of a full queue (the
+// same single rounding as the tile path).
+__device__ __noinline__ void deposit_wide(const SubTet &Q, const SpecArgs &S) {
+    SpecTet T;
+    spec_setup(Q, S, T);
+    for (int i = T.i0; i < T.i1; ++i) {
+        const float x = spec_value(T, S.om, S.mode == TETRA_BIN, i);
+        if (fabsf(x) < 4.0e18f) {
+            const long long qv = __float2ll_rn(x);
+            if (qv) atomicAdd(reinterpret_cast<unsigned long long *>(&S.sums[i]), static_cast<unsigned long long>(qv));
         } else {
             atomicOr(S.status, kFlagRange);
-            qv = 0;
         }
-        if (qv) atomicAdd(reinterpret_cast<unsigned long long *>(&S.tile[i]), static_cast<unsigned long long>(qv));
     }
+}
+
+// Rounds to nearest even by adding 1.5 * 2^23 (exact below 2^22) and adds.
+__device__ __forceinline__ void spec_add(int *tile, int i, float x) {
+    const int qv = __float_as_int(x + 12582912.f) - 0x4B400000;
+    if (qv) atomicAdd(&tile[i], qv);
 }
 
 // Queues sign * nu * (distribution of D) of one sub-tetrahedron in this
@@ -251,7 +261,7 @@ __device__ void deposit(const SubTet &T, const SpecArgs &S) {
 // this lane's own segment, in the order the clipping produces them.
 template <int KIND>
 __device__ __noinline__ void accumulate(P5 v0, P5 v1, P5 v2, P5 v3, float sign, uint32_t key,
-                                        const SpecArgs S) {
+                                        const SpecArgs &S) {
     const float u00 = v0.l0 - v3.l0, u01 = v0.l1 - v3.l1, u02 = v0.l2 - v3.l2;
     const float u10 = v1.l0 - v3.l0, u11 = v1.l1 - v3.l1, u12 = v1.l2 - v3.l2;
     const float u20 = v2.l0 - v3.l0, u21 = v2.l1 - v3.l1, u22 = v2.l2 - v3.l2;
@@ -264,8 +274,8 @@ __device__ __noinline__ void accumulate(P5 v0, P5 v1, P5 v2, P5 v3, float sign, 
 #undef SPEC_CS
     if constexpr (KIND == kKindRe) {
         // every sub-tetrahedron reaches every energy (a flat one as 1/(w - d))
-        const int slot = (*S.qn)++;
-        S.rq[slot] = ReSeg{d[0], d[1], d[2], d[3], sign * nu * S.scale};
+        const int lane = threadIdx.x & 31, slot = S.qn[lane]++;
+        S.rq[lane * kSubPerPair + slot] = ReSeg{d[0], d[1], d[2], d[3], sign * nu * S.scale};
         return;
     }
     // a flat transition energy is a delta: measure zero in point mode, its
@@ -276,16 +286,65 @@ __device__ __noinline__ void accumulate(P5 v0, P5 v1, P5 v2, P5 v3, float sign, 
     const SubTet T{d[0], d[1], d[2], d[3], sign * nu * S.scale, key};
     const int slot = atomicAdd(S.qn, 1);
     if (slot < kQueueCap) S.q[slot] = T;
-    else deposit(T, S);
+    else deposit_wide(T, S);
 }
 
-// Every lane of the warp takes queued sub-tetrahedra in turn; the queue is
-// empty afterwards. Called by all 32 lanes together.
+// Empties the queue, 32 sub-tetrahedra at a time. Called by all 32 lanes
+// together. Each lane sets one up; those with many energies are then taken
+// by the whole warp, a lane per energy (consecutive tile entries: no bank
+// conflict, no lane idle for another's longer window), the short ones by
+// their own lane. The sums are 32-bit (64-bit shared atomics take about 20
+// cycles a warp, 32-bit ones 1 to 4); a warp about to push the tile's bound
+// past kTileLimit moves the tile to the 64-bit accumulator first. Adds that
+// other warps have announced but not made yet may land after that, uncounted:
+// at most 2^27 for each of the four warps.
 __device__ __forceinline__ void drain(const SpecArgs &S, int lane) {
+    constexpr unsigned kAll = 0xffffffffu;
     __syncwarp();
     const int n = min(*S.qn, kQueueCap);
-    for (int e = lane; e < n; e += 32) deposit(S.q[e], S);
-    __syncwarp();
+    const float *om = S.om;
+    int *tile = S.tile32;
+    const bool bin = S.mode == TETRA_BIN;
+    for (int base = 0; base < n; base += 32) {
+        SpecTet T;
+        int K = 0;
+        unsigned qb = 0;
+        if (base + lane < n) {
+            const SubTet Q = S.q[base + lane];
+            spec_setup(Q, S, T);
+            K = T.i1 - T.i0;
+            // (a density is at most 3 / E41, a bin's average that or its step over it)
+            const float most = fabsf(T.amp) * (bin ? 1.01f * fminf(S.max_iw, 3.f * T.r41) : 1.01f);
+            if (K > 0 && !(most < kEntryCap)) {
+                deposit_wide(Q, S);
+                K = 0;
+            }
+            if (K > 0) qb = (unsigned)most + 2u;
+            S.st[lane] = T;
+        }
+        const unsigned announce = __reduce_add_sync(kAll, qb);
+        unsigned old = 0;
+        if (lane == 0) old = atomicAdd(S.bound, announce);
+        old = __shfl_sync(kAll, old, 0);
+        if (old + announce > kTileLimit) {
+            if (lane == 0) atomicExch(S.bound, announce);
+            for (int i = lane; i < S.n_om; i += 32) {
+                const int v = atomicExch(&tile[i], 0);
+                if (v) atomicAdd(reinterpret_cast<unsigned long long *>(&S.sums[i]), static_cast<unsigned long long>((long long)v));
+            }
+        }
+        __syncwarp();
+        unsigned wide = __ballot_sync(kAll, K >= kWide);
+        while (wide) {
+            const int j = __ffs(wide) - 1;
+            wide &= wide - 1;
+            const SpecTet W = S.st[j];
+            for (int i = W.i0 + lane; i < W.i1; i += 32) spec_add(tile, i, spec_value(W, om, bin, i));
+        }
+        if (K > 0 && K < kWide)
+            for (int i = T.i0; i < T.i1; ++i) spec_add(tile, i, spec_value(T, om, bin, i));
+        __syncwarp();
+    }
     if (lane == 0) *S.qn = 0;
     __syncwarp();
 }
@@ -294,7 +353,7 @@ __device__ __forceinline__ void drain(const SpecArgs &S, int lane) {
 // sub-tetrahedra (second and last cut).
 template <int KIND>
 __device__ __noinline__ void clip_second(P5 v0, P5 v1, P5 v2, P5 v3, int which, float sign, uint32_t key,
-                                         const SpecArgs S) {
+                                         const SpecArgs &S) {
     float s0 = field(v0, which), s1 = field(v1, which), s2 = field(v2, which), s3 = field(v3, which);
     cswap5(v0, v1, s0, s1);
     cswap5(v2, v3, s2, s3);
@@ -325,7 +384,7 @@ __device__ __noinline__ void clip_second(P5 v0, P5 v1, P5 v2, P5 v3, int which, 
 // every kept tetrahedron by `second`.
 template <int KIND>
 __device__ __noinline__ void region(P5 v0, P5 v1, P5 v2, P5 v3, int first, int second, float sign,
-                                    uint32_t key, const SpecArgs S) {
+                                    uint32_t key, const SpecArgs &S) {
     float s0 = field(v0, first), s1 = field(v1, first), s2 = field(v2, first), s3 = field(v3, first);
     cswap5(v0, v1, s0, s1);
     cswap5(v2, v3, s2, s3);
@@ -593,47 +652,91 @@ __host__ __device__ constexpr int queue_counts() { return KIND == kKindS ? 2 : 3
 template <int KIND>
 __host__ __device__ constexpr size_t queue_entry_bytes() { return KIND == kKindS ? sizeof(SubTet) : sizeof(ReSeg); }
 
-// S: queues, counts, tile, energies. Real part: lane segments, counts,
-// staged set-ups, FP32 sums, tile, energies.
+// Queues (lane segments), counts, staged set-ups, real part: FP32 sums, tile
+// (int64; S: int32), energies.
 template <int KIND>
 size_t spec_smem_bytes(int n_om, int mode) {
     return queue_entry_bytes<KIND>() * kSpecWarps * queue_entries<KIND>() +
            sizeof(int) * kSpecWarps * queue_counts<KIND>() +
-           (KIND == kKindRe ? sizeof(ReStage) * kSpecWarps * 32 + sizeof(float) * kSpecWarps * (size_t)n_om : 0) +
-           sizeof(long long) * (size_t)n_om + sizeof(float) * (size_t)(mode == TETRA_BIN ? n_om + 1 : n_om);
+           (KIND == kKindRe ? sizeof(ReStage) * kSpecWarps * 32 + sizeof(float) * kSpecWarps * (size_t)n_om
+                            : sizeof(SpecTet) * kSpecWarps * 32) +
+           (KIND == kKindRe ? sizeof(long long) : sizeof(int)) * (size_t)n_om +
+           sizeof(float) * (size_t)(mode == TETRA_BIN ? n_om + 1 : n_om);
+}
+// The longest grid a call takes: 12 bytes per energy beside the queues of S
+// (about 17000 energies), 28 of the real part.
+template <int KIND>
+bool spec_grid_fits(int n_om, int mode, size_t optin) {
+    return spec_smem_bytes<KIND>(n_om, mode) + (KIND == kKindS ? 4 * (size_t)n_om - sizeof(SpecTet) * kSpecWarps * 32 : 0) <= optin;
+}
+
+// Fraction bits of S's unit. A value is a sum of items of size ~2^bits / K (K
+// energies per tetrahedron, about 2 n_om / N for N points a side), each
+// rounded without bias to one unit: its relative error is about
+// sqrt(K n_om / items) / 2^(bits + 1), here kept near 1e-9 (the items that
+// reach an energy are some percent of all). At 64^3 points, 8 bands, 400
+// energies that is 22 bits; 20 bits doubled the error against 64 bits, 3e-8.
+// An item of a tetrahedron with K energies is at most 3 2^bits / K, which has
+// to stay below kEntryCap.
+int spec_bits(const Plan &P, int n_om) {
+    const double points = (double)P.d.n1 * P.d.n2 * P.d.n3, K = std::max(1.0, 2.0 * n_om / std::cbrt(points));
+    const double items = 6.0 * points * P.d.n_bands * P.d.n_bands;
+    const int need = (int)std::ceil(std::log2(5e8 * std::sqrt(K * n_om / items)));
+    return std::max(20, std::min(std::min(26, need), 20 + (int)std::log2(K)));
 }
 
 template <int NB, int KIND>
 __global__ void __launch_bounds__(kSpecThreads, KIND == kKindS ? kSpecBlocksPerSM : kReBlocksPerSM)
     spectral_t0_kernel(const float *eps, int eps_stride, int n1, int n2, int n3, int nx, int ny, int z0, int z1,
                        int qx, int qy, int qz, float mu, const float *omega, int n_om, int mode,
-                       double vtvg, long long *sums, float *out, int *status) {
+                       double vtvg, int bits, long long *sums, float *out, int *status) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int QW = queue_entries<KIND>(), QC = queue_counts<KIND>();
     unsigned char *qraw = smem;                                             // [warps][QW] entries
     int *qcount = reinterpret_cast<int *>(qraw + queue_entry_bytes<KIND>() * kSpecWarps * QW);   // [warps][QC]
     ReStage *stage = reinterpret_cast<ReStage *>(qcount + kSpecWarps * QC); // real part: [warps][32]
-    float *racc = reinterpret_cast<float *>(stage + (KIND == kKindRe ? kSpecWarps * 32 : 0));   // [warps][n_om]
+    SpecTet *stet = reinterpret_cast<SpecTet *>(stage);                     // S: [warps][32]
+    float *racc = reinterpret_cast<float *>(stage + kSpecWarps * 32);       // real part: [warps][n_om]
     long long *tile = reinterpret_cast<long long *>(racc + (KIND == kKindRe ? kSpecWarps * n_om : 0));
-    float *om = reinterpret_cast<float *>(tile + n_om);
+    int *tile32 = reinterpret_cast<int *>(tile);                            // S
+    float *om = KIND == kKindRe ? reinterpret_cast<float *>(tile + n_om) : reinterpret_cast<float *>(tile32 + n_om);
+    static_assert(sizeof(SpecTet) == sizeof(ReStage), "one staging area for both");
+    __shared__ unsigned s_bound;
+    __shared__ float s_iw[kSpecWarps];
     const int n_edges = (mode == TETRA_BIN) ? n_om + 1 : n_om;
-    for (int i = threadIdx.x; i < n_om; i += blockDim.x) tile[i] = 0;
+    for (int i = threadIdx.x; i < n_om; i += blockDim.x) {
+        if constexpr (KIND == kKindRe) tile[i] = 0;
+        else tile32[i] = 0;
+    }
     for (int i = threadIdx.x; i < n_edges; i += blockDim.x) om[i] = omega[i];
+    if (threadIdx.x == 0) s_bound = 0u;
     for (int i = threadIdx.x; i < kSpecWarps * QC; i += blockDim.x) qcount[i] = 0;
     if constexpr (KIND == kKindRe)
         for (int i = threadIdx.x; i < kSpecWarps * n_om; i += blockDim.x) racc[i] = 0.f;
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // V_T/V_G in fixed-point units: de * 2^26
+    // V_T/V_G in fixed-point units: de * 2^bits
     const double de = mean_spacing(om, n_om, mode);
-    const float scale = (float)ldexp(de, kSpecBits);
+    const float scale = (float)ldexp(de, bits);
+    float max_iw = 0.f;
+    if (KIND == kKindS && mode == TETRA_BIN) {
+        for (int i = threadIdx.x; i < n_om; i += blockDim.x) max_iw = fmaxf(max_iw, 1.0f / (om[i + 1] - om[i]));
+        max_iw = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(max_iw)));   // (not negative)
+        if (lane == 0) s_iw[warp] = max_iw;
+        __syncthreads();
+        for (int i = 0; i < kSpecWarps; ++i) max_iw = fmaxf(max_iw, s_iw[i]);
+    }
     const float om_lo = om[0], om_hi = om[n_edges - 1];
     SubTet *wq = reinterpret_cast<SubTet *>(qraw) + warp * QW;   // S
     ReSeg *wr = reinterpret_cast<ReSeg *>(qraw) + warp * QW;     // real part
     int *wn = qcount + warp * QC;
-    const SpecArgs S{om, tile, n_om, mode, scale, status, om_lo, om_hi, (float)(1.0 / de), wq,
-                     KIND == kKindS ? wn : wn + lane, racc + warp * n_om, wr + lane * kSubPerPair,
-                     stage + warp * 32};
+    // (in shared memory: the clipping's calls pass an address, not 120 bytes)
+    __shared__ SpecArgs s_args[kSpecWarps];
+    if (lane == 0)
+        s_args[warp] = SpecArgs{om, tile, tile32, &s_bound, sums, n_om, mode, scale, max_iw, status, om_lo, om_hi,
+                                (float)(1.0 / de), wq, wn, stet + warp * 32, racc + warp * n_om, wr, stage + warp * 32};
+    __syncwarp();
+    const SpecArgs &S = s_args[warp];
     int since_flush = 0;   // real part: entries in the per-warp FP32 sums
     // energy range of the grid: a band pair whose transition energies over a
     // tetrahedron miss it contributes nothing (the clipped regions' values
@@ -742,8 +845,10 @@ __global__ void __launch_bounds__(kSpecThreads, KIND == kKindS ? kSpecBlocksPerS
     // by the CTA that finishes last: out[i] = unit * sum. (A row of partials per
     // CTA and a kernel that added the 608 rows took 0.16 ms at 400 energies.)
     __syncthreads();
-    for (int i = threadIdx.x; i < n_om; i += blockDim.x)
-        if (tile[i]) atomicAdd(reinterpret_cast<unsigned long long *>(sums + i), static_cast<unsigned long long>(tile[i]));
+    for (int i = threadIdx.x; i < n_om; i += blockDim.x) {
+        const long long v = KIND == kKindRe ? tile[i] : (long long)tile32[i];
+        if (v) atomicAdd(reinterpret_cast<unsigned long long *>(sums + i), static_cast<unsigned long long>(v));
+    }
     __threadfence();
     __syncthreads();
     __shared__ int s_last;
@@ -751,7 +856,7 @@ __global__ void __launch_bounds__(kSpecThreads, KIND == kKindS ? kSpecBlocksPerS
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    const double unit = vtvg / de * ldexp(1.0, -kSpecBits);
+    const double unit = vtvg / de * ldexp(1.0, -bits);
     for (int i = threadIdx.x; i < n_om; i += blockDim.x) out[i] = (float)((double)__ldcg(sums + i) * unit);
 }
 
@@ -761,8 +866,8 @@ int spectral_grid(const Plan &P) { return (KIND == kKindS ? kSpecBlocksPerSM : k
 
 template <int NB, int KIND>
 cudaError_t launch_spectral_nb(const Plan &P, const float *eps, const int q[3], float mu, const float *omega,
-                               int n_om, int mode, double vtvg, long long *sums, float *out, int *status,
-                               int grid, size_t smem, cudaStream_t stream) {
+                               int n_om, int mode, double vtvg, int bits, long long *sums, float *out,
+                               int *status, int grid, size_t smem, cudaStream_t stream) {
     auto k = spectral_t0_kernel<NB, KIND>;
     static std::atomic<int> opted[64];
     int dev = 0;
@@ -778,7 +883,8 @@ cudaError_t launch_spectral_nb(const Plan &P, const float *eps, const int q[3], 
         }
     }
     k<<<grid, kSpecThreads, smem, stream>>>(eps, P.eps_stride, P.d.n1, P.d.n2, P.d.n3, P.nx, P.ny, P.z0, P.z1,
-                                           q[0], q[1], q[2], mu, omega, n_om, mode, vtvg, sums, out, status);
+                                           q[0], q[1], q[2], mu, omega, n_om, mode, vtvg, bits, sums, out,
+                                           status);
     return cudaGetLastError();
 }
 
@@ -800,24 +906,24 @@ tetra_status_t launch_spectral(const Plan &P, const float *eps, const int q_in[3
     // the bands at k + q come from every plane of the grid
     if (P.z0 != 0 || P.z1 != P.d.n3) return TETRA_EUNSUPPORTED;
     const size_t smem = spec_smem_bytes<KIND>(n_om, mode);
-    if (smem > P.smem_optin) return TETRA_EUNSUPPORTED;
+    if (!spec_grid_fits<KIND>(n_om, mode, P.smem_optin)) return TETRA_EUNSUPPORTED;
     if (ws_bytes < spectral_workspace<KIND>(P, n_om)) return TETRA_ENOMEM;
     const double vtvg = 1.0 / (6.0 * (double)P.d.n1 * (double)P.d.n2 * (double)P.d.n3);
     const int q[3] = {mod_q(q_in[0], P.d.n1), mod_q(q_in[1], P.d.n2), mod_q(q_in[2], P.d.n3)};
-    const int grid = spectral_grid<KIND>(P);
+    const int grid = spectral_grid<KIND>(P), bits = KIND == kKindS ? spec_bits(P, n_om) : kReBits;
     int *status = reinterpret_cast<int *>(ws);
     long long *sums = reinterpret_cast<long long *>(static_cast<unsigned char *>(ws) + kStatusBytes);
     if (cudaMemsetAsync(ws, 0, spectral_workspace<KIND>(P, n_om), stream) != cudaSuccess) return TETRA_ECUDA;
     cudaError_t e;
     switch (P.d.n_bands) {
-        case 1: e = launch_spectral_nb<1, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, sums, S, status, grid, smem, stream); break;
-        case 2: e = launch_spectral_nb<2, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, sums, S, status, grid, smem, stream); break;
-        case 3: e = launch_spectral_nb<3, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, sums, S, status, grid, smem, stream); break;
-        case 4: e = launch_spectral_nb<4, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, sums, S, status, grid, smem, stream); break;
-        case 5: e = launch_spectral_nb<5, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, sums, S, status, grid, smem, stream); break;
-        case 6: e = launch_spectral_nb<6, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, sums, S, status, grid, smem, stream); break;
-        case 7: e = launch_spectral_nb<7, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, sums, S, status, grid, smem, stream); break;
-        default: e = launch_spectral_nb<8, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, sums, S, status, grid, smem, stream); break;
+        case 1: e = launch_spectral_nb<1, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, bits, sums, S, status, grid, smem, stream); break;
+        case 2: e = launch_spectral_nb<2, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, bits, sums, S, status, grid, smem, stream); break;
+        case 3: e = launch_spectral_nb<3, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, bits, sums, S, status, grid, smem, stream); break;
+        case 4: e = launch_spectral_nb<4, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, bits, sums, S, status, grid, smem, stream); break;
+        case 5: e = launch_spectral_nb<5, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, bits, sums, S, status, grid, smem, stream); break;
+        case 6: e = launch_spectral_nb<6, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, bits, sums, S, status, grid, smem, stream); break;
+        case 7: e = launch_spectral_nb<7, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, bits, sums, S, status, grid, smem, stream); break;
+        default: e = launch_spectral_nb<8, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, bits, sums, S, status, grid, smem, stream); break;
     }
     return e == cudaSuccess ? TETRA_OK : TETRA_ECUDA;
 }
