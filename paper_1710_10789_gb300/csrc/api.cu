@@ -65,6 +65,12 @@ int pow2_floor(int v) {
     return p;
 }
 
+static int pow2_ceil(int v) {
+    int p = 1;
+    while (p < v) p *= 2;
+    return p;
+}
+
 // Default box of cubes for a band count: 4 x 4 x BZ with at most ~1536 work
 // items per box (a work item is a (tetrahedron pair, band) with up to 8
 // orbitals, a (tetrahedron, band) with more), which keeps the per-item
@@ -111,6 +117,14 @@ static tetra_status_t plan_geometry(Plan &P, const int box[3], int ctas_per_sm) 
     if (fixed + per_w * 64 > P.smem_optin) return TETRA_EUNSUPPORTED;
     int cw = (int)std::min<size_t>((P.smem_optin - fixed - 8) / per_w, (size_t)d.n_omega);
     P.n_chunks = (d.n_omega + cw - 1) / cw;
+    // whether a tile row of the next power of two of orbitals would fit them
+    // all (a batch takes no more energies with 3, 5 or 6 orbitals than with 4
+    // or 8, although their rows are shorter)
+    {
+        const int row = pow2_ceil(tetra::norb_template(d.n_orb));
+        const size_t more = 4 * (size_t)(row + 1 - P.tile_stride) * (d.mode == TETRA_INTEGRATED ? 2 : 1);
+        P.one_tile = (P.smem_optin - fixed - 8 - 4 * (size_t)(row + 1 - P.tile_stride)) / (per_w + more) >= (size_t)d.n_omega;
+    }
     P.chunk_w = (d.n_omega + P.n_chunks - 1) / P.n_chunks;
     P.smem_bytes = fixed + per_w * P.chunk_w + 8;
     // Bin mode: neighbouring pairs of a band tend to fall into the same bin,
@@ -366,7 +380,7 @@ tetra_status_t tetra_plan_batched(tetra_batch_plan_t *plan, const tetra_desc_t *
     }
     // the largest energy grid must fit one shared tile (no energy chunks)
     const Plan &Pb = B->models[B->big];
-    if (Pb.n_chunks != 1) return fail(TETRA_EUNSUPPORTED);
+    if (!Pb.one_tile) return fail(TETRA_EUNSUPPORTED);
     B->chunk_w = Pb.chunk_w;
     B->smem_bytes = Pb.smem_bytes;
     // work items: every box of every model, models in order; the CTAs claim

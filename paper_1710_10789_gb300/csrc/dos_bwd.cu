@@ -106,6 +106,9 @@ struct BwdArgs {
     int staged;              // edges, G and D staged in shared memory
 };
 
+// Orbitals of the kernel instantiation that takes n_orb.
+int bwd_norb(int n_orb) { return n_orb <= 1 ? 1 : n_orb <= 2 ? 2 : n_orb <= 4 ? 4 : n_orb <= 8 ? 8 : 16; }
+
 // Shared-memory bytes of the staged edges, G and D (n_bins + 1 rows each;
 // row e of the first holds G_{e-1}), or 0 when they do not fit the 64 KB
 // budget.
@@ -359,7 +362,7 @@ tetra_status_t launch_dos_backward(const Plan &P, const float *eps, const void *
     A.f = (float)(0.25 / (6.0 * (double)P.d.n1 * (double)P.d.n2 * (double)P.d.n3));
     A.eps = eps; A.w = w; A.edges = omega; A.grad_dos = grad_dos; A.geps = grad_eps; A.gw = grad_w;
     A.vec = (reinterpret_cast<uintptr_t>(grad_w) & 15u) == 0;
-    A.staged = bwd_stage_bytes(norb_template(A.n_orb), A.n_bins) > 0;
+    A.staged = bwd_stage_bytes(bwd_norb(A.n_orb), A.n_bins) > 0;
     if (cudaMemsetAsync(ws, 0, kStatusBytes, stream) != cudaSuccess) return TETRA_ECUDA;
     // the parity classes add into the arrays: start from zero (halo and
     // padding entries stay zero)
@@ -368,12 +371,13 @@ tetra_status_t launch_dos_backward(const Plan &P, const float *eps, const void *
         cudaMemsetAsync(grad_w, 0, sizeof(float) * pts * P.w_stride, stream) != cudaSuccess)
         return TETRA_ECUDA;
     cudaError_t e;
-    const int no = P.d.n_orb;
-    if (no <= 1) e = launch_bwd_n<1>(P, A, stream);
-    else if (no <= 2) e = launch_bwd_n<2>(P, A, stream);
-    else if (no <= 4) e = launch_bwd_n<4>(P, A, stream);
-    else if (no <= 8) e = launch_bwd_n<8>(P, A, stream);
-    else e = launch_bwd_n<16>(P, A, stream);
+    switch (bwd_norb(P.d.n_orb)) {
+        case 1: e = launch_bwd_n<1>(P, A, stream); break;
+        case 2: e = launch_bwd_n<2>(P, A, stream); break;
+        case 4: e = launch_bwd_n<4>(P, A, stream); break;
+        case 8: e = launch_bwd_n<8>(P, A, stream); break;
+        default: e = launch_bwd_n<16>(P, A, stream); break;
+    }
     return e == cudaSuccess ? TETRA_OK : TETRA_ECUDA;
 }
 

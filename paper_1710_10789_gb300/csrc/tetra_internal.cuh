@@ -22,6 +22,7 @@ struct tetra_plan_s {
     int BX, BY, BZ;             // box of cubes
     int nbx, nby, nbz, n_boxes;
     int chunk_w, n_chunks;      // energy chunking of the shared-memory tile
+    bool one_tile;              // all energies in one tile (batches need it)
     int grid_x;                 // persistent CTAs per energy chunk
     int fixed_bits;             // fixed-point fraction bits (see dos.cu)
     int flush_bits;             // a tile block is flushed once its bound reaches 2^flush_bits
