@@ -29,13 +29,16 @@ struct BatchOut {
 __global__ void tetra_dos_reduce_batched(const __grid_constant__ Batch<kMaxBatch> B, const BatchOut O,
                                          const long long *G, int n_orb, int chunk_w, int mode) {
     const ModelP &M = B.m[blockIdx.y];
-    const double u = fixed_unit(M.omega, M.n_omega, mode, M.vtvg, M.fixed_bits);
+    __shared__ float s_unit[2];
+    if (threadIdx.x == 0) unit_pair(fixed_unit(M.omega, M.n_omega, mode, M.vtvg, M.fixed_bits), s_unit[0], s_unit[1]);
+    __syncthreads();
+    const float uh = s_unit[0], ul = s_unit[1];
     const long total = (long)n_orb * M.n_omega;
     for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < total;
          idx += (long)gridDim.x * blockDim.x) {
         const int s = (int)(idx / M.n_omega), i = (int)(idx - (long)s * M.n_omega);
         const long long g = G[((long)blockIdx.y * n_orb + s) * chunk_w + i];
-        O.dos[blockIdx.y][idx] = (float)((double)g * u);
+        O.dos[blockIdx.y][idx] = scale_units(g, uh, ul);
     }
 }
 

@@ -340,6 +340,7 @@ __global__ void __maxnreg__(kMaxRegs)
     __shared__ float red_f[kThreads / 32];
     __shared__ int s_wsum[kThreads / 32];
     __shared__ int s_abort, s_active, s_slot;
+    __shared__ float s_fq, s_unit[2];   // of the current model
     __shared__ int s_cdelta[8];   // staged-box point offset of cube corner c
     __shared__ int n_issued[3];   // TMA loads issued per mbarrier (thread 0 keeps them)
 
@@ -433,7 +434,6 @@ __global__ void __maxnreg__(kMaxRegs)
 
     // state of the model whose boxes are being accumulated
     int cur = -1, w0 = 0, wc = 0;
-    double u = 1.0;
     float fq = 0.f, om0 = 0.f, inv_de = 0.f, max_iw = 0.f;
     long long *Gc = A.G;
     // The count column of rows 0..wc: differences (as the walks update it)
@@ -543,8 +543,11 @@ __global__ void __maxnreg__(kMaxRegs)
             __syncthreads();
             if (MODE == TETRA_BIN)
                 for (int i = tid; i < wc; i += blockDim.x) iw[i] = 1.0f / (om[i + 1] - om[i]);
-            u = fixed_unit(M.omega, M.n_omega, MODE, M.vtvg, M.fixed_bits);
-            fq = (float)(0.25 * M.vtvg / u);   // V_T/(4 V_G) in fixed-point units
+            if (tid == 0) {
+                const double u = fixed_unit(M.omega, M.n_omega, MODE, M.vtvg, M.fixed_bits);
+                s_fq = (float)(0.25 * M.vtvg / u);   // V_T/(4 V_G) in fixed-point units
+                unit_pair(u, s_unit[0], s_unit[1]);
+            }
             om0 = M.omega[0];
             const float omN = (MODE != TETRA_BIN) ? M.omega[M.n_omega - 1] : M.omega[M.n_omega];
             inv_de = (MODE != TETRA_BIN) ? (M.n_omega > 1 ? (float)(M.n_omega - 1) / (omN - om0) : 0.f)
@@ -561,6 +564,7 @@ __global__ void __maxnreg__(kMaxRegs)
                 for (int i = 0; i < (int)(blockDim.x >> 5); ++i) max_iw = fmaxf(max_iw, red_f[i]);
             }
             __syncthreads();
+            fq = s_fq;
         }
         const int st = k & 1;
         for (int i = tid; i < kKBins; i += blockDim.x) khist[i] = 0;
@@ -966,25 +970,38 @@ __global__ void __maxnreg__(kMaxRegs)
                 Tet TA, TB;
                 tet_setup<MODE>(TA, ea[0], ea[1], ea[2], ea[3], fq);
                 tet_setup<MODE>(TB, eb[0], eb[1], eb[2], eb[3], fq);
+                // one orbital: the weights' differences along the edges (tet_value)
+                const TetDiff bda = tet_diff(bw[0][0], bw[1][0], bw[2][0], bw[3][0]);
+                const TetDiff bdb = tet_diff(bw[ROWS - 4][0], bw[ROWS - 3][0], bw[ROWS - 2][0], bw[ROWS - 1][0]);
                 if (fast) {
                     // lane-dependent start, wrapping walk (see below)
                     const int K = (hi - lo - part + (1 << ls)) >> ls, i0 = lo + part, i1 = i0 + ((K - 1) << ls);
                     int i = i0 + (((lane * K) >> 5) << ls);
                     for (int j = 0; j < K; ++j) {
-                        float da[4], db[4], d5[ROWS];   // zero outside a tetrahedron's own window
-                        tet_dw(TA, om[i - w0], da);
-                        tet_dw(TB, om[i - w0], db);
-                        merge_pair(oa, ob, da, db, d5);
                         int *col = tile + (i - w0) * TS;
+                        if constexpr (NORB == 1) {
+                            const float acc = tet_value(TA, om[i - w0], bda) + (tet_value(TB, om[i - w0], bdb) + dith);
+                            atomicAdd(col, __float_as_int(acc + kMagic));
+                        } else {
+                            float da[4], db[4], d5[ROWS];   // zero outside a tetrahedron's own window
+                            tet_dw(TA, om[i - w0], da);
+                            tet_dw(TB, om[i - w0], db);
+                            merge_pair(oa, ob, da, db, d5);
 #pragma unroll
-                        for (int s = 0; s < NORB; ++s) {
-                            const float acc = project(d5, s, dith);
-                            atomicAdd(col + s, __float_as_int(acc + kMagic));
+                            for (int s = 0; s < NORB; ++s) {
+                                const float acc = project(d5, s, dith);
+                                atomicAdd(col + s, __float_as_int(acc + kMagic));
+                            }
                         }
                         i = (i == i1) ? i0 : i + (1 << ls);
                     }
                 } else {
                     for (int i = lo + part; i <= hi; i += 1 << ls) {
+                        if constexpr (NORB == 1) {   // (the same sum as the tile path)
+                            const float acc = tet_value(TA, om[i - w0], bda) + (tet_value(TB, om[i - w0], bdb) + dith);
+                            deposit_one(acc, Gc + (i - w0), A.status);
+                            continue;
+                        }
                         float da[4], db[4], d5[ROWS];   // zero outside a tetrahedron's own window
                         tet_dw(TA, om[i - w0], da);
                         tet_dw(TB, om[i - w0], db);
@@ -1245,7 +1262,7 @@ __global__ void __maxnreg__(kMaxRegs)
         if (!s_active) return;
         __threadfence();
         const ModelP &M = B.m[0];
-        u = fixed_unit(M.omega, M.n_omega, MODE, M.vtvg, M.fixed_bits);
+        const float uh = s_unit[0], ul = s_unit[1];   // (every CTA has a box)
         for (int c = group; c < (int)gridDim.y; c += kDoneGroups) {
             const int f0 = c * A.chunk_w, fn = min(A.chunk_w, M.n_omega - f0);
             const long long *G = A.G + (long)c * A.n_orb * A.chunk_w;
@@ -1283,7 +1300,7 @@ __global__ void __maxnreg__(kMaxRegs)
                 const int s = i / fn, j = i - s * fn;
                 long long v = __ldcg(G + (long)s * A.chunk_w + j);
                 if (MODE == TETRA_INTEGRATED) v += reinterpret_cast<const long long *>(tile)[i];
-                A.dos[(long)s * M.n_omega + f0 + j] = (float)((double)v * u);
+                A.dos[(long)s * M.n_omega + f0 + j] = scale_units(v, uh, ul);
             }
         }
     }

@@ -90,6 +90,29 @@ __device__ __forceinline__ void tet_dw(const Tet &T, float E, float (&d)[4]) {
     d[3] = fmaf(f42 + f43, b, f41 * s);
 }
 
+// sum_l b_l dw_l/dE of one orbital (28 operations instead of 30 and 4): the
+// weight is linear along the edges, so the section's corners take b at their
+// crossing points from the differences along the edges.
+struct TetDiff {
+    float b1, b2, b21, b31, b41, b32, b42, b43;
+};
+__device__ __forceinline__ TetDiff tet_diff(float b1, float b2, float b3, float b4) {
+    return TetDiff{b1, b2, b2 - b1, b3 - b1, b4 - b1, b3 - b2, b4 - b2, b4 - b3};
+}
+__device__ __forceinline__ float tet_value(const Tet &T, float E, const TetDiff &D) {
+    const float x = E - T.e1, t = E - T.e2, y = E - T.e3;
+    const float f21 = __saturatef(x * T.r21), f31 = __saturatef(x * T.r31), f41 = __saturatef(x * T.r41);
+    const float f32 = __saturatef(t * T.r32), f42 = __saturatef(t * T.r42), f43 = __saturatef(y * T.r43);
+    const float p = fmaf(-f21, f32, f21), q = fmaf(-f32, f43, f32);
+    const float qs = q * T.scale;
+    const float a = (p * T.scale) * f31, b = fmaf(-qs, f42, qs);
+    const float k14 = fmaf(f41, D.b41, D.b1), step = f32 * D.b32;
+    // corners 13, 14, 12|23 and 14, 24, 23|34
+    const float ka = (fmaf(f31, D.b31, D.b1) + k14) + (fmaf(f21, D.b21, D.b1) + step);
+    const float kb = (fmaf(f42, D.b42, D.b2) + k14) + (fmaf(f43, D.b43, D.b2) + step);
+    return fmaf(a, ka, b * kb);
+}
+
 // w_l(E) at any E (0 below E1, f above E4), sorted corners (49 operations).
 __device__ __forceinline__ void tet_w(const Tet &T, float E, float (&w)[4]) {
     const float x = E - T.e1, t = E - T.e2, y = E - T.e3;
@@ -104,6 +127,21 @@ __device__ __forceinline__ void tet_w(const Tet &T, float E, float (&w)[4]) {
     w[1] = fmaf(v4, f24, fmaf(v3, g23 + f24, fmaf(v2, g23, v1 * f21)));
     w[2] = fmaf(v4, 2.f - f43, fmaf(v3, f32, fmaf(v2, f31 + f32, v1 * f31)));
     w[3] = fmaf(v4, s42 + f43, fmaf(v3, s42, (v1 + v2) * f41));
+}
+
+// A fixed-point unit as two floats, and v units as a float: products and remainders in
+// FP32 pairs (v = float(v) + rest, exact product by fused multiply-add), good
+// to the last place. FP64 runs at 1/64 of the FP32 rate here: the unit's
+// divisions by every warp of a CTA took microseconds of each launch, and v * u
+// for 8 x 4000 values by the CTA that finishes 23 us.
+__device__ __forceinline__ void unit_pair(double u, float &hi, float &lo) {
+    hi = (float)u;
+    lo = (float)(u - (double)hi);
+}
+__device__ __forceinline__ float scale_units(long long v, float uh, float ul) {
+    const float vh = __ll2float_rn(v), rest = __ll2float_rn(v - __float2ll_rn(vh));
+    const float p = vh * uh;
+    return p + fmaf(rest, uh, fmaf(vh, ul, fmaf(vh, uh, -p)));
 }
 
 }  // namespace tetra
