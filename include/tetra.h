@@ -278,11 +278,11 @@ tetra_status_t tetra_dos_batched(tetra_batch_plan_t plan, const float *const *ep
  *   ef     : host float, the result.
  *   ws     : device workspace of at least tetra_fermi_workspace_bytes(plan)
  *            bytes, 16-byte aligned.
- * Method: the band minimum and maximum bracket E_F; each round evaluates N at
- * 64 equidistant energies of the bracket in one TETRA_INTEGRATED launch and
- * keeps the sub-interval where N crosses n_electrons, until the bracket is at
- * the FP32 resolution of the energies (about six rounds). Synchronises
- * `stream` once per round. Returns TETRA_EINVAL for null/misaligned pointers
+ * Method: the band minimum and maximum bracket E_F; each round (one launch)
+ * evaluates N at 16 equidistant energies of the bracket, from the tetrahedra
+ * that straddle it, and keeps the sub-interval where N crosses n_electrons,
+ * until the bracket is at the FP32 resolution of the energies (about eight
+ * rounds). Synchronises `stream`. Returns TETRA_EINVAL for null/misaligned pointers
  * or n_electrons outside [0, N(max eps)], TETRA_ENOMEM if ws_bytes is too
  * small, TETRA_EUNSUPPORTED for a slab plan (the count needs the whole grid). */
 size_t tetra_fermi_workspace_bytes(tetra_plan_t plan);
@@ -347,17 +347,17 @@ tetra_status_t tetra_spectral_t0(tetra_plan_t plan, const float *eps, const int 
  * the Hilbert transform of tetra_spectral_t0's S (chi0 = int S(w')/(w - w' + i0) dw').
  * Same clipping into sub-tetrahedra as tetra_spectral_t0; each sub-tetrahedron
  * of volume fraction nu adds sign * nu * P<1/(w - D)>, the principal-value
- * average of 1/(w - D) over it (D linear there): a moment series beyond four
- * half-widths of its D range, the closed form of its density's three
- * quadratic pieces (logarithms) nearer. Every sub-tetrahedron reaches every
+ * average of 1/(w - D) over it (D linear there): a moment series beyond two
+ * half-widths of its D range (farther away one for several together), the
+ * closed form of its density's three quadratic pieces (logarithms) nearer. Every sub-tetrahedron reaches every
  * energy, so the cost grows with n_omega x sub-tetrahedra.
  *   plan, eps, q, mu : as tetra_spectral_t0 (whole-grid plan, n_bands <= 8).
  *   omega   : [n_omega] float, device, the energies (eV); any order.
  *   R       : [n_omega] float, overwritten.
  *   ws      : at least tetra_chi0_real_t0_workspace_bytes(plan, n_omega)
  *             bytes, 16-byte aligned.
- * The sub-tetrahedra of a warp are summed in FP32 in a fixed order (64 at a
- * time) and added to exact 64-bit integer tiles: reproducible for a given
+ * The sub-tetrahedra of a warp are summed in FP32 in a fixed order (64 band
+ * pairs at a time) and added to exact 64-bit integer tiles: reproducible for a given
  * plan and device, not bitwise independent of the launch shape. Returns
  * TETRA_EINVAL for null/misaligned pointers, TETRA_EUNSUPPORTED for
  * n_bands > 8, slab plans or n_omega beyond about 6000 (shared memory);

@@ -43,7 +43,7 @@
 #include <atomic>
 #include <cmath>
 
-#include "tetra_internal.cuh"
+#include "tet_common.cuh"
 
 namespace tetra {
 
@@ -62,9 +62,12 @@ constexpr unsigned kTileLimit = 1u << 30;   // the int32 tile is flushed before 
 constexpr int kKindS = 0, kKindRe = 1;
 constexpr int kReBlocksPerSM = 3;
 constexpr int kSubPerPair = 18;  // sub-tetrahedra one (tetrahedron, band pair) can give: 2 regions x 3 x 3
-constexpr int kReFlush = 64;     // entries summed in FP32 before the per-warp sums go to the tile
-constexpr int kReMom = 12;       // highest moment of the far-field series
-constexpr int kRePiece = 15;     // highest term of a density piece's own series
+constexpr int kReFlush = 64;     // band pairs summed in FP32 before the per-warp sums go to the tile
+constexpr int kReGroup = 8;      // lanes whose sub-tetrahedra are taken together far away
+constexpr int kReCluster = 20;   // highest moment of such a group
+constexpr int kReMom = 16;       // highest moment of one sub-tetrahedron
+constexpr int kRePiece = 8;      // terms of a density piece's own series
+constexpr int kReBatch = 16;     // sub-tetrahedra set up at a time
 
 // Table I (corner labels minus one, label c at offset (c&1, (c>>1)&1, (c>>2)&1)).
 __constant__ int kSpecTable[6][4] = {{0, 1, 2, 5}, {1, 2, 3, 5}, {0, 2, 4, 5},
@@ -112,14 +115,18 @@ struct ReSeg {
     float d0, d1, d2, d3, amp;
 };
 
-// Far-field set-up of one entry as the warp's lanes read it (16 words):
-// mean c, (4 R)^2, amplitude, segment slot, moments mu_0 and mu_2..mu_kReMom
-// (mu_1 vanishes about the mean).
+// Set-up of one entry as the warp's lanes read it (32 words): mean c,
+// amplitude, (2 R)^2, moments mu_2..mu_kReMom (mu_0 = 1, and mu_1 vanishes
+// about the mean), its group's centre and (twice the half-width)^2, and the
+// density pieces: corner values, reciprocal lengths (0 for an empty one),
+// g(d1), g(d2) and the middle piece's value at its centre.
 struct __align__(16) ReStage {
-    float c, far2, amp;
-    int loc;
-    float mu0, mu[kReMom - 1];
+    float c, amp, far2;
+    float mu[kReMom - 1];
+    float gc, gfar2;
+    float d[4], r[3], G1, G2, A2, pad[2];
 };
+static_assert(sizeof(ReStage) == 128, "32 words");
 
 // Constants of a launch that the sub-tetrahedron accumulation needs.
 struct SpecArgs {
@@ -135,12 +142,13 @@ struct SpecArgs {
     int *status;
     float om0, om_last;     // first and last grid energy (edge)
     float inv_de;           // 1 / mean spacing, for the index estimates
-    SubTet *q;              // shared: this warp's queue [kQueueCap]
-    int *qn;                // shared: its fill count (real part: each lane's)
+    SubTet *q;              // shared, S: this warp's queue [kQueueCap]
+    int *qn;                // shared, S: its fill count
     struct SpecTet *st;     // shared, S: this warp's set-ups [32]
-    float *racc;            // shared, real part: this warp's FP32 sums per energy
-    ReSeg *rq;              // shared, real part: the lanes' segments [32][kSubPerPair]
-    ReStage *stage;         // shared, real part: this warp's set-ups [32]
+    float *racc;            // shared, real part: the warps' FP32 sums per energy
+    ReSeg *rq;              // shared, real part: the lanes' segments [warps][32][kSubPerPair]
+    unsigned char *rn;      // shared, real part: their counts [warps][32]
+    ReStage *stage;         // shared, real part: the warps' set-ups [warps][kReBatch]
 };
 
 // One sub-tetrahedron set up for its energies [i0, i1): the density of D, and
@@ -256,9 +264,33 @@ __device__ __forceinline__ void spec_add(int *tile, int i, float x) {
     if (qv) atomicAdd(&tile[i], qv);
 }
 
-// Queues sign * nu * (distribution of D) of one sub-tetrahedron in this
-// warp's queue (or adds it at once when the queue is full). Real part: in
-// this lane's own segment, in the order the clipping produces them.
+// Queues one sub-tetrahedron with corner values d of D in this warp's queue (or
+// adds it at once when the queue is full). Real part: in this lane's own
+// segment, in the order the clipping produces them.
+template <int KIND>
+__device__ __forceinline__ void keep(float (&d)[4], float amp, uint32_t key, const SpecArgs &S) {
+#define SPEC_CS(i, j) { const float lo_ = fminf(d[i], d[j]), hi_ = fmaxf(d[i], d[j]); d[i] = lo_; d[j] = hi_; }
+    SPEC_CS(0, 1) SPEC_CS(2, 3) SPEC_CS(0, 2) SPEC_CS(1, 3) SPEC_CS(1, 2)
+#undef SPEC_CS
+    if constexpr (KIND == kKindRe) {
+        // every sub-tetrahedron reaches every energy (a flat one as 1/(w - d))
+        const int slot = S.rn[threadIdx.x]++;
+        S.rq[threadIdx.x * kSubPerPair + slot] = ReSeg{d[0], d[1], d[2], d[3], amp};
+    } else {
+        // a flat transition energy is a delta: measure zero in point mode, its
+        // whole weight in the bin that holds it in bin mode
+        if (S.mode != TETRA_BIN && !(d[3] > d[0])) return;
+        // no grid energy (bin) in reach
+        if (d[3] < S.om0 || d[0] > S.om_last) return;
+        const SubTet T{d[0], d[1], d[2], d[3], amp, key};
+        const int slot = atomicAdd(S.qn, 1);
+        if (slot < kQueueCap) S.q[slot] = T;
+        else deposit_wide(T, S);
+    }
+}
+
+// Keeps sign * nu * (distribution of D) of the sub-tetrahedron v0..v3, nu its
+// volume fraction.
 template <int KIND>
 __device__ __noinline__ void accumulate(P5 v0, P5 v1, P5 v2, P5 v3, float sign, uint32_t key,
                                         const SpecArgs &S) {
@@ -269,24 +301,7 @@ __device__ __noinline__ void accumulate(P5 v0, P5 v1, P5 v2, P5 v3, float sign, 
                            u02 * (u10 * u21 - u11 * u20));
     if (!(nu > 0.f)) return;
     float d[4] = {v0.c - v0.a, v1.c - v1.a, v2.c - v2.a, v3.c - v3.a};
-#define SPEC_CS(i, j) { const float lo_ = fminf(d[i], d[j]), hi_ = fmaxf(d[i], d[j]); d[i] = lo_; d[j] = hi_; }
-    SPEC_CS(0, 1) SPEC_CS(2, 3) SPEC_CS(0, 2) SPEC_CS(1, 3) SPEC_CS(1, 2)
-#undef SPEC_CS
-    if constexpr (KIND == kKindRe) {
-        // every sub-tetrahedron reaches every energy (a flat one as 1/(w - d))
-        const int lane = threadIdx.x & 31, slot = S.qn[lane]++;
-        S.rq[lane * kSubPerPair + slot] = ReSeg{d[0], d[1], d[2], d[3], sign * nu * S.scale};
-        return;
-    }
-    // a flat transition energy is a delta: measure zero in point mode, its
-    // whole weight in the bin that holds it in bin mode
-    if (S.mode != TETRA_BIN && !(d[3] > d[0])) return;
-    // no grid energy (bin) in reach
-    if (d[3] < S.om[0] || d[0] > S.om_last) return;
-    const SubTet T{d[0], d[1], d[2], d[3], sign * nu * S.scale, key};
-    const int slot = atomicAdd(S.qn, 1);
-    if (slot < kQueueCap) S.q[slot] = T;
-    else deposit_wide(T, S);
+    keep<KIND>(d, sign * nu * S.scale, key, S);
 }
 
 // Empties the queue, 32 sub-tetrahedra at a time. Called by all 32 lanes
@@ -300,6 +315,8 @@ __device__ __noinline__ void accumulate(P5 v0, P5 v1, P5 v2, P5 v3, float sign, 
 // at most 2^27 for each of the four warps.
 __device__ __forceinline__ void drain(const SpecArgs &S, int lane) {
     constexpr unsigned kAll = 0xffffffffu;
+    const SubTet *queue = S.q;
+    SpecTet *st = S.st;
     __syncwarp();
     const int n = min(*S.qn, kQueueCap);
     const float *om = S.om;
@@ -310,7 +327,7 @@ __device__ __forceinline__ void drain(const SpecArgs &S, int lane) {
         int K = 0;
         unsigned qb = 0;
         if (base + lane < n) {
-            const SubTet Q = S.q[base + lane];
+            const SubTet Q = queue[base + lane];
             spec_setup(Q, S, T);
             K = T.i1 - T.i0;
             // (a density is at most 3 / E41, a bin's average that or its step over it)
@@ -320,7 +337,7 @@ __device__ __forceinline__ void drain(const SpecArgs &S, int lane) {
                 K = 0;
             }
             if (K > 0) qb = (unsigned)most + 2u;
-            S.st[lane] = T;
+            st[lane] = T;
         }
         const unsigned announce = __reduce_add_sync(kAll, qb);
         unsigned old = 0;
@@ -338,7 +355,7 @@ __device__ __forceinline__ void drain(const SpecArgs &S, int lane) {
         while (wide) {
             const int j = __ffs(wide) - 1;
             wide &= wide - 1;
-            const SpecTet W = S.st[j];
+            const SpecTet W = st[j];
             for (int i = W.i0 + lane; i < W.i1; i += 32) spec_add(tile, i, spec_value(W, om, bin, i));
         }
         if (K > 0 && K < kWide)
@@ -418,109 +435,124 @@ __device__ __noinline__ void region(P5 v0, P5 v1, P5 v2, P5 v3, int first, int s
 // 1/(w - x). g is a quadratic spline on the sorted corner values d0..d3 with
 // Bernstein coefficients (0, 0, G1) on [d0, d1], (G1, 3/d41, G2) on [d1, d2]
 // and (G2, 0, 0) on [d2, d3], G1 = 3 d21/(d31 d41) = g(d1), G2 = 3 d43/(d41
-// d42) = g(d2). Far from the sub-tetrahedron (|w - c| > 4 R, c the mean of
+// d42) = g(d2). Far from the sub-tetrahedron (|w - c| > 2 R, c the mean of
 // the corner values, R the largest |d_k - c|) the average is the moment
 // series sum_n mu_n / (w - c)^(n+1), mu_n = <(D - c)^n> = 6 n!/(n+3)!
 // h_n(d - c) (h_n the complete homogeneous symmetric polynomial), whose
-// terms shrink by 1/4 or more. Near it each piece [a, b] (h = b - a,
-// s = (w - a)/h) gives, within 3/2 of its own centre,
-//   p(s) [ln|w - a| - ln|w - b|] + b0 (3/2 - s) + b1 (2s - 1) - b2 (s + 1/2),
-// p the piece's polynomial continued to t = s, and beyond that its own
-// moment series in 1/(s - 1/2) (a thin piece far from w, where the closed
-// form would cancel). At a knot the two pieces meeting there drop their
+// terms shrink by 1/2 or more. Near it each piece [a, b] gives its closed
+// form with the logarithm of |w - a| / |w - b|, or, beyond 3/2 of its length
+// from its centre, that form's series (re_piece). At a knot the two pieces meeting there drop their
 // equal-and-opposite ln|w - knot| terms.
-// Far-field data of a sub-tetrahedron: mean c of its corner values, (4 R)^2
-// and the moments mu_0..mu_kReMom about c.
-struct ReFar {
-    float c, far2;
-    float mu[kReMom + 1];
-};
+//
+// Neighbouring lanes keep neighbouring tetrahedra of one band pair, whose D
+// lie close together: far from all of a group of kReGroup lanes (beyond twice
+// the half-width of their joint range) they add one series, of their summed
+// moments about its centre; only the energies nearer than that take them one
+// by one: beyond 2 R of a sub-tetrahedron by its own series, within by the
+// density pieces. Series are cut where their terms, (R/u)^n times moments
+// that fall as n^-3 (joint range: n^-1), drop below 2^-23 of the first.
+// (One series per sub-tetrahedron at every energy, pieces within 4 R: 33.8 ms
+// at 48^3 points, 8 bands, 400 energies on a 4 eV window; with the whole warp
+// as the group and the pieces' series in 16 terms 14.0 ms.)
 
-__device__ __forceinline__ void re_far_setup(const ReSeg &T, ReFar &F) {
-    F.c = 0.25f * ((T.d0 + T.d1) + (T.d2 + T.d3));
-    const float e[4] = {T.d0 - F.c, T.d1 - F.c, T.d2 - F.c, T.d3 - F.c};
-    const float R = fmaxf(-e[0], e[3]);
-    F.far2 = 16.f * R * R;
-    // h_n(e) from prod_k 1 / (1 - e_k t), one factor at a time
-    float h[kReMom + 1];
+// h_n of the values e_0..e_3 (h_0 = 1), from prod_k 1 / (1 - e_k t).
+template <int K>
+__device__ __forceinline__ void re_homogeneous(const float (&e)[4], float (&h)[K + 1]) {
     h[0] = 1.f;
 #pragma unroll
-    for (int n = 1; n <= kReMom; ++n) h[n] = 0.f;
+    for (int n = 1; n <= K; ++n) h[n] = 0.f;
 #pragma unroll
     for (int k = 0; k < 4; ++k)
 #pragma unroll
-        for (int n = 1; n <= kReMom; ++n) h[n] = fmaf(e[k], h[n - 1], h[n]);
-#pragma unroll
-    for (int n = 0; n <= kReMom; ++n) F.mu[n] = h[n] * (6.f / (float)((n + 1) * (n + 2) * (n + 3)));
+        for (int n = 1; n <= K; ++n) h[n] = fmaf(e[k], h[n - 1], h[n]);
 }
+__host__ __device__ constexpr float re_coef(int n) { return 6.f / (float)((n + 1) * (n + 2) * (n + 3)); }
 
-// int_0^1 p(t) / (s - t) dt for a piece with Bernstein coefficients b0..b2.
-__device__ __forceinline__ float re_piece(float b0, float b1, float b2, float a, float rh, float La, float Lb,
-                                          float w) {
-    if (rh == 0.f) return 0.f;
-    const float s = (w - a) * rh, up = s - 0.5f;
-    if (fabsf(up) >= 1.5f) {
-        // p = A + B tau + C tau^2, tau = t - 1/2; moments of tau^k over
-        // [-1/2, 1/2]: 2^-k / (k + 1) for even k, 0 for odd k
-        const float A = 0.25f * (b0 + 2.f * b1 + b2), B = b2 - b0, C = b0 - 2.f * b1 + b2;
-        const float v = 1.f / up;
-        float acc = 0.f;
+__device__ __forceinline__ void re_setup(const ReSeg &T, ReStage &st) {
+    const float c = 0.25f * ((T.d0 + T.d1) + (T.d2 + T.d3));
+    const float e[4] = {T.d0 - c, T.d1 - c, T.d2 - c, T.d3 - c};
+    const float R = fmaxf(-e[0], e[3]);
+    st.c = c;
+    st.amp = T.amp;
+    st.far2 = 4.f * R * R;
+    float h[kReMom + 1];
+    re_homogeneous<kReMom>(e, h);
 #pragma unroll
-        for (int j = kRePiece; j >= 0; --j) {
-            float m;
-            if (j % 2 == 0)
-                m = A * (ldexpf(1.f, -j) / (float)(j + 1)) + C * (ldexpf(1.f, -(j + 2)) / (float)(j + 3));
-            else
-                m = B * (ldexpf(1.f, -(j + 1)) / (float)(j + 2));
-            acc = fmaf(acc, v, m);
-        }
-        return acc * v;
-    }
-    const float t1 = 1.f - s;
-    const float ps = fmaf(b0 * t1, t1, fmaf(2.f * b1 * s, t1, b2 * s * s));
-    return fmaf(ps, La - Lb, fmaf(b0, 1.5f - s, fmaf(b1, 2.f * s - 1.f, -b2 * (s + 0.5f))));
-}
-
-__device__ __forceinline__ float re_log(float w, float d) { return (w == d) ? 0.f : __logf(fabsf(w - d)); }
-
-// P<1/(w - D)> within four half-widths of the sub-tetrahedron (or for a
-// flat one): the three density pieces.
-__device__ float re_near(const ReSeg &T, float w) {
+    for (int n = 2; n <= kReMom; ++n) st.mu[n - 2] = h[n] * re_coef(n);
     const float d21 = T.d1 - T.d0, d31 = T.d2 - T.d0, d41 = T.d3 - T.d0;
     const float d32 = T.d2 - T.d1, d42 = T.d3 - T.d1, d43 = T.d3 - T.d2;
-    if (!(d41 > 0.f)) return (w == T.d0) ? 0.f : 1.f / (w - T.d0);
-    const float G1 = d31 > 0.f ? __fdividef(3.f * d21, d31 * d41) : 0.f;
-    const float G2 = d42 > 0.f ? __fdividef(3.f * d43, d41 * d42) : 0.f;
-    const float mid = __fdividef(3.f, d41);
-    const float r1 = d21 > 0.f ? __fdividef(1.f, d21) : 0.f;
-    const float r2 = d32 > 0.f ? __fdividef(1.f, d32) : 0.f;
-    const float r3 = d43 > 0.f ? __fdividef(1.f, d43) : 0.f;
-    const float L0 = re_log(w, T.d0), L1 = re_log(w, T.d1), L2 = re_log(w, T.d2), L3 = re_log(w, T.d3);
-    return re_piece(0.f, 0.f, G1, T.d0, r1, L0, L1, w) + re_piece(G1, mid, G2, T.d1, r2, L1, L2, w) +
-           re_piece(G2, 0.f, 0.f, T.d2, r3, L2, L3, w);
+    st.d[0] = T.d0; st.d[1] = T.d1; st.d[2] = T.d2; st.d[3] = T.d3;
+    st.G1 = d31 > 0.f ? __fdividef(3.f * d21, d31 * d41) : 0.f;
+    st.G2 = d42 > 0.f ? __fdividef(3.f * d43, d41 * d42) : 0.f;
+    st.A2 = 0.25f * (st.G1 + st.G2) + (d41 > 0.f ? __fdividef(1.5f, d41) : 0.f);
+    st.r[0] = d21 > 0.f ? __fdividef(1.f, d21) : 0.f;
+    st.r[1] = d32 > 0.f ? __fdividef(1.f, d32) : 0.f;
+    st.r[2] = d43 > 0.f ? __fdividef(1.f, d43) : 0.f;
 }
 
-// The moment series with terms mu_0..mu_K at v = 1/(w - c), four energies at once.
-template <int K>
-__device__ __forceinline__ void re_series4(const float (&mu)[kReMom + 1], const float (&v)[4], float (&r)[4]) {
-    float acc[4];
+// int p(tau) / (up - tau) dtau over [-1/2, 1/2], p = A + B tau + C tau^2, up
+// the distance from the piece's centre in lengths, L = log2 of the ratio of
+// the distances to its ends. With P = int 1/(up - tau) = ln 2 L the integral
+// is p(up) P - B - C up; beyond 3/2 lengths, where that would cancel, P =
+// v (1 + t S), v = 1/up, t = v^2/4, S = 1/3 + t/5 + t^2/7 + ..., and the
+// integral A P + (B t + C v/4) S.
+__device__ __forceinline__ float re_piece(float A, float B, float C, float up, float L) {
+    if (fabsf(up) >= 1.5f) {
+        const float v = __fdividef(1.f, up), t = 0.25f * v * v;
+        float S = 1.f / (2 * kRePiece + 1);
 #pragma unroll
-    for (int k = 0; k < 4; ++k) acc[k] = mu[K];
+        for (int j = kRePiece - 1; j >= 1; --j) S = fmaf(S, t, 1.f / (2 * j + 1));
+        return fmaf(A * v, fmaf(t, S, 1.f), fmaf(B, t, 0.25f * C * v) * S);
+    }
+    return fmaf(fmaf(fmaf(C, up, B), up, A), 0.693147181f * L, -fmaf(C, up, B));
+}
+
+// log2 |w - d|; 0 at a knot (also for a subnormal difference, which the
+// approximation would take as 0)
+__device__ __forceinline__ float re_log2(float w, float d) {
+    const float x = fabsf(w - d);
+    float l;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(l) : "f"(x));
+    return x < 1.2e-38f ? 0.f : l;
+}
+
+// P<1/(w - D)> within two half-widths of the sub-tetrahedron (or of a flat
+// one): the three density pieces.
+__device__ __forceinline__ float re_near(const ReStage &T, float w) {
+    if (!(T.d[3] > T.d[0])) return (w == T.d[0]) ? 0.f : 1.f / (w - T.d[0]);
+    float L[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) L[k] = re_log2(w, T.d[k]);
+    float up[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) up[k] = fmaf(-0.5f, T.d[k + 1] - T.d[k], w - T.d[k]) * T.r[k];
+    float sum = 0.f;
+    if (T.r[0] != 0.f) sum += re_piece(0.25f * T.G1, T.G1, T.G1, up[0], L[0] - L[1]);
+    if (T.r[1] != 0.f)
+        sum += re_piece(T.A2, T.G2 - T.G1, 2.f * (T.G1 + T.G2) - 4.f * T.A2, up[1], L[1] - L[2]);
+    if (T.r[2] != 0.f) sum += re_piece(0.25f * T.G2, -T.G2, T.G2, up[2], L[2] - L[3]);
+    return sum;
+}
+
+// sum_{n <= K} m[n] z^n for several z at once.
+template <int K, int U, int N>
+__device__ __forceinline__ void re_series(const float (&m)[N], const float (&z)[U], float (&r)[U]) {
+#pragma unroll
+    for (int k = 0; k < U; ++k) r[k] = m[K];
 #pragma unroll
     for (int n = K - 1; n >= 0; --n)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) acc[k] = fmaf(acc[k], v[k], mu[n]);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) r[k] = acc[k] * v[k];
+        for (int k = 0; k < U; ++k) r[k] = fmaf(r[k], z[k], m[n]);
 }
 
 // Adds the per-warp FP32 sums to the tile (one rounding per energy and
 // flush) and clears them. Every lane owns the energies lane, lane + 32, ...
 __device__ __forceinline__ void re_flush(const SpecArgs &S, int lane) {
+    float *racc = S.racc + (threadIdx.x >> 5) * S.n_om;
     __syncwarp();
     for (int i = lane; i < S.n_om; i += 32) {
-        const float x = S.racc[i];
-        S.racc[i] = 0.f;
+        const float x = racc[i];
+        racc[i] = 0.f;
         if (fabsf(x) < 4.0e18f) {
             const long long qv = __float2ll_rn(x);
             if (qv) atomicAdd(reinterpret_cast<unsigned long long *>(&S.tile[i]), static_cast<unsigned long long>(qv));
@@ -531,123 +563,193 @@ __device__ __forceinline__ void re_flush(const SpecArgs &S, int lane) {
     __syncwarp();
 }
 
-// The warp takes the sub-tetrahedra its lanes queued for the last band
-// pair in lane order (a fixed order: the FP32 sums are reproducible), up to
-// 32 at a time: each lane sets up one entry's far field into the warp's
-// staging area; then every lane runs over its energies (lane, lane + 32,
-// lane + 64, lane + 96 of each chunk of 128) and, for each staged entry in
-// order, adds its average there into four register sums, which go to the
-// warp's FP32 sums once per chunk. Series terms (truncation below 2^-23 of
-// the leading 1/(w - c), terms shrinking by R/|w - c|): 6 when the warp's 128
-// energies are all beyond 16 R, 8 beyond 8 R, 13 beyond 4 R; nearer, the
-// density pieces.
-__device__ __forceinline__ void re_process(const SpecArgs &S, const ReSeg *wq, int *wn, int lane,
-                                           int &since_flush) {
+// The warp takes the sub-tetrahedra its lanes kept of the last band pair, in
+// lane order (a fixed order: the FP32 sums are reproducible). Every lane owns
+// the energies lane, lane + 32, ...
+__device__ __forceinline__ void re_process(const SpecArgs &S, int lane, int &since_flush) {
     constexpr unsigned kAll = 0xffffffffu;
+    const int warp = threadIdx.x >> 5;
+    const ReSeg *wq = S.rq + warp * 32 * kSubPerPair;
+    ReStage *stage = S.stage + warp * kReBatch;
+    const float *om = S.om;
+    const int n_om = S.n_om;
+    float *racc = S.racc + warp * n_om;
     __syncwarp();
-    const int mine = wn[lane];
-    // exclusive prefix of the lanes' counts
+    const int mine = S.rn[threadIdx.x];
+    if (!__any_sync(kAll, mine)) return;
+    // exclusive prefix of the lanes' counts, and the group's joint range
     int incl = mine;
+    float lo = INFINITY, hi = -INFINITY;
+    for (int i = 0; i < mine; ++i) {
+        lo = fminf(lo, wq[lane * kSubPerPair + i].d0);
+        hi = fmaxf(hi, wq[lane * kSubPerPair + i].d3);
+    }
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
         const int y = __shfl_up_sync(kAll, incl, d);
         if (lane >= d) incl += y;
+        if (d < kReGroup) {
+            lo = fminf(lo, __shfl_xor_sync(kAll, lo, d));
+            hi = fmaxf(hi, __shfl_xor_sync(kAll, hi, d));
+        }
     }
     const int start = incl - mine, total = __shfl_sync(kAll, incl, 31);
-    for (int base = 0; base < total; base += 32) {
-        // this lane's entry: the last lane whose segment starts at or before it
-        const int e = base + lane;
-        int src = 0;
+    // joint moments about the group's centre in units of its half-width, of
+    // this lane's entries first
+    const bool some = hi >= lo;
+    const float C = some ? 0.5f * (lo + hi) : 0.f, rho = some ? 0.5f * (hi - lo) : 0.f;
+    const float inv = rho > 0.f ? 1.f / rho : 0.f;
+    constexpr int kM = 24;   // kReCluster + 1 in whole thirds of the exchange below
+    float M[kM];
 #pragma unroll
-        for (int step = 16; step >= 1; step >>= 1) {
-            const int cand = src + step;
-            if (__shfl_sync(kAll, start, cand) <= e) src = cand;
+    for (int n = 0; n < kM; ++n) M[n] = 0.f;
+    for (int i = 0; i < mine; ++i) {
+        const ReSeg T = wq[lane * kSubPerPair + i];
+        const float e[4] = {(T.d0 - C) * inv, (T.d1 - C) * inv, (T.d2 - C) * inv, (T.d3 - C) * inv};
+        float h[kReCluster + 1];
+        re_homogeneous<kReCluster>(e, h);
+#pragma unroll
+        for (int n = 0; n <= kReCluster; ++n) M[n] = fmaf(T.amp * re_coef(n), h[n], M[n]);
+    }
+    // summed over the group's lanes: three moments end up in each
+#pragma unroll
+    for (int step = 0; step < 3; ++step) {
+        const int half = kM >> (step + 1), mask = kReGroup >> (step + 1);
+        const bool upper = lane & mask;
+#pragma unroll
+        for (int i = 0; i < half; ++i) {
+            const float send = upper ? M[i] : M[i + half], keep = upper ? M[i + half] : M[i];
+            M[i] = keep + __shfl_xor_sync(kAll, send, mask);
         }
-        const int src_start = __shfl_sync(kAll, start, src);
-        if (e < total) {
-            const int loc = src * kSubPerPair + (e - src_start);
-            const ReSeg T = wq[loc];
-            ReFar F;
-            re_far_setup(T, F);
-            ReStage &st = S.stage[lane];
-            st.c = F.c; st.far2 = F.far2; st.amp = T.amp; st.loc = loc; st.mu0 = F.mu[0];
+    }
+    float *joint = reinterpret_cast<float *>(stage);   // [group][kM]
+    {
+        const int first = 12 * ((lane >> 2) & 1) + 6 * ((lane >> 1) & 1) + 3 * (lane & 1);
 #pragma unroll
-            for (int n = 2; n <= kReMom; ++n) st.mu[n - 2] = F.mu[n];
-        }
-        __syncwarp();
-        const int n_here = min(32, total - base);
-        for (int c0 = 0; c0 < S.n_om; c0 += 128) {
-            float w[4], sum[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int i = 0; i < 3; ++i) joint[(lane / kReGroup) * kM + first + i] = M[i];
+    }
+    __syncwarp();
+    bool near_any = false;
+#pragma unroll 1
+    for (int g = 0; g < 32 / kReGroup; ++g) {
+        const float gC = __shfl_sync(kAll, C, g * kReGroup), grho = __shfl_sync(kAll, rho, g * kReGroup);
+        if (!__shfl_sync(kAll, (int)some, g * kReGroup)) continue;
+        float m[kReCluster + 1];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) w[k] = S.om[min(c0 + lane + 32 * k, S.n_om - 1)];
-            for (int j = 0; j < n_here; ++j) {
-                const ReStage &st = S.stage[j];
-                float mu[kReMom + 1];
-                mu[0] = st.mu0;
-                mu[1] = 0.f;
-#pragma unroll
-                for (int n = 2; n <= kReMom; ++n) mu[n] = st.mu[n - 2];
-                float v[4], r[4];
-                float umin = INFINITY;
-                bool lane_far = true;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const float u = w[k] - st.c;
-                    v[k] = __fdividef(1.f, u);
-                    if (c0 + lane + 32 * k < S.n_om) {
-                        umin = fminf(umin, u * u);
-                        lane_far = lane_far && (u * u > st.far2);
-                    }
-                }
-                // the warp's nearest energy (non-negative floats order as integers)
-                const float wmin = __uint_as_float(__reduce_min_sync(kAll, __float_as_uint(umin)));
-                const float R2 = st.far2 * (1.f / 16.f);
-                if (R2 * 256.f < wmin) {
-                    re_series4<5>(mu, v, r);
-                } else if (R2 * 64.f < wmin) {
-                    re_series4<7>(mu, v, r);
-                } else if (lane_far) {
-                    re_series4<kReMom>(mu, v, r);
-                } else {
-                    const ReSeg T = wq[st.loc];
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const float u = w[k] - st.c;
-                        if (u * u > st.far2) {
-                            float p = mu[kReMom];
-#pragma unroll
-                            for (int n = kReMom - 1; n >= 0; --n) p = fmaf(p, v[k], mu[n]);
-                            r[k] = p * v[k];
-                        } else {
-                            r[k] = re_near(T, w[k]);
-                        }
-                    }
-                }
-#pragma unroll
-                for (int k = 0; k < 4; ++k) sum[k] = fmaf(st.amp, r[k], sum[k]);
-            }
+        for (int n = 0; n <= kReCluster; ++n) m[n] = joint[g * kM + n];
+        const float far2 = 4.f * grho * grho;
+        for (int c0 = 0; c0 < n_om; c0 += 128) {
+            float z[4], v[4], r[4];
+            float umin = INFINITY;
+            bool far[4];
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int i = c0 + lane + 32 * k;
-                if (i < S.n_om) S.racc[i] += sum[k];
+                const float u = om[min(i, n_om - 1)] - gC;
+                v[k] = __fdividef(1.f, u);
+                z[k] = grho * v[k];
+                far[k] = i < n_om && u * u > far2;
+                near_any = near_any || (i < n_om && !far[k]);
+                if (far[k]) umin = fminf(umin, u * u);
             }
+            // the warp's nearest far energy (non-negative floats order as integers)
+            const float wmin = __uint_as_float(__reduce_min_sync(kAll, __float_as_uint(umin)));
+            if (wmin == INFINITY) continue;
+            if (wmin > 16.f * far2) re_series<7>(m, z, r);
+            else if (wmin > 4.f * far2) re_series<11>(m, z, r);
+            else re_series<kReCluster>(m, z, r);
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (far[k]) racc[c0 + lane + 32 * k] += r[k] * v[k];
         }
-        __syncwarp();
-        since_flush += n_here;
-        if (since_flush >= kReFlush) {
-            re_flush(S, lane);
-            since_flush = 0;
+    }
+    if (__any_sync(kAll, near_any)) {
+        for (int base = 0; base < total; base += kReBatch) {
+            const int n_here = min(kReBatch, total - base);
+            // entry's place: the last lane whose segment starts at or before it
+            const int e = base + (lane & (kReBatch - 1));
+            int src = 0;
+#pragma unroll
+            for (int step = 16; step >= 1; step >>= 1) {
+                const int cand = src + step;
+                if (__shfl_sync(kAll, start, cand) <= e) src = cand;
+            }
+            const int loc = src * kSubPerPair + (e - __shfl_sync(kAll, start, src));
+            const float gC = __shfl_sync(kAll, C, src), grho = __shfl_sync(kAll, rho, src);
+            __syncwarp();   // the joint moments, the last batch are read
+            if (lane < n_here) {
+                re_setup(wq[loc], stage[lane]);
+                stage[lane].gc = gC;
+                stage[lane].gfar2 = 4.f * grho * grho;
+            }
+            __syncwarp();
+            for (int c0 = 0; c0 < n_om; c0 += 64) {
+                float w[2], sum[2] = {0.f, 0.f};
+                bool touched = false;
+#pragma unroll
+                for (int k = 0; k < 2; ++k) w[k] = om[min(c0 + lane + 32 * k, n_om - 1)];
+                for (int j = 0; j < n_here; ++j) {
+                    const ReStage &st = stage[j];
+                    bool near[2];
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        const float u = w[k] - st.gc;
+                        near[k] = c0 + lane + 32 * k < n_om && !(u * u > st.gfar2);
+                    }
+                    if (!__any_sync(kAll, near[0] || near[1])) continue;
+                    touched = true;
+                    float v[2], r[2] = {0.f, 0.f}, umin = INFINITY;
+                    bool own[2];   // by its own series
+                    bool pieces = false;
+#pragma unroll
+                    for (int k = 0; k < 2; ++k) {
+                        const float u = w[k] - st.c;
+                        v[k] = __fdividef(1.f, u);
+                        own[k] = u * u > st.far2;
+                        pieces = pieces || (near[k] && !own[k]);
+                        if (near[k] && own[k]) umin = fminf(umin, u * u);
+                    }
+                    const float wmin = __uint_as_float(__reduce_min_sync(kAll, __float_as_uint(umin)));
+                    if (wmin != INFINITY) {
+                        float mu[kReMom + 1];
+                        mu[0] = 1.f;
+                        mu[1] = 0.f;
+#pragma unroll
+                        for (int n = 2; n <= kReMom; ++n) mu[n] = st.mu[n - 2];
+                        if (wmin > 4.f * st.far2) re_series<8>(mu, v, r);
+                        else re_series<kReMom>(mu, v, r);
+#pragma unroll
+                        for (int k = 0; k < 2; ++k) r[k] *= v[k];
+                    }
+                    if (__any_sync(kAll, pieces)) {
+#pragma unroll
+                        for (int k = 0; k < 2; ++k)
+                            if (near[k] && !own[k]) r[k] = re_near(st, w[k]);
+                    }
+#pragma unroll
+                    for (int k = 0; k < 2; ++k)
+                        if (near[k]) sum[k] = fmaf(st.amp, r[k], sum[k]);
+                }
+                if (touched) {
+#pragma unroll
+                    for (int k = 0; k < 2; ++k)
+                        if (c0 + lane + 32 * k < n_om) racc[c0 + lane + 32 * k] += sum[k];
+                }
+            }
         }
     }
     __syncwarp();
-    wn[lane] = 0;
-    __syncwarp();
+    S.rn[threadIdx.x] = 0;
+    if (++since_flush >= kReFlush) {
+        re_flush(S, lane);
+        since_flush = 0;
+    }
 }
 
 template <int KIND>
 __host__ __device__ constexpr int queue_entries() { return KIND == kKindS ? kQueueCap : 32 * kSubPerPair; }
-template <int KIND>
-__host__ __device__ constexpr int queue_counts() { return KIND == kKindS ? 2 : 32; }
+template <int KIND>   // in ints; real part: a byte per lane
+__host__ __device__ constexpr int queue_counts() { return KIND == kKindS ? 2 : 8; }
 
 template <int KIND>
 __host__ __device__ constexpr size_t queue_entry_bytes() { return KIND == kKindS ? sizeof(SubTet) : sizeof(ReSeg); }
@@ -658,7 +760,7 @@ template <int KIND>
 size_t spec_smem_bytes(int n_om, int mode) {
     return queue_entry_bytes<KIND>() * kSpecWarps * queue_entries<KIND>() +
            sizeof(int) * kSpecWarps * queue_counts<KIND>() +
-           (KIND == kKindRe ? sizeof(ReStage) * kSpecWarps * 32 + sizeof(float) * kSpecWarps * (size_t)n_om
+           (KIND == kKindRe ? sizeof(ReStage) * kSpecWarps * kReBatch + sizeof(float) * kSpecWarps * (size_t)n_om
                             : sizeof(SpecTet) * kSpecWarps * 32) +
            (KIND == kKindRe ? sizeof(long long) : sizeof(int)) * (size_t)n_om +
            sizeof(float) * (size_t)(mode == TETRA_BIN ? n_om + 1 : n_om);
@@ -694,14 +796,15 @@ __global__ void __launch_bounds__(kSpecThreads, KIND == kKindS ? kSpecBlocksPerS
     constexpr int QW = queue_entries<KIND>(), QC = queue_counts<KIND>();
     unsigned char *qraw = smem;                                             // [warps][QW] entries
     int *qcount = reinterpret_cast<int *>(qraw + queue_entry_bytes<KIND>() * kSpecWarps * QW);   // [warps][QC]
-    ReStage *stage = reinterpret_cast<ReStage *>(qcount + kSpecWarps * QC); // real part: [warps][32]
+    ReStage *stage = reinterpret_cast<ReStage *>(qcount + kSpecWarps * QC); // real part: [warps][kReBatch]
     SpecTet *stet = reinterpret_cast<SpecTet *>(stage);                     // S: [warps][32]
-    float *racc = reinterpret_cast<float *>(stage + kSpecWarps * 32);       // real part: [warps][n_om]
+    float *racc = reinterpret_cast<float *>(stage + kSpecWarps * kReBatch); // real part: [warps][n_om]
     long long *tile = reinterpret_cast<long long *>(racc + (KIND == kKindRe ? kSpecWarps * n_om : 0));
     int *tile32 = reinterpret_cast<int *>(tile);                            // S
     float *om = KIND == kKindRe ? reinterpret_cast<float *>(tile + n_om) : reinterpret_cast<float *>(tile32 + n_om);
-    static_assert(sizeof(SpecTet) == sizeof(ReStage), "one staging area for both");
+    static_assert(sizeof(SpecTet) * 32 == sizeof(ReStage) * kReBatch, "one staging area for both");
     __shared__ unsigned s_bound;
+    __shared__ float s_grid[4];   // V_T/V_G in units, 1 / mean spacing, the unit as a pair
     __shared__ float s_iw[kSpecWarps];
     const int n_edges = (mode == TETRA_BIN) ? n_om + 1 : n_om;
     for (int i = threadIdx.x; i < n_om; i += blockDim.x) {
@@ -709,15 +812,19 @@ __global__ void __launch_bounds__(kSpecThreads, KIND == kKindS ? kSpecBlocksPerS
         else tile32[i] = 0;
     }
     for (int i = threadIdx.x; i < n_edges; i += blockDim.x) om[i] = omega[i];
-    if (threadIdx.x == 0) s_bound = 0u;
+    if (threadIdx.x == 0) {
+        s_bound = 0u;
+        const double de = mean_spacing(omega, n_om, mode);
+        s_grid[0] = (float)ldexp(de, bits);
+        s_grid[1] = (float)(1.0 / de);
+        unit_pair(vtvg / de * ldexp(1.0, -bits), s_grid[2], s_grid[3]);
+    }
     for (int i = threadIdx.x; i < kSpecWarps * QC; i += blockDim.x) qcount[i] = 0;
     if constexpr (KIND == kKindRe)
         for (int i = threadIdx.x; i < kSpecWarps * n_om; i += blockDim.x) racc[i] = 0.f;
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    // V_T/V_G in fixed-point units: de * 2^bits
-    const double de = mean_spacing(om, n_om, mode);
-    const float scale = (float)ldexp(de, bits);
+    const float scale = s_grid[0];
     float max_iw = 0.f;
     if (KIND == kKindS && mode == TETRA_BIN) {
         for (int i = threadIdx.x; i < n_om; i += blockDim.x) max_iw = fmaxf(max_iw, 1.0f / (om[i + 1] - om[i]));
@@ -727,17 +834,21 @@ __global__ void __launch_bounds__(kSpecThreads, KIND == kKindS ? kSpecBlocksPerS
         for (int i = 0; i < kSpecWarps; ++i) max_iw = fmaxf(max_iw, s_iw[i]);
     }
     const float om_lo = om[0], om_hi = om[n_edges - 1];
-    SubTet *wq = reinterpret_cast<SubTet *>(qraw) + warp * QW;   // S
-    ReSeg *wr = reinterpret_cast<ReSeg *>(qraw) + warp * QW;     // real part
-    int *wn = qcount + warp * QC;
-    // (in shared memory: the clipping's calls pass an address, not 120 bytes)
-    __shared__ SpecArgs s_args[kSpecWarps];
-    if (lane == 0)
-        s_args[warp] = SpecArgs{om, tile, tile32, &s_bound, sums, n_om, mode, scale, max_iw, status, om_lo, om_hi,
-                                (float)(1.0 / de), wq, wn, stet + warp * 32, racc + warp * n_om, wr, stage + warp * 32};
-    __syncwarp();
-    const SpecArgs &S = s_args[warp];
-    int since_flush = 0;   // real part: entries in the per-warp FP32 sums
+    // (in shared memory: the clipping's calls pass an address, not 120 bytes;
+    // S: one per warp with its own queue, which measured 2.1 ms at 64^3 against
+    // 2.8 with one per block; real part: one, to leave the room to its sums)
+    constexpr int kArgs = KIND == kKindS ? kSpecWarps : 1;
+    __shared__ SpecArgs s_args[kArgs];
+    if (threadIdx.x < kArgs) {
+        const int wp = threadIdx.x;
+        s_args[wp] = SpecArgs{om, tile, tile32, &s_bound, sums, n_om, mode, scale, max_iw, status, om_lo, om_hi,
+                              s_grid[1], reinterpret_cast<SubTet *>(qraw) + wp * QW, qcount + wp * QC,
+                              stet + wp * 32, racc, reinterpret_cast<ReSeg *>(qraw),
+                              reinterpret_cast<unsigned char *>(qcount), stage};
+    }
+    __syncthreads();
+    const SpecArgs &S = s_args[KIND == kKindS ? warp : 0];
+    int since_flush = 0;   // real part: band pairs in the per-warp FP32 sums
     // energy range of the grid: a band pair whose transition energies over a
     // tetrahedron miss it contributes nothing (the clipped regions' values
     // lie between the corner minimum and maximum); the +1 region has positive
@@ -776,7 +887,7 @@ __global__ void __launch_bounds__(kSpecThreads, KIND == kKindS ? kSpecBlocksPerS
         }
         // per band: some corner occupied (an), some corner empty (ap); the
         // same for the bands at k + q (cn: occupied, cp: empty)
-        uint32_t an = 0, ap = 0, cn = 0, cp = 0, a_all = 0, c_all = 0;
+        uint32_t an = 0, ap = 0, cn = 0, cp = 0, a_all = 0, c_all = 0, a_none = 0, c_none = 0;
         if (valid) {
 #pragma unroll
             for (int n = 0; n < NB; ++n) {
@@ -790,12 +901,27 @@ __global__ void __launch_bounds__(kSpecThreads, KIND == kKindS ? kSpecBlocksPerS
                 cp |= (cmax > 0.f ? 1u : 0u) << n;
                 a_all |= (amax < 0.f ? 1u : 0u) << n;   // occupied at every corner
                 c_all |= (cmin > 0.f ? 1u : 0u) << n;   // empty at every corner
+                a_none |= (amin > 0.f ? 1u : 0u) << n;  // and the converse
+                c_none |= (cmax < 0.f ? 1u : 0u) << n;
             }
         }
-        // band pairs in a loop that is not unrolled (one copy of the code);
-        // the queue is drained between pairs once it holds kDrainAt entries
+        // band pairs with a region in some lane's tetrahedron, in a loop that is
+        // not unrolled (one copy of the code); the queue is drained between pairs
+        // once it holds kDrainAt entries. (The +1 region has positive transition
+        // energies, the -1 region negative ones.)
+        const bool above = KIND == kKindRe || om_hi > 0.f, below = KIND == kKindRe || om_lo < 0.f;
+        uint64_t mine = 0;
+#pragma unroll
+        for (int n = 0; n < NB; ++n) {
+            const uint32_t row = (above && ((an >> n) & 1u) ? cp : 0u) | (below && ((ap >> n) & 1u) ? cn : 0u);
+            mine |= (uint64_t)row << (n * NB);
+        }
+        uint64_t pairs = (uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)mine) |
+                         (uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(mine >> 32)) << 32;
 #pragma unroll 1
-        for (int pr = 0; pr < NB * NB; ++pr) {
+        while (pairs) {
+            const int pr = __ffsll((long long)pairs) - 1;
+            pairs &= pairs - 1;
             if constexpr (KIND == kKindS) {
                 // lane 0's count, read after every push of the previous pair
                 // and before any of this one: the same decision in every lane
@@ -803,33 +929,36 @@ __global__ void __launch_bounds__(kSpecThreads, KIND == kKindS ? kSpecBlocksPerS
                 const int queued = __shfl_sync(0xffffffffu, *S.qn, 0);
                 if (queued >= kDrainAt) drain(S, lane);
             } else {
-                re_process(S, wr, wn, lane, since_flush);   // the previous pair's sub-tetrahedra
+                re_process(S, lane, since_flush);   // the previous pair's sub-tetrahedra
             }
             const int n = pr / NB, m = pr - (pr / NB) * NB;
-            bool plus = ((an >> n) & 1u) && ((cp >> m) & 1u);
-            bool minus = ((ap >> n) & 1u) && ((cn >> m) & 1u);
+            const bool plus = above && ((an >> n) & 1u) && ((cp >> m) & 1u);
+            const bool minus = below && ((ap >> n) & 1u) && ((cn >> m) & 1u);
             if (!plus && !minus) continue;
+            float d[4];
+#pragma unroll
+            for (int v = 0; v < 4; ++v) d[v] = c[v][m] - a[v][n];
             if constexpr (KIND == kKindS) {
-                const float d0 = c[0][m] - a[0][n], d1 = c[1][m] - a[1][n];
-                const float d2 = c[2][m] - a[2][n], d3 = c[3][m] - a[3][n];
-                const float dlo = fminf(fminf(d0, d1), fminf(d2, d3)), dhi = fmaxf(fmaxf(d0, d1), fmaxf(d2, d3));
+                const float dlo = fminf(fminf(d[0], d[1]), fminf(d[2], d[3]));
+                const float dhi = fmaxf(fmaxf(d[0], d[1]), fmaxf(d[2], d[3]));
                 if (dhi < om_lo || dlo > om_hi) continue;
-                plus = plus && om_hi > 0.f;
-                minus = minus && om_lo < 0.f;
-                if (!plus && !minus) continue;
+            }
+            const uint32_t key = ((uint32_t)it * (uint32_t)(NB * NB) + (uint32_t)(n * NB + m)) * 2u;
+            // band n occupied and band m empty at every corner (or the converse):
+            // the region is the whole tetrahedron, with the dither key that the two
+            // cuts would produce
+            if (((a_all >> n) & 1u) && ((c_all >> m) & 1u)) {
+                keep<KIND>(d, scale, key * 16u, S);
+                continue;
+            }
+            if (((a_none >> n) & 1u) && ((c_none >> m) & 1u)) {
+                keep<KIND>(d, -scale, (key + 1u) * 16u, S);
+                continue;
             }
             const P5 v0{1.f, 0.f, 0.f, a[0][n], c[0][m]};
             const P5 v1{0.f, 1.f, 0.f, a[1][n], c[1][m]};
             const P5 v2{0.f, 0.f, 1.f, a[2][n], c[2][m]};
             const P5 v3{0.f, 0.f, 0.f, a[3][n], c[3][m]};
-            const uint32_t key = ((uint32_t)it * (uint32_t)(NB * NB) + (uint32_t)(n * NB + m)) * 2u;
-            // band n occupied and band m empty at every corner: the +1
-            // region is the whole tetrahedron (the same sub-tetrahedron and
-            // dither key the two cuts would produce)
-            if (((a_all >> n) & 1u) && ((c_all >> m) & 1u)) {
-                accumulate<KIND>(v0, v1, v2, v3, 1.f, key * 16u, S);
-                continue;
-            }
             // +1 on {a < 0, c > 0}; -1 on {a > 0, c < 0}
             if (plus) region<KIND>(v0, v1, v2, v3, 0, 3, 1.f, key, S);
             if (minus) region<KIND>(v0, v1, v2, v3, 1, 2, -1.f, key + 1u, S);
@@ -838,7 +967,7 @@ __global__ void __launch_bounds__(kSpecThreads, KIND == kKindS ? kSpecBlocksPerS
     if constexpr (KIND == kKindS) {
         drain(S, lane);
     } else {
-        re_process(S, wr, wn, lane, since_flush);
+        re_process(S, lane, since_flush);
         re_flush(S, lane);
     }
     // one accumulator for all CTAs (integer atomics: exact in any order), scaled
@@ -856,8 +985,7 @@ __global__ void __launch_bounds__(kSpecThreads, KIND == kKindS ? kSpecBlocksPerS
     __syncthreads();
     if (!s_last) return;
     __threadfence();
-    const double unit = vtvg / de * ldexp(1.0, -bits);
-    for (int i = threadIdx.x; i < n_om; i += blockDim.x) out[i] = (float)((double)__ldcg(sums + i) * unit);
+    for (int i = threadIdx.x; i < n_om; i += blockDim.x) out[i] = scale_units(__ldcg(sums + i), s_grid[2], s_grid[3]);
 }
 
 // persistent blocks, as many as fit an SM at the register bound
