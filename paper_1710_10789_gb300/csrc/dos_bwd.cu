@@ -7,7 +7,7 @@
 //   L = sum_{T,n} sum_l sum_s b_{l,s} sum_e D_{e,s} w_l(e),
 // where edges at or below a tetrahedron's E1 give nothing and those at or
 // above E4 telescope to f G_{j-1,s} (w_l = f = V_T/(4 V_G) there; e_j the first
-// of them). So only the edges inside (E1, E4) cost work, a few or none:
+// of them; so do edges inside with w_l - f in the sum instead of w_l). So only the edges inside (E1, E4) cost work, a few or none:
 //   dL/db_{l,s} = f G_{j-1,s} + sum_e w_l(e) D_{e,s},
 //   dL/de_r     = - sum_e sum_l M_rl(e) k_l(e),  k_l(e) = sum_s b_{l,s} D_{e,s},
 // with M_rl(E) = int lambda_r lambda_l delta(E - D) over the tetrahedron, since
@@ -36,20 +36,19 @@ namespace tetra {
 namespace {
 
 constexpr int kBwdThreads = 128;
-constexpr int kBwdBlocks = 3;   // per SM
+// blocks per SM (16 orbitals do not fit the registers of four)
+constexpr int bwd_blocks(int norb_t) { return norb_t <= 8 ? 4 : 3; }
 
-// Sorted corner energies, the reciprocals of their differences and
+// Sorted corner energies, the reciprocals of their differences,
 // V_T/(4 V_G) (f) and f / E41. A difference of zero gives an infinite
 // reciprocal, which the clamped products below turn into a step.
 struct TetB {
-    float e1, e2, e3;
+    float e1, e2, e3, e4;
     float r21, r31, r41, r32, r42, r43;
     float f, fr;
 };
 __device__ __forceinline__ void tetb_setup(TetB &T, const float e[4], float f) {
-    T.e1 = e[0]; T.e3 = e[2];
-    // E2 = E3 = E4: no edge below E4 may see f32 > 0, and at E4 it is 1
-    T.e2 = e[1] < e[3] ? e[1] : nextafterf(e[3], -INFINITY);
+    T.e1 = e[0]; T.e2 = e[1]; T.e3 = e[2]; T.e4 = e[3];
     T.r21 = __fdividef(1.f, e[1] - e[0]); T.r31 = __fdividef(1.f, e[2] - e[0]);
     T.r41 = __fdividef(1.f, e[3] - e[0]); T.r32 = __fdividef(1.f, e[2] - e[1]);
     T.r42 = __fdividef(1.f, e[3] - e[1]); T.r43 = __fdividef(1.f, e[3] - e[2]);
@@ -57,12 +56,22 @@ __device__ __forceinline__ void tetb_setup(TetB &T, const float e[4], float f) {
     T.fr = f * T.r41;
 }
 
-// At an edge E inside (E1, E4): the corner weights w and m = M k (both for the
-// sorted corners).
-__device__ __forceinline__ void edge_terms(const TetB &T, float E, const float (&k)[4], float (&w)[4], float (&m)[4]) {
-    const float x = E - T.e1, t = E - T.e2, y = E - T.e3;
-    const float f21 = __saturatef(x * T.r21), f31 = __saturatef(x * T.r31), f41 = __saturatef(x * T.r41);
-    const float f32 = __saturatef(t * T.r32), f42 = __saturatef(t * T.r42), f43 = __saturatef(y * T.r43);
+// At an edge E inside (E1, E4): w, the corner weights, or from the middle of
+// the tetrahedron's range on the corner weights minus f, and m = M k (both for
+// the sorted corners). The upper half is the lower half of the mirrored
+// tetrahedron (energies -E4 <= -E3 <= -E2 <= -E1 at -E, w - f of it the
+// negative weights in reverse order), so w is small and accurate towards
+// either end: the sums over many edges cancel.
+__device__ __forceinline__ void edge_terms(const TetB &T, float E, bool mir, const float (&kk)[4], float (&ww)[4],
+                                           float (&mm)[4]) {
+    const float x = mir ? T.e4 - E : E - T.e1, t = mir ? T.e3 - E : E - T.e2, y = mir ? T.e2 - E : E - T.e3;
+    const float r21 = mir ? T.r43 : T.r21, r31 = mir ? T.r42 : T.r31, r42 = mir ? T.r31 : T.r42,
+                r43 = mir ? T.r21 : T.r43;
+    float k[4], w[4], m[4];
+#pragma unroll
+    for (int l = 0; l < 4; ++l) k[l] = mir ? kk[3 - l] : kk[l];
+    const float f21 = __saturatef(x * r21), f31 = __saturatef(x * r31), f41 = __saturatef(x * T.r41);
+    const float f32 = __saturatef(t * T.r32), f42 = __saturatef(t * r42), f43 = __saturatef(y * r43);
     const float f12 = 1.f - f21, f13 = 1.f - f31, f14 = 1.f - f41, f23 = 1.f - f32, f24 = 1.f - f42;
     // volume below E: four simplices (forward kernel, tet_w)
     const float fa = T.f * f41, fb = T.f * f14;
@@ -87,6 +96,11 @@ __device__ __forceinline__ void edge_terms(const TetB &T, float E, const float (
     m[1] = fmaf(p, tx, fmaf(f24, t24, f23 * ty));
     m[2] = fmaf(f31, t13, fmaf(f32, tx, q * ty));
     m[3] = fmaf(f41, t14, fmaf(f42, t24, f43 * ty));
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+        ww[l] = mir ? -w[3 - l] : w[l];
+        mm[l] = mir ? m[3 - l] : m[l];
+    }
 }
 
 // Table I corner labels minus one.
@@ -122,7 +136,7 @@ inline size_t bwd_stage_bytes(int norb_t, int n_bins) {
 inline size_t bwd_scratch_bytes(int n_orb) { return sizeof(float) * (1 + (size_t)n_orb) * 8 * kBwdThreads; }
 
 template <int NORB, typename WT>
-__global__ void __launch_bounds__(kBwdThreads, kBwdBlocks) tetra_dos_bwd_kernel(const BwdArgs A, int px, int py, int pz) {
+__global__ void __launch_bounds__(kBwdThreads, bwd_blocks(NORB)) tetra_dos_bwd_kernel(const BwdArgs A, int px, int py, int pz) {
     extern __shared__ __align__(16) float s_mem[];
     const int n_e = A.n_bins + 1;
     const int ed_words = (n_e + 3) & ~3;
@@ -208,16 +222,11 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdBlocks) tetra_dos_bwd_kernel(
             if (hi == 0 || lo == n_e) continue;
             float acc_e[4] = {0.f, 0.f, 0.f, 0.f};
             float acc_w[4][NORB];
-            {
-                float g[NORB];   // f G_{hi-1}: the edges at or above E4
 #pragma unroll
-                for (int s = 0; s < NORB; ++s) g[s] = 0.f;
-                if (hi < n_e) row(false, hi, g);
+            for (int r = 0; r < 4; ++r)
 #pragma unroll
-                for (int s = 0; s < NORB; ++s)
-#pragma unroll
-                    for (int r = 0; r < 4; ++r) acc_w[r][s] = A.f * g[s];
-            }
+                for (int s = 0; s < NORB; ++s) acc_w[r][s] = 0.f;
+            int full = hi;   // first edge that counts as full (w - f instead of w)
             if (lo < hi) {
                 float b[4][NORB];
 #pragma unroll
@@ -225,6 +234,7 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdBlocks) tetra_dos_bwd_kernel(
                     load_weights<NORB, WT>(W + (long)pt[slot[r]] * A.w_stride + (long)n * A.n_orb, A.n_orb, b[r]);
                 TetB T;
                 tetb_setup(T, e, A.f);
+                const float mid = 0.5f * (e[0] + e[3]);
                 for (int i = lo; i < hi; ++i) {
                     float g[NORB], k[4] = {0.f, 0.f, 0.f, 0.f}, w[4], m[4];
                     row(true, i, g);
@@ -232,7 +242,9 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdBlocks) tetra_dos_bwd_kernel(
                     for (int s = 0; s < NORB; ++s)
 #pragma unroll
                         for (int l = 0; l < 4; ++l) k[l] = fmaf(g[s], b[l][s], k[l]);
-                    edge_terms(T, ed[i], k, w, m);
+                    const bool mir = ed[i] >= mid;
+                    if (mir) full = min(full, i);
+                    edge_terms(T, ed[i], mir, k, w, m);
 #pragma unroll
                     for (int l = 0; l < 4; ++l) {
                         acc_e[l] -= m[l];
@@ -240,6 +252,16 @@ __global__ void __launch_bounds__(kBwdThreads, kBwdBlocks) tetra_dos_bwd_kernel(
                         for (int s = 0; s < NORB; ++s) acc_w[l][s] = fmaf(g[s], w[l], acc_w[l][s]);
                     }
                 }
+            }
+            // the edges that count as full: their D telescope to G below the first
+            // (0 below the first edge of all, 0 if there is none)
+            if (full > 0 && full < n_e) {
+                float g[NORB];
+                row(false, full, g);
+#pragma unroll
+                for (int r = 0; r < 4; ++r)
+#pragma unroll
+                    for (int s = 0; s < NORB; ++s) acc_w[r][s] = fmaf(A.f, g[s], acc_w[r][s]);
             }
             // add the sorted corners' sums to the cube-corner accumulators
 #pragma unroll
@@ -329,7 +351,7 @@ cudaError_t launch_bwd_n(const Plan &P, const BwdArgs &A, cudaStream_t stream) {
             const long total = cubes * A.nb;
             if (total == 0) continue;
             // as many blocks as run at once: each stages the bin tables once
-            const int grid = (int)std::min<long>((total + kBwdThreads - 1) / kBwdThreads, (long)kBwdBlocks * P.sm_count);
+            const int grid = (int)std::min<long>((total + kBwdThreads - 1) / kBwdThreads, (long)bwd_blocks(NORB) * P.sm_count);
             kfn<<<grid, kBwdThreads, smem, stream>>>(A, px, py, pz);
             e = cudaGetLastError();
             if (e != cudaSuccess) return e;

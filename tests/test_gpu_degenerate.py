@@ -16,7 +16,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("n_orb", [1, 8, 16])
+@pytest.mark.parametrize("n_orb", [1, 3, 5, 6, 8, 16])
 @pytest.mark.parametrize("mode", ["point", "bin", "integrated"])
 def test_coinciding_corner_energies(mode, n_orb):
     import paper_1710_10789_gb300 as T
