@@ -36,8 +36,8 @@ namespace {
 
 constexpr int kPts = 16;           // energies per round: bracket / 16
 constexpr int kPer = 4;            // energies per task
-constexpr int kRounds = 64;        // at most; FP32 resolution takes about six
-constexpr int kRoundsPerSync = 7;
+constexpr int kRounds = 64;        // at most; FP32 resolution takes about five
+constexpr int kRoundsPerSync = 6;
 constexpr int kFermiThreads = 256;
 constexpr int kFermiBlocks = 3;    // per SM
 constexpr int kUnitBits = 26;
@@ -55,7 +55,8 @@ __device__ __forceinline__ float unordered(unsigned u) {
 struct FermiState {
     unsigned mm[2];            // complemented minimum, maximum of the bands (ordered; both from 0 up)
     float lo, hi;              // bracket
-    long long base;            // N(lo) in units
+    long long base, top;       // N(lo), N(hi) in units
+    int guess;                 // whether the round's energies cluster about the interpolated level
     int round, done, bad;      // bad: no such count, or no valid band energy
     int ticket;
     unsigned long long sums[kPts];   // N(E_j) - N(lo) of the running round
@@ -100,9 +101,20 @@ struct FermiArgs {
     FermiState *S;
 };
 
-// Energy j of a round's grid, ascending to hi.
-__device__ __forceinline__ float grid_energy(float lo, float hi, int j) {
-    return j == kPts - 1 ? hi : lo + (hi - lo) * ((float)(j + 1) * (1.0f / kPts));
+// Energy j of a round, ascending to hi: equidistant, or about the level that
+// the line through N(lo) and N(hi) gives, at distances shrinking to 2^-16 of
+// the bracket. N is smooth on the scale of a small bracket, so the crossing
+// lies close to that level and a round narrows the bracket by far more than
+// 16 (three rounds less in eight at 95 x 97 x 96); a round that narrows it by
+// less than 8 is followed by an equidistant one.
+__device__ __forceinline__ float round_energy(float lo, float hi, bool guess, float level, int j) {
+    if (j == kPts - 1) return hi;
+    const float h = hi - lo;
+    if (!guess) return lo + h * ((float)(j + 1) * (1.0f / kPts));
+    constexpr int kMid = kPts / 2 - 1;
+    const int k = j < kMid ? kMid - j : j - kMid;   // distance from the middle: 1 nearest
+    const float d = k == 0 ? 0.f : h * exp2f(-16.f + 2.25f * (float)(k - 1));
+    return fminf(fmaxf(j < kMid ? level - d : level + d, lo), hi);
 }
 
 // Sum of n_orb weights, 16 bytes at a time where they fill whole vectors (the
@@ -148,7 +160,14 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
     }
     if (tid < kPts) {
         s_sum[tid] = 0ull;
-        s_om[tid] = grid_energy(lo, hi, tid);
+        const bool guess = !first && S->guess;
+        float level = lo;
+        if (guess) {   // (one thread group; FP64 is slow but this is a few operations)
+            const double below = (double)S->base, above = (double)S->top;
+            const double n = A.n_electrons / (A.vtvg * ldexp(1.0, -kUnitBits));
+            level = lo + (hi - lo) * (float)((n - below) / (above - below));
+        }
+        s_om[tid] = round_energy(lo, hi, guess, level, tid);
     }
     // tile points (x, row) at 32 row + x, band by band: a warp reads and
     // writes consecutive words
@@ -335,6 +354,8 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
     while (j < kPts - 1 && (double)N[j] * unit < A.n_electrons) ++j;
     const float nlo = j == 0 ? lo : s_om[j - 1], nhi = s_om[j];
     S->base = j == 0 ? base : N[j - 1];
+    S->top = N[j];
+    S->guess = (nhi - nlo) * 8.f <= hi - lo && S->top > S->base;
     S->lo = nlo;
     S->hi = nhi;
     // FP32 resolution reached: the bracket no longer shrinks
