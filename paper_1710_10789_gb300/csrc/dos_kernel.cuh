@@ -300,6 +300,8 @@ __global__ void __maxnreg__(kMaxRegs)
     // them or, for odd NORB, in an array after the rows: the odd row length
     // spreads consecutive rows over the shared-memory banks
     constexpr int TS = NORB | 1;
+    // one orbital, point and bin mode: items of zero weight dropped before the ranking
+    constexpr bool kFilter = NORB == 1 && MODE != TETRA_INTEGRATED;
     auto count_of = [&](int *t, int row) -> int & {
         return (NORB & 1) ? t[TS * (A.chunk_w + 1) + row] : t[row * TS + NORB];
     };
@@ -652,10 +654,35 @@ __global__ void __maxnreg__(kMaxRegs)
                         if (act && K > 0) atomicAdd(&khist[min(K, kKBins - 1)], 1);
                         if (zm && lane == __ffs(zm) - 1) atomicAdd(&khist[0], __popc(zm));
                     } else {
-                        if (act) atomicAdd(&khist[min(K, kKBins - 1)], 1);
+                        if (!kFilter && act) atomicAdd(&khist[min(K, kKBins - 1)], 1);
                     }
                 }
             }
+        }
+        if constexpr (kFilter) {
+            // The box's weights, waited for here instead of before pass B: items
+            // whose weights are all zero are dropped (every contribution rounds
+            // to zero, the dither being at most 1/2) before the ranking counts
+            // the others, so that the warps stay full. Two thirds of a
+            // susceptibility's transition bands have both ends occupied or both
+            // empty.
+            if (mbar_wait_bounded(&mbar[2], k & 1, A.status))
+                for (int it = tid; it < A.items_per_box; it += blockDim.x) {
+                    const int K = s_K[it];
+                    if (K == 0) continue;
+                    const int cube = it & (ncube - 1), rest = it >> lcube;
+                    const int cx = cube & (A.BX - 1), cy = (cube >> A.lbx) & (A.BY - 1), cz = cube >> (A.lbx + A.lby);
+                    const int n = rest / 3, p0 = cx + PX * (cy + PY * cz);
+                    const uint32_t code = pair_code(rest - 3 * n);
+                    bool any = false;
+#pragma unroll
+                    for (int q = 0; q < 5; ++q) {
+                        const int p = p0 + s_cdelta[(code >> (3 * q)) & 7];
+                        any = any || to_f32<WT>(Ws[(long)p * A.w_stride + n]) != 0.f;
+                    }
+                    if (any) atomicAdd(&khist[min(K, kKBins - 1)], 1);
+                    else s_K[it] = 0;
+                }
         }
         __syncthreads();
         // Items ranked by window length K: an exclusive scan of the K histogram
@@ -802,15 +829,6 @@ __global__ void __maxnreg__(kMaxRegs)
                     for (int q = 1; q < ROWS; ++q) acc = fmaf(bw[q][s], d[q], acc);
                     return acc;
                 };
-                if constexpr (NORB == 1) {
-                    // all weights zero: every contribution rounds to zero (the dither
-                    // is at most 1/2). Two thirds of a susceptibility's transition
-                    // bands have both ends occupied or both empty.
-                    float any = 0.f;
-#pragma unroll
-                    for (int q = 0; q < ROWS; ++q) any = fmaxf(any, fabsf(bw[q][0]));
-                    if (MODE != TETRA_INTEGRATED && any == 0.f) continue;
-                }
                 const float dith = item_dither((gcube * 3u + (uint32_t)pr) * (uint32_t)A.nb + (uint32_t)n);
                 if constexpr (MODE == TETRA_INTEGRATED) {
                     // Occupation: the walk over the union window adds both
