@@ -131,9 +131,9 @@ inline size_t bwd_stage_bytes(int norb_t, int n_bins) {
     return b <= 64 * 1024 ? b : 0;
 }
 
-// Thread-private corner accumulators: (1 + n_orb) values for each of the
-// cube's 8 corners, interleaved over the block's threads.
-inline size_t bwd_scratch_bytes(int n_orb) { return sizeof(float) * (1 + (size_t)n_orb) * 8 * kBwdThreads; }
+// Thread-private corner accumulators and energies: (1 + n_orb) and one value
+// for each of the cube's 8 corners, interleaved over the block's threads.
+inline size_t bwd_scratch_bytes(int n_orb) { return sizeof(float) * (2 + (size_t)n_orb) * 8 * kBwdThreads; }
 
 template <int NORB, typename WT>
 __global__ void __launch_bounds__(kBwdThreads, bwd_blocks(NORB)) tetra_dos_bwd_kernel(const BwdArgs A, int px, int py, int pz) {
@@ -142,6 +142,7 @@ __global__ void __launch_bounds__(kBwdThreads, bwd_blocks(NORB)) tetra_dos_bwd_k
     const int ed_words = (n_e + 3) & ~3;
     const size_t stage = A.staged ? (size_t)ed_words + 2 * (size_t)NORB * n_e : 0;
     float *scr = s_mem + stage;   // [(1 + n_orb) * 8][blockDim]
+    float *sce = scr + (1 + A.n_orb) * 8 * blockDim.x;   // corner energies, [8][blockDim]
     // G_{e-1,s}, from the gradient (0 beyond either end)
     auto g_below = [&](int e, int s) -> float {
         return e > 0 ? A.grad_dos[(long)s * A.n_bins + e - 1] / (A.edges[e] - A.edges[e - 1]) : 0.f;
@@ -188,14 +189,26 @@ __global__ void __launch_bounds__(kBwdThreads, bwd_blocks(NORB)) tetra_dos_bwd_k
         const int x = px + 2 * (int)(cube % cxn), y = py + 2 * (int)((cube / cxn) % cyn),
                   z = pz + 2 * (int)(cube / ((long)cxn * cyn));
         for (int v = 0; v < nv * 8; ++v) scr[v * nt + tid] = 0.f;
+        // the cube's corner energies, read together (the loads overlap)
+        const long p0 = x + (long)A.nx * (y + (long)A.ny * z);
+        const int sy = A.nx, sz = A.nx * A.ny;
+        {
+            float e8[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+                e8[c] = A.eps[(p0 + (c & 1) + ((c >> 1) & 1) * sy + (long)(c >> 2) * sz) * A.eps_stride + n];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) sce[c * nt + tid] = e8[c];
+        }
         for (int t = 0; t < 6; ++t) {
             float e[4];
-            int pt[4], slot[4];
+            long pt[4];
+            int slot[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int cc = c_tab[t][q];
-                pt[q] = (x + (cc & 1)) + A.nx * ((y + ((cc >> 1) & 1)) + A.ny * (z + ((cc >> 2) & 1)));
-                e[q] = A.eps[(long)pt[q] * A.eps_stride + n];
+                pt[q] = p0 + (cc & 1) + ((cc >> 1) & 1) * sy + (long)(cc >> 2) * sz;
+                e[q] = sce[cc * nt + tid];
                 slot[q] = q;
             }
             // sort corners by energy, carrying their Table-I slot (stable for ties)
@@ -231,7 +244,7 @@ __global__ void __launch_bounds__(kBwdThreads, bwd_blocks(NORB)) tetra_dos_bwd_k
                 float b[4][NORB];
 #pragma unroll
                 for (int r = 0; r < 4; ++r)
-                    load_weights<NORB, WT>(W + (long)pt[slot[r]] * A.w_stride + (long)n * A.n_orb, A.n_orb, b[r]);
+                    load_weights<NORB, WT>(W + pt[slot[r]] * A.w_stride + (long)n * A.n_orb, A.n_orb, b[r]);
                 TetB T;
                 tetb_setup(T, e, A.f);
                 const float mid = 0.5f * (e[0] + e[3]);
@@ -273,24 +286,43 @@ __global__ void __launch_bounds__(kBwdThreads, bwd_blocks(NORB)) tetra_dos_bwd_k
                     if (s < A.n_orb) scr[((1 + s) * 8 + c) * nt + tid] += acc_w[r][s];
             }
         }
-        // this class's cubes share no point: plain read-modify-write
-        for (int c = 0; c < 8; ++c) {
-            const long p = (x + (c & 1)) + (long)A.nx * ((y + ((c >> 1) & 1)) + (long)A.ny * (z + (c >> 2)));
-            A.geps[p * A.eps_stride + n] += scr[(0 * 8 + c) * nt + tid];
-            float *gwp = A.gw + p * A.w_stride + (long)n * A.n_orb;
-            if (NORB % 4 == 0 && A.vec && A.n_orb == NORB) {
+        // this class's cubes share no point: plain read-modify-write, the loads
+        // of four corners together
+#pragma unroll 1
+        for (int h = 0; h < 8; h += 4) {
+            float ge[4];
+            float4 g4[4][NORB / 4 > 0 ? NORB / 4 : 1];
+            const bool whole = NORB % 4 == 0 && A.vec && A.n_orb == NORB;
+            long p[4];
 #pragma unroll
-                for (int v = 0; v < NORB / 4; ++v) {
-                    float4 *g4 = reinterpret_cast<float4 *>(gwp) + v;
-                    float4 g = *g4;
-                    g.x += scr[((1 + 4 * v) * 8 + c) * nt + tid];
-                    g.y += scr[((2 + 4 * v) * 8 + c) * nt + tid];
-                    g.z += scr[((3 + 4 * v) * 8 + c) * nt + tid];
-                    g.w += scr[((4 + 4 * v) * 8 + c) * nt + tid];
-                    *g4 = g;
+            for (int i = 0; i < 4; ++i) {
+                const int c = h + i;
+                p[i] = p0 + (c & 1) + ((c >> 1) & 1) * sy + (long)(c >> 2) * sz;
+                ge[i] = A.geps[p[i] * A.eps_stride + n];
+                if (whole) {
+#pragma unroll
+                    for (int v = 0; v < NORB / 4; ++v)
+                        g4[i][v] = reinterpret_cast<const float4 *>(A.gw + p[i] * A.w_stride + (long)n * A.n_orb)[v];
                 }
-            } else {
-                for (int s = 0; s < A.n_orb; ++s) gwp[s] += scr[((1 + s) * 8 + c) * nt + tid];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int c = h + i;
+                A.geps[p[i] * A.eps_stride + n] = ge[i] + scr[(0 * 8 + c) * nt + tid];
+                float *gwp = A.gw + p[i] * A.w_stride + (long)n * A.n_orb;
+                if (whole) {
+#pragma unroll
+                    for (int v = 0; v < NORB / 4; ++v) {
+                        float4 g = g4[i][v];
+                        g.x += scr[((1 + 4 * v) * 8 + c) * nt + tid];
+                        g.y += scr[((2 + 4 * v) * 8 + c) * nt + tid];
+                        g.z += scr[((3 + 4 * v) * 8 + c) * nt + tid];
+                        g.w += scr[((4 + 4 * v) * 8 + c) * nt + tid];
+                        reinterpret_cast<float4 *>(gwp)[v] = g;
+                    }
+                } else {
+                    for (int s = 0; s < A.n_orb; ++s) gwp[s] += scr[((1 + s) * 8 + c) * nt + tid];
+                }
             }
         }
     }
