@@ -117,14 +117,12 @@ struct ReSeg {
 
 // Set-up of one entry as the warp's lanes read it (32 words): mean c,
 // amplitude, (2 R)^2, moments mu_2..mu_kReMom (mu_0 = 1, and mu_1 vanishes
-// about the mean), its group's centre and (twice the half-width)^2, and the
-// density pieces: corner values, reciprocal lengths (0 for an empty one),
+// about the mean), and the density pieces: corner values, reciprocal lengths (0 for an empty one),
 // g(d1), g(d2) and the middle piece's value at its centre.
 struct __align__(16) ReStage {
     float c, amp, far2;
     float mu[kReMom - 1];
-    float gc, gfar2;
-    float d[4], r[3], G1, G2, A2, pad[2];
+    float d[4], r[3], G1, G2, A2, pad[4];
 };
 static_assert(sizeof(ReStage) == 128, "32 words");
 
@@ -593,7 +591,7 @@ __device__ __forceinline__ void re_process(const SpecArgs &S, int lane, int &sin
             hi = fmaxf(hi, __shfl_xor_sync(kAll, hi, d));
         }
     }
-    const int start = incl - mine, total = __shfl_sync(kAll, incl, 31);
+    const int start = incl - mine;
     // joint moments about the group's centre in units of its half-width, of
     // this lane's entries first
     const bool some = hi >= lo;
@@ -622,22 +620,18 @@ __device__ __forceinline__ void re_process(const SpecArgs &S, int lane, int &sin
             M[i] = keep + __shfl_xor_sync(kAll, send, mask);
         }
     }
-    float *joint = reinterpret_cast<float *>(stage);   // [group][kM]
-    {
-        const int first = 12 * ((lane >> 2) & 1) + 6 * ((lane >> 1) & 1) + 3 * (lane & 1);
-#pragma unroll
-        for (int i = 0; i < 3; ++i) joint[(lane / kReGroup) * kM + first + i] = M[i];
-    }
-    __syncwarp();
-    bool near_any = false;
 #pragma unroll 1
     for (int g = 0; g < 32 / kReGroup; ++g) {
-        const float gC = __shfl_sync(kAll, C, g * kReGroup), grho = __shfl_sync(kAll, rho, g * kReGroup);
-        if (!__shfl_sync(kAll, (int)some, g * kReGroup)) continue;
+        const int g0 = g * kReGroup;
+        if (!__shfl_sync(kAll, (int)some, g0)) continue;
+        const float gC = __shfl_sync(kAll, C, g0), grho = __shfl_sync(kAll, rho, g0);
+        // the group's moments: n in M[n % 3] of the lane that the exchange left it in
         float m[kReCluster + 1];
 #pragma unroll
-        for (int n = 0; n <= kReCluster; ++n) m[n] = joint[g * kM + n];
+        for (int n = 0; n <= kReCluster; ++n)
+            m[n] = __shfl_sync(kAll, M[n % 3], g0 + 4 * (n / 12) + 2 * ((n % 12) / 6) + (n % 6) / 3);
         const float far2 = 4.f * grho * grho;
+        bool near_any = false;
         for (int c0 = 0; c0 < n_om; c0 += 128) {
             float z[4], v[4], r[4];
             float umin = INFINITY;
@@ -662,42 +656,35 @@ __device__ __forceinline__ void re_process(const SpecArgs &S, int lane, int &sin
             for (int k = 0; k < 4; ++k)
                 if (far[k]) racc[c0 + lane + 32 * k] += r[k] * v[k];
         }
-    }
-    if (__any_sync(kAll, near_any)) {
-        for (int base = 0; base < total; base += kReBatch) {
-            const int n_here = min(kReBatch, total - base);
-            // entry's place: the last lane whose segment starts at or before it
+        if (!__any_sync(kAll, near_any)) continue;
+        // the group's entries one by one at the nearer energies, 16 set up at a
+        // time, in lane order
+        const int first = __shfl_sync(kAll, start, g0), last = __shfl_sync(kAll, incl, g0 + kReGroup - 1);
+        for (int base = first; base < last; base += kReBatch) {
+            const int n_here = min(kReBatch, last - base);
+            // entry's place: the group's last lane whose segment starts at or before it
             const int e = base + (lane & (kReBatch - 1));
-            int src = 0;
+            int src = g0;
 #pragma unroll
-            for (int step = 16; step >= 1; step >>= 1) {
-                const int cand = src + step;
-                if (__shfl_sync(kAll, start, cand) <= e) src = cand;
-            }
+            for (int step = kReGroup / 2; step >= 1; step >>= 1)
+                if (__shfl_sync(kAll, start, src + step) <= e) src += step;
             const int loc = src * kSubPerPair + (e - __shfl_sync(kAll, start, src));
-            const float gC = __shfl_sync(kAll, C, src), grho = __shfl_sync(kAll, rho, src);
-            __syncwarp();   // the joint moments, the last batch are read
-            if (lane < n_here) {
-                re_setup(wq[loc], stage[lane]);
-                stage[lane].gc = gC;
-                stage[lane].gfar2 = 4.f * grho * grho;
-            }
+            __syncwarp();   // the last batch is read
+            if (lane < n_here) re_setup(wq[loc], stage[lane]);
             __syncwarp();
             for (int c0 = 0; c0 < n_om; c0 += 64) {
                 float w[2], sum[2] = {0.f, 0.f};
-                bool touched = false;
+                bool near[2];
 #pragma unroll
-                for (int k = 0; k < 2; ++k) w[k] = om[min(c0 + lane + 32 * k, n_om - 1)];
+                for (int k = 0; k < 2; ++k) {
+                    const int i = c0 + lane + 32 * k;
+                    w[k] = om[min(i, n_om - 1)];
+                    const float u = w[k] - gC;
+                    near[k] = i < n_om && !(u * u > far2);
+                }
+                if (!__any_sync(kAll, near[0] || near[1])) continue;
                 for (int j = 0; j < n_here; ++j) {
                     const ReStage &st = stage[j];
-                    bool near[2];
-#pragma unroll
-                    for (int k = 0; k < 2; ++k) {
-                        const float u = w[k] - st.gc;
-                        near[k] = c0 + lane + 32 * k < n_om && !(u * u > st.gfar2);
-                    }
-                    if (!__any_sync(kAll, near[0] || near[1])) continue;
-                    touched = true;
                     float v[2], r[2] = {0.f, 0.f}, umin = INFINITY;
                     bool own[2];   // by its own series
                     bool pieces = false;
@@ -727,14 +714,11 @@ __device__ __forceinline__ void re_process(const SpecArgs &S, int lane, int &sin
                             if (near[k] && !own[k]) r[k] = re_near(st, w[k]);
                     }
 #pragma unroll
-                    for (int k = 0; k < 2; ++k)
-                        if (near[k]) sum[k] = fmaf(st.amp, r[k], sum[k]);
+                    for (int k = 0; k < 2; ++k) sum[k] = fmaf(st.amp, r[k], sum[k]);
                 }
-                if (touched) {
 #pragma unroll
-                    for (int k = 0; k < 2; ++k)
-                        if (c0 + lane + 32 * k < n_om) racc[c0 + lane + 32 * k] += sum[k];
-                }
+                for (int k = 0; k < 2; ++k)
+                    if (near[k]) racc[c0 + lane + 32 * k] += sum[k];
             }
         }
     }
