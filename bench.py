@@ -43,12 +43,11 @@ OPS_PER_ITEM = 40
 # capture of the 128^3, 4000-energy, FP32, point-mode launch, scaled by the
 # number of boxes to other cubic grids (the traffic is per box: halo reads of
 # the TMA boxes). Valid only for the kernel source it was taken from: first 16
-# hex digits of the SHA-256 of csrc/dos.cu up to the reduce kernels (the
-# forward kernel and every device function it calls); otherwise the bench
+# hex digits of the SHA-256 of csrc/dos_kernel.cuh and csrc/tet_common.cuh (the
+# forward kernel and the device functions it calls); otherwise the bench
 # reports null.
 DOS_TRAFFIC_CAPTURE = {"dos_fwd_sha256": "3ddeea97f2fb5a4a", "grid": 128, "n_omega": 4000,
                        "bytes": 691929856 + 4707840}
-DOS_FWD_END = b"// Single model: dos[s][w0+j] = u * sum over CTAs of the int64 partials (exact)."
 
 
 def parse():
@@ -178,10 +177,10 @@ def dos_traffic(n, n_omega, mode, weight_dtype):
     when the capture does not describe this kernel source or configuration."""
     import hashlib
     c = DOS_TRAFFIC_CAPTURE
-    src = os.path.join(ROOT, "paper_1710_10789_gb300", "csrc", "dos.cu")
-    text = open(src, "rb").read()
-    end = text.find(DOS_FWD_END)
-    sha = hashlib.sha256(text[:end]).hexdigest()[:16] if end > 0 else None
+    h = hashlib.sha256()
+    for name in ("dos_kernel.cuh", "tet_common.cuh"):
+        h.update(open(os.path.join(ROOT, "paper_1710_10789_gb300", "csrc", name), "rb").read())
+    sha = h.hexdigest()[:16]
     if sha != c["dos_fwd_sha256"] or n_omega != c["n_omega"] or mode != "point" or weight_dtype != "f32":
         return None
     return c["bytes"] * (n / c["grid"]) ** 3
@@ -993,7 +992,7 @@ def main():
         "dense_updates_per_s_dos_only": dense / (dos_ms * 1e-3),
         "in_window_triples": triples,
         "roofline": roof, "eig_roofline": eig_roof, "cpu_baseline": cb, "e2e": e2e, "clocks": clocks, "variants": variants,
-        "gpu_launches": 3 * args.steps,
+        "gpu_launches": 2 * args.steps,   # eigensolver, DOS
     }
     print(json.dumps(line), flush=True)
 
