@@ -30,7 +30,10 @@ __global__ void tetra_dos_reduce_batched(const __grid_constant__ Batch<kMaxBatch
                                          const long long *G, int n_orb, int chunk_w, int mode) {
     const ModelP &M = B.m[blockIdx.y];
     __shared__ float s_unit[2];
-    if (threadIdx.x == 0) unit_pair(fixed_unit(M.omega, M.n_omega, mode, M.vtvg, M.fixed_bits), s_unit[0], s_unit[1]);
+    if (threadIdx.x == 0) {
+        float fq;
+        unit_pair(fixed_unit(M.omega, M.n_omega, mode, M.vtvg, M.fixed_bits, fq), s_unit[0], s_unit[1]);
+    }
     __syncthreads();
     const float uh = s_unit[0], ul = s_unit[1];
     const long total = (long)n_orb * M.n_omega;

@@ -13,11 +13,11 @@
 //    order), so the work stays balanced whatever the models' costs; when the
 //    model changes the CTA flushes its tile into that model's int64
 //    accumulator with integer atomics and reloads the energy grid.
-//  * One thread handles one (tetrahedron, band) item: it reads the four corner
-//    energies, sorts them with a 5-comparator network carrying the corner
-//    positions (Sec. II.C sorts E1 <= E2 <= E3 <= E4), reads the orbital
-//    weights in sorted order, and visits only the energies strictly inside
-//    (E1, E4) (bins overlapping it in bin mode); all others get zero weight.
+//  * One thread handles one item: it reads the corner energies and orbital
+//    weights, sorts the energies (Sec. II.C sorts E1 <= E2 <= E3 <= E4), and
+//    visits only the energies strictly inside (E1, E4) (bins overlapping it in
+//    bin mode); all others get zero weight. With more than 8 orbitals the item
+//    is a (tetrahedron, band).
 //  * Up to 8 orbitals (every mode): the item is a pair of tetrahedra sharing
 //    a face (Table I's six form three such pairs). Their windows overlap
 //    heavily, so one walk over the union of the two windows adds both
@@ -71,9 +71,13 @@ constexpr uint32_t kSmemAlign = 1024;
 // and constants in registers; 16 orbitals would not fit, so there a unit is
 // one tetrahedron. Each of the SM's four sub-partitions has 16K registers for
 // its warps: 16 warps can use 128 registers per thread. (A pair with 8
-// orbitals fits them since its corner derivatives need ten constants per
-// tetrahedron; 64^3 points, 8 bands, 2000 energies: 1742 us with 12 warps of
-// 168 registers, 1670 us with 16; 256^3 and 4000 energies 45.8 and 43.8 ms.)
+// orbitals fits them with ten constants per tetrahedron and five weight rows;
+// 64^3 points, 8 bands, 2000 energies: 1742 us with 12 warps of 168 registers
+// against 1670 us with 16, 1477 us with the five rows and 1408 us with 20
+// warps of 96 registers; at 256^3 and 4000 energies, with the eigensolver,
+// those are 57.1, 55.0, 50.5 and 52.0 ms. At 64^3 the kernel issues in 75 % of
+// its cycles and uses 63 % of the shared-memory wavefronts: 3.5 of them for
+// each add of 32 lanes to unrelated rows.)
 constexpr int kThreads = 512;
 constexpr int kMaxRegs = 128;
 template <int NORB>
@@ -122,12 +126,15 @@ struct FwdArgs {
     float *dos;          // single model: the result, written by the CTA that finishes a chunk
 };
 
-// Fixed-point unit, identical in every kernel that uses it. The DOS modes
-// scale with the mean energy spacing (their values are per energy); the
-// integrated occupation is dimensionless, so its unit does not depend on the
-// grid (a narrow grid, as in a Fermi-level search, keeps full resolution).
+// Fixed-point unit, identical in every kernel that uses it, and fq, V_T/(4 V_G)
+// in units. The DOS modes scale with the mean energy spacing (their values are
+// per energy); the integrated occupation is dimensionless, so its unit does
+// not depend on the grid (a narrow grid, as in a Fermi-level search, keeps full
+// resolution). The unit is what makes fq exact: fq is the float that the
+// kernel multiplies with, and its rounding would shift every value by up to
+// 6e-8.
 __device__ __forceinline__ double fixed_unit(const float *omega, int n_omega, int mode, double vtvg,
-                                             int bits) {
+                                             int bits, float &fq) {
     double de;
     if (mode == TETRA_INTEGRATED)
         de = 1.0;
@@ -136,7 +143,8 @@ __device__ __forceinline__ double fixed_unit(const float *omega, int n_omega, in
     else
         de = ((double)omega[n_omega] - (double)omega[0]) / n_omega;
     if (!(de > 0.0)) de = 1.0;
-    return vtvg / de * ldexp(1.0, -bits);
+    fq = (float)(0.25 * ldexp(de, bits));
+    return 0.25 * vtvg / (double)fq;
 }
 
 // One rounded contribution added to the CTA's int64 partial (global 64-bit
@@ -546,9 +554,7 @@ __global__ void __maxnreg__(kMaxRegs)
             if (MODE == TETRA_BIN)
                 for (int i = tid; i < wc; i += blockDim.x) iw[i] = 1.0f / (om[i + 1] - om[i]);
             if (tid == 0) {
-                const double u = fixed_unit(M.omega, M.n_omega, MODE, M.vtvg, M.fixed_bits);
-                s_fq = (float)(0.25 * M.vtvg / u);   // V_T/(4 V_G) in fixed-point units
-                unit_pair(u, s_unit[0], s_unit[1]);
+                unit_pair(fixed_unit(M.omega, M.n_omega, MODE, M.vtvg, M.fixed_bits, s_fq), s_unit[0], s_unit[1]);
             }
             om0 = M.omega[0];
             const float omN = (MODE != TETRA_BIN) ? M.omega[M.n_omega - 1] : M.omega[M.n_omega];

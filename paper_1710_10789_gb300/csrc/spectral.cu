@@ -801,7 +801,8 @@ __global__ void __launch_bounds__(kSpecThreads, KIND == kKindS ? kSpecBlocksPerS
         const double de = mean_spacing(omega, n_om, mode);
         s_grid[0] = (float)ldexp(de, bits);
         s_grid[1] = (float)(1.0 / de);
-        unit_pair(vtvg / de * ldexp(1.0, -bits), s_grid[2], s_grid[3]);
+        // (the unit that makes the float the kernel multiplies with exact)
+        unit_pair(vtvg / (double)s_grid[0], s_grid[2], s_grid[3]);
     }
     for (int i = threadIdx.x; i < kSpecWarps * QC; i += blockDim.x) qcount[i] = 0;
     if constexpr (KIND == kKindRe)
