@@ -19,26 +19,32 @@
 // a tetrahedron (the total of Sec. II.C's corner weight derivatives divided
 // by V_T / V_G), or nu * [G(w_hi) - G(w_lo)] / (w_hi - w_lo) as a bin average.
 //
-// One thread per (cube, tetrahedron) runs over the band pairs in a loop that
-// is not unrolled (the unrolled 64-pair loop overflowed the instruction
-// cache); a pair whose regions are empty (band n nowhere occupied or band m
-// nowhere empty for the +1 region, and the converse for -1) is skipped from
-// four corner minima and maxima. The clipping only queues the kept
+// One thread per (cube, tetrahedron) runs over the band pairs that have a
+// region in some lane's tetrahedron (four corner minima and maxima: band n
+// occupied somewhere and band m empty somewhere for the +1 region, the
+// converse for -1), in a loop that is not unrolled (the unrolled 64-pair loop
+// overflowed the instruction cache). A whole tetrahedron (occupied, empty at
+// every corner) needs no cuts. The clipping only queues the kept
 // sub-tetrahedra (sorted transition energies, amplitude, dither key) in a
 // per-warp queue in shared memory; between band pairs, once the queue holds
-// kDrainAt entries, all 32 lanes drain it, one sub-tetrahedron per lane, so
-// the per-energy work is not serialised behind the lanes' different clip
-// paths. Contributions are rounded once to integers of a fixed-point unit
-// (a dither hashed from the contribution's identity makes the rounding
-// unbiased) and added with 64-bit integer atomics into a per-CTA shared
-// tile, then over the CTAs in one accumulator: the result does not depend on
-// the schedule or on the order in which queues are drained.
+// kDrainAt entries, the warp drains it: long windows a lane per energy, short
+// ones a lane each, so the per-energy work is not serialised behind the
+// lanes' different clip paths. Contributions are rounded once to integers of
+// a fixed-point unit (a dither hashed from the contribution's identity makes
+// the rounding unbiased) and added with 32-bit integer atomics into a per-CTA
+// shared tile, which goes to one 64-bit accumulator before it could overflow
+// and at the end: the result does not depend on the schedule or on the order
+// in which queues are drained. At 64^3 points, 8 bands and 400 energies 3.7
+// -> 2.2 ms (64-bit shared atomics, one lane per sub-tetrahedron before); 1.3
+// ms of it is clipping, which fetches instructions and branches (issue active
+// 34 %).
 //
 // The real part runs the same clipping with KIND = kKindRe: every
 // sub-tetrahedron reaches every energy (its principal-value average of
 // 1/(w - D), below), so the sub-tetrahedra are kept in per-lane segments and
-// the whole warp evaluates them, lane by lane in a fixed order, at all
-// energies (each lane owning every 32nd energy).
+// the whole warp evaluates them in a fixed order, neighbours jointly far away
+// and one by one near (each lane owning every 32nd energy). At 48^3 points, 8
+// bands and 400 energies 33.2 -> 10.7 ms.
 #include <algorithm>
 #include <atomic>
 #include <cmath>
