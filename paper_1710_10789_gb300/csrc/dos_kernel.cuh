@@ -359,7 +359,8 @@ __global__ void __maxnreg__(kMaxRegs)
         const uintptr_t need = reinterpret_cast<uintptr_t>(mbar + 3) - reinterpret_cast<uintptr_t>(smem_raw);
         const bool bad = need > dynamic_smem_bytes() || (smem_u32(estage[0]) & 127u) != 0 ||
                          (A.e_stage & 127u) != 0 || (A.w_stage & 127u) != 0 || A.e_box_bytes > A.e_stage ||
-                         A.w_box_bytes > A.w_stage || (smem_u32(mbar) & 7u) != 0 || A.items_per_box > 65535;
+                         A.w_box_bytes > A.w_stage || (smem_u32(mbar) & 7u) != 0 || A.items_per_box > 65535 ||
+                         (MAXM > 1 && n_blk > (int)blockDim.x);   // (a batch's flush: a thread per block)
         if (bad) {
             if (tid == 0) atomicOr(A.status, kFlagConfig);
             return;
@@ -1349,9 +1350,12 @@ cudaError_t launch_t(size_t smem, dim3 grid, const Batch<MAXM> &Bt, const FwdArg
             }
         }
     }
-    // no more warps than a box has items for (idle ones only slow its barriers)
+    // no more warps than a box has items for (idle ones only slow its barriers);
+    // in a batch, whose flush looks at one block of 64 energies per thread, as
+    // many threads as blocks (at most about 280: a tile takes 13 bytes per energy)
     const int items = A.items_per_box << (MODE != TETRA_BIN && Cfg<NORB>::pairs ? A.split : 0);
-    const int threads = std::min(kThreads, std::max(128, (items + 31) & ~31));
+    const int least = MAXM > 1 ? std::max(128, (((A.chunk_w + 63) >> 6) + 31) & ~31) : 128;
+    const int threads = std::min(kThreads, std::max(least, (items + 31) & ~31));
     k<<<grid, threads, smem, stream>>>(Bt, A);
     return cudaGetLastError();
 }

@@ -1,0 +1,45 @@
+"""Value ranges and table sizes at which the kernels' counters, units and
+shared tables change, against the general path or the oracle."""
+import numpy as np
+import pytest
+
+import oracle
+import tbgen
+from helpers import to_layout
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def T():
+    import paper_1710_10789_gb300 as T
+    T.build()
+    return T
+
+
+@pytest.mark.parametrize("box,bins", [((4, 4, 4), 12900), ((2, 2, 2), 9000)])
+def test_batch_flushes_every_block_of_a_long_grid(T, box, bins):
+    """A batch whose tile has more blocks of 64 bins than its boxes have work
+    items for threads (201 and 141 blocks; 192 and 24 items): one narrow band
+    near the top of the grid puts more than 2^31 units into one bin of every
+    CTA's 32-bit tile, so the result is right only if that bin's block is
+    flushed on the way. The batch equals the single plan bit for bit; the
+    band's weight is all in its bin, to the fixed-point unit's 5e-6."""
+    n = 64
+    top = np.float32(bins * 1e-3 - 0.05)
+    edges = (np.arange(bins + 1) * 1e-3).astype(np.float32)
+    i = int(np.searchsorted(edges, top, side="right")) - 1
+    mid, width = 0.5 * (edges[i] + edges[i + 1]), edges[i + 1] - edges[i]
+    noise = np.random.default_rng(3).uniform(-0.3, 0.3, (n ** 3, 1))
+    eps = (mid + noise * width).astype(np.float32)
+    w = np.full((n ** 3, 1, 1), 0.9, np.float32)
+    plan = T.BatchPlan([(n, n, n)], [bins], 1, 1, mode="bin", tune={"box": box})
+    E, W = to_layout(eps, w, n, n, n, plan.layouts[0].eps_stride, plan.layouts[0].w_stride)
+    Et, Wt, om = torch.from_numpy(E).cuda(), torch.from_numpy(W).cuda(), torch.from_numpy(edges).cuda()
+    out, = plan.dos([Et], [Wt], [om])
+    assert plan.status() == T.TETRA_OK
+    single = T.Plan(n, n, n, 1, 1, bins, mode="bin").dos(Et, Wt, om)
+    assert torch.equal(out, single)
+    g = out.cpu().numpy()[0].astype(np.float64)
+    assert abs(g[i] * float(width) - 0.9) <= 5e-6 * 0.9 and np.count_nonzero(g) == 1
