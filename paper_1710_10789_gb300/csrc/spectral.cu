@@ -122,13 +122,14 @@ struct ReSeg {
 };
 
 // Set-up of one entry as the warp's lanes read it (32 words): mean c,
-// amplitude, (2 R)^2, moments mu_2..mu_kReMom (mu_0 = 1, and mu_1 vanishes
-// about the mean), and the density pieces: corner values, reciprocal lengths (0 for an empty one),
-// g(d1), g(d2) and the middle piece's value at its centre.
+// amplitude, (2 R)^2, half-width R, moments mu_2..mu_kReMom in units of R (mu_0
+// = 1, and mu_1 vanishes about the mean), and the density pieces: corner
+// values, reciprocal lengths (0 for an empty one), g(d1), g(d2) and the middle
+// piece's value at its centre.
 struct __align__(16) ReStage {
-    float c, amp, far2;
+    float c, amp, far2, R;
     float mu[kReMom - 1];
-    float d[4], r[3], G1, G2, A2, pad[4];
+    float d[4], r[3], G1, G2, A2, pad[3];
 };
 static_assert(sizeof(ReStage) == 128, "32 words");
 
@@ -474,11 +475,14 @@ __host__ __device__ constexpr float re_coef(int n) { return 6.f / (float)((n + 1
 
 __device__ __forceinline__ void re_setup(const ReSeg &T, ReStage &st) {
     const float c = 0.25f * ((T.d0 + T.d1) + (T.d2 + T.d3));
-    const float e[4] = {T.d0 - c, T.d1 - c, T.d2 - c, T.d3 - c};
-    const float R = fmaxf(-e[0], e[3]);
+    const float R = fmaxf(c - T.d0, T.d3 - c), inv = R > 1e-37f ? __fdividef(1.f, R) : 0.f;
+    // (in units of R: order 16 in the units of the energies would overflow for
+    // half-widths above 250 of them and underflow below 1e-2)
+    const float e[4] = {(T.d0 - c) * inv, (T.d1 - c) * inv, (T.d2 - c) * inv, (T.d3 - c) * inv};
     st.c = c;
     st.amp = T.amp;
     st.far2 = 4.f * R * R;
+    st.R = R;
     float h[kReMom + 1];
     re_homogeneous<kReMom>(e, h);
 #pragma unroll
@@ -602,7 +606,7 @@ __device__ __forceinline__ void re_process(const SpecArgs &S, int lane, int &sin
     // this lane's entries first
     const bool some = hi >= lo;
     const float C = some ? 0.5f * (lo + hi) : 0.f, rho = some ? 0.5f * (hi - lo) : 0.f;
-    const float inv = rho > 0.f ? 1.f / rho : 0.f;
+    const float inv = rho > 1e-37f ? 1.f / rho : 0.f;
     constexpr int kM = 24;   // kReCluster + 1 in whole thirds of the exchange below
     float M[kM];
 #pragma unroll
@@ -709,8 +713,9 @@ __device__ __forceinline__ void re_process(const SpecArgs &S, int lane, int &sin
                         mu[1] = 0.f;
 #pragma unroll
                         for (int n = 2; n <= kReMom; ++n) mu[n] = st.mu[n - 2];
-                        if (wmin > 4.f * st.far2) re_series<8>(mu, v, r);
-                        else re_series<kReMom>(mu, v, r);
+                        const float z[2] = {st.R * v[0], st.R * v[1]};
+                        if (wmin > 4.f * st.far2) re_series<8>(mu, z, r);
+                        else re_series<kReMom>(mu, z, r);
 #pragma unroll
                         for (int k = 0; k < 2; ++k) r[k] *= v[k];
                     }

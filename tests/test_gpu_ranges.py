@@ -5,7 +5,7 @@ import pytest
 
 import oracle
 import tbgen
-from helpers import to_layout
+from helpers import tb_problem, to_layout
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -43,3 +43,31 @@ def test_batch_flushes_every_block_of_a_long_grid(T, box, bins):
     assert torch.equal(out, single)
     g = out.cpu().numpy()[0].astype(np.float64)
     assert abs(g[i] * float(width) - 0.9) <= 5e-6 * 0.9 and np.count_nonzero(g) == 1
+
+
+@pytest.mark.parametrize("power", [10, -17])
+def test_chi0_real_does_not_depend_on_the_unit_of_energy(T, power):
+    """Bands, chemical potential and energies times s (eV as meV: sub-tetrahedra
+    hundreds of units wide on a coarse grid; or as 1e5 eV) give Re chi0 / s. s
+    is a power of two, so all FP32 products scale exactly and only the
+    logarithms round differently: log2 of arguments 2^power larger, rounded at
+    |log2| < 32 to 2e-6, in sums that keep 2e-5 of the largest value. The
+    oracle at the bar of test_gpu_chi0_real.py, 1e-4."""
+    n, q, s = (10, 9, 8), (3, 0, 1), np.float32(2.0 ** power)
+    _, eps, _ = tb_problem(3, n)
+    mu = float(np.float32(np.median(eps)))
+    omega = np.concatenate([tbgen.uniform_grid(-3.0, 3.0, 97), [-25.0, 40.0]]).astype(np.float32)
+
+    def run(s):
+        plan = T.Plan(*n, eps.shape[1], 1, 16)
+        E, _ = to_layout(eps * s, np.zeros(eps.shape + (1,), np.float32), *n, plan.layout.eps_stride, plan.layout.w_stride)
+        r = plan.chi0_real_t0(torch.from_numpy(E).cuda(), q, mu * float(s), torch.from_numpy(omega * s).cuda())
+        assert plan.spectral_status() == T.TETRA_OK
+        return r.cpu().numpy().astype(np.float64) * float(s)
+
+    one, other = run(np.float32(1)), run(s)
+    r = oracle.chi0_real_t0(eps.astype(np.float64), *n, q, mu, omega.astype(np.float64))
+    scale = np.max(np.abs(r))
+    print(f"2^{power}: {np.max(np.abs(other - one)) / scale:.1e} from 1, {np.max(np.abs(other - r)) / scale:.1e} from the oracle")
+    assert np.max(np.abs(other - one)) <= 2e-5 * scale
+    assert np.max(np.abs(other - r)) <= 1e-4 * scale
