@@ -279,10 +279,15 @@ tetra_status_t tetra_dos_batched(tetra_batch_plan_t plan, const float *const *ep
  *   ws     : device workspace of at least tetra_fermi_workspace_bytes(plan)
  *            bytes, 16-byte aligned.
  * Method: the band minimum and maximum bracket E_F; each round (one launch)
- * evaluates N at 16 equidistant energies of the bracket, from the tetrahedra
- * that straddle it, and keeps the sub-interval where N crosses n_electrons,
- * until the bracket is at the FP32 resolution of the energies (about eight
- * rounds). Synchronises `stream`. Returns TETRA_EINVAL for null/misaligned pointers
+ * evaluates N at 16 energies of the bracket, from the tetrahedra that straddle
+ * it, and keeps the sub-interval where N crosses n_electrons, until the bracket
+ * is at the FP32 resolution of the energies (four to six rounds). The energies
+ * are equidistant, or close to the level that the line through N at the
+ * bracket's ends gives. N is summed in integers of 2^-26 of a tetrahedron of
+ * weight one, or of a larger unit where weights are so large that 64 bits would
+ * not hold the sums. A weight that is not finite leaves its cubes out and is
+ * recorded in the workspace (TETRA_ERANGE from tetra_workspace_status).
+ * Synchronises `stream`. Returns TETRA_EINVAL for null/misaligned pointers
  * or n_electrons outside [0, N(max eps)], TETRA_ENOMEM if ws_bytes is too
  * small, TETRA_EUNSUPPORTED for a slab plan (the count needs the whole grid). */
 size_t tetra_fermi_workspace_bytes(tetra_plan_t plan);

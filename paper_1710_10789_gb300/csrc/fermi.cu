@@ -19,7 +19,10 @@
 // weight. The corner weights need no energy cases (tet_common.cuh). Each
 // cube's N(E) - N(lo) is rounded once to an integer of 2^-26 of a full
 // tetrahedron, summed over the warp by two 32-bit reductions, over the
-// block's warps and over the grid by integer adds: exact in any order.
+// block's warps and over the grid by integer adds: exact in any order. Weights
+// so large that the 64-bit sums could wrap (above about 20 per band at 1024^3
+// points, 10^6 on a small grid) take a coarser unit: the first round, which
+// stages every weight, finds the largest one and is then repeated.
 //
 // At 95 x 97 x 96 points, 8 bands and 8 orbitals the five rounds of the
 // integrated-mode DOS kernel before (64 energies, every orbital, every
@@ -41,7 +44,6 @@ constexpr int kRounds = 64;        // at most; FP32 resolution takes about five
 constexpr int kRoundsPerSync = 6;
 constexpr int kFermiThreads = 256;
 constexpr int kFermiBlocks = 3;    // per SM
-constexpr int kUnitBits = 26;
 
 // Order-preserving map of a float to an unsigned int (for atomic min / max).
 __device__ __forceinline__ unsigned ordered(float f) {
@@ -59,6 +61,9 @@ struct FermiState {
     long long base, top;       // N(lo), N(hi) in units
     int guess;                 // whether the round's energies cluster about the interpolated level
     int round, done, bad;      // bad: no such count, or no valid band energy
+    int drop;                  // the unit is 2^-(kFermiBits - drop) of a full tetrahedron
+    unsigned wmax;             // largest |sum of a corner's weights| (a float's bits), first round
+    int range;                 // a cube's value was not finite and was left out
     int ticket;
     unsigned long long sums[kPts];   // N(E_j) - N(lo) of the running round
 };
@@ -100,6 +105,7 @@ struct FermiArgs {
     const float *eps;
     const void *w;
     FermiState *S;
+    int *status;
 };
 
 // Energy j of a round, ascending to hi: equidistant, or about the level that
@@ -145,10 +151,12 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
     __shared__ unsigned s_band[2][2];   // bands with an item, of two tiles in turn
     __shared__ int s_count[2];          // items, of two tiles in turn
     __shared__ int s_last;
+    __shared__ unsigned s_wmax;         // first round: the largest |weight sum| staged (a float's bits)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int nwarp = kFermiThreads / 32;
     FermiState *S = A.S;
     const bool first = S->round == 0;
+    const int drop = S->drop, bits = kFermiBits - drop;
     if (S->done) return;   // (set by an earlier launch only)
     float lo, hi;
     if (first) {
@@ -159,13 +167,14 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
         lo = S->lo;
         hi = S->hi;
     }
+    if (tid == 0) s_wmax = 0u;
     if (tid < kPts) {
         s_sum[tid] = 0ull;
         const bool guess = !first && S->guess;
         float level = lo;
         if (guess) {   // (one thread group; FP64 is slow but this is a few operations)
             const double below = (double)S->base, above = (double)S->top;
-            const double n = A.n_electrons / (A.vtvg * ldexp(1.0, -kUnitBits));
+            const double n = A.n_electrons / (A.vtvg * ldexp(1.0, -bits));
             level = lo + (hi - lo) * (float)((n - below) / (above - below));
         }
         s_om[tid] = round_energy(lo, hi, guess, level, tid);
@@ -176,7 +185,7 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
     const int lcol = A.lty + A.ltz;   // log2 of the (y, z) columns
     float *se = s_pt, *sw = s_pt + A.nb * ps;
     unsigned short *item = reinterpret_cast<unsigned short *>(sw + A.nb * ps);   // (band, column, x)
-    const float fq = (float)(1 << kUnitBits) * 0.25f;
+    const float fq = ldexpf(0.25f, bits);
     const WT *W = static_cast<const WT *>(A.w);
     const bool vec = (A.n_orb * sizeof(WT)) % 16 == 0;
     // an item's first corner in the tile
@@ -185,6 +194,13 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
         return (it >> (5 + lcol)) * ps + (it & 31) + 32 * (cy + py * cz);
     };
     const int dy = 32, dz = 32 * py;
+    // a cube's value in units; one that is not finite is left out (a finite one
+    // is below 2^48 once the unit is chosen, see fermi_drop)
+    auto units = [&](float v) -> long long {
+        if (fabsf(v) < 5.6e14f) return __float2ll_rn(v);
+        atomicOr(&S->range, 1);
+        return 0;
+    };
     long long acc = 0;   // lane j: this warp's sum at energy j
     int par = 0;
     for (int tile = blockIdx.x; tile < A.n_tiles; tile += gridDim.x, par ^= 1) {
@@ -243,9 +259,16 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
 #pragma unroll 2
             for (int r = warp; r < rows; r += nwarp) {
                 const int y = min(y0 + r % py, A.n2), z = min(z0 + r / py, A.n3);
-                if (in_x)
-                    sw[n * ps + r * 32 + lane] = sum_weights<WT>(
+                float t = 0.f;
+                if (in_x) {
+                    t = sum_weights<WT>(
                         W + (x0 + lane + (long)A.nx * (y + (long)A.ny * z)) * A.w_stride + n * A.n_orb, A.n_orb, vec);
+                    sw[n * ps + r * 32 + lane] = t;
+                }
+                if (first) {
+                    const unsigned m = __reduce_max_sync(0xffffffffu, fabsf(t) < INFINITY ? __float_as_uint(fabsf(t)) : 0u);
+                    if (lane == 0) atomicMax(&s_wmax, m);
+                }
             }
         }
         __syncthreads();
@@ -312,11 +335,11 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
             for (int t = 0; t < 6; ++t)
 #pragma unroll
                 for (int k = 0; k < 4; ++k) full += fq * b[(tet_code(t) >> (3 * k)) & 7];
-            const long long q_lo = __float2ll_rn(at_lo), q_full = __float2ll_rn(full);
+            const long long q_lo = act ? units(at_lo) : 0, q_full = act ? units(full) : 0;
 #pragma unroll
             for (int j = 0; j < kPer; ++j) {
                 // (a flat tetrahedron at E is empty there: only above emax all is full)
-                const long long q = act ? (in[j] ? __float2ll_rn(v[j]) : (E[j] > emax ? q_full : 0)) - q_lo : 0;
+                const long long q = act ? (in[j] ? units(v[j]) : (E[j] > emax ? q_full : 0)) - q_lo : 0;
                 // q = high 2^24 + low, low in [0, 2^24): sums of 32 fit 32 bits
                 const long long sum = ((long long)__reduce_add_sync(0xffffffffu, (int)(q >> 24)) << 24) +
                                       (long long)__reduce_add_sync(0xffffffffu, (unsigned)(q & 0xFFFFFF));
@@ -328,6 +351,7 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
     if (lane < kPts && acc) atomicAdd(&s_sum[lane], (unsigned long long)acc);
     __syncthreads();
     if (tid < kPts && s_sum[tid]) atomicAdd(&S->sums[tid], s_sum[tid]);
+    if (first && tid == 0) atomicMax(&S->wmax, s_wmax);
     __threadfence();
     __syncthreads();
     if (tid == 0) s_last = atomicAdd(&S->ticket, 1) == (int)gridDim.x - 1;
@@ -336,7 +360,7 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
     __threadfence();
     // the last block narrows the bracket to the sub-interval where N crosses
     // n_electrons (N does not decrease)
-    const double unit = A.vtvg * ldexp(1.0, -kUnitBits);
+    const double unit = A.vtvg * ldexp(1.0, -bits);
     const long long base = first ? 0 : S->base;
     long long N[kPts];
     for (int j = 0; j < kPts; ++j) {
@@ -344,7 +368,16 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
         S->sums[j] = 0ull;
     }
     S->ticket = 0;
+    if (first && drop == 0) {
+        const int d = fermi_drop(__uint_as_float(__ldcg(&S->wmax)), (double)A.n1 * A.n2 * A.n3 * A.nb);
+        if (d > 0) {   // the sums may have wrapped: the round again with the coarser unit
+            S->drop = d;
+            S->range = 0;
+            return;
+        }
+    }
     S->round = S->round + 1;
+    if (__ldcg(&S->range)) atomicOr(A.status, kFlagRange);
     const double top = (double)N[kPts - 1] * unit;
     if (first && (!(lo <= hi) || !(A.n_electrons >= 0.0) || A.n_electrons > top * (1.0 + 1e-6))) {
         S->bad = 1;
@@ -422,6 +455,7 @@ tetra_status_t fermi_level(const Plan &P, const float *eps, const void *w, doubl
     A.vtvg = 1.0 / (6.0 * (double)P.d.n1 * (double)P.d.n2 * (double)P.d.n3);
     A.eps = eps; A.w = w;
     A.S = reinterpret_cast<FermiState *>(static_cast<unsigned char *>(ws) + kStatusBytes);
+    A.status = reinterpret_cast<int *>(ws);
     choose_tile(P, A);
     const size_t smem = tile_bytes(A);
     const int grid = std::min(A.n_tiles, kFermiBlocks * P.sm_count);

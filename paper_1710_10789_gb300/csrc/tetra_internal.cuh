@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
+#include <math.h>
 #include <stdint.h>
 #include "../../include/tetra.h"
 
@@ -178,6 +179,20 @@ __device__ __forceinline__ void load_weights(const WT *src, int n_orb, float (&b
 #pragma unroll
         for (int s = 0; s < NORB; ++s) b[s] = (s < n_orb) ? to_f32<WT>(src[s]) : 0.f;
     }
+}
+
+// Fermi level: the unit of the count is 2^-(kFermiBits - drop) of a full
+// tetrahedron of weight one, 0 <= drop the least for which no sum of the count
+// can pass 2^61 (cells = cubes x bands, a cell's six tetrahedra full and all
+// weights wmax) and no cell 2^48 (32 of its upper parts, value >> 24, are added in
+// 32 bits).
+constexpr int kFermiBits = 26;
+__host__ __device__ inline int fermi_drop(float wmax, double cells) {
+    if (!(wmax > 0.f)) return 0;
+    const double one = log2(6.0 * (double)wmax), all = one + log2(cells);
+    const int a = (int)ceil(all) + kFermiBits - 61, b = (int)ceil(one) + kFermiBits - 48;
+    const int d = a > b ? a : b;
+    return d > 0 ? d : 0;
 }
 
 // ---------------------------------------------------------------- host helpers

@@ -71,3 +71,23 @@ def test_chi0_real_does_not_depend_on_the_unit_of_energy(T, power):
     print(f"2^{power}: {np.max(np.abs(other - one)) / scale:.1e} from 1, {np.max(np.abs(other - r)) / scale:.1e} from the oracle")
     assert np.max(np.abs(other - one)) <= 2e-5 * scale
     assert np.max(np.abs(other - r)) <= 1e-4 * scale
+
+
+@pytest.mark.parametrize("power", [24, 100])
+@pytest.mark.parametrize("n_electrons", [0.37, 5.25])
+def test_fermi_level_does_not_depend_on_the_scale_of_the_weights(T, n_electrons, power):
+    """Weights and electron count times 2^power: the same level. 2^24 puts the
+    count of this grid at 2^66 units of 2^-26 of a tetrahedron. The unit is
+    never coarser than 2^-21 of the scaled weight here, 10^5 cells of which
+    shift N by 1e-7 of a state at most, and E_F by 1e-6 eV at one state per 10 eV."""
+    n = (12, 11, 10)
+    _, eps, w = tb_problem(4, n)
+    plan = T.Plan(*n, 8, 8, 16)
+    E, W = to_layout(eps, w, *n, plan.layout.eps_stride, plan.layout.w_stride)
+    Et, Wt = torch.from_numpy(E).cuda(), torch.from_numpy(W).cuda()
+    one = plan.fermi_level(Et, Wt, n_electrons)
+    s = 2.0 ** power
+    assert abs(plan.fermi_level(Et, Wt * s, n_electrons * s) - one) <= 5e-6
+    with pytest.raises(T.TetraError) as ex:
+        plan.fermi_level(Et, Wt * s, 8.01 * s)
+    assert ex.value.status == T.TETRA_EINVAL
