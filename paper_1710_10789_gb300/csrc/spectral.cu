@@ -31,13 +31,15 @@
 // ones a lane each, so the per-energy work is not serialised behind the
 // lanes' different clip paths. Contributions are rounded once to integers of
 // a fixed-point unit (a dither hashed from the contribution's identity makes
-// the rounding unbiased) and added with 32-bit integer atomics into a per-CTA
-// shared tile, which goes to one 64-bit accumulator before it could overflow
-// and at the end: the result does not depend on the schedule or on the order
-// in which queues are drained. At 64^3 points, 8 bands and 400 energies 3.7
-// -> 2.2 ms (64-bit shared atomics, one lane per sub-tetrahedron before); 1.3
+// the rounding unbiased) and added to exact 64-bit sums, whose low halves are
+// 32-bit words of a per-CTA shared tile and whose carries go to the accumulator
+// in global memory: the result does not depend on the schedule or on the order
+// in which queues are drained. At 64^3 points, 8 bands and 400 energies 3.6
+// -> 2.3 ms (64-bit shared atomics, one lane per sub-tetrahedron before); 1.3
 // ms of it is clipping, which fetches instructions and branches (issue active
-// 34 %).
+// 34 %). (Units up to 64 times coarser, so that a bounded 32-bit tile holds
+// the sums, took 2.2 ms, but the error against 64 bits was 4.6e-8 instead of
+// 3.0e-8 there and up to four times larger on small grids of few energies.)
 //
 // The real part runs the same clipping with KIND = kKindRe: every
 // sub-tetrahedron reaches every energy (its principal-value average of
@@ -58,17 +60,19 @@ namespace {
 constexpr int kSpecThreads = 128;
 constexpr int kSpecWarps = kSpecThreads / 32;
 constexpr int kSpecBlocksPerSM = 4;
-constexpr int kReBits = 26;     // fixed-point fraction bits of the real part's unit (S: spec_bits)
+constexpr int kSpecBits = 26;   // fixed-point fraction bits of the unit
 constexpr int kQueueCap = 256;  // sub-tetrahedra per warp queue
 constexpr int kDrainAt = 64;    // a queue this full is drained before the next band pair
 constexpr int kWide = 20;       // a sub-tetrahedron with this many energies is taken by the whole warp
-constexpr float kEntryCap = 4.1e6f;         // below 2^22: larger contributions go to the 64-bit accumulator
-constexpr unsigned kTileLimit = 1u << 30;   // the int32 tile is flushed before its sums could pass this
+constexpr float kEntryCap = 1.0e9f;   // below 2^30: larger contributions go to the 64-bit accumulator
 // the real part of chi0 (kKindRe) next to the spectral function (kKindS)
 constexpr int kKindS = 0, kKindRe = 1;
 constexpr int kReBlocksPerSM = 3;
 constexpr int kSubPerPair = 18;  // sub-tetrahedra one (tetrahedron, band pair) can give: 2 regions x 3 x 3
-constexpr int kReFlush = 64;     // band pairs summed in FP32 before the per-warp sums go to the tile
+// band pairs summed in FP32 before the per-warp sums go to the tile (error against 64
+// bits at 48^3 points, 8 bands, 400 energies: 3.8e-8, and no more when they go after
+// every 64 sub-tetrahedra)
+constexpr int kReFlush = 64;
 constexpr int kReGroup = 8;      // lanes whose sub-tetrahedra are taken together far away
 constexpr int kReCluster = 20;   // highest moment of such a group
 constexpr int kReMom = 16;       // highest moment of one sub-tetrahedron
@@ -137,8 +141,7 @@ static_assert(sizeof(ReStage) == 128, "32 words");
 struct SpecArgs {
     const float *om;        // shared: energies (point) or bin edges (bin)
     long long *tile;        // shared, real part: int64 accumulators per energy
-    int *tile32;            // shared, S: int32 accumulators per energy / bin
-    unsigned *bound;        // shared, S: bound on what any entry of tile32 holds
+    unsigned *tile32;       // shared, S: low halves of the sums per energy / bin
     long long *sums;        // global: int64 accumulators per energy / bin
     int n_om;               // energies or bins
     int mode;               // TETRA_POINT or TETRA_BIN
@@ -183,7 +186,7 @@ __device__ __forceinline__ float spec_below(const SpecTet &T, float E) {
 }
 
 // Mean spacing of the energy grid (or bin width), the scale of the
-// fixed-point unit = (V_T/V_G) / de * 2^-bits.
+// fixed-point unit = (V_T/V_G) / de * 2^-26.
 __device__ __forceinline__ double mean_spacing(const float *om, int n_om, int mode) {
     const int spacings = mode == TETRA_BIN ? n_om : n_om - 1;
     double de = spacings > 0 ? ((double)om[spacings] - (double)om[0]) / spacings : 1.0;
@@ -234,7 +237,8 @@ __device__ __forceinline__ void spec_setup(const SubTet &Q, const SpecArgs &S, S
         T.i0 = max(0, upper_index(S.om, S.n_om + 1, Q.d0, S.om0, S.inv_de) - 1);   // bins with upper edge > d0
         T.i1 = min(S.n_om, upper_index(S.om, S.n_om + 1, Q.d3, S.om0, S.inv_de));   // and lower edge <= d3
     } else {
-        T.amp = Q.amp * 3.f * T.r41;
+        // (3 / E41 first: 3 amp would round alike for all whole tetrahedra)
+        T.amp = Q.amp * (3.f * T.r41);
         T.i0 = upper_index(S.om, S.n_om, Q.d0, S.om0, S.inv_de);
         T.i1 = lower_index(S.om, S.n_om, Q.d3, S.om0, S.inv_de);
     }
@@ -263,11 +267,28 @@ __device__ __noinline__ void deposit_wide(const SubTet &Q, const SpecArgs &S) {
     }
 }
 
-// Rounds to nearest even by adding 1.5 * 2^23 (exact below 2^22) and adds.
-__device__ __forceinline__ void spec_add(int *tile, int i, float x) {
-    const int qv = __float_as_int(x + 12582912.f) - 0x4B400000;
-    if (qv) atomicAdd(&tile[i], qv);
-}
+// Adds values (below 2^31), rounded to integers, to the exact 64-bit sums: the
+// low halves in the tile, whose carries and borrows (the old value says when) go
+// to the accumulator in global memory. They are rare, about one per 2^32 / |x|
+// adds, so that nothing has to bound or flush the tile. The old value is looked
+// at one add later, when it has arrived.
+struct SpecAdd {
+    unsigned *tile;
+    long long *sums;
+    int q = 0, i = 0;
+    unsigned old = 0;
+    __device__ __forceinline__ void settle() {
+        const int carry = (old + (unsigned)q < old ? 1 : 0) + (q >> 31);
+        if (carry) atomicAdd(reinterpret_cast<unsigned long long *>(&sums[i]), (unsigned long long)((long long)carry << 32));
+    }
+    __device__ __forceinline__ void add(int j, float x) {
+        const int v = __float2int_rn(x);
+        settle();
+        old = atomicAdd(&tile[j], (unsigned)v);
+        q = v;
+        i = j;
+    }
+};
 
 // Queues one sub-tetrahedron with corner values d of D in this warp's queue (or
 // adds it at once when the queue is full). Real part: in this lane's own
@@ -313,11 +334,8 @@ __device__ __noinline__ void accumulate(P5 v0, P5 v1, P5 v2, P5 v3, float sign, 
 // together. Each lane sets one up; those with many energies are then taken
 // by the whole warp, a lane per energy (consecutive tile entries: no bank
 // conflict, no lane idle for another's longer window), the short ones by
-// their own lane. The sums are 32-bit (64-bit shared atomics take about 20
-// cycles a warp, 32-bit ones 1 to 4); a warp about to push the tile's bound
-// past kTileLimit moves the tile to the 64-bit accumulator first. Adds that
-// other warps have announced but not made yet may land after that, uncounted:
-// at most 2^27 for each of the four warps.
+// their own lane. The atomics are 32-bit (64-bit shared ones take about 20
+// cycles a warp, 32-bit ones 1 to 4).
 __device__ __forceinline__ void drain(const SpecArgs &S, int lane) {
     constexpr unsigned kAll = 0xffffffffu;
     const SubTet *queue = S.q;
@@ -325,12 +343,11 @@ __device__ __forceinline__ void drain(const SpecArgs &S, int lane) {
     __syncwarp();
     const int n = min(*S.qn, kQueueCap);
     const float *om = S.om;
-    int *tile = S.tile32;
+    SpecAdd acc{S.tile32, S.sums};
     const bool bin = S.mode == TETRA_BIN;
     for (int base = 0; base < n; base += 32) {
         SpecTet T;
         int K = 0;
-        unsigned qb = 0;
         if (base + lane < n) {
             const SubTet Q = queue[base + lane];
             spec_setup(Q, S, T);
@@ -341,19 +358,7 @@ __device__ __forceinline__ void drain(const SpecArgs &S, int lane) {
                 deposit_wide(Q, S);
                 K = 0;
             }
-            if (K > 0) qb = (unsigned)most + 2u;
             st[lane] = T;
-        }
-        const unsigned announce = __reduce_add_sync(kAll, qb);
-        unsigned old = 0;
-        if (lane == 0) old = atomicAdd(S.bound, announce);
-        old = __shfl_sync(kAll, old, 0);
-        if (old + announce > kTileLimit) {
-            if (lane == 0) atomicExch(S.bound, announce);
-            for (int i = lane; i < S.n_om; i += 32) {
-                const int v = atomicExch(&tile[i], 0);
-                if (v) atomicAdd(reinterpret_cast<unsigned long long *>(&S.sums[i]), static_cast<unsigned long long>((long long)v));
-            }
         }
         __syncwarp();
         unsigned wide = __ballot_sync(kAll, K >= kWide);
@@ -361,12 +366,13 @@ __device__ __forceinline__ void drain(const SpecArgs &S, int lane) {
             const int j = __ffs(wide) - 1;
             wide &= wide - 1;
             const SpecTet W = st[j];
-            for (int i = W.i0 + lane; i < W.i1; i += 32) spec_add(tile, i, spec_value(W, om, bin, i));
+            for (int i = W.i0 + lane; i < W.i1; i += 32) acc.add(i, spec_value(W, om, bin, i));
         }
         if (K > 0 && K < kWide)
-            for (int i = T.i0; i < T.i1; ++i) spec_add(tile, i, spec_value(T, om, bin, i));
+            for (int i = T.i0; i < T.i1; ++i) acc.add(i, spec_value(T, om, bin, i));
         __syncwarp();
     }
+    acc.settle();
     if (lane == 0) *S.qn = 0;
     __syncwarp();
 }
@@ -767,26 +773,11 @@ bool spec_grid_fits(int n_om, int mode, size_t optin) {
     return spec_smem_bytes<KIND>(n_om, mode) + (KIND == kKindS ? 4 * (size_t)n_om - sizeof(SpecTet) * kSpecWarps * 32 : 0) <= optin;
 }
 
-// Fraction bits of S's unit. A value is a sum of items of size ~2^bits / K (K
-// energies per tetrahedron, about 2 n_om / N for N points a side), each
-// rounded without bias to one unit: its relative error is about
-// sqrt(K n_om / items) / 2^(bits + 1), here kept near 1e-9 (the items that
-// reach an energy are some percent of all). At 64^3 points, 8 bands, 400
-// energies that is 22 bits; 20 bits doubled the error against 64 bits, 3e-8.
-// An item of a tetrahedron with K energies is at most 3 2^bits / K, which has
-// to stay below kEntryCap.
-int spec_bits(const Plan &P, int n_om) {
-    const double points = (double)P.d.n1 * P.d.n2 * P.d.n3, K = std::max(1.0, 2.0 * n_om / std::cbrt(points));
-    const double items = 6.0 * points * P.d.n_bands * P.d.n_bands;
-    const int need = (int)std::ceil(std::log2(5e8 * std::sqrt(K * n_om / items)));
-    return std::max(20, std::min(std::min(26, need), 20 + (int)std::log2(K)));
-}
-
 template <int NB, int KIND>
 __global__ void __launch_bounds__(kSpecThreads, KIND == kKindS ? kSpecBlocksPerSM : kReBlocksPerSM)
     spectral_t0_kernel(const float *eps, int eps_stride, int n1, int n2, int n3, int nx, int ny, int z0, int z1,
                        int qx, int qy, int qz, float mu, const float *omega, int n_om, int mode,
-                       double vtvg, int bits, long long *sums, float *out, int *status) {
+                       double vtvg, long long *sums, float *out, int *status) {
     extern __shared__ __align__(16) unsigned char smem[];
     constexpr int QW = queue_entries<KIND>(), QC = queue_counts<KIND>();
     unsigned char *qraw = smem;                                             // [warps][QW] entries
@@ -795,22 +786,20 @@ __global__ void __launch_bounds__(kSpecThreads, KIND == kKindS ? kSpecBlocksPerS
     SpecTet *stet = reinterpret_cast<SpecTet *>(stage);                     // S: [warps][32]
     float *racc = reinterpret_cast<float *>(stage + kSpecWarps * kReBatch); // real part: [warps][n_om]
     long long *tile = reinterpret_cast<long long *>(racc + (KIND == kKindRe ? kSpecWarps * n_om : 0));
-    int *tile32 = reinterpret_cast<int *>(tile);                            // S
+    unsigned *tile32 = reinterpret_cast<unsigned *>(tile);                  // S
     float *om = KIND == kKindRe ? reinterpret_cast<float *>(tile + n_om) : reinterpret_cast<float *>(tile32 + n_om);
     static_assert(sizeof(SpecTet) * 32 == sizeof(ReStage) * kReBatch, "one staging area for both");
-    __shared__ unsigned s_bound;
     __shared__ float s_grid[4];   // V_T/V_G in units, 1 / mean spacing, the unit as a pair
     __shared__ float s_iw[kSpecWarps];
     const int n_edges = (mode == TETRA_BIN) ? n_om + 1 : n_om;
     for (int i = threadIdx.x; i < n_om; i += blockDim.x) {
         if constexpr (KIND == kKindRe) tile[i] = 0;
-        else tile32[i] = 0;
+        else tile32[i] = 0u;
     }
     for (int i = threadIdx.x; i < n_edges; i += blockDim.x) om[i] = omega[i];
     if (threadIdx.x == 0) {
-        s_bound = 0u;
         const double de = mean_spacing(omega, n_om, mode);
-        s_grid[0] = (float)ldexp(de, bits);
+        s_grid[0] = (float)ldexp(de, kSpecBits);
         s_grid[1] = (float)(1.0 / de);
         // (the unit that makes the float the kernel multiplies with exact)
         unit_pair(vtvg / (double)s_grid[0], s_grid[2], s_grid[3]);
@@ -837,7 +826,7 @@ __global__ void __launch_bounds__(kSpecThreads, KIND == kKindS ? kSpecBlocksPerS
     __shared__ SpecArgs s_args[kArgs];
     if (threadIdx.x < kArgs) {
         const int wp = threadIdx.x;
-        s_args[wp] = SpecArgs{om, tile, tile32, &s_bound, sums, n_om, mode, scale, max_iw, status, om_lo, om_hi,
+        s_args[wp] = SpecArgs{om, tile, tile32, sums, n_om, mode, scale, max_iw, status, om_lo, om_hi,
                               s_grid[1], reinterpret_cast<SubTet *>(qraw) + wp * QW, qcount + wp * QC,
                               stet + wp * 32, racc, reinterpret_cast<ReSeg *>(qraw),
                               reinterpret_cast<unsigned char *>(qcount), stage};
@@ -971,7 +960,7 @@ __global__ void __launch_bounds__(kSpecThreads, KIND == kKindS ? kSpecBlocksPerS
     // CTA and a kernel that added the 608 rows took 0.16 ms at 400 energies.)
     __syncthreads();
     for (int i = threadIdx.x; i < n_om; i += blockDim.x) {
-        const long long v = KIND == kKindRe ? tile[i] : (long long)tile32[i];
+        const long long v = KIND == kKindRe ? tile[i] : (long long)(unsigned long long)tile32[i];
         if (v) atomicAdd(reinterpret_cast<unsigned long long *>(sums + i), static_cast<unsigned long long>(v));
     }
     __threadfence();
@@ -990,7 +979,7 @@ int spectral_grid(const Plan &P) { return (KIND == kKindS ? kSpecBlocksPerSM : k
 
 template <int NB, int KIND>
 cudaError_t launch_spectral_nb(const Plan &P, const float *eps, const int q[3], float mu, const float *omega,
-                               int n_om, int mode, double vtvg, int bits, long long *sums, float *out,
+                               int n_om, int mode, double vtvg, long long *sums, float *out,
                                int *status, int grid, size_t smem, cudaStream_t stream) {
     auto k = spectral_t0_kernel<NB, KIND>;
     static std::atomic<int> opted[64];
@@ -1007,7 +996,7 @@ cudaError_t launch_spectral_nb(const Plan &P, const float *eps, const int q[3], 
         }
     }
     k<<<grid, kSpecThreads, smem, stream>>>(eps, P.eps_stride, P.d.n1, P.d.n2, P.d.n3, P.nx, P.ny, P.z0, P.z1,
-                                           q[0], q[1], q[2], mu, omega, n_om, mode, vtvg, bits, sums, out,
+                                           q[0], q[1], q[2], mu, omega, n_om, mode, vtvg, sums, out,
                                            status);
     return cudaGetLastError();
 }
@@ -1034,20 +1023,20 @@ tetra_status_t launch_spectral(const Plan &P, const float *eps, const int q_in[3
     if (ws_bytes < spectral_workspace<KIND>(P, n_om)) return TETRA_ENOMEM;
     const double vtvg = 1.0 / (6.0 * (double)P.d.n1 * (double)P.d.n2 * (double)P.d.n3);
     const int q[3] = {mod_q(q_in[0], P.d.n1), mod_q(q_in[1], P.d.n2), mod_q(q_in[2], P.d.n3)};
-    const int grid = spectral_grid<KIND>(P), bits = KIND == kKindS ? spec_bits(P, n_om) : kReBits;
+    const int grid = spectral_grid<KIND>(P);
     int *status = reinterpret_cast<int *>(ws);
     long long *sums = reinterpret_cast<long long *>(static_cast<unsigned char *>(ws) + kStatusBytes);
     if (cudaMemsetAsync(ws, 0, spectral_workspace<KIND>(P, n_om), stream) != cudaSuccess) return TETRA_ECUDA;
     cudaError_t e;
     switch (P.d.n_bands) {
-        case 1: e = launch_spectral_nb<1, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, bits, sums, S, status, grid, smem, stream); break;
-        case 2: e = launch_spectral_nb<2, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, bits, sums, S, status, grid, smem, stream); break;
-        case 3: e = launch_spectral_nb<3, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, bits, sums, S, status, grid, smem, stream); break;
-        case 4: e = launch_spectral_nb<4, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, bits, sums, S, status, grid, smem, stream); break;
-        case 5: e = launch_spectral_nb<5, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, bits, sums, S, status, grid, smem, stream); break;
-        case 6: e = launch_spectral_nb<6, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, bits, sums, S, status, grid, smem, stream); break;
-        case 7: e = launch_spectral_nb<7, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, bits, sums, S, status, grid, smem, stream); break;
-        default: e = launch_spectral_nb<8, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, bits, sums, S, status, grid, smem, stream); break;
+        case 1: e = launch_spectral_nb<1, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, sums, S, status, grid, smem, stream); break;
+        case 2: e = launch_spectral_nb<2, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, sums, S, status, grid, smem, stream); break;
+        case 3: e = launch_spectral_nb<3, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, sums, S, status, grid, smem, stream); break;
+        case 4: e = launch_spectral_nb<4, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, sums, S, status, grid, smem, stream); break;
+        case 5: e = launch_spectral_nb<5, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, sums, S, status, grid, smem, stream); break;
+        case 6: e = launch_spectral_nb<6, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, sums, S, status, grid, smem, stream); break;
+        case 7: e = launch_spectral_nb<7, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, sums, S, status, grid, smem, stream); break;
+        default: e = launch_spectral_nb<8, KIND>(P, eps, q, mu, omega, n_om, mode, vtvg, sums, S, status, grid, smem, stream); break;
     }
     return e == cudaSuccess ? TETRA_OK : TETRA_ECUDA;
 }

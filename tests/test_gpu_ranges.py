@@ -91,3 +91,23 @@ def test_fermi_level_does_not_depend_on_the_scale_of_the_weights(T, n_electrons,
     with pytest.raises(T.TetraError) as ex:
         plan.fermi_level(Et, Wt * s, 8.01 * s)
     assert ex.value.status == T.TETRA_EINVAL
+
+
+@pytest.mark.parametrize("mode", ["point", "bin"])
+def test_spectral_t0_units_do_not_depend_on_the_length_of_the_grid(T, mode):
+    """The unit is 2^-26 of a tetrahedron over the mean spacing, whatever the
+    number of energies: a slice of a grid of exact spacing gives the same bits as the
+    whole grid does there, down to two energies."""
+    n, q = (10, 9, 8), (3, 1, 0)
+    _, eps, _ = tb_problem(3, n)
+    mu = float(np.median(eps))
+    om = torch.arange(-128, 129, device="cuda").float() / 64   # spacing 2^-6
+    plan = T.Plan(*n, eps.shape[1], 1, 16)
+    E, _ = to_layout(eps, np.zeros(eps.shape + (1,), np.float32), *n, plan.layout.eps_stride, plan.layout.w_stride)
+    Et = torch.from_numpy(E).cuda()
+    whole = plan.spectral_t0(Et, q, mu, om, mode=mode)
+    bins = mode == "bin"
+    for a, b in ((0, 256), (20, 90), (100, 117), (160, 162)):
+        part = plan.spectral_t0(Et, q, mu, om[a:b + bins].clone(), mode=mode)
+        assert plan.spectral_status() == T.TETRA_OK
+        assert torch.equal(part, whole[a:b]) and whole[a:b].any(), (a, b)
