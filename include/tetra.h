@@ -285,8 +285,8 @@ tetra_status_t tetra_dos_batched(tetra_batch_plan_t plan, const float *const *ep
  * are equidistant, or close to the level that the line through N at the
  * bracket's ends gives. N is summed in integers of 2^-26 of a tetrahedron of
  * weight one, or of a larger unit where weights are so large that 64 bits would
- * not hold the sums. A weight that is not finite leaves its cubes out and is
- * recorded in the workspace (TETRA_ERANGE from tetra_workspace_status).
+ * not hold the sums. A weight that is not finite counts as zero and is recorded
+ * in the workspace (TETRA_ERANGE from tetra_workspace_status).
  * Synchronises `stream`. Returns TETRA_EINVAL for null/misaligned pointers
  * or n_electrons outside [0, N(max eps)], TETRA_ENOMEM if ws_bytes is too
  * small, TETRA_EUNSUPPORTED for a slab plan (the count needs the whole grid). */

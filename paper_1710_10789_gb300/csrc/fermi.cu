@@ -20,9 +20,9 @@
 // cube's N(E) - N(lo) is rounded once to an integer of 2^-26 of a full
 // tetrahedron, summed over the warp by two 32-bit reductions, over the
 // block's warps and over the grid by integer adds: exact in any order. Weights
-// so large that the 64-bit sums could wrap (above about 20 per band at 1024^3
-// points, 10^6 on a small grid) take a coarser unit: the first round, which
-// stages every weight, finds the largest one and is then repeated.
+// so large that the 64-bit sums could wrap (above about 20 a band at 1024^3
+// points, 10^6 on a small grid) are scaled down by a power of two: the first
+// round, which stages every weight, finds the largest and is then repeated.
 //
 // At 95 x 97 x 96 points, 8 bands and 8 orbitals the five rounds of the
 // integrated-mode DOS kernel before (64 energies, every orbital, every
@@ -61,9 +61,9 @@ struct FermiState {
     long long base, top;       // N(lo), N(hi) in units
     int guess;                 // whether the round's energies cluster about the interpolated level
     int round, done, bad;      // bad: no such count, or no valid band energy
-    int drop;                  // the unit is 2^-(kFermiBits - drop) of a full tetrahedron
-    unsigned wmax;             // largest |sum of a corner's weights| (a float's bits), first round
-    int range;                 // a cube's value was not finite and was left out
+    int drop;                  // weights are staged times 2^-drop
+    unsigned wmax;             // largest finite |weight sum| of a corner (a float's bits), before the scaling
+    int range;                 // a weight was not finite (and taken as zero)
     int ticket;
     unsigned long long sums[kPts];   // N(E_j) - N(lo) of the running round
 };
@@ -151,12 +151,13 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
     __shared__ unsigned s_band[2][2];   // bands with an item, of two tiles in turn
     __shared__ int s_count[2];          // items, of two tiles in turn
     __shared__ int s_last;
-    __shared__ unsigned s_wmax;         // first round: the largest |weight sum| staged (a float's bits)
+    __shared__ float s_scale;           // 2^-drop
+    __shared__ unsigned s_wmax;         // first pass: wmax of the block
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     constexpr int nwarp = kFermiThreads / 32;
     FermiState *S = A.S;
     const bool first = S->round == 0;
-    const int drop = S->drop, bits = kFermiBits - drop;
+    const int drop = S->drop;
     if (S->done) return;   // (set by an earlier launch only)
     float lo, hi;
     if (first) {
@@ -167,14 +168,17 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
         lo = S->lo;
         hi = S->hi;
     }
-    if (tid == 0) s_wmax = 0u;
+    if (tid == 0) {
+        s_scale = exp2f((float)-drop);
+        s_wmax = 0u;
+    }
     if (tid < kPts) {
         s_sum[tid] = 0ull;
         const bool guess = !first && S->guess;
         float level = lo;
         if (guess) {   // (one thread group; FP64 is slow but this is a few operations)
             const double below = (double)S->base, above = (double)S->top;
-            const double n = A.n_electrons / (A.vtvg * ldexp(1.0, -bits));
+            const double n = A.n_electrons / (A.vtvg * ldexp(1.0, drop - kFermiBits));
             level = lo + (hi - lo) * (float)((n - below) / (above - below));
         }
         s_om[tid] = round_energy(lo, hi, guess, level, tid);
@@ -185,7 +189,7 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
     const int lcol = A.lty + A.ltz;   // log2 of the (y, z) columns
     float *se = s_pt, *sw = s_pt + A.nb * ps;
     unsigned short *item = reinterpret_cast<unsigned short *>(sw + A.nb * ps);   // (band, column, x)
-    const float fq = ldexpf(0.25f, bits);
+    const float fq = (float)(1 << kFermiBits) * 0.25f;
     const WT *W = static_cast<const WT *>(A.w);
     const bool vec = (A.n_orb * sizeof(WT)) % 16 == 0;
     // an item's first corner in the tile
@@ -194,13 +198,6 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
         return (it >> (5 + lcol)) * ps + (it & 31) + 32 * (cy + py * cz);
     };
     const int dy = 32, dz = 32 * py;
-    // a cube's value in units; one that is not finite is left out (a finite one
-    // is below 2^48 once the unit is chosen, see fermi_drop)
-    auto units = [&](float v) -> long long {
-        if (fabsf(v) < 5.6e14f) return __float2ll_rn(v);
-        atomicOr(&S->range, 1);
-        return 0;
-    };
     long long acc = 0;   // lane j: this warp's sum at energy j
     int par = 0;
     for (int tile = blockIdx.x; tile < A.n_tiles; tile += gridDim.x, par ^= 1) {
@@ -253,23 +250,28 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
         const int count = s_count[par];
         if (count == 0) continue;
         unsigned long long bands = ((unsigned long long)s_band[par][1] << 32) | s_band[par][0];
+        unsigned wmax = 0u;
         while (bands) {
             const int n = __ffsll((long long)bands) - 1;
             bands &= bands - 1;
 #pragma unroll 2
             for (int r = warp; r < rows; r += nwarp) {
                 const int y = min(y0 + r % py, A.n2), z = min(z0 + r / py, A.n3);
-                float t = 0.f;
                 if (in_x) {
-                    t = sum_weights<WT>(
+                    float t = sum_weights<WT>(
                         W + (x0 + lane + (long)A.nx * (y + (long)A.ny * z)) * A.w_stride + n * A.n_orb, A.n_orb, vec);
-                    sw[n * ps + r * 32 + lane] = t;
-                }
-                if (first) {
-                    const unsigned m = __reduce_max_sync(0xffffffffu, fabsf(t) < INFINITY ? __float_as_uint(fabsf(t)) : 0u);
-                    if (lane == 0) atomicMax(&s_wmax, m);
+                    if (!(fabsf(t) < INFINITY)) {
+                        t = 0.f;
+                        S->range = 1;
+                    }
+                    wmax = max(wmax, __float_as_uint(fabsf(t)));
+                    sw[n * ps + r * 32 + lane] = t * s_scale;
                 }
             }
+        }
+        if (first) {
+            wmax = __reduce_max_sync(0xffffffffu, wmax);
+            if (lane == 0) atomicMax(&s_wmax, wmax);
         }
         __syncthreads();
         const int groups = (count + 31) >> 5;
@@ -335,11 +337,11 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
             for (int t = 0; t < 6; ++t)
 #pragma unroll
                 for (int k = 0; k < 4; ++k) full += fq * b[(tet_code(t) >> (3 * k)) & 7];
-            const long long q_lo = act ? units(at_lo) : 0, q_full = act ? units(full) : 0;
+            const long long q_lo = __float2ll_rn(at_lo), q_full = __float2ll_rn(full);
 #pragma unroll
             for (int j = 0; j < kPer; ++j) {
                 // (a flat tetrahedron at E is empty there: only above emax all is full)
-                const long long q = act ? (in[j] ? units(v[j]) : (E[j] > emax ? q_full : 0)) - q_lo : 0;
+                const long long q = act ? (in[j] ? __float2ll_rn(v[j]) : (E[j] > emax ? q_full : 0)) - q_lo : 0;
                 // q = high 2^24 + low, low in [0, 2^24): sums of 32 fit 32 bits
                 const long long sum = ((long long)__reduce_add_sync(0xffffffffu, (int)(q >> 24)) << 24) +
                                       (long long)__reduce_add_sync(0xffffffffu, (unsigned)(q & 0xFFFFFF));
@@ -360,7 +362,7 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
     __threadfence();
     // the last block narrows the bracket to the sub-interval where N crosses
     // n_electrons (N does not decrease)
-    const double unit = A.vtvg * ldexp(1.0, -bits);
+    const double unit = A.vtvg * ldexp(1.0, drop - kFermiBits);
     const long long base = first ? 0 : S->base;
     long long N[kPts];
     for (int j = 0; j < kPts; ++j) {
@@ -370,9 +372,8 @@ __global__ void __launch_bounds__(kFermiThreads, kFermiBlocks) fermi_round_kerne
     S->ticket = 0;
     if (first && drop == 0) {
         const int d = fermi_drop(__uint_as_float(__ldcg(&S->wmax)), (double)A.n1 * A.n2 * A.n3 * A.nb);
-        if (d > 0) {   // the sums may have wrapped: the round again with the coarser unit
+        if (d > 0) {   // the sums may have wrapped: the round again
             S->drop = d;
-            S->range = 0;
             return;
         }
     }

@@ -181,16 +181,15 @@ __device__ __forceinline__ void load_weights(const WT *src, int n_orb, float (&b
     }
 }
 
-// Fermi level: the unit of the count is 2^-(kFermiBits - drop) of a full
-// tetrahedron of weight one, 0 <= drop the least for which no sum of the count
-// can pass 2^61 (cells = cubes x bands, a cell's six tetrahedra full and all
-// weights wmax) and no cell 2^48 (32 of its upper parts, value >> 24, are added in
-// 32 bits).
+// Fermi level: the count is in units of 2^-kFermiBits of a full tetrahedron of
+// weight 2^drop. drop is the least (not below 0) for which no sum of `cells` (cube,
+// band) values can pass 2^62 and no value 2^48 (32 of their upper parts, value
+// >> 24, are added in 32 bits); wmax: the largest summed weight of a corner.
 constexpr int kFermiBits = 26;
 __host__ __device__ inline int fermi_drop(float wmax, double cells) {
     if (!(wmax > 0.f)) return 0;
-    const double one = log2(6.0 * (double)wmax), all = one + log2(cells);
-    const int a = (int)ceil(all) + kFermiBits - 61, b = (int)ceil(one) + kFermiBits - 48;
+    const double one = log2(6.0 * (double)wmax) + kFermiBits;   // a cube's six tetrahedra, full
+    const int a = (int)ceil(one + log2(cells)) - 62, b = (int)ceil(one) - 48;
     const int d = a > b ? a : b;
     return d > 0 ? d : 0;
 }
