@@ -116,7 +116,7 @@ struct BwdArgs {
     const float *eps;
     const void *w;
     const float *edges;      // n_bins + 1
-    const float *grad_dos;   // [n_orb][n_bins]
+    const float *grad_dos;   // [n_orb][n_bins] (TABLE: rows of G, see tetra_dos_bwd_table)
     float *geps, *gw;
     int vec;                 // gw is 16-byte aligned (the caller's array may not be)
     int staged;              // edges, G and D staged in shared memory
@@ -137,12 +137,13 @@ inline size_t bwd_stage_bytes(int norb_t, int n_bins) {
 // for each of the cube's 8 corners, interleaved over the block's threads.
 inline size_t bwd_scratch_bytes(int n_orb) { return sizeof(float) * (2 + (size_t)n_orb) * 8 * kBwdThreads; }
 
-template <int NORB, typename WT>
+// TABLE: G from rows in global memory instead of shared memory or the gradient.
+template <int NORB, typename WT, bool TABLE>
 __global__ void __launch_bounds__(kBwdThreads, bwd_blocks(NORB)) tetra_dos_bwd_kernel(const BwdArgs A, int px, int py, int pz) {
     extern __shared__ __align__(16) float s_mem[];
     const int n_e = A.n_bins + 1;
     const int ed_words = (n_e + 3) & ~3;
-    const size_t stage = A.staged ? (size_t)ed_words + 2 * (size_t)NORB * n_e : 0;
+    const size_t stage = !TABLE && A.staged ? (size_t)ed_words + 2 * (size_t)NORB * n_e : 0;
     float *scr = s_mem + stage;   // [(1 + n_orb) * 8][blockDim]
     float *sce = scr + (1 + A.n_orb) * 8 * blockDim.x;   // corner energies, [8][blockDim]
     // G_{e-1,s}, from the gradient (0 beyond either end)
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(kBwdThreads, bwd_blocks(NORB)) tetra_dos_bwd_k
         return e > 0 ? A.grad_dos[(long)s * A.n_bins + e - 1] / (A.edges[e] - A.edges[e - 1]) : 0.f;
     };
     const float *ed = A.edges, *sG = nullptr, *sD = nullptr;
-    if (A.staged) {
+    if (!TABLE && A.staged) {
         for (int i = threadIdx.x; i < n_e; i += blockDim.x) s_mem[i] = A.edges[i];
         float *G = s_mem + ed_words, *D = G + (size_t)NORB * n_e;
         for (int i = threadIdx.x; i < NORB * n_e; i += blockDim.x) {
@@ -167,7 +168,15 @@ __global__ void __launch_bounds__(kBwdThreads, bwd_blocks(NORB)) tetra_dos_bwd_k
     }
     // row e of G_{e-1} or D_e
     auto row = [&](bool diff, int e, float (&r)[NORB]) {
-        if (A.staged) {
+        if constexpr (TABLE) {
+            load_weights<NORB, float>(A.grad_dos + (size_t)e * NORB, NORB, r);
+            if (diff) {
+                float hi[NORB];
+                load_weights<NORB, float>(A.grad_dos + (size_t)(e + 1) * NORB, NORB, hi);
+#pragma unroll
+                for (int s = 0; s < NORB; ++s) r[s] -= hi[s];
+            }
+        } else if (A.staged) {
             load_weights<NORB, float>((diff ? sD : sG) + (size_t)e * NORB, NORB, r);
         } else {
 #pragma unroll
@@ -330,6 +339,18 @@ __global__ void __launch_bounds__(kBwdThreads, bwd_blocks(NORB)) tetra_dos_bwd_k
     }
 }
 
+// Rows G_{e-1}, e = 0 .. n_bins + 1, for more bins than the kernel stages in
+// shared memory (8 orbitals: 962); D_e is the difference of two. 64^3 points, 8
+// bands, 8 orbitals: 6.5 ms at 900 bins, staged, 6.1 ms at 1000 from these
+// rows, which the first-level cache serves; forming the values at every edge and
+// orbital, two divisions and strided loads each, took 31.7 ms.
+__global__ void tetra_dos_bwd_table(const BwdArgs A, int norb_t, float *rows) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x, e = i / norb_t, s = i - e * norb_t;
+    if (e > A.n_bins + 1) return;
+    rows[i] = s < A.n_orb && e > 0 && e <= A.n_bins
+                  ? A.grad_dos[(long)s * A.n_bins + e - 1] / (A.edges[e] - A.edges[e - 1]) : 0.f;
+}
+
 // Folds the periodic images (x = n1, y = n2, z = n3 in the padded layout) onto
 // the interior point they copy and zeroes them: one thread per (interior
 // point on a face x = 0, y = 0 or z = 0, value of its rows of both arrays),
@@ -374,7 +395,14 @@ __global__ void tetra_dos_bwd_fold(const BwdArgs A) {
 }
 
 template <int NORB>
-cudaError_t launch_bwd_n(const Plan &P, const BwdArgs &A, cudaStream_t stream) {
+cudaError_t launch_bwd_n(const Plan &P, const BwdArgs &A0, float *table, cudaStream_t stream) {
+    BwdArgs A = A0;
+    if (table) {
+        tetra_dos_bwd_table<<<((A.n_bins + 2) * NORB + 255) / 256, 256, 0, stream>>>(A, NORB, table);
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        A.grad_dos = table;
+    }
     const size_t smem = (A.staged ? bwd_stage_bytes(NORB, A.n_bins) : 0) + bwd_scratch_bytes(A.n_orb);
     auto go = [&](auto kfn) {
         cudaError_t e = cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
@@ -396,9 +424,12 @@ cudaError_t launch_bwd_n(const Plan &P, const BwdArgs &A, cudaStream_t stream) {
         return cudaGetLastError();
     };
     switch (P.d.weight_dtype) {
-        case TETRA_F16: return go(tetra_dos_bwd_kernel<NORB, __half>);
-        case TETRA_BF16: return go(tetra_dos_bwd_kernel<NORB, __nv_bfloat16>);
-        default: return go(tetra_dos_bwd_kernel<NORB, float>);
+        case TETRA_F16:
+            return table ? go(tetra_dos_bwd_kernel<NORB, __half, true>) : go(tetra_dos_bwd_kernel<NORB, __half, false>);
+        case TETRA_BF16:
+            return table ? go(tetra_dos_bwd_kernel<NORB, __nv_bfloat16, true>) : go(tetra_dos_bwd_kernel<NORB, __nv_bfloat16, false>);
+        default:
+            return table ? go(tetra_dos_bwd_kernel<NORB, float, true>) : go(tetra_dos_bwd_kernel<NORB, float, false>);
     }
 }
 
@@ -419,6 +450,11 @@ tetra_status_t launch_dos_backward(const Plan &P, const float *eps, const void *
     A.eps = eps; A.w = w; A.edges = omega; A.grad_dos = grad_dos; A.geps = grad_eps; A.gw = grad_w;
     A.vec = (reinterpret_cast<uintptr_t>(grad_w) & 15u) == 0;
     A.staged = bwd_stage_bytes(bwd_norb(A.n_orb), A.n_bins) > 0;
+    // the rows of G go behind the status words if the caller's workspace has the
+    // room (tetra_workspace_bytes has; the call takes less)
+    float *table = nullptr;
+    if (!A.staged && ws_bytes >= kStatusBytes + sizeof(float) * bwd_norb(A.n_orb) * ((size_t)A.n_bins + 2))
+        table = reinterpret_cast<float *>(static_cast<unsigned char *>(ws) + kStatusBytes);
     if (cudaMemsetAsync(ws, 0, kStatusBytes, stream) != cudaSuccess) return TETRA_ECUDA;
     // the parity classes add into the arrays: start from zero (halo and
     // padding entries stay zero)
@@ -428,11 +464,11 @@ tetra_status_t launch_dos_backward(const Plan &P, const float *eps, const void *
         return TETRA_ECUDA;
     cudaError_t e;
     switch (bwd_norb(P.d.n_orb)) {
-        case 1: e = launch_bwd_n<1>(P, A, stream); break;
-        case 2: e = launch_bwd_n<2>(P, A, stream); break;
-        case 4: e = launch_bwd_n<4>(P, A, stream); break;
-        case 8: e = launch_bwd_n<8>(P, A, stream); break;
-        default: e = launch_bwd_n<16>(P, A, stream); break;
+        case 1: e = launch_bwd_n<1>(P, A, table, stream); break;
+        case 2: e = launch_bwd_n<2>(P, A, table, stream); break;
+        case 4: e = launch_bwd_n<4>(P, A, table, stream); break;
+        case 8: e = launch_bwd_n<8>(P, A, table, stream); break;
+        default: e = launch_bwd_n<16>(P, A, table, stream); break;
     }
     return e == cudaSuccess ? TETRA_OK : TETRA_ECUDA;
 }

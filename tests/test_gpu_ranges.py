@@ -93,6 +93,26 @@ def test_fermi_level_does_not_depend_on_the_scale_of_the_weights(T, n_electrons,
     assert ex.value.status == T.TETRA_EINVAL
 
 
+@pytest.mark.parametrize("no,bins", [(1, 5600), (3, 2500), (5, 1000), (8, 963), (8, 2000), (16, 600)])
+def test_adjoint_tables_too_long_for_shared_memory(T, no, bins):
+    """More bins than the adjoint stages in shared memory: its rows in the
+    workspace, and without the room for them the values formed at every edge,
+    give the same bits."""
+    n, nb = (4, 5, 3), 2
+    eps, w = (a.astype(np.float32) for a in tbgen.synthetic_bands(29, *n, nb, no))
+    edges = tbgen.bin_edges(float(eps.min()) + 0.4, float(eps.max()) - 0.3, bins)
+    g = np.random.default_rng(6).normal(0, 1, (no, bins)).astype(np.float32)
+    plan = T.Plan(*n, nb, no, bins, mode="bin")
+    E, W = to_layout(eps, w, *n, plan.layout.eps_stride, plan.layout.w_stride)
+    Et, Wt, om, gt = (torch.from_numpy(a).cuda() for a in (E, W, edges, g))
+    ge, gw = plan.dos_backward(Et, Wt, om, gt)
+    he, hw = torch.empty_like(ge), torch.empty_like(gw)
+    ws = torch.empty(256, dtype=torch.uint8, device="cuda")
+    assert T.tetra_dos_backward(plan.handle, Et.data_ptr(), Wt.data_ptr(), om.data_ptr(), gt.data_ptr(), he.data_ptr(),
+                                hw.data_ptr(), ws.data_ptr(), 256, torch.cuda.current_stream().cuda_stream) == T.TETRA_OK
+    assert torch.equal(ge, he) and torch.equal(gw, hw)
+
+
 @pytest.mark.parametrize("mode", ["point", "bin"])
 def test_spectral_t0_units_do_not_depend_on_the_length_of_the_grid(T, mode):
     """The unit is 2^-26 of a tetrahedron over the mean spacing, whatever the
