@@ -83,6 +83,26 @@ void default_box(const tetra_desc_t &d, int box[3]) {
     box[2] = env_int("TETRA_BOX_Z", std::max(1, std::min(4, 1536 / (16 * per_cube))));
 }
 
+// Largest bound, in fixed-point units, of an item that may use the int32 tile,
+// whose blocks are flushed at 2^flush_bits: a box's items together stay below
+// 2^31 - 2^flush_bits - 2^20, and the rounding to integers is exact.
+static int fast_cap(int items_per_box, int flush_bits) {
+    const long sum = (1L << 31) - (1L << flush_bits) - (1L << 20);
+    return (int)std::min<long>(sum / items_per_box, 1L << 21);
+}
+
+// Bin and integrated mode: the bound of an item whose weights are at most one (a
+// pair of tetrahedra, or one, with its full step).
+static double unit_bound(const Plan &P) {
+    return (tetra::norb_template(P.d.n_orb) <= 8 ? 2.02 : 1.01) * std::ldexp(1.0, P.fixed_bits);
+}
+
+// Energies per k-point of a side of the grid: about how many lie in a
+// tetrahedron's window.
+static double energies_per_side(const tetra_desc_t &d, int planes) {
+    return d.n_omega / std::cbrt((double)d.n1 * d.n2 * planes);
+}
+
 // Chooses the box shape, energy chunking and grid of the forward kernel. Box
 // sides are powers of two (items are decoded with shifts), clipped to the grid.
 static tetra_status_t plan_geometry(Plan &P, const int box[3], int ctas_per_sm) {
@@ -127,19 +147,6 @@ static tetra_status_t plan_geometry(Plan &P, const int box[3], int ctas_per_sm) 
     }
     P.chunk_w = (d.n_omega + P.n_chunks - 1) / P.n_chunks;
     P.smem_bytes = fixed + per_w * P.chunk_w + 8;
-    // Bin mode: neighbouring pairs of a band tend to fall into the same bin,
-    // so a warp's tile adds hit the same addresses; up to 8 copies of the
-    // tile (as shared memory allows), one per lane residue, spread them.
-    // Each copy has its own block bounds (4 bytes per 64 energies).
-    P.tile_copies = 1;
-    if (d.mode == TETRA_BIN && pairs) {
-        const size_t copy = 4 * (size_t)P.tile_stride * (P.chunk_w + 1) + 4 * (size_t)((P.chunk_w + 63) / 64);
-        const size_t room = P.smem_optin > P.smem_bytes ? P.smem_optin - P.smem_bytes : 0;
-        P.tile_copies = (int)std::min<size_t>(8, 1 + room / copy);
-        P.smem_bytes += (size_t)(P.tile_copies - 1) * copy;
-    }
-    const int ctas = std::max(1, ctas_per_sm) * P.sm_count;
-    P.grid_x = std::max(1, std::min(P.n_boxes, (ctas + P.n_chunks - 1) / P.n_chunks));
     // Fixed-point fraction bits. A DOS value is a sum of N contributions of
     // size ~2^F / K units (K = energies per tetrahedron window), each rounded
     // with an unbiased dithered error below one unit, so its relative error is
@@ -157,21 +164,54 @@ static tetra_status_t plan_geometry(Plan &P, const int box[3], int ctas_per_sm) 
         if (d.mode == TETRA_INTEGRATED) F = 18;
         P.fixed_bits = env_int("TETRA_FIXED_BITS", F);
     }
-    // tile blocks are flushed at a bound of 2^30 (a lower value, for tests of
-    // the flush path, from TETRA_FLUSH_BITS)
-    P.flush_bits = std::max(8, std::min(30, env_int("TETRA_FLUSH_BITS", 30)));
+    // The tile's blocks are flushed at a bound of 2^30, or at 2^28 where only that
+    // keeps items of weights up to 1.15 in the tile: boxes of 3072 items in
+    // integrated mode, where weights above 0.66 went to global memory
+    // (occupation at 128^3 points, 8 bands, 1000 energies: 45 -> 5.8 ms for 8
+    // orbitals of weight one, 23.6 -> 4.5 ms for one; 4 x 4 x 4 boxes take 6.4
+    // and 4.7 ms; weights of a half pay 2 % for the flushes).
+    int flush = 30;
+    P.fast_cap = fast_cap(P.items_per_box, flush);
+    if (d.mode != TETRA_POINT && unit_bound(P) > P.fast_cap && fast_cap(P.items_per_box, 28) >= 1.15 * unit_bound(P)) {
+        flush = 28;
+        P.fast_cap = fast_cap(P.items_per_box, flush);
+    }
+    // (a lower value, for tests of the flush path, from TETRA_FLUSH_BITS)
+    P.flush_bits = std::max(8, std::min(flush, env_int("TETRA_FLUSH_BITS", 30)));
+    // Bin mode: neighbouring pairs of a band tend to fall into the same bin,
+    // so a warp's tile adds hit the same addresses; up to 8 copies of the
+    // tile (as shared memory allows), one per lane residue, spread them.
+    // Each copy has its own block bounds (4 bytes per 64 energies).
+    P.tile_copies = 1;
+    if (d.mode == TETRA_BIN && pairs) {
+        const size_t copy = 4 * (size_t)P.tile_stride * (P.chunk_w + 1) + 4 * (size_t)((P.chunk_w + 63) / 64);
+        const size_t room = P.smem_optin > P.smem_bytes ? P.smem_optin - P.smem_bytes : 0;
+        P.tile_copies = (int)std::min<size_t>(8, 1 + room / copy);
+        P.smem_bytes += (size_t)(P.tile_copies - 1) * copy;
+    }
+    const int ctas = std::max(1, ctas_per_sm) * P.sm_count;
+    P.grid_x = std::max(1, std::min(P.n_boxes, (ctas + P.n_chunks - 1) / P.n_chunks));
     return TETRA_OK;
+}
+
+// Whether box P keeps the items of box P0 in the int32 tile: in bin and
+// integrated mode those of weights up to 1.15, or all that P0 takes; in point mode
+// all, where most would be beyond a smaller cap.
+static bool keeps_items(const Plan &P, const Plan &P0) {
+    if (P.d.mode == TETRA_POINT) return P.fast_cap >= P0.fast_cap || energies_per_side(P.d, P.z1 - P.z0) >= 1.5;
+    return P.fast_cap >= std::min((double)P0.fast_cap, 1.15 * unit_bound(P));
 }
 
 // Box of a single-model plan. CTAs take boxes in rounds of grid_x, so the time
 // goes with rounds x (cubes per box + overhead of a box): a small grid wants
 // boxes that fill a round (60x60x10 points, 4x4x4 boxes: 4.4 rounds and every
 // sixth cube plane off the grid; 8x4x2: 3.9), a large one wants large boxes
-// (256^3, 200 bins: 26.3 ms with 4x4x4, 23.8 ms with 8x4x4, from which the
-// overhead of about 8 cubes; less in point mode, more in bin mode). A shape
-// may hold up to twice the default's items where the shared memory has room
-// beside the same energy tile and tile copies. The result does not depend on
-// the shape.
+// (256^3, 200 bins: 24.8 ms with 4x4x4, 22.6 ms with 2x8x8, which this takes,
+// and with 8x4x4 and 4x4x8, from which the overhead of about 8 cubes; less in
+// point mode). A shape may hold up to twice the default's items where the
+// shared memory has room beside the same energy tile and tile copies and the
+// tile still takes the items (keeps_items). The result does not depend on the
+// shape.
 static void choose_box(const Plan &P0, int box[3]) {
     if (std::getenv("TETRA_BOX_X") || std::getenv("TETRA_BOX_Y") || std::getenv("TETRA_BOX_Z")) return;
     auto cost = [](const Plan &P) {
@@ -188,7 +228,7 @@ static void choose_box(const Plan &P0, int box[3]) {
                 Plan P = P0;
                 const int b[3] = {bx, by, bz};
                 if (plan_geometry(P, b, env_int("TETRA_CTAS_PER_SM", 1)) != TETRA_OK) continue;
-                if (P.n_chunks != P0.n_chunks || P.tile_copies < P0.tile_copies) continue;
+                if (P.n_chunks != P0.n_chunks || P.tile_copies < P0.tile_copies || !keeps_items(P, P0)) continue;
                 const double c = cost(P);
                 if (c < best) {
                     best = c;

@@ -65,9 +65,7 @@ void fill_common(const Plan &P, FwdArgs &A) {
     A.split = 0;
     while (A.split < 3 && (P.items_per_box << (A.split + 1)) <= kThreads) ++A.split;
     A.flush_at = 1u << P.flush_bits;
-    long cap = ((1L << 30) - (1L << 20)) / A.items_per_box;
-    if (cap > (1L << 21)) cap = 1L << 21;
-    A.fast_cap = (int)cap;
+    A.fast_cap = P.fast_cap;
 }
 
 ModelP model_of(const Plan &P, const float *omega) {
@@ -93,10 +91,6 @@ tetra_status_t encode_maps(const Plan &P, const float *eps, const void *w, MapPa
 }
 
 }  // namespace
-
-int norb_template(int n_orb) {
-    return n_orb <= 6 ? std::max(1, n_orb) : n_orb <= 8 ? 8 : 16;
-}
 
 size_t dos_forward_workspace(const Plan &P) {
     // integrated mode: a second array of the same size for the step sums

@@ -26,6 +26,7 @@ struct tetra_plan_s {
     bool one_tile;              // all energies in one tile (batches need it)
     int grid_x;                 // persistent CTAs per energy chunk
     int fixed_bits;             // fixed-point fraction bits (see dos.cu)
+    int fast_cap;               // largest bound of an item that uses the int32 tile
     int flush_bits;             // a tile block is flushed once its bound reaches 2^flush_bits
     int items_per_box;          // work units per box: (pair, band) in point mode, (tetrahedron, band) in bin mode
     int tile_stride;            // ints per energy in the shared tile
@@ -224,7 +225,8 @@ tetra_status_t encode_point_map(CUtensorMap *map, const void *base, CUtensorMapD
                                 int elem_bytes, int stride_elems, int nx, int ny, int nz,
                                 int box_x, int box_y, int box_z);
 
-int norb_template(int n_orb);
+// Orbitals of the kernel instantiation that takes n_orb.
+inline int norb_template(int n_orb) { return n_orb < 1 ? 1 : n_orb <= 6 ? n_orb : n_orb <= 8 ? 8 : 16; }
 
 // Launchers implemented in dos.cu / eig.cu.
 tetra_status_t launch_dos_forward(const Plan &P, const float *eps, const void *w,
