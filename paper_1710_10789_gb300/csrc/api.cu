@@ -225,6 +225,8 @@ static void choose_box(const Plan &P0, int box[3]) {
         for (int by = 2; by <= 8; by *= 2)
             for (int bz = 1; bz <= 8; bz *= 2) {
                 if ((long)bx * by * bz * per_cube > most) continue;
+                // (small boxes of a grid near the largest: their count is an int)
+                if (((long)P0.d.n1 + bx - 1) / bx * ((P0.d.n2 + by - 1) / by) * ((P0.z1 - P0.z0 + bz - 1) / bz) > (1L << 30)) continue;
                 Plan P = P0;
                 const int b[3] = {bx, by, bz};
                 if (plan_geometry(P, b, env_int("TETRA_CTAS_PER_SM", 1)) != TETRA_OK) continue;

@@ -57,7 +57,7 @@ def fields(lib, n, bands, orbitals, energies, mode):
     return None if st else dict(zip(NAMES, out))
 
 
-@pytest.mark.parametrize("n", [(1, 1, 1), (60, 60, 10), (256, 256, 256), (4096, 3, 4095)])
+@pytest.mark.parametrize("n", [(1, 1, 1), (60, 60, 10), (2048, 2048, 2048), (4096, 4096, 4096), (4096, 3, 4095)])
 def test_boxes_cover_the_grid(lib, n):
     for bands, energies, mode in ((1, 400, POINT), (1, 4000, BIN), (8, 200, INTEGRATED)):
         p = fields(lib, n, bands, 1, energies, mode)
