@@ -135,10 +135,12 @@ tetra_status_t tetra_dos(tetra_plan_t plan, const float *eps, const void *w,
  *   GPU that loads the library until the process exits). The call allocates
  *   nothing. If the plan's accumulators do not fit, returns TETRA_ENOMEM; they
  *   take
- *     256 + m * 8 * n_orb * n_chunks * ceil(n_omega / n_chunks)  bytes,
+ *     256 + m * c * 8 * n_orb * n_chunks * ceil(n_omega / n_chunks)  bytes,
  *   m = 2 in TETRA_INTEGRATED mode and 1 otherwise, where n_chunks is the
  *   number of shared-memory energy tiles of the plan (1 up to about 4300
- *   energies for 8 orbitals and 8 bands in F32).
+ *   energies for 8 orbitals and 8 bands in F32) and c the number of copies of
+ *   the accumulators (up to 16 for short grids, together at most 1 MiB; 1 for
+ *   the others).
  *   Set-up: the first call on a device looks up the array's device address
  *   (cudaGetSymbolAddress) with that device current; make that first call
  *   before any stream capture. The address is kept with the device's context;

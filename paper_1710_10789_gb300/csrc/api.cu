@@ -103,6 +103,23 @@ static double energies_per_side(const tetra_desc_t &d, int planes) {
     return d.n_omega / std::cbrt((double)d.n1 * d.n2 * planes);
 }
 
+// Whether many items may be too large for the int32 tile: in point mode on a
+// grid of few energies, in integrated mode for weights above one. (In bin mode for many bins
+// only, whose adds do not collide.)
+static bool many_large(const tetra_desc_t &d, int planes) {
+    return d.mode == TETRA_INTEGRATED || (d.mode == TETRA_POINT && energies_per_side(d, planes) < 4.0);
+}
+
+// Copies of the int64 accumulator, over which the adds of such items spread: up
+// to 16 that together have at most 2^17 entries and few for the work (the CTA
+// that finishes last adds them up).
+static int accumulator_copies(const Plan &P) {
+    if (P.n_chunks > 1 || !many_large(P.d, P.z1 - P.z0)) return 1;
+    const long entries = (long)P.d.n_orb * P.chunk_w * (P.d.mode == TETRA_INTEGRATED ? 2 : 1);
+    const long work = (long)P.n_boxes * P.items_per_box / 256;
+    return (int)std::max(1L, std::min<long>(kMaxCopies, std::min(1L << 17, work) / entries));
+}
+
 // Chooses the box shape, energy chunking and grid of the forward kernel. Box
 // sides are powers of two (items are decoded with shifts), clipped to the grid.
 static tetra_status_t plan_geometry(Plan &P, const int box[3], int ctas_per_sm) {
@@ -191,6 +208,7 @@ static tetra_status_t plan_geometry(Plan &P, const int box[3], int ctas_per_sm) 
     }
     const int ctas = std::max(1, ctas_per_sm) * P.sm_count;
     P.grid_x = std::max(1, std::min(P.n_boxes, (ctas + P.n_chunks - 1) / P.n_chunks));
+    P.copies = accumulator_copies(P);
     return TETRA_OK;
 }
 
@@ -434,6 +452,11 @@ tetra_status_t tetra_plan_batched(tetra_batch_plan_t *plan, const tetra_desc_t *
         if (total > (1L << 30)) return fail(TETRA_EUNSUPPORTED);
     }
     B->total_boxes = (int)total;
+    // copies of the accumulators if a model has many large items, up to 32 MB
+    bool large = false;
+    for (int m = 0; m < n_models; ++m) large = large || tetra::many_large(descs[m], B->models[m].z1 - B->models[m].z0);
+    const long entries = (long)n_models * d0.n_orb * B->chunk_w;
+    B->copies = large ? (int)std::max(1L, std::min<long>(tetra::kMaxCopies, (4L << 20) / entries)) : 1;
     B->grid_x = (int)std::max<long>(1, std::min<long>(total, (long)ctas_per_sm * Pb.sm_count));
     *plan = B;
     return TETRA_OK;

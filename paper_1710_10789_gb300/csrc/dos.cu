@@ -6,14 +6,16 @@ namespace tetra {
 
 namespace fwd {
 
-#define TETRA_FWD_EXTERN(MODE, MAXM)                                                                          \
-    extern template cudaError_t launch_norb<MODE, MAXM>(int, int, size_t, dim3, const Batch<MAXM> &, const FwdArgs &, \
-                                                        cudaStream_t);
-TETRA_FWD_EXTERN(TETRA_POINT, 1)
-TETRA_FWD_EXTERN(TETRA_BIN, 1)
-TETRA_FWD_EXTERN(TETRA_INTEGRATED, 1)
-TETRA_FWD_EXTERN(TETRA_POINT, kMaxBatch)
-TETRA_FWD_EXTERN(TETRA_BIN, kMaxBatch)
+#define TETRA_FWD_EXTERN(MODE, MAXM, COPIES)                                                                           \
+    extern template cudaError_t launch_norb<MODE, MAXM, COPIES>(int, int, size_t, dim3, const Batch<MAXM> &,              \
+                                                                const FwdArgs &, cudaStream_t);
+TETRA_FWD_EXTERN(TETRA_POINT, 1, false)
+TETRA_FWD_EXTERN(TETRA_POINT, 1, true)
+TETRA_FWD_EXTERN(TETRA_BIN, 1, false)
+TETRA_FWD_EXTERN(TETRA_INTEGRATED, 1, true)
+TETRA_FWD_EXTERN(TETRA_POINT, kMaxBatch, false)
+TETRA_FWD_EXTERN(TETRA_POINT, kMaxBatch, true)
+TETRA_FWD_EXTERN(TETRA_BIN, kMaxBatch, false)
 #undef TETRA_FWD_EXTERN
 
 }  // namespace fwd
@@ -27,7 +29,7 @@ struct BatchOut {
     float *dos[kMaxBatch];
 };
 __global__ void tetra_dos_reduce_batched(const __grid_constant__ Batch<kMaxBatch> B, const BatchOut O,
-                                         const long long *G, int n_orb, int chunk_w, int mode) {
+                                         const long long *G, int copies, int n_orb, int chunk_w, int mode) {
     const ModelP &M = B.m[blockIdx.y];
     __shared__ float s_unit[2];
     if (threadIdx.x == 0) {
@@ -40,7 +42,8 @@ __global__ void tetra_dos_reduce_batched(const __grid_constant__ Batch<kMaxBatch
     for (long idx = blockIdx.x * (long)blockDim.x + threadIdx.x; idx < total;
          idx += (long)gridDim.x * blockDim.x) {
         const int s = (int)(idx / M.n_omega), i = (int)(idx - (long)s * M.n_omega);
-        const long long g = G[((long)blockIdx.y * n_orb + s) * chunk_w + i];
+        long long g = 0;
+        for (int r = 0; r < copies; ++r) g += G[(((long)blockIdx.y * copies + r) * n_orb + s) * chunk_w + i];
         O.dos[blockIdx.y][idx] = scale_units(g, uh, ul);
     }
 }
@@ -74,6 +77,7 @@ ModelP model_of(const Plan &P, const float *omega) {
     m.nbx = P.nbx; m.nby = P.nby; m.n_boxes = P.n_boxes; m.n_omega = P.d.n_omega;
     m.fixed_bits = P.fixed_bits;
     m.box_base = 0;
+    m.copies = P.copies;
     m.vtvg = 1.0 / (6.0 * (double)P.d.n1 * (double)P.d.n2 * (double)P.d.n3);
     m.omega = omega;
     return m;
@@ -94,7 +98,7 @@ tetra_status_t encode_maps(const Plan &P, const float *eps, const void *w, MapPa
 
 size_t dos_forward_workspace(const Plan &P) {
     // integrated mode: a second array of the same size for the step sums
-    const size_t parts = sizeof(long long) * (size_t)P.n_chunks * P.d.n_orb * (size_t)P.chunk_w;
+    const size_t parts = sizeof(long long) * (size_t)P.n_chunks * P.copies * P.d.n_orb * (size_t)P.chunk_w;
     return kStatusBytes + (P.d.mode == TETRA_INTEGRATED ? 2 : 1) * parts;
 }
 
@@ -114,22 +118,26 @@ tetra_status_t launch_dos_forward(const Plan &P, const float *eps, const void *w
     A.status = reinterpret_cast<int *>(ws);
     A.queue = nullptr;
     A.G = reinterpret_cast<long long *>(static_cast<unsigned char *>(ws) + kStatusBytes);
-    A.Gs = A.G + (size_t)P.n_chunks * P.d.n_orb * (size_t)P.chunk_w;
+    A.Gs = A.G + (size_t)P.n_chunks * P.copies * P.d.n_orb * (size_t)P.chunk_w;
     A.done = reinterpret_cast<int *>(static_cast<unsigned char *>(ws) + kDoneOffset);
     A.dos = dos;
     cudaError_t e = cudaMemsetAsync(ws, 0, need, stream);
     if (e != cudaSuccess) return TETRA_ECUDA;
     const dim3 grid(P.grid_x, P.n_chunks);
-    const int mode = P.d.mode;
-    e = mode == TETRA_POINT ? launch_norb<TETRA_POINT, 1>(P.d.n_orb, P.d.weight_dtype, P.smem_bytes, grid, Bt, A, stream)
-        : mode == TETRA_BIN ? launch_norb<TETRA_BIN, 1>(P.d.n_orb, P.d.weight_dtype, P.smem_bytes, grid, Bt, A, stream)
-                            : launch_norb<TETRA_INTEGRATED, 1>(P.d.n_orb, P.d.weight_dtype, P.smem_bytes, grid, Bt,
-                                                               A, stream);
+    const int n_orb = P.d.n_orb, wdt = P.d.weight_dtype;
+    switch (P.d.mode) {
+        case TETRA_POINT:
+            e = P.copies > 1 ? launch_norb<TETRA_POINT, 1, true>(n_orb, wdt, P.smem_bytes, grid, Bt, A, stream)
+                             : launch_norb<TETRA_POINT, 1, false>(n_orb, wdt, P.smem_bytes, grid, Bt, A, stream);
+            break;
+        case TETRA_BIN: e = launch_norb<TETRA_BIN, 1, false>(n_orb, wdt, P.smem_bytes, grid, Bt, A, stream); break;
+        default: e = launch_norb<TETRA_INTEGRATED, 1, true>(n_orb, wdt, P.smem_bytes, grid, Bt, A, stream);
+    }
     return e == cudaSuccess ? TETRA_OK : TETRA_ECUDA;
 }
 
 size_t dos_batched_workspace(const BatchPlan &B) {
-    return kStatusBytes + sizeof(long long) * (size_t)B.n_models * B.models[0].d.n_orb * (size_t)B.chunk_w;
+    return kStatusBytes + sizeof(long long) * (size_t)B.n_models * B.copies * B.models[0].d.n_orb * (size_t)B.chunk_w;
 }
 
 tetra_status_t launch_dos_batched(const BatchPlan &BP, const float *const *eps, const void *const *w,
@@ -148,6 +156,7 @@ tetra_status_t launch_dos_batched(const BatchPlan &BP, const float *const *eps, 
         if (st != TETRA_OK) return st;
         ModelP mp = model_of(P, omega[m]);
         mp.box_base = BP.box_base[m];
+        mp.copies = BP.copies;
         Bt->m[m] = mp;
         O->dos[m] = dos[m];
     }
@@ -165,14 +174,14 @@ tetra_status_t launch_dos_batched(const BatchPlan &BP, const float *const *eps, 
     if (e != cudaSuccess) return TETRA_ECUDA;
     const dim3 grid(BP.grid_x, 1);
     const int n_orb = P0.d.n_orb, wdt = P0.d.weight_dtype;
-    e = (P0.d.mode == TETRA_POINT)
-            ? launch_norb<TETRA_POINT, kMaxBatch>(n_orb, wdt, BP.smem_bytes, grid, *Bt, A, stream)
-            : launch_norb<TETRA_BIN, kMaxBatch>(n_orb, wdt, BP.smem_bytes, grid, *Bt, A, stream);
+    e = P0.d.mode == TETRA_BIN ? launch_norb<TETRA_BIN, kMaxBatch, false>(n_orb, wdt, BP.smem_bytes, grid, *Bt, A, stream)
+        : BP.copies > 1        ? launch_norb<TETRA_POINT, kMaxBatch, true>(n_orb, wdt, BP.smem_bytes, grid, *Bt, A, stream)
+                               : launch_norb<TETRA_POINT, kMaxBatch, false>(n_orb, wdt, BP.smem_bytes, grid, *Bt, A, stream);
     if (e != cudaSuccess) return TETRA_ECUDA;
     const long total = (long)n_orb * BP.chunk_w;
     const int rb = 256;
     const int rg = (int)std::max<long>(1, std::min<long>((total + rb - 1) / rb, 64));
-    tetra_dos_reduce_batched<<<dim3(rg, BP.n_models), rb, 0, stream>>>(*Bt, *O, A.G, n_orb,
+    tetra_dos_reduce_batched<<<dim3(rg, BP.n_models), rb, 0, stream>>>(*Bt, *O, A.G, BP.copies, n_orb,
                                                                         BP.chunk_w, P0.d.mode);
     if (cudaGetLastError() != cudaSuccess) return TETRA_ECUDA;
     return TETRA_OK;

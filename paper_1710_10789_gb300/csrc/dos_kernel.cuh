@@ -42,12 +42,20 @@
 //    flushed.
 //  * A per-item bound q_max (|b| <= Bmax of the box, and the tetrahedron DOS
 //    is at most 3/E41 of V_T/V_G) decides between this fast path and a 64-bit
-//    global integer path for rare near-flat tetrahedra. The sum of q_max over
-//    processed items bounds every tile entry; the tile is flushed into the
-//    int64 accumulator in global memory before it could overflow.
+//    global integer path for tetrahedra flat on the scale of the grid: few on a
+//    fine grid, many where the grid has about as many energies as points a
+//    side. The sum of q_max over processed items bounds every tile entry; the
+//    tile is flushed into the int64 accumulator in global memory before it
+//    could overflow.
 //  * The CTAs flush into one int64 accumulator (integer atomics: exact, any
 //    order); the CTA that finishes last scales it by u. For a batch a second
-//    kernel scales each model's accumulator.
+//    kernel scales each model's accumulator. Where the global path may take
+//    many items of few energies (COPIES), all CTAs would add to the same few
+//    addresses: the accumulator has up to 16 copies that they take in turn
+//    (8 bands, one orbital of weight one: 64^3 points, 128 energies 0.99 ->
+//    0.33 ms, 128^3, 256 energies 5.2 -> 2.4 ms). A kernel of its own, because
+//    the code of the others' walks suffers from the few instructions more
+//    (64^3 points, 8 orbitals, 2000 energies: 1.59 -> 1.67 ms).
 //
 // The instantiations of a mode are compiled in a file of their own
 // (dos_point.cu, ...), so that they build in parallel.
@@ -118,7 +126,7 @@ struct FwdArgs {
     int split;           // log2 of the lanes that share a pair's walk (point and integrated mode)
     int fast_cap;
     unsigned flush_at;   // a 64-energy block is flushed once its bound reaches this
-    long long *G;        // int64 accumulators, [slot][n_orb][chunk_w]; slot = chunk, or model of a batch
+    long long *G;        // int64 accumulators, [slot][copy][n_orb][chunk_w]; slot = chunk, or model of a batch
     long long *Gs;       // integrated mode: int64 accumulators of the step sums, the same shape
     int *status;
     int *queue;          // batched: next unclaimed (model, box) work item
@@ -284,6 +292,7 @@ struct ModelP {
     int n1, n2, n3, z0, z1, nbx, nby, n_boxes, n_omega;
     int fixed_bits;
     int box_base;    // first global work index of the model (batched launches)
+    int copies;      // copies of its accumulator (COPIES): CTA b adds into copy b % copies
     double vtvg;
     const float *omega;
 };
@@ -301,7 +310,7 @@ struct Batch {
     int total_work;   // batched: (model, box) items of the launch
 };
 
-template <int NORB, typename WT, int MODE, int MAXM>
+template <int NORB, typename WT, int MODE, int MAXM, bool COPIES>
 __global__ void __maxnreg__(kMaxRegs)
     tetra_dos_fwd_kernel(const __grid_constant__ Batch<MAXM> B, const FwdArgs A) {
     // tile row: NORB orbitals, and the row's add count (differences) behind
@@ -542,7 +551,8 @@ __global__ void __maxnreg__(kMaxRegs)
             wc = min(A.chunk_w, M.n_omega - w0);
             // accumulator: one per energy chunk of a single model, one per model
             // of a batch (CTAs flush into it with integer atomics)
-            const long slot = (MAXM == 1) ? (long)chunk : (long)mi;
+            long slot = (MAXM == 1) ? (long)chunk : (long)mi;
+            if constexpr (COPIES) slot = slot * M.copies + blockIdx.x % M.copies;
             Gc = A.G + slot * (long)A.n_orb * A.chunk_w;
             if (MODE == TETRA_INTEGRATED) Gsc = A.Gs + slot * (long)A.n_orb * A.chunk_w;
             for (int i = tid; i < copy_ints * n_copies; i += blockDim.x) tile[i] = 0;
@@ -1290,17 +1300,26 @@ __global__ void __maxnreg__(kMaxRegs)
         const float uh = s_unit[0], ul = s_unit[1];   // (every CTA has a box)
         for (int c = group; c < (int)gridDim.y; c += kDoneGroups) {
             const int f0 = c * A.chunk_w, fn = min(A.chunk_w, M.n_omega - f0);
-            const long long *G = A.G + (long)c * A.n_orb * A.chunk_w;
+            const long copy = (long)A.n_orb * A.chunk_w;
+            const int copies = COPIES ? M.copies : 1;
+            const long long *G = A.G + (long)c * copies * copy;
+            // an entry summed over the copies
+            auto total = [&](const long long *g) {
+                long long v = __ldcg(g);
+                if constexpr (COPIES)
+                    for (int r = 1; r < copies; ++r) v += __ldcg(g + r * copy);
+                return v;
+            };
             if constexpr (MODE == TETRA_INTEGRATED) {
                 // running sum of the chunk's steps (a chunk's first energy holds the
                 // steps of every tetrahedron below the chunk): one warp per orbital,
                 // in the shared memory of the two tiles
-                const long long *Gs = A.Gs + (long)c * A.n_orb * A.chunk_w;
+                const long long *Gs = A.Gs + (long)c * copies * copy;
                 long long *buf = reinterpret_cast<long long *>(tile);
                 __syncthreads();
                 for (int i = tid; i < A.n_orb * fn; i += blockDim.x) {
                     const int s = i / fn;
-                    buf[i] = __ldcg(Gs + (long)s * A.chunk_w + (i - s * fn));
+                    buf[i] = total(Gs + (long)s * A.chunk_w + (i - s * fn));
                 }
                 __syncthreads();
                 const int lane = tid & 31;
@@ -1323,7 +1342,7 @@ __global__ void __maxnreg__(kMaxRegs)
             }
             for (int i = tid; i < A.n_orb * fn; i += blockDim.x) {
                 const int s = i / fn, j = i - s * fn;
-                long long v = __ldcg(G + (long)s * A.chunk_w + j);
+                long long v = total(G + (long)s * A.chunk_w + j);
                 if (MODE == TETRA_INTEGRATED) v += reinterpret_cast<const long long *>(tile)[i];
                 A.dos[(long)s * M.n_omega + f0 + j] = scale_units(v, uh, ul);
             }
@@ -1331,10 +1350,10 @@ __global__ void __maxnreg__(kMaxRegs)
     }
 }
 
-template <int NORB, typename WT, int MODE, int MAXM>
+template <int NORB, typename WT, int MODE, int MAXM, bool COPIES>
 cudaError_t launch_t(size_t smem, dim3 grid, const Batch<MAXM> &Bt, const FwdArgs &A,
                      cudaStream_t stream) {
-    auto k = tetra_dos_fwd_kernel<NORB, WT, MODE, MAXM>;
+    auto k = tetra_dos_fwd_kernel<NORB, WT, MODE, MAXM, COPIES>;
     // The shared-memory opt-in is set once per device and size, so that a
     // launch inside a CUDA-graph capture makes no attribute call.
     static std::atomic<int> opted[64];
@@ -1360,28 +1379,28 @@ cudaError_t launch_t(size_t smem, dim3 grid, const Batch<MAXM> &Bt, const FwdArg
     return cudaGetLastError();
 }
 
-template <int NORB, int MODE, int MAXM>
+template <int NORB, int MODE, int MAXM, bool COPIES>
 cudaError_t launch_wt(int wdtype, size_t smem, dim3 grid, const Batch<MAXM> &Bt, const FwdArgs &A,
                       cudaStream_t stream) {
     switch (wdtype) {
-        case TETRA_F16: return launch_t<NORB, __half, MODE, MAXM>(smem, grid, Bt, A, stream);
-        case TETRA_BF16: return launch_t<NORB, __nv_bfloat16, MODE, MAXM>(smem, grid, Bt, A, stream);
-        default: return launch_t<NORB, float, MODE, MAXM>(smem, grid, Bt, A, stream);
+        case TETRA_F16: return launch_t<NORB, __half, MODE, MAXM, COPIES>(smem, grid, Bt, A, stream);
+        case TETRA_BF16: return launch_t<NORB, __nv_bfloat16, MODE, MAXM, COPIES>(smem, grid, Bt, A, stream);
+        default: return launch_t<NORB, float, MODE, MAXM, COPIES>(smem, grid, Bt, A, stream);
     }
 }
 
-template <int MODE, int MAXM>
+template <int MODE, int MAXM, bool COPIES>
 cudaError_t launch_norb(int n_orb, int wdtype, size_t smem, dim3 grid, const Batch<MAXM> &Bt,
                         const FwdArgs &A, cudaStream_t stream) {
     switch (norb_template(n_orb)) {
-        case 1: return launch_wt<1, MODE, MAXM>(wdtype, smem, grid, Bt, A, stream);
-        case 2: return launch_wt<2, MODE, MAXM>(wdtype, smem, grid, Bt, A, stream);
-        case 3: return launch_wt<3, MODE, MAXM>(wdtype, smem, grid, Bt, A, stream);
-        case 4: return launch_wt<4, MODE, MAXM>(wdtype, smem, grid, Bt, A, stream);
-        case 5: return launch_wt<5, MODE, MAXM>(wdtype, smem, grid, Bt, A, stream);
-        case 6: return launch_wt<6, MODE, MAXM>(wdtype, smem, grid, Bt, A, stream);
-        case 8: return launch_wt<8, MODE, MAXM>(wdtype, smem, grid, Bt, A, stream);
-        default: return launch_wt<16, MODE, MAXM>(wdtype, smem, grid, Bt, A, stream);
+        case 1: return launch_wt<1, MODE, MAXM, COPIES>(wdtype, smem, grid, Bt, A, stream);
+        case 2: return launch_wt<2, MODE, MAXM, COPIES>(wdtype, smem, grid, Bt, A, stream);
+        case 3: return launch_wt<3, MODE, MAXM, COPIES>(wdtype, smem, grid, Bt, A, stream);
+        case 4: return launch_wt<4, MODE, MAXM, COPIES>(wdtype, smem, grid, Bt, A, stream);
+        case 5: return launch_wt<5, MODE, MAXM, COPIES>(wdtype, smem, grid, Bt, A, stream);
+        case 6: return launch_wt<6, MODE, MAXM, COPIES>(wdtype, smem, grid, Bt, A, stream);
+        case 8: return launch_wt<8, MODE, MAXM, COPIES>(wdtype, smem, grid, Bt, A, stream);
+        default: return launch_wt<16, MODE, MAXM, COPIES>(wdtype, smem, grid, Bt, A, stream);
     }
 }
 

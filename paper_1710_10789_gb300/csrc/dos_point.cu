@@ -3,6 +3,6 @@
 
 namespace tetra {
 namespace fwd {
-template cudaError_t launch_norb<TETRA_POINT, 1>(int, int, size_t, dim3, const Batch<1> &, const FwdArgs &, cudaStream_t);
+template cudaError_t launch_norb<TETRA_POINT, 1, false>(int, int, size_t, dim3, const Batch<1> &, const FwdArgs &, cudaStream_t);
 }  // namespace fwd
 }  // namespace tetra

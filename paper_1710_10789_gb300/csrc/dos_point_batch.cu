@@ -1,8 +1,8 @@
-// Forward kernel: point mode, batched.
+// Forward kernel: point mode, batches.
 #include "dos_kernel.cuh"
 
 namespace tetra {
 namespace fwd {
-template cudaError_t launch_norb<TETRA_POINT, kMaxBatch>(int, int, size_t, dim3, const Batch<kMaxBatch> &, const FwdArgs &, cudaStream_t);
+template cudaError_t launch_norb<TETRA_POINT, kMaxBatch, false>(int, int, size_t, dim3, const Batch<kMaxBatch> &, const FwdArgs &, cudaStream_t);
 }  // namespace fwd
 }  // namespace tetra

@@ -31,6 +31,7 @@ struct tetra_plan_s {
     int items_per_box;          // work units per box: (pair, band) in point mode, (tetrahedron, band) in bin mode
     int tile_stride;            // ints per energy in the shared tile
     int tile_copies;            // copies of the tile (bin mode: lanes spread over them)
+    int copies;                 // copies of the int64 accumulator
     size_t smem_bytes;
 };
 
@@ -39,6 +40,7 @@ struct tetra_plan_s {
 // CTAs take (model, box) work items from a global counter at run time.
 namespace tetra {
 constexpr int kMaxBatch = 64;
+constexpr int kMaxCopies = 16;   // of an int64 accumulator
 }  // namespace tetra
 struct tetra_batch_plan_s {
     int n_models;
@@ -46,6 +48,7 @@ struct tetra_batch_plan_s {
     tetra_plan_s models[tetra::kMaxBatch];   // common box shape, one energy chunk each
     int big;                                 // model with the most energies
     int chunk_w;                             // energies per shared tile (= max n_omega)
+    int copies;                              // copies of each int64 accumulator
     size_t smem_bytes;
     int grid_x;                              // persistent CTAs
     int total_boxes;                         // work items of the whole batch

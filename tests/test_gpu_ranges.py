@@ -113,6 +113,39 @@ def test_adjoint_tables_too_long_for_shared_memory(T, no, bins):
     assert torch.equal(ge, he) and torch.equal(gw, hw)
 
 
+@pytest.mark.parametrize("mode", ["point", "bin", "integrated"])
+@pytest.mark.parametrize("no", [1, 3, 8, 16])
+def test_large_contributions(T, mode, no, monkeypatch):
+    """Contributions beyond the 32-bit tile's bound: weights up to 40 and a
+    narrow band, on a coarse energy grid (several copies of the accumulator)
+    and on a long one (one). The same bits with a small FLUSH_BITS and other
+    boxes, and the oracle within 2e-5 of the largest value."""
+    n, nb = (9, 8, 7), 3
+    eps, w = (a.astype(np.float32) for a in tbgen.synthetic_bands(41, *n, nb, no))
+    w *= 40.0
+    eps[:, 0] = eps[:, 0].min() + 1e-3 * (eps[:, 0] - eps[:, 0].min())
+    lo, hi = float(eps.min()) - 0.3, float(eps.max()) + 0.3
+    for ne in (9, 12000 // (no + 2)):
+        om = tbgen.uniform_grid(lo, hi, ne + (mode == "bin"))
+        omt = torch.from_numpy(om).cuda()
+
+        def run():
+            plan = T.Plan(*n, nb, no, ne, mode=mode)
+            E, W = to_layout(eps, w, *n, plan.layout.eps_stride, plan.layout.w_stride)
+            out = plan.dos(torch.from_numpy(E).cuda(), torch.from_numpy(W).cuda(), omt)
+            assert plan.status() == T.TETRA_OK
+            return out
+
+        out = run()
+        r = oracle.dos(eps, w, *n, om.astype(np.float64), mode=mode)
+        assert np.max(np.abs(out.cpu().numpy() - r)) <= 2e-5 * np.max(np.abs(r))
+        for key, value in (("TETRA_FLUSH_BITS", "10"), ("TETRA_BOX_X", "2"), ("TETRA_BOX_Z", "1")):
+            monkeypatch.setenv(key, value)
+            assert torch.equal(run(), out), key
+        for key in ("TETRA_FLUSH_BITS", "TETRA_BOX_X", "TETRA_BOX_Z"):
+            monkeypatch.delenv(key)
+
+
 @pytest.mark.parametrize("mode", ["point", "bin"])
 def test_spectral_t0_units_do_not_depend_on_the_length_of_the_grid(T, mode):
     """The unit is 2^-26 of a tetrahedron over the mean spacing, whatever the

@@ -28,13 +28,13 @@ extern "C" int plan_fields(const int *desc, long *out) {
     const int st = tetra_plan(&p, reinterpret_cast<const tetra_desc_t *>(desc), 0);
     if (st) return st;
     const long v[] = {p->BX, p->BY, p->BZ, p->n_boxes, p->nbx, p->nby, p->nbz, p->grid_x, p->items_per_box, p->fixed_bits,
-                      p->fast_cap, p->flush_bits, p->n_chunks, p->chunk_w, (long)p->smem_bytes};
+                      p->fast_cap, p->flush_bits, p->copies, p->n_chunks, p->chunk_w, (long)p->smem_bytes};
     for (unsigned i = 0; i < sizeof v / sizeof *v; ++i) out[i] = v[i];
     return tetra_plan_destroy(p);
 }
 extern "C" int drop(float wmax, double cells) { return tetra::fermi_drop(wmax, cells); }
 """
-NAMES = "BX BY BZ n_boxes nbx nby nbz grid items bits cap flush chunks width smem".split()
+NAMES = "BX BY BZ n_boxes nbx nby nbz grid items bits cap flush copies chunks width smem".split()
 POINT, BIN, INTEGRATED = 0, 1, 2
 
 
@@ -85,7 +85,7 @@ def test_larger_boxes_keep_unit_weights_in_the_tile(lib, monkeypatch):
         assert p["bits"] == base["bits"]
         assert p["cap"] >= unit or base["cap"] < unit, (side, bands, orbitals, energies, mode, p, base)
         assert p["cap"] * p["items"] + 2 ** p["flush"] < 2 ** 31 and p["cap"] <= 2 ** 21
-        assert p["smem"] <= 232448
+        assert p["smem"] <= 232448 and 1 <= p["copies"] <= 16
 
 
 def test_fermi_unit(lib):
