@@ -164,3 +164,13 @@ def test_spectral_t0_units_do_not_depend_on_the_length_of_the_grid(T, mode):
         part = plan.spectral_t0(Et, q, mu, om[a:b + bins].clone(), mode=mode)
         assert plan.spectral_status() == T.TETRA_OK
         assert torch.equal(part, whole[a:b]) and whole[a:b].any(), (a, b)
+
+
+def test_one_point_has_no_density_of_states(T):
+    """A grid of one point: flat bands, a delta that point mode leaves out."""
+    plan = T.Plan(1, 1, 1, 2, 3, 5)
+    E, W = plan.empty_inputs()
+    E[..., :2] = torch.tensor([-0.25, 0.5], device="cuda")
+    W += 0.5
+    om = torch.tensor([-1.0, -0.25, 0.0, 0.5, 1.0], device="cuda")
+    assert not plan.dos(E, W, om).any()
