@@ -46,8 +46,8 @@ OPS_PER_ITEM = 40
 # hex digits of the SHA-256 of csrc/dos_kernel.cuh and csrc/tet_common.cuh (the
 # forward kernel and the device functions it calls); otherwise the bench
 # reports null.
-DOS_TRAFFIC_CAPTURE = {"dos_fwd_sha256": "1e00607290971754", "grid": 128, "n_omega": 4000,
-                       "bytes": 653975040 + 4716800}
+DOS_TRAFFIC_CAPTURE = {"dos_fwd_sha256": "82f91e8f7a5ddc16", "grid": 128, "n_omega": 4000,
+                       "bytes": 653802752 + 4445440}
 
 
 def parse():

@@ -20,9 +20,10 @@
 // cube's N(E) - N(lo) is rounded once to an integer of 2^-26 of a full
 // tetrahedron, summed over the warp by two 32-bit reductions, over the
 // block's warps and over the grid by integer adds: exact in any order. Weights
-// so large that the 64-bit sums could wrap (above about 20 a band at 1024^3
-// points, 10^6 on a small grid) are scaled down by a power of two: the first
-// round, which stages every weight, finds the largest and is then repeated.
+// so large that the 64-bit sums could wrap (corner sums above 1.3 at 1024^3
+// points and 8 bands, 7 10^5 on a small grid) are scaled down by a power of
+// two: the first round, which stages every weight, finds the largest and is
+// then repeated.
 //
 // At 95 x 97 x 96 points, 8 bands and 8 orbitals the five rounds of the
 // integrated-mode DOS kernel before (64 energies, every orbital, every
