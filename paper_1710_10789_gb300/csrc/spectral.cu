@@ -246,7 +246,13 @@ __device__ __forceinline__ void spec_setup(const SubTet &Q, const SpecArgs &S, S
 
 // Its contribution to energy (bin) i, before rounding.
 __device__ __forceinline__ float spec_value(const SpecTet &T, const float *om, bool bin, int i) {
-    if (bin) return fmaf(T.amp, __fdividef(spec_below(T, om[i + 1]) - spec_below(T, om[i]), om[i + 1] - om[i]), T.dith);
+    if (bin) {
+        // the quotient with its residual added once: the approximate reciprocal's
+        // error is the same for all items of a bin
+        const float width = om[i + 1] - om[i], r = __fdividef(1.f, width);
+        const float step = spec_below(T, om[i + 1]) - spec_below(T, om[i]), v = step * r;
+        return fmaf(T.amp, fmaf(fmaf(-width, v, step), r, v), T.dith);
+    }
     return fmaf(T.amp, spec_density(T, om[i]), T.dith);
 }
 

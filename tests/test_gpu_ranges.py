@@ -174,3 +174,25 @@ def test_one_point_has_no_density_of_states(T):
     W += 0.5
     om = torch.tensor([-1.0, -0.25, 0.0, 0.5, 1.0], device="cuda")
     assert not plan.dos(E, W, om).any()
+
+
+def test_spectral_t0_average_over_one_wide_bin(T):
+    """A bin that holds every transition: the average is their total over its
+    width, the same factor for all items, so that an error of the quotient does
+    not average out. Two roundings of 2^-24 (quotient, result) and 6e-9 for the
+    items' own, which do."""
+    n, q = (10, 9, 8), (3, 1, 0)
+    _, eps, _ = tb_problem(3, n)
+    mu, span = float(np.median(eps)), float(eps.max() - eps.min())
+    plan = T.Plan(*n, eps.shape[1], 1, 16)
+    E, _ = to_layout(eps, np.zeros(eps.shape + (1,), np.float32), *n, plan.layout.eps_stride, plan.layout.w_stride)
+    Et = torch.from_numpy(E).cuda()
+    total = oracle.spectral_t0(eps.astype(np.float64), *n, q, mu, np.array([0.0, 64.0]), mode="bin")[0] * 64.0
+    widths = (span + np.random.default_rng(8).uniform(0.1, 20.0, 64)).astype(np.float32)
+    worst = 0.0
+    for width in widths:
+        om = torch.tensor([0.0, float(width)], device="cuda")
+        g = float(plan.spectral_t0(Et, q, mu, om, mode="bin")[0])
+        worst = max(worst, abs(g * float(width) / total - 1.0))
+    print(f"{worst:.2e}")
+    assert worst <= 2.0 ** -23 + 6e-9
